@@ -71,7 +71,11 @@ extern "C" {
 #define CLS_OPT_BLOCK 3         /* threads per block, multiple of 32 in [32, 256]; the FP64
                                    history tracker uses at most 128, the FP32 history tracker
                                    for the 3D box at most 224 (their launch bounds)          */
-#define CLS_OPT_CHUNK 4         /* histories a warp claims at once: 32, 64, ..., 1024       */
+#define CLS_OPT_CHUNK 4         /* histories a warp claims at once: 32, 64, ..., 1024.  The  */
+                                /* history tracker claims at most 32 times as many while a  */
+                                /* run is long, and fewer (down to 32, or to 1 in runs too   */
+                                /* small to go round) as it ends; the event tracker exactly  */
+                                /* this many                                                */
 #define CLS_OPT_NBATCH 5        /* statistics batches per run, 2..1024 (default 64)         */
 #define CLS_OPT_MAX_EVENTS 6    /* per-history event cap, 1..2^28 (default 1e8)             */
 #define CLS_OPT_BLOCKS_PER_SM 7 /* persistent grid = SMs x this; 0 = occupancy maximum     */
@@ -409,7 +413,7 @@ int cls_debug_fixed32(const float *c, int n, unsigned long long *out);
  * options; per-history event cap 1e8).  The call is asynchronous, so it cannot
  * report capped histories as CLS_E_EVENT_LIMIT: they show in d_counters[k][7].
  *
- * Scratch (case parameters, work list, work counter; about 16 KB) lives in a
+ * Scratch (case parameters, work list, work counters; about 48 KB) lives in a
  * static device array that every GPU loading the library holds until the
  * process exits.  The first call on each device looks up that array's device
  * address (with the device current) and keeps it for the life of the process;

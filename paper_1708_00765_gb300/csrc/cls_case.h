@@ -44,6 +44,42 @@ inline double cost_estimate(const CaseParams &c) {
     return 1.0 + rate * path;
 }
 
+// How a history-tracker launch of n histories in each of `nruns` run entries is
+// claimed by about `warps` warps (LaunchArgs): pieces of whole statistics
+// batches, at most max_pieces of them; as many warps start on a piece as it
+// takes to employ all; and the least a warp claims is 32 histories, a warp's
+// lanes, or where that would not go round, a power of two below.
+inline void plan_pieces(LaunchArgs &a, uint64_t n, uint64_t batch_len, uint64_t warps, uint64_t max_pieces) {
+    const uint64_t used = (n + batch_len - 1) / batch_len;  // batches
+    const uint64_t per_run = std::max<uint64_t>(1, std::min<uint64_t>(std::min<uint64_t>(used, 64), max_pieces / a.nruns));
+    const uint64_t batches = (used + per_run - 1) / per_run;
+    a.piece_len = batches * batch_len;
+    a.pieces_per_run = (uint32_t)((used + batches - 1) / batches);
+    const uint64_t pieces = (uint64_t)a.pieces_per_run * a.nruns;
+    a.team = (uint32_t)((warps + pieces - 1) / pieces);
+    const double per_warp = (double)n * a.nruns / (double)warps;
+    a.chunk = 32;
+    while (a.chunk > 1 && (double)a.chunk > per_warp) a.chunk >>= 1;
+}
+
+// Claim limit and refill threshold of a run entry (RunCase), from the
+// estimated cost of its histories and of all histories of the launch.  A claim
+// takes at most 1/8 of a warp's share of the launch by that estimate (a sweep's
+// longest cases have a hundred times its shortest's events), and at most 32
+// times the chunk option.  Events per history are about cost^(3/4)
+// (measured: the estimate is within a factor of two for short histories and
+// several times too high for scattering media).
+inline void plan_claims(RunCase &r, const CaseParams &c, double launch_cost, uint64_t warps, uint32_t chunk,
+                        uint32_t option) {
+    const double share = launch_cost / (8.0 * (double)warps * std::max(c.cost, 1.0) * chunk);
+    const double most = std::min(share, 32.0 * option / chunk);
+    int bits = 0;
+    while (bits < 40 && std::ldexp(1.0, bits + 1) <= most) ++bits;
+    r.claim_bits = (uint16_t)bits;
+    const double events = std::pow(std::max(c.cost, 1.0), 0.75);
+    r.refill_min = (uint16_t)std::min(12.0, std::max(2.0, std::floor(5.2 * std::sqrt(32.0 / events) + 0.5)));
+}
+
 // The kernels' view of one validated case: p_0 = Lambda_0 / (Lambda_0 +
 // Lambda_1) (paper Sec. 2), the mesh width, FP32 copies, reciprocals and the
 // integer thresholds of the draw comparisons.  Case k of a launch draws with

@@ -355,6 +355,24 @@ struct Flight {
     bool tail;  // k1 is the mesh's last bin: the difference array's end marker falls past the mesh
 };
 
+// FP64 walk: the same in fixed point, units of 2^-kFixed64Bits bin widths,
+// formed in integer arithmetic (plan_flight).  A flight that scores straight
+// into the global bins (`real`) holds the bit patterns of the doubles instead.
+template <>
+struct Flight<double> {
+    int k0, k1;
+    unsigned long long a0, a1, c;
+    bool tail, real;
+};
+
+__device__ __forceinline__ double flight_real(unsigned long long a) { return __longlong_as_double((long long)a); }
+__device__ __forceinline__ double flight_real(float a) { return (double)a; }
+
+// whether the flight scores straight into the global bins (a lane whose region
+// was handed to a newer key; FP64 also flights too long for the fixed point)
+__device__ __forceinline__ bool scores_global(const Flight<float> &, int lreg) { return lreg == 2; }
+__device__ __forceinline__ bool scores_global(const Flight<double> &f, int) { return f.real; }
+
 // Output words (hi, lo) of draw j = s.j of the history; advances j.  Even
 // draws compute a Philox block and keep its words 2, 3 for the odd draw.
 template <typename P>
@@ -585,20 +603,23 @@ __device__ __forceinline__ void trace_row(TraceSink *tr, int ev, const History<P
 // its length l itself, which stays exact for grazing flights (|wx| -> 0).  A
 // flight with wx == 0 scores its whole length in the bin that contains x0.
 template <typename P>
-__device__ __forceinline__ void plan_flight(Flight<P> &f, History<P> &s, const CaseParams &cp, P x0, P x1, P l,
-                                            int m) {
-    using R = Real<P>;
+__device__ __forceinline__ void add_track(History<P> &s, P l, int m) {
     const P t = (m == 0 ? s.track0 : s.track1) + l;  // one add, the sum selected
     s.track0 = (m == 0) ? t : s.track0;
     s.track1 = (m == 0) ? s.track1 : t;
+}
+
+__device__ __forceinline__ void plan_flight(Flight<float> &f, History<float> &s, const CaseParams &cp, float x0,
+                                            float x1, float l, int m, bool) {
+    using R = Real<float>;
+    add_track(s, l, m);
     f.k0 = 0;
     f.k1 = -1;
     if (!R::pos(l)) return;
     const int nb = cp.nbins;
-    const P inv_dx = R::inv_dx(cp);
-    // the x-extent clipped to [0, L]; every value below is >= 0, so min and
-    // max are the integer comparisons of R::lt
-    const P a = R::nonneg(x0), b = R::nonneg(x1);
+    const float inv_dx = R::inv_dx(cp);
+    // the x-extent clipped to [0, L]
+    const float a = R::nonneg(x0), b = R::nonneg(x1);
     if (R::is_zero(s.w[0])) {
         const int k = R::floor_index(a * inv_dx, nb - 1);
         f.k0 = f.k1 = k;
@@ -606,13 +627,13 @@ __device__ __forceinline__ void plan_flight(Flight<P> &f, History<P> &s, const C
         f.a0 = l;
         return;
     }
-    const P L = R::L(cp);
-    const P lo = R::lt(a, b) ? a : b;
-    P hi = R::lt(a, b) ? b : a;
+    const float L = R::L(cp);
+    const float lo = R::lt(a, b) ? a : b;
+    float hi = R::lt(a, b) ? b : a;
     hi = R::lt(L, hi) ? L : hi;
     // bin coordinates x / dx: bin index = integer part; the end bins receive
     // (1 - frac) dx / |wx| and frac dx / |wx|
-    const P ulo = lo * inv_dx, uhi = hi * inv_dx;
+    const float ulo = lo * inv_dx, uhi = hi * inv_dx;
     const int k0 = R::floor_index(ulo, nb - 1);
     const int k1 = R::floor_index(uhi, nb - 1);
     f.k0 = k0;
@@ -622,10 +643,99 @@ __device__ __forceinline__ void plan_flight(Flight<P> &f, History<P> &s, const C
         f.a0 = l;
         return;
     }
-    const P c = R::dx(cp) * R::abs(s.iw[0]);
-    f.a0 = R::nonneg(fma(-R::frac(ulo, k0), c, c));
+    const float c = R::dx(cp) * R::abs(s.iw[0]);
+    f.a0 = R::nonneg(fmaf(-R::frac(ulo, k0), c, c));
     f.a1 = R::frac(uhi, k1) * c;
     f.c = c;
+}
+
+// FP64 walk.  Fixed point: 48 fraction bits of a bin width, a rounding of
+// 2^-49 bin widths per deposit, below the 2^-53 relative rounding of a sum of
+// more than 16 bin widths; and 2^15 bin widths of headroom per bin between two
+// flushes (DepositBound).  Lengths of 2^kFixed64MaxExp bin widths and more (a
+// grazing flight, |wx| < 2^-9) go to the global bins in FP64.
+constexpr int kFixed64Bits = 48;
+constexpr int kFixed64MaxExp = 9;
+
+// A bin coordinate u = x / dx >= 0 (below 2^12): its integer part, and its
+// fraction with 64 bits.
+__device__ __forceinline__ unsigned long long split_coordinate(double u, int *k) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(u);
+    const int e = (int)(b >> 52) - 1023;
+    const unsigned long long M = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    *k = e >= 0 ? (int)(M >> (52 - e)) : 0;
+    return e >= -12 ? M << (12 + e) : M >> min(-12 - e, 63);
+}
+
+// round(v 2^kFixed64Bits) for 0 <= v < 2^kFixed64MaxExp, half up
+__device__ __forceinline__ unsigned long long fixed64(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int sh = 52 - kFixed64Bits - ((int)(b >> 52) - 1023);
+    const unsigned long long M = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    return sh <= 0 ? M << -sh : ((M >> min(sh - 1, 63)) + 1ull) >> 1;
+}
+
+// round(F c 2^-64), half up
+__device__ __forceinline__ unsigned long long mul_fraction(unsigned long long F, unsigned long long c) {
+    return __umul64hi(F, c) + ((F * c) >> 63);
+}
+
+// The flight in FP64, for the global bins: bit patterns of a0, a1 and c.
+__device__ __forceinline__ void plan_flight_real(Flight<double> &f, double ulo, double uhi, double l, double c) {
+    using R = Real<double>;
+    f.real = true;
+    if (f.k0 == f.k1) {
+        f.a0 = (unsigned long long)__double_as_longlong(l);
+        return;
+    }
+    f.a0 = (unsigned long long)__double_as_longlong(R::nonneg(fma(-R::frac(ulo, f.k0), c, c)));
+    f.a1 = (unsigned long long)__double_as_longlong(R::frac(uhi, f.k1) * c);
+    f.c = (unsigned long long)__double_as_longlong(c);
+}
+
+__device__ __forceinline__ void plan_flight(Flight<double> &f, History<double> &s, const CaseParams &cp, double x0,
+                                            double x1, double l, int m, bool global) {
+    using R = Real<double>;
+    add_track(s, l, m);
+    f.k0 = 0;
+    f.k1 = -1;
+    f.real = global;
+    if (!R::pos(l)) return;
+    const int nb = cp.nbins;
+    const double inv_dx = R::inv_dx(cp);
+    // the x-extent clipped to [0, L]; every value below is >= 0, so min and
+    // max are the integer comparisons of R::lt
+    const double a = R::nonneg(x0), b = R::nonneg(x1);
+    const double L = R::L(cp);
+    const double lo = R::lt(a, b) ? a : b;
+    double hi = R::lt(a, b) ? b : a;
+    hi = R::lt(L, hi) ? L : hi;
+    // bin coordinates x / dx: bin index = integer part; the end bins receive
+    // (1 - frac) dx / |wx| and frac dx / |wx|
+    const double ulo = lo * inv_dx, uhi = hi * inv_dx;
+    int k0, k1;
+    const unsigned long long F0 = split_coordinate(ulo, &k0);
+    unsigned long long F1 = split_coordinate(uhi, &k1);
+    if (k1 >= nb) {  // x = L: the whole of the last bin
+        k1 = nb - 1;
+        F1 = ~0ull;
+    }
+    k0 = min(k0, nb - 1);
+    if (R::is_zero(s.w[0])) k1 = k0 = (R::lt(a, b) ? k0 : k1);  // the bin that contains x0
+    f.k0 = k0;
+    f.k1 = k1;
+    f.tail = k1 == nb - 1;
+    // in bin widths: a flight inside one bin scores its length itself, else
+    // 1/|wx| in a whole bin
+    const double v = k0 == k1 ? l * inv_dx : R::abs(s.iw[0]);
+    if (global || (int)((unsigned long long)__double_as_longlong(v) >> 52) >= 1023 + kFixed64MaxExp) {
+        plan_flight_real(f, ulo, uhi, l, R::dx(cp) * R::abs(s.iw[0]));
+        return;
+    }
+    const unsigned long long q = fixed64(v);
+    f.a0 = k0 == k1 ? q : q - mul_fraction(F0, q);
+    f.a1 = mul_fraction(F1, q);
+    f.c = q;
 }
 
 // Distance along the flight to the face ahead on one axis: (L - r)/omega
@@ -641,10 +751,10 @@ __device__ __forceinline__ P face_distance(P r, P w, P iw, P L) {
 
 // One event of Algorithm A.  Fills the flight to score and returns -1 while
 // the history continues, else the terminating event (EV_LEAK_X0, EV_LEAK_XL,
-// EV_ABSORB, EV_CAPPED).
+// EV_ABSORB, EV_CAPPED).  global: the lane scores into the global bins.
 template <typename P, bool TRACE, int G = 0, bool DEFER = false>
 __device__ __forceinline__ int step(History<P> &s, const CaseParams &cp, const RoundKeys &key, uint32_t max_events,
-                                    Flight<P> &f, TraceSink *tr) {
+                                    Flight<P> &f, TraceSink *tr, bool global = false) {
     using R = Real<P>;
     const int gd = geometry<G>(cp);
     f.k0 = 0;
@@ -708,7 +818,7 @@ __device__ __forceinline__ int step(History<P> &s, const CaseParams &cp, const R
     const bool leak = bnd && face != 2;
     const P l = bnd ? l_b : (coll ? l_c : l_i);
     const P x1 = leak ? ((face == 0) ? P(0) : L) : s.r[0] + l * s.w[0];
-    plan_flight(f, s, cp, s.r[0], x1, l, m);
+    plan_flight(f, s, cp, s.r[0], x1, l, m, global);
     s.r[0] = x1;
     if (lateral) {
         if (bnd && face == 2 && R::eq(l_y, l_b)) {  // specular reflection on a y face
@@ -767,17 +877,42 @@ __device__ __forceinline__ int step(History<P> &s, const CaseParams &cp, const R
 
 // ------------------------------------------------------- tally regions
 // A warp-private shared-memory region (layout: region_bytes() in
-// cls_internal.h): the bins, FP64 statistics, u64 counters and the lanes' own
-// FP64 copies of the per-history statistics.  The FP64 walk's bins are
-// doubles; the FP32 walk's are a fixed-point difference array (u64 with 32
-// fraction bits), added with native integer atomics -- no retry loop when a
-// warp's flights share an entry, as on thin slabs -- and prefix-summed exactly
-// at the flush.
-template <typename P>
-constexpr bool kFixedBins = sizeof(P) == 4;
+// cls_internal.h): the bins, FP64 statistics, counters and the lanes' own
+// copies of the per-history statistics.  The bins are a fixed-point difference
+// array, prefix-summed exactly at the flush: the FP32 walk's with 32 fraction
+// bits of track length, the FP64 walk's with kFixed64Bits of a bin width.
+//
+// 64-bit additions in shared memory go through 32-bit halves: the low half's
+// atomic returns the old value, whose carry joins the high half.  Every wrap
+// of a low half is seen by exactly one addition, so the pair holds the sum
+// modulo 2^64 whatever the order.  Measured at full occupancy on random
+// entries of 200: 14 cycles per warp and scheduler, against 62 for a 64-bit
+// integer atomic and 94 for a double (both are compare-and-swap loops, and
+// slow down further where lanes meet: 90 and 250 on 20 entries; the halves
+// stay at 14).
+__device__ __forceinline__ void add_halves(uint32_t *lo, uint32_t *hi, unsigned long long x) {
+    const uint32_t xl = (uint32_t)x;
+    const uint32_t old = atomicAdd(lo, xl);
+    const uint32_t h = (uint32_t)(x >> 32) + (old + xl < old ? 1u : 0u);
+    if (h != 0u) atomicAdd(hi, h);
+}
 
-__device__ __forceinline__ unsigned long long *region_fixed(unsigned char *region) {
-    return reinterpret_cast<unsigned long long *>(region);
+template <typename P>
+constexpr bool kFixedStats = sizeof(P) == 4;
+
+// difference array entry k (k <= nbs)
+__device__ __forceinline__ void add_entry(unsigned char *region, int nbs, int k, unsigned long long x) {
+    uint32_t *lo = reinterpret_cast<uint32_t *>(region) + k;
+    add_halves(lo, lo + nbs + 1, x);
+}
+
+__device__ __forceinline__ uint32_t *region_counters(unsigned char *region, int nbs) {
+    return reinterpret_cast<uint32_t *>(region + region_bins_bytes(nbs) + 8 * S_NUM);
+}
+
+// counter c of the region += x (C_MAXEV: maximum, below 2^32)
+__device__ __forceinline__ void add_count(uint32_t *ct, int c, unsigned long long x) {
+    add_halves(ct + c, ct + C_NUM + c, x);
 }
 
 // round(c 2^32), ties to even, for 0 <= c < 2^32, in two 32-bit halves: the
@@ -799,11 +934,11 @@ __device__ __forceinline__ unsigned long long fixed32(float c) {
 // 24; the slot of t stays unused, its sum being that of t0 and t1 -- so that
 // the FP32 walk sums them exactly.
 template <typename P>
-using LaneStat = typename std::conditional<kFixedBins<P>, unsigned long long, double>::type;
+using LaneStat = typename std::conditional<kFixedStats<P>, unsigned long long, double>::type;
 
 template <typename P>
 __device__ __forceinline__ LaneStat<P> *region_lane_stats(unsigned char *region, int nbs) {
-    return reinterpret_cast<LaneStat<P> *>(region + region_lane_stats_offset(kFixedBins<P>, nbs));
+    return reinterpret_cast<LaneStat<P> *>(region + region_lane_stats_offset(nbs));
 }
 
 // A history longer than this (in track length) keeps its statistics out of the
@@ -812,9 +947,8 @@ __device__ __forceinline__ LaneStat<P> *region_lane_stats(unsigned char *region,
 // histories between flushes (FP32 regions flush every 1024).
 constexpr float kFixedTrackMax = 8192.0f;
 
-template <typename P>
 __device__ __forceinline__ double *region_stats(unsigned char *region, int nbs) {
-    return reinterpret_cast<double *>(region + region_bins_bytes(kFixedBins<P>, nbs));
+    return reinterpret_cast<double *>(region + region_bins_bytes(nbs));
 }
 
 // The history's track length t and t^2 into this lane's own copy of the
@@ -827,7 +961,7 @@ __device__ __forceinline__ double *region_stats(unsigned char *region, int nbs) 
 template <typename P>
 __device__ __forceinline__ bool finish_history(unsigned char *region, int nbs, const History<P> &s, int lane) {
     LaneStat<P> *ls = region_lane_stats<P>(region, nbs) + lane;
-    if constexpr (kFixedBins<P>) {
+    if constexpr (kFixedStats<P>) {
         const float t = s.track0 + s.track1;
         if (!(t <= kFixedTrackMax)) return false;
         const unsigned long long q0 = fixed32(s.track0), q1 = fixed32(s.track1);
@@ -847,20 +981,37 @@ __device__ __forceinline__ bool finish_history(unsigned char *region, int nbs, c
     return true;
 }
 
+// A finished history's collisions and reflections, from its draw index and its
+// other counters (the walk need not count them): the source takes a fixed
+// number of draws, every event two, every collision one and every scatter one
+// more (a direction cosine) or two (mu and phi); and every event is a
+// collision, an interface crossing, a reflection or the final leak.
+template <typename P, int G>
+__device__ __forceinline__ void derive_counts(const History<P> &s, const CaseParams &cp, int outcome, uint32_t *n_coll,
+                                              uint32_t *n_refl) {
+    const int gd = geometry<G>(cp);
+    const bool wide = gd == 3 || gd == 2, volume = cp.source == 1;
+    const uint32_t source = gd == 3 ? 5u + volume : gd == 2 ? 4u + volume : gd == 1 ? 1u + 2u * volume : 2u + volume;
+    const uint32_t absorbed = outcome == EV_ABSORB, leaked = outcome == EV_LEAK_X0 || outcome == EV_LEAK_XL;
+    const uint32_t extra = s.j - source - 2u * s.events;  // of collisions and scatters
+    *n_coll = wide ? (extra + 2u * absorbed) / 3u : (extra + absorbed) / 2u;
+    *n_refl = s.events - *n_coll - s.n_int - leaked;
+}
+
 // Outcome and event counters of the lanes whose history ended this step
 // (`ended`, scoring into region lreg < 2).  When several lanes ended they are
 // summed over the warp per region (ballot counts, warp reductions of 16-bit
 // halves) and one lane adds each to the region, else each lane adds its own:
 // short histories that end together do not serialise on shared atomics.
-__device__ __forceinline__ void count_one(unsigned long long *ct, int outcome, uint32_t n_coll, uint32_t n_int,
-                                          uint32_t n_refl, uint32_t events) {
+__device__ __forceinline__ void count_one(uint32_t *ct, int outcome, uint32_t n_coll, uint32_t n_int, uint32_t n_refl,
+                                          uint32_t events) {
     const int c = (outcome == EV_LEAK_X0) ? C_R : (outcome == EV_LEAK_XL) ? C_T : (outcome == EV_ABSORB) ? C_A : C_CAPPED;
-    atomicAdd(&ct[c], 1ull);
-    if (n_coll) atomicAdd(&ct[C_COLL], (unsigned long long)n_coll);
-    if (n_int) atomicAdd(&ct[C_INT], (unsigned long long)n_int);
-    if (n_refl) atomicAdd(&ct[C_REFL], (unsigned long long)n_refl);
-    atomicAdd(&ct[C_EVENTS], (unsigned long long)events);
-    atomicMax(&ct[C_MAXEV], (unsigned long long)events);
+    add_count(ct, c, 1ull);
+    if (n_coll) add_count(ct, C_COLL, n_coll);
+    if (n_int) add_count(ct, C_INT, n_int);
+    if (n_refl) add_count(ct, C_REFL, n_refl);
+    add_count(ct, C_EVENTS, events);
+    atomicMax(&ct[C_MAXEV], events);
 }
 
 __device__ __forceinline__ unsigned long long warp_sum32(bool mine, uint32_t x, bool small) {
@@ -872,13 +1023,13 @@ __device__ __forceinline__ unsigned long long warp_sum32(bool mine, uint32_t x, 
 
 template <typename P>
 __device__ __forceinline__ void warp_count(unsigned char *regions, int rbytes, int nbs, bool ended, int lreg,
-                                           const History<P> &s, int outcome, int lane, bool small) {
+                                           const History<P> &s, uint32_t n_coll, uint32_t n_refl, int outcome, int lane,
+                                           bool small) {
     const unsigned em = __ballot_sync(CLS_FULL_MASK, ended);
     if (em == 0u) return;
     if (__popc(em) < 4) {
         if (ended)
-            count_one(reinterpret_cast<unsigned long long *>(region_stats<P>(regions + lreg * rbytes, nbs) + S_NUM),
-                      outcome, s.n_coll, s.n_int, s.n_refl, s.events);
+            count_one(region_counters(regions + lreg * rbytes, nbs), outcome, n_coll, s.n_int, n_refl, s.events);
         return;
     }
 #pragma unroll 1
@@ -890,33 +1041,29 @@ __device__ __forceinline__ void warp_count(unsigned char *regions, int rbytes, i
         const unsigned nt = __popc(__ballot_sync(CLS_FULL_MASK, mine && outcome == EV_LEAK_XL));
         const unsigned na = __popc(__ballot_sync(CLS_FULL_MASK, mine && outcome == EV_ABSORB));
         const unsigned ncap = __popc(m) - nr - nt - na;
-        const unsigned long long nc = warp_sum32(mine, s.n_coll, small), ni = warp_sum32(mine, s.n_int, small);
-        const unsigned long long nf = warp_sum32(mine, s.n_refl, small), ne = warp_sum32(mine, s.events, small);
+        const unsigned long long nc = warp_sum32(mine, n_coll, small), ni = warp_sum32(mine, s.n_int, small);
+        const unsigned long long nf = warp_sum32(mine, n_refl, small), ne = warp_sum32(mine, s.events, small);
         const unsigned mx = __reduce_max_sync(CLS_FULL_MASK, mine ? s.events : 0u);
         if (lane == __ffs(m) - 1) {
-            unsigned long long *ct = reinterpret_cast<unsigned long long *>(region_stats<P>(regions + r * rbytes, nbs) + S_NUM);
-            if (nr) atomicAdd(&ct[C_R], (unsigned long long)nr);
-            if (nt) atomicAdd(&ct[C_T], (unsigned long long)nt);
-            if (na) atomicAdd(&ct[C_A], (unsigned long long)na);
-            if (ncap) atomicAdd(&ct[C_CAPPED], (unsigned long long)ncap);
-            if (nc) atomicAdd(&ct[C_COLL], nc);
-            if (ni) atomicAdd(&ct[C_INT], ni);
-            if (nf) atomicAdd(&ct[C_REFL], nf);
-            atomicAdd(&ct[C_EVENTS], ne);
-            atomicMax(&ct[C_MAXEV], (unsigned long long)mx);
+            uint32_t *ct = region_counters(regions + r * rbytes, nbs);
+            if (nr) add_count(ct, C_R, nr);
+            if (nt) add_count(ct, C_T, nt);
+            if (na) add_count(ct, C_A, na);
+            if (ncap) add_count(ct, C_CAPPED, ncap);
+            if (nc) add_count(ct, C_COLL, nc);
+            if (ni) add_count(ct, C_INT, ni);
+            if (nf) add_count(ct, C_REFL, nf);
+            add_count(ct, C_EVENTS, ne);
+            atomicMax(&ct[C_MAXEV], mx);
         }
     }
 }
 
-// The interior bins of all lanes' flights, spread evenly over the 32 lanes:
-// lane t of each round scores interior task base + t, found by a 5-step
-// shuffle search over the warp's inclusive prefix sum of the interior counts.
-// Lanes with lreg < 2 score into their FP64 region (FP64 walk only: the FP32
-// walk's region lanes take the difference array and bring no tasks here);
-// lanes with lreg == 2 into the FP64 global bins.
-template <typename P>
-__device__ __forceinline__ void spread_interior(unsigned char *regions, int rbytes, int lreg, double *gflux,
-                                                uint64_t goff, int k0, P c, int ni, int lane) {
+// The interior bins of the flights that score into the global bins, spread
+// evenly over the 32 lanes: lane t of each round scores interior task base +
+// t, found by a 5-step shuffle search over the warp's inclusive prefix sum of
+// the interior counts ni.
+__device__ __forceinline__ void spread_interior(double *gflux, uint64_t goff, int k0, double c, int ni, int lane) {
     int incl = ni;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -924,8 +1071,6 @@ __device__ __forceinline__ void spread_interior(unsigned char *regions, int rbyt
         if (lane >= o) incl += v;
     }
     const int total = __shfl_sync(CLS_FULL_MASK, incl, 31);
-    if (total == 0) return;
-    const bool any_global = __any_sync(CLS_FULL_MASK, lreg == 2 && ni > 0);
     const int base_bin = k0 + 1 - (incl - ni);  // interior task t of this lane goes to base_bin + t
     for (int base = 0; base < total; base += 32) {
         const int t = base + lane;
@@ -936,81 +1081,79 @@ __device__ __forceinline__ void spread_interior(unsigned char *regions, int rbyt
             if (v <= t) o += sft;
         }
         const int ob = __shfl_sync(CLS_FULL_MASK, base_bin, o);
-        const P oc = __shfl_sync(CLS_FULL_MASK, c, o);
-        const int oreg = __shfl_sync(CLS_FULL_MASK, lreg, o);
-        uint64_t ogoff = 0;
-        if (any_global) ogoff = __shfl_sync(CLS_FULL_MASK, goff, o);
-        if (t < total) {
-            if (!kFixedBins<P> && oreg < 2) {
-                double *bins = reinterpret_cast<double *>(regions + oreg * rbytes);
-                atomicAdd(&bins[ob + t], (double)oc);
-            } else {
-                atomicAdd(&gflux[ogoff + ob + t], (double)oc);
-            }
-        }
+        const double oc = __shfl_sync(CLS_FULL_MASK, c, o);
+        const uint64_t ogoff = __shfl_sync(CLS_FULL_MASK, goff, o);
+        if (t < total) atomicAdd(&gflux[ogoff + ob + t], oc);
     }
 }
 
+// Bound on a region's bins between two flushes (FP64 walk): each lane sums the
+// high words of its flights' largest deposits, at most 2^(kFixed64Bits - 32 +
+// kFixed64MaxExp) = 2^25 each, and the warp flushes once a lane's sum has
+// reached 2^25: no lane's passes 2^26, so no bin of the warp passes 2^63 units.
+// FP32 regions are flushed by the histories fed into them.
+constexpr uint32_t kDepositBound = 1u << (kFixed64Bits - 32 + kFixed64MaxExp);
+static_assert(32ull * 2 * kDepositBound <= 1ull << 31, "a bin's sum stays below 2^63 units");
+
 // Score the warp's flights.
-//   FP32 walk, region lanes: the flight's bins are a0 in k0, c in each interior
-//   bin k0 < k < k1 and a1 in k1, each rounded once to 32 fraction bits (q0,
-//   qc, q1; zero where the flight has no such bin); as a difference array D
+//   Region lanes: the flight's bins are a0 in k0, c in each interior bin
+//   k0 < k < k1 and a1 in k1, each rounded once to fixed point (q0, qc, q1;
+//   zero where the flight has no such bin); as a difference array D
 //   (bin k = D[0] + ... + D[k]) that is D[k0] += q0, D[k0+1] += qc - q0 (or
 //   q1 - q0 when k1 = k0 + 1), D[k1] += q1 - qc, D[k1+1] -= q1 -- two integer
-//   atomics for a flight inside one bin, three when it spans two, four
+//   additions for a flight inside one bin, three when it spans two, four
 //   otherwise -- and the flush's prefix sum returns exactly the rounded
-//   deposits, whatever the order of the atomics.  With SKIP, an entry that
+//   deposits, whatever the order of the additions.  With SKIP, an entry that
 //   adds zero is left out (q0 = qc when the flight covers its first bin
 //   whole, q1 = qc when it covers its last bin whole), and so is the end
 //   marker D[k1+1] of a flight whose last bin is the mesh's (the flush never
 //   reads past the last bin).
-//   FP64 walk: each lane adds its two end bins, and the interior bins of all
-//   lanes' flights are spread evenly over the 32 lanes (spread_interior), so
-//   long flights do not serialise the warp; each interior bin is added
-//   exactly (a difference array's prefix sums would cancel between near and
-//   far bins, and FP64 parity holds to 1e-12 per bin).
-// A lane with lreg == 2 scores straight into the FP64 global bins at
-// gflux + goff, those of its (case, batch) (see the region eviction in the
-// trackers).
+//   Lanes that score globally (scores_global) add FP64 values to the bins of
+//   their (case, batch) at gflux + goff, interior bins spread over the warp.
+// Returns the lane's share of DepositBound.
 template <typename P, bool SKIP = false>
-__device__ __forceinline__ void warp_deposit(unsigned char *regions, int rbytes, int nbs, int lreg, double *gflux,
-                                             uint64_t goff, const Flight<P> &f, int lane) {
-    const bool has = f.k1 >= f.k0;
+__device__ __forceinline__ uint32_t warp_deposit(unsigned char *regions, int rbytes, int nbs, int lreg, double *gflux,
+                                                 uint64_t goff, const Flight<P> &f, int lane) {
+    const bool has = f.k1 >= f.k0, global = scores_global(f, lreg);
+    uint32_t bound = 0;
     if (has) {
-        if (lreg < 2) {
-            if constexpr (kFixedBins<P>) {
-                // predicated, not branched: every lane with a flight runs the same code
-                unsigned long long *D = region_fixed(regions + lreg * rbytes);
-                const bool multi = f.k1 > f.k0, inter = f.k1 > f.k0 + 1;
-                const unsigned long long q0 = fixed32((float)f.a0);
-                const unsigned long long q1 = fixed32(multi ? (float)f.a1 : 0.0f);
-                const unsigned long long qc = fixed32(inter ? (float)f.c : 0.0f);
-                const unsigned long long d1 = (inter ? qc : q1) - q0;  // modulo 2^64: exact
-                if constexpr (SKIP) {
-                    if (q0 != 0ull) atomicAdd(&D[f.k0], q0);
-                    if (d1 != 0ull && (multi || !f.tail)) atomicAdd(&D[f.k0 + 1], d1);
-                    if (inter && q1 != qc) atomicAdd(&D[f.k1], q1 - qc);
-                    if (multi && !f.tail) atomicAdd(&D[f.k1 + 1], 0ull - q1);
-                } else {
-                    atomicAdd(&D[f.k0], q0);
-                    atomicAdd(&D[f.k0 + 1], d1);
-                    if (inter) atomicAdd(&D[f.k1], q1 - qc);
-                    if (multi) atomicAdd(&D[f.k1 + 1], 0ull - q1);
-                }
+        if (!global) {
+            // predicated, not branched: every lane with a flight runs the same code
+            unsigned char *region = regions + lreg * rbytes;
+            const bool multi = f.k1 > f.k0, inter = f.k1 > f.k0 + 1;
+            unsigned long long q0, q1, qc;
+            if constexpr (sizeof(P) == 4) {
+                q0 = fixed32(f.a0);
+                q1 = fixed32(multi ? f.a1 : 0.0f);
+                qc = fixed32(inter ? f.c : 0.0f);
             } else {
-                double *bins = reinterpret_cast<double *>(regions + lreg * rbytes);
-                atomicAdd(&bins[f.k0], (double)f.a0);
-                if (f.k1 > f.k0) atomicAdd(&bins[f.k1], (double)f.a1);
+                bound = (uint32_t)(f.c >> 32) + 1u;
+                q0 = f.a0;
+                q1 = multi ? f.a1 : 0ull;
+                qc = inter ? f.c : 0ull;
+            }
+            const unsigned long long d1 = (inter ? qc : q1) - q0;  // modulo 2^64: exact
+            if constexpr (SKIP) {
+                if (q0 != 0ull) add_entry(region, nbs, f.k0, q0);
+                if (d1 != 0ull && (multi || !f.tail)) add_entry(region, nbs, f.k0 + 1, d1);
+                if (inter && q1 != qc) add_entry(region, nbs, f.k1, q1 - qc);
+                if (multi && !f.tail) add_entry(region, nbs, f.k1 + 1, 0ull - q1);
+            } else {
+                add_entry(region, nbs, f.k0, q0);
+                add_entry(region, nbs, f.k0 + 1, d1);
+                if (inter) add_entry(region, nbs, f.k1, q1 - qc);
+                if (multi) add_entry(region, nbs, f.k1 + 1, 0ull - q1);
             }
         } else {
             double *gbins = gflux + goff;
-            atomicAdd(&gbins[f.k0], (double)f.a0);
-            if (f.k1 > f.k0) atomicAdd(&gbins[f.k1], (double)f.a1);
+            atomicAdd(&gbins[f.k0], flight_real(f.a0));
+            if (f.k1 > f.k0) atomicAdd(&gbins[f.k1], flight_real(f.a1));
         }
     }
-    const int ni = (has && !(kFixedBins<P> && lreg < 2)) ? max(f.k1 - f.k0 - 1, 0) : 0;
-    if (!__any_sync(CLS_FULL_MASK, ni > 0)) return;  // one vote instead of the scan when no lane has any
-    spread_interior<P>(regions, rbytes, lreg, gflux, goff, f.k0, f.c, ni, lane);
+    const int ni = (has && global) ? max(f.k1 - f.k0 - 1, 0) : 0;
+    // one vote instead of the scan when no lane has any
+    if (__any_sync(CLS_FULL_MASK, ni > 0)) spread_interior(gflux, goff, f.k0, flight_real(f.c), ni, lane);
+    return bound;
 }
 
 // A finished history's outcome into the caller's record, when one is bound
@@ -1027,11 +1170,21 @@ __device__ __forceinline__ void record_outcome(const LaunchArgs &a, int case_ind
     r.codes[(uint64_t)case_index * r.stride + (h - r.first)] = code;
 }
 
+// This warp's copy of a case's global statistics.  All warps of a launch work
+// on the same case or two at a time, and an FP64 addition to one address of
+// global memory takes 16 ns, whoever asks (0.7 ns for integers): with one copy
+// per case a sweep's flushes queued on it (38 ns per flush; 256 cases x 1e6 in
+// chunks of 256 histories ran at that rate, 38 ms).
+__device__ __forceinline__ double *global_stats(const Tallies &t, int case_index) {
+    const unsigned w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    return t.stats + ((size_t)case_index * t.stats_copies + w % (unsigned)t.stats_copies) * S_NUM;
+}
+
 // A history's track-length statistics added straight to the case's global
 // FP64 tally block.
 template <typename P>
 __device__ __forceinline__ void add_history_stats_global(const LaunchArgs &a, int case_index, const History<P> &s) {
-    double *st = a.t.stats + (size_t)case_index * S_NUM;
+    double *st = global_stats(a.t, case_index);
     const double t0 = (double)s.track0;
     const double t1 = (double)s.track1;
     const double t = t0 + t1;
@@ -1045,86 +1198,84 @@ __device__ __forceinline__ void add_history_stats_global(const LaunchArgs &a, in
 // and counters as finish_history, added to the case's global tally block.
 template <typename P>
 __device__ __forceinline__ void finish_history_global(const LaunchArgs &a, int case_index, const History<P> &s,
-                                                      int outcome, bool with_event_counts) {
+                                                      int outcome, bool with_event_counts, uint32_t n_coll = 0,
+                                                      uint32_t n_refl = 0) {
     add_history_stats_global<P>(a, case_index, s);
     unsigned long long *ct = a.t.counters + (size_t)case_index * C_NUM;
     const int c = (outcome == EV_LEAK_X0) ? C_R : (outcome == EV_LEAK_XL) ? C_T : (outcome == EV_ABSORB) ? C_A : C_CAPPED;
     atomicAdd(&ct[c], 1ull);
     if (with_event_counts) {
-        if (s.n_coll) atomicAdd(&ct[C_COLL], (unsigned long long)s.n_coll);
+        if (n_coll) atomicAdd(&ct[C_COLL], (unsigned long long)n_coll);
         if (s.n_int) atomicAdd(&ct[C_INT], (unsigned long long)s.n_int);
-        if (s.n_refl) atomicAdd(&ct[C_REFL], (unsigned long long)s.n_refl);
+        if (n_refl) atomicAdd(&ct[C_REFL], (unsigned long long)n_refl);
         atomicAdd(&ct[C_EVENTS], (unsigned long long)s.events);
     }
     atomicMax(&ct[C_MAXEV], (unsigned long long)s.events);
 }
 
 // Flush a warp region into the global tally block of (case, batch): one global
-// FP64 atomic per non-zero bin, statistic and counter; the region is zeroed.
+// FP64 atomic per non-zero bin and, with `ends`, per statistic and counter
+// (these belong to the case: a region that moves on to another batch of the
+// same case keeps them); what is flushed is zeroed.
 template <typename P>
 __device__ __forceinline__ void flush_region(unsigned char *region, const LaunchArgs &a, int case_index,
-                                             uint32_t batch, int lane) {
+                                             uint32_t batch, int lane, bool ends = true) {
     const int nbs = a.t.nbins_stride;
     const int nb = a.cases[case_index].nbins;
     double *g = a.t.flux + ((size_t)case_index * a.t.nbatch + batch) * (size_t)nbs;
-    if constexpr (kFixedBins<P>) {
-        // the exact prefix sum of the fixed-point difference array, 32 bins at a
-        // time; its entry nb (past the last bin) sums to zero and is cleared
-        unsigned long long *D = region_fixed(region);
-        unsigned long long carry = 0ull;
-        for (int base = 0; base <= nb; base += 32) {
-            const int k = base + lane;
-            unsigned long long d = (k <= nb) ? D[k] : 0ull;
+    // the exact prefix sum of the fixed-point difference array, 32 bins at a
+    // time; its entry nb (past the last bin) sums to zero and is cleared
+    const double unit = sizeof(P) == 4 ? 0x1p-32 : a.cases[case_index].dx * (1.0 / (double)(1ull << kFixed64Bits));
+    uint32_t *lo = reinterpret_cast<uint32_t *>(region), *hi = lo + nbs + 1;
+    unsigned long long carry = 0ull;
+    for (int base = 0; base <= nb; base += 32) {
+        const int k = base + lane;
+        unsigned long long d = (k <= nb) ? (unsigned long long)hi[k] << 32 | lo[k] : 0ull;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long v = __shfl_up_sync(CLS_FULL_MASK, d, o);
-                if (lane >= o) d += v;
-            }
-            const long long q = (long long)(carry + d);  // the bin's deposits, 2^-32 units
-            carry += __shfl_sync(CLS_FULL_MASK, d, 31);
-            if (k < nb && q != 0) atomicAdd(&g[k], (double)q * 0x1p-32);
-            if (k <= nb) D[k] = 0ull;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long v = __shfl_up_sync(CLS_FULL_MASK, d, o);
+            if (lane >= o) d += v;
         }
-    } else {
-        double *bins = reinterpret_cast<double *>(region);
-        for (int k = lane; k < nb; k += 32) {
-            const double v = bins[k];
-            if (v != 0.0) {
-                atomicAdd(&g[k], v);
-                bins[k] = 0.0;
-            }
-        }
+        const long long q = (long long)(carry + d);  // the bin's deposits, in units
+        carry += __shfl_sync(CLS_FULL_MASK, d, 31);
+        if (k < nb && q != 0) atomicAdd(&g[k], (double)q * unit);
+        if (k <= nb) lo[k] = hi[k] = 0u;
+    }
+    if (!ends) {
+        __syncwarp();
+        return;
     }
     // the lanes' own copies of the per-history statistics, summed over the warp
+    double *gst = global_stats(a.t, case_index);
     LaneStat<P> *ls = region_lane_stats<P>(region, nbs);
 #pragma unroll
     for (int q = 0; q < S_NUM; ++q) {
         double v;
-        if constexpr (kFixedBins<P>)
+        if constexpr (kFixedStats<P>)
             v = (q == S_T) ? (double)(ls[32 * S_TRACK0 + lane] + ls[32 * S_TRACK1 + lane]) * 0x1p-32
                            : (double)ls[32 * q + lane] * (q == S_T2 ? 0x1p-24 : 0x1p-32);
         else v = ls[32 * q + lane];
         ls[32 * q + lane] = 0;
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(CLS_FULL_MASK, v, o);
-        if (lane == 0 && __double_as_longlong(v) != 0) atomicAdd(&a.t.stats[(size_t)case_index * S_NUM + q], v);
+        if (lane == 0 && __double_as_longlong(v) != 0) atomicAdd(&gst[q], v);
     }
-    double *st = region_stats<P>(region, nbs);
+    double *st = region_stats(region, nbs);
     if (lane < S_NUM) {
         const double v = st[lane];
         if (v != 0.0) {
-            atomicAdd(&a.t.stats[(size_t)case_index * S_NUM + lane], v);
+            atomicAdd(&gst[lane], v);
             st[lane] = 0.0;
         }
     } else if (lane < S_NUM + C_NUM) {
         const int c = lane - S_NUM;
-        unsigned long long *ct = reinterpret_cast<unsigned long long *>(st + S_NUM);
-        const unsigned long long v = ct[c];
+        uint32_t *ct = region_counters(region, nbs);
+        const unsigned long long v = (unsigned long long)ct[C_NUM + c] << 32 | ct[c];
         if (v != 0ull) {
             unsigned long long *gc = &a.t.counters[(size_t)case_index * C_NUM + c];
             if (c == C_MAXEV) atomicMax(gc, v);
             else atomicAdd(gc, v);
-            ct[c] = 0ull;
+            ct[c] = ct[C_NUM + c] = 0u;
         }
     }
     __syncwarp();
@@ -1141,13 +1292,206 @@ __device__ __forceinline__ int find_run(const LaunchArgs &a, uint64_t ch) {
     return lo;
 }
 
+// A warp's feeding state in the history tracker: the ids being fed, its claim
+// still to be fed (positions in its run entry), its piece and the histories
+// known to be claimed of it (piece < 0: none yet), the regions' keys (run entry
+// and batch; run < 0: none) and the histories fed into each since its last full
+// flush, and the region, run entry and batch being fed.
+struct WarpFeed {
+    uint64_t cursor, end;
+    uint64_t pos, pos_end;
+    uint64_t known;
+    int run[2];
+    uint32_t batch[2];
+    uint32_t fed[2];
+    int piece;
+    int reg, cur_run;
+    uint32_t cur_batch;
+    int stealing;
+};
+static_assert(sizeof(WarpFeed) <= kWarpFeedBytes, "WarpFeed outgrew its shared memory");
+
+// Lane states beside the terminating events (>= 0).
+constexpr int kWalking = -1, kEmpty = -2;
+
+__device__ __forceinline__ uint64_t piece_size(const LaunchArgs &a, uint32_t piece) {
+    const RunCase &rc = a.runs[piece / a.pieces_per_run];
+    return min(a.piece_len, rc.n - (piece % a.pieces_per_run) * a.piece_len);
+}
+
+// A piece with unclaimed histories, the one with the most among the first 128
+// from this warp's starting point that have any; -1 if there is none.
+__device__ __forceinline__ int find_piece(const LaunchArgs &a, int lane) {
+    const uint32_t np = (uint32_t)a.nruns * a.pieces_per_run;
+    const uint32_t start = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 128u % np;
+    for (uint32_t o = 0; o < np; o += 128) {
+        uint32_t most = 0, best = 0;
+#pragma unroll 4
+        for (uint32_t i = 0; i < 4; ++i) {
+            const uint32_t q = o + 32 * i + lane;
+            if (q >= np) break;
+            const uint32_t p = (start + q) % np;
+            const uint64_t size = piece_size(a, p), used = __ldcg(&a.claimed[p]);
+            const uint32_t left = used < size ? (uint32_t)min(size - used, (uint64_t)0xFFFFFFFFu) : 0u;
+            if (left > most) {
+                most = left;
+                best = p;
+            }
+        }
+        const uint32_t top = __reduce_max_sync(CLS_FULL_MASK, most);
+        if (top > 0) {
+            const unsigned who = __ballot_sync(CLS_FULL_MASK, most == top);
+            return __shfl_sync(CLS_FULL_MASK, (int)best, __ffs(who) - 1);
+        }
+    }
+    return -1;
+}
+
+// The warp's next claim, into feed->pos .. pos_end of piece feed->piece;
+// false when nothing is left to claim.
+//
+// Pieces are handed out in the order of the work list, each to `team` warps in
+// turn; a warp stays with its piece until all of it is claimed, and when all
+// pieces are handed out it helps with those that have histories left.  So a
+// warp's histories mostly lie in one statistics batch (it flushes its bins
+// seldom, and histories seldom outlive their region), and the warps work on
+// many batches at a time: a bin in global memory takes an FP64 addition only
+// every 16 ns, and chunks dealt out one by one sent all warps' flushes to the
+// same batch (1e7 rod histories in FP32: chunks of 32 8.9 ms, of 256 1.6 ms;
+// pieces 1.25 ms).  A claim takes half of the team's even share of what is
+// left of the piece, so that claims shrink as it ends, within claim_bits.
+__device__ __forceinline__ bool claim(WarpFeed *feed, const LaunchArgs &a, int lane) {
+    const uint32_t np = (uint32_t)a.nruns * a.pieces_per_run;
+    int piece = feed->piece;
+    uint64_t known = feed->known;
+    bool stealing = feed->stealing != 0;
+    while (true) {
+        if (piece >= 0) {
+            const uint64_t size = piece_size(a, piece);
+            const RunCase &rc = a.runs[piece / a.pieces_per_run];
+            const uint64_t share = (known < size ? size - known : 0ull) / (stealing ? max(2 * a.team, 64u) : 2 * a.team);
+            const uint64_t k = max(min(share, (uint64_t)a.chunk << rc.claim_bits), (uint64_t)a.chunk);
+            unsigned long long got;
+            if (lane == 0) got = atomicAdd(&a.claimed[piece], (unsigned long long)k);
+            got = __shfl_sync(CLS_FULL_MASK, got, 0);
+            if (got < size) {
+                if (lane == 0) {
+                    const uint64_t base = (piece % a.pieces_per_run) * a.piece_len;
+                    feed->pos = base + got;
+                    feed->pos_end = base + min((uint64_t)got + k, size);
+                    feed->known = got + k;
+                    feed->piece = piece;
+                    feed->stealing = stealing;
+                }
+                __syncwarp();
+                return true;
+            }
+        }
+        known = 0;
+        if (!stealing) {
+            unsigned long long t;
+            if (lane == 0) t = atomicAdd(a.chunk_counter, 1ull);
+            t = __shfl_sync(CLS_FULL_MASK, t, 0);
+            stealing = t >= (unsigned long long)np * a.team;
+            piece = stealing ? -1 : (int)(t / a.team);
+        }
+        if (stealing) {
+            piece = find_piece(a, lane);
+            if (piece < 0) return false;
+        }
+    }
+}
+
+// Empty lanes take the next histories of the warp's claims, in lane order.
+// Returns whether the launch has no histories left to claim.
+template <typename P, int G>
+__device__ __forceinline__ bool refill(unsigned char *regions, int rb, WarpFeed *feed, const LaunchArgs &a,
+                                       History<P> &s, int &out, int &lreg, int &lcase, uint32_t &lbatch, int &refill_min,
+                                       int lane) {
+    const unsigned lt_mask = (1u << lane) - 1u;
+    unsigned need = __ballot_sync(CLS_FULL_MASK, out == kEmpty);
+    while (need != 0u) {
+        uint64_t cursor = feed->cursor, end = feed->end;
+        int reg = feed->reg;
+        if (cursor == end) {
+            if (feed->pos == feed->pos_end && !claim(feed, a, lane)) return true;
+            const int run = feed->piece / a.pieces_per_run;
+            const RunCase &rc = a.runs[run];
+            const uint64_t pos = feed->pos;
+            const uint32_t batch = (uint32_t)(pos / rc.batch_len);
+            // the claim's histories of this batch
+            const uint64_t stop = min(feed->pos_end, (uint64_t)(batch + 1ull) * rc.batch_len);
+            refill_min = rc.refill_min;
+            int r = -1;
+            if (feed->run[0] == run && feed->batch[0] == batch) r = 0;
+            else if (feed->run[1] == run && feed->batch[1] == batch) r = 1;
+            if (r < 0) {
+                const bool live0 = __any_sync(CLS_FULL_MASK, out == kWalking && lreg == 0);
+                const bool live1 = __any_sync(CLS_FULL_MASK, out == kWalking && lreg == 1);
+                const int other = reg ^ 1;
+                if (!(other ? live1 : live0)) r = other;
+                else if (!(reg ? live1 : live0)) r = reg;
+                else r = other;  // both referenced: evict the older region
+                const int old_run = feed->run[r];
+                if (old_run >= 0) {
+                    flush_region<P>(regions + r * rb, a, a.runs[old_run].case_index, feed->batch[r], lane, old_run != run);
+                    // lanes still walking a history of the old key go on in global memory
+                    if (out == kWalking && lreg == r) lreg = 2;
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    if (old_run != run) feed->fed[r] = 0;
+                    feed->run[r] = run;
+                    feed->batch[r] = batch;
+                }
+            }
+            reg = r;
+            cursor = rc.first + pos;
+            end = rc.first + stop;
+            __syncwarp();
+            if (lane == 0) {
+                feed->pos = stop;
+                feed->end = end;
+                feed->reg = reg;
+                feed->cur_run = run;
+                feed->cur_batch = batch;
+            }
+            __syncwarp();
+        }
+        const uint64_t avail = end - cursor;
+        const uint32_t nneed = __popc(need);
+        const uint32_t take = (avail < nneed) ? (uint32_t)avail : nneed;
+        const uint32_t rank = __popc(need & lt_mask);
+        if (((need >> lane) & 1u) && rank < take) {
+            lcase = a.runs[feed->cur_run].case_index;
+            lreg = reg;
+            lbatch = feed->cur_batch;
+            source<P, G, true>(s, a.cases[lcase], a.rk, cursor + rank);
+            out = kWalking;
+        }
+        const uint32_t fed = feed->fed[reg] + take;
+        __syncwarp();
+        // FP32 regions flush before a bin's sum can outgrow its 64 bits
+        const bool full = sizeof(P) == 4 && fed >= a.flush_every;
+        if (full) flush_region<P>(regions + reg * rb, a, a.runs[feed->cur_run].case_index, feed->cur_batch, lane);
+        if (lane == 0) {
+            feed->cursor = cursor + take;
+            feed->fed[reg] = full ? 0u : fed;
+        }
+        __syncwarp();
+        need = __ballot_sync(CLS_FULL_MASK, out == kEmpty);
+    }
+    return false;
+}
+
 // ------------------------------------------------- history-based tracker
-// Persistent kernel.  Each warp claims chunks of consecutive histories from a
-// global counter; a lane whose history ends immediately takes the next history
-// of the warp's current chunk (ballot + prefix popcount), so lanes stay busy
-// across history and chunk boundaries.  Each warp owns two shared-memory tally
+// Persistent kernel.  Each warp claims ranges of consecutive histories (claim);
+// lanes whose histories have ended take the next histories of the warp's claim
+// (ballot + prefix popcount), several lanes at a time, so lanes stay busy across
+// history and claim boundaries.  Each warp owns two shared-memory tally
 // regions keyed by (case, batch); a region is flushed to global memory when
-// its key changes, after flush_every histories, or when the warp retires.
+// its key changes, after flush_every histories (FP32) or kDepositBound (FP64),
+// or when the warp retires.
 // When a new key arrives while both regions still serve live histories, the
 // older region is flushed and re-keyed, and its remaining histories score
 // straight into the FP64 global tallies: the warp never waits for a straggler
@@ -1194,139 +1538,83 @@ __global__ void __launch_bounds__(HistoryBounds<P, G>::threads, HistoryBounds<P,
     if constexpr (sizeof(P) == 8) __syncthreads();
     __syncwarp();
 
-    // warp-uniform feeding state
-    int key_run0 = -1, key_run1 = -1;
-    uint32_t key_batch0 = 0, key_batch1 = 0;
-    int fed0 = 0, fed1 = 0;
-    uint64_t cursor = 0, end = 0;  // history ids of the chunk being fed
-    int feed_reg = 0, feed_run = 0;
-    uint32_t feed_batch = 0;
-    bool exhausted = false;
+    // warp-uniform feeding state, in shared memory: it is needed where lanes
+    // take new histories only, and would hold a dozen registers of every lane
+    WarpFeed *feed = reinterpret_cast<WarpFeed *>(smem + (size_t)(blockDim.x >> 5) * 2 * rb + (size_t)warp * kWarpFeedBytes);
+    if (lane == 0) *feed = WarpFeed{0, 0, 0, 0, 0, {-1, -1}, {0, 0}, {0, 0}, -1, 0, 0, 0, 0};
+    __syncwarp();
 
-    // lane state: lreg is the lane's tally region, or 2 once that region was
-    // handed to a newer key (the lane then scores into global memory)
+    // lane state: `out` is kWalking, kEmpty or the terminating event of a
+    // history still to be counted; lreg is the lane's tally region, or 2 once
+    // that region was handed to a newer key (the lane then scores into global
+    // memory)
     History<P> s;
     Flight<P> f;
-    bool alive = false;
+    int out = kEmpty;
+    bool exhausted = false;
+    int refill_min = 1;
     int lreg = 0, lcase = 0;
     uint32_t lbatch = 0;
+    uint32_t deposited = 0;  // FP64 walk: this lane's share of kDepositBound
     const RoundKeys &key = a.rk;
-    const unsigned lt_mask = (1u << lane) - 1u;
 
     while (true) {
-        unsigned need = __ballot_sync(CLS_FULL_MASK, !alive);
-        while (need != 0u && !exhausted) {
-            if (cursor == end) {
-                unsigned long long ch;
-                if (lane == 0) ch = atomicAdd(a.chunk_counter, 1ull);
-                ch = __shfl_sync(CLS_FULL_MASK, ch, 0);
-                if (ch >= a.total_chunks) {
-                    exhausted = true;
-                    break;
+        const unsigned idle = __ballot_sync(CLS_FULL_MASK, out != kWalking);
+        // History ends and births, together, once refill_min lanes (of the run
+        // entry last fed) wait for them: both are long stretches of code for the few lanes concerned.
+        if (idle == CLS_FULL_MASK || (!exhausted && __popc(idle) >= refill_min)) {
+            uint32_t n_coll = 0, n_refl = 0;
+            if (out >= 0) {
+                derive_counts<P, G>(s, a.cases[lcase], out, &n_coll, &n_refl);
+                record_outcome(a, lcase, s.h_lo, s.h_hi, out);
+                if (lreg < 2) {
+                    if (!finish_history<P>(regions + lreg * rb, a.t.nbins_stride, s, lane))
+                        add_history_stats_global<P>(a, lcase, s);
+                    if constexpr (!(WC || G == 0))
+                        count_one(region_counters(regions + lreg * rb, a.t.nbins_stride), out, n_coll, s.n_int,
+                                  n_refl, s.events);
+                } else {
+                    finish_history_global<P>(a, lcase, s, out, true, n_coll, n_refl);
                 }
-                const int run = find_run(a, ch);
-                const RunCase &rc = a.runs[run];
-                const uint64_t local0 = (ch - rc.chunk_begin) * (uint64_t)a.chunk;
-                const uint64_t cnt = min((uint64_t)a.chunk, rc.n - local0);
-                const uint32_t batch = (uint32_t)(local0 / rc.batch_len);
-                int r = -1;
-                if (key_run0 == run && key_batch0 == batch) r = 0;
-                else if (key_run1 == run && key_batch1 == batch) r = 1;
-                if (r < 0) {
-                    const bool live0 = __any_sync(CLS_FULL_MASK, alive && lreg == 0);
-                    const bool live1 = __any_sync(CLS_FULL_MASK, alive && lreg == 1);
-                    const int other = feed_reg ^ 1;
-                    if (!(other ? live1 : live0)) r = other;
-                    else if (!(feed_reg ? live1 : live0)) r = feed_reg;
-                    else r = other;  // both referenced: evict the older region
-                    const int old_run = r ? key_run1 : key_run0;
-                    const uint32_t old_batch = r ? key_batch1 : key_batch0;
-                    if (old_run >= 0) {
-                        flush_region<P>(regions + r * rb, a, a.runs[old_run].case_index, old_batch, lane);
-                        // lanes still walking a history of the old key go on in global memory
-                        if (alive && lreg == r) lreg = 2;
-                    }
-                    if (r == 0) {
-                        key_run0 = run;
-                        key_batch0 = batch;
-                        fed0 = 0;
-                    } else {
-                        key_run1 = run;
-                        key_batch1 = batch;
-                        fed1 = 0;
-                    }
-                }
-                feed_reg = r;
-                feed_run = run;
-                feed_batch = batch;
-                cursor = rc.first + local0;
-                end = cursor + cnt;
             }
-            const uint64_t avail = end - cursor;
-            const uint32_t nneed = __popc(need);
-            const uint32_t take = (avail < nneed) ? (uint32_t)avail : nneed;
-            const uint32_t rank = __popc(need & lt_mask);
-            if (((need >> lane) & 1u) && rank < take) {
-                lcase = a.runs[feed_run].case_index;
-                lreg = feed_reg;
-                lbatch = feed_batch;
-                source<P, G, true>(s, a.cases[lcase], key, cursor + rank);
-                alive = true;
-            }
-            if (feed_reg == 0) fed0 += (int)take;
-            else fed1 += (int)take;
-            cursor += take;
-            need = __ballot_sync(CLS_FULL_MASK, !alive);
+            // short histories often end together: their counters are then summed
+            // over the warp first (the host asks for it when a launch's cases average
+            // few events per history, and always for the mixed-geometry kernel)
+            if constexpr (WC || G == 0)
+                warp_count<P>(regions, rb, a.t.nbins_stride, out >= 0 && lreg < 2, lreg, s, n_coll, n_refl, out, lane,
+                              a.max_events < (1u << 27));
+            out = out >= 0 ? kEmpty : out;
+            if (!exhausted) exhausted = refill<P, G>(regions, rb, feed, a, s, out, lreg, lcase, lbatch, refill_min, lane);
+            if (__all_sync(CLS_FULL_MASK, out != kWalking)) break;
         }
-        if (!__any_sync(CLS_FULL_MASK, alive)) break;
         f.k0 = 0;
         f.k1 = -1;
-        int out = -1;
-        if (alive) {
+        if (out == kWalking) {
             // directions of the lanes born in this round and of those that scattered in the last
             resolve_direction<P, G>(s, a.cases[lcase], key);
-            out = step<P, false, G, true>(s, a.cases[lcase], key, a.max_events, f, nullptr);
+            const int ev = step<P, false, G, true>(s, a.cases[lcase], key, a.max_events, f, nullptr, lreg == 2);
+            out = ev < 0 ? kWalking : ev;
         }
-        const uint64_t goff =
-            (lreg == 2) ? ((uint64_t)lcase * (uint64_t)a.t.nbatch + lbatch) * (uint64_t)a.t.nbins_stride : 0ull;
-        warp_deposit<P, WC>(regions, rb, a.t.nbins_stride, lreg, a.t.flux, goff, f, lane);
-        if (out >= 0) {
-            record_outcome(a, lcase, s.h_lo, s.h_hi, out);
-            if (lreg < 2) {
-                if (!finish_history<P>(regions + lreg * rb, a.t.nbins_stride, s, lane))
-                    add_history_stats_global<P>(a, lcase, s);
-                if constexpr (!(WC || G == 0))
-                    count_one(reinterpret_cast<unsigned long long *>(region_stats<P>(regions + lreg * rb, a.t.nbins_stride) + S_NUM),
-                              out, s.n_coll, s.n_int, s.n_refl, s.events);
-            } else {
-                finish_history_global<P>(a, lcase, s, out, true);
-            }
-        }
-        // short histories often end together: their counters are then summed
-        // over the warp first (the host asks for it when a launch's cases average
-        // few events per history, and always for the mixed-geometry kernel)
-        if constexpr (WC || G == 0)
-            warp_count<P>(regions, rb, a.t.nbins_stride, out >= 0 && lreg < 2, lreg, s, out, lane,
-                          a.max_events < (1u << 27));
-        if (out >= 0) alive = false;
-        // only FP32 regions flush early (their float partial sums stay short);
-        // the host sets no flush interval for FP64 regions
-        if (sizeof(P) == 4 && a.flush_every) {
-            if (fed0 >= a.flush_every) {
+        const uint64_t goff = scores_global(f, lreg)
+                                  ? ((uint64_t)lcase * (uint64_t)a.t.nbatch + lbatch) * (uint64_t)a.t.nbins_stride
+                                  : 0ull;
+        deposited += warp_deposit<P, WC>(regions, rb, a.t.nbins_stride, lreg, a.t.flux, goff, f, lane);
+        if constexpr (sizeof(P) == 8) {  // before a bin's sum can outgrow its 64 bits
+            if (__any_sync(CLS_FULL_MASK, deposited >= kDepositBound)) {
                 __syncwarp();
-                flush_region<P>(regions, a, a.runs[key_run0].case_index, key_batch0, lane);
-                fed0 = 0;
-            }
-            if (fed1 >= a.flush_every) {
-                __syncwarp();
-                flush_region<P>(regions + rb, a, a.runs[key_run1].case_index, key_batch1, lane);
-                fed1 = 0;
+#pragma unroll 1
+                for (int r = 0; r < 2; ++r)
+                    if (feed->run[r] >= 0)
+                        flush_region<P>(regions + r * rb, a, a.runs[feed->run[r]].case_index, feed->batch[r], lane, false);
+                deposited = 0;
             }
         }
     }
     __syncwarp();
-    if (key_run0 >= 0) flush_region<P>(regions, a, a.runs[key_run0].case_index, key_batch0, lane);
-    if (key_run1 >= 0) flush_region<P>(regions + rb, a, a.runs[key_run1].case_index, key_batch1, lane);
+#pragma unroll 1
+    for (int r = 0; r < 2; ++r)
+        if (feed->run[r] >= 0)
+            flush_region<P>(regions + r * rb, a, a.runs[feed->run[r]].case_index, feed->batch[r], lane);
 }
 
 // ------------------------------------------------------------ trace kernel

@@ -144,8 +144,8 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
 // event maximum (event and collision counts are added per pass).
 template <typename P>
 __device__ __forceinline__ void finish_event_history(unsigned char *region, int nbs, const History<P> &s, int outcome) {
-    double *st = region_stats<P>(region, nbs);
-    unsigned long long *ct = reinterpret_cast<unsigned long long *>(st + S_NUM);
+    double *st = region_stats(region, nbs);
+    uint32_t *ct = region_counters(region, nbs);
     const double t0 = (double)s.track0;
     const double t1 = (double)s.track1;
     const double t = t0 + t1;
@@ -154,8 +154,8 @@ __device__ __forceinline__ void finish_event_history(unsigned char *region, int 
     if (__double_as_longlong(t0) != 0) atomicAdd(&st[S_TRACK0], t0);
     if (__double_as_longlong(t1) != 0) atomicAdd(&st[S_TRACK1], t1);
     const int c = (outcome == EV_LEAK_X0) ? C_R : (outcome == EV_LEAK_XL) ? C_T : (outcome == EV_ABSORB) ? C_A : C_CAPPED;
-    atomicAdd(&ct[c], 1ull);
-    atomicMax(&ct[C_MAXEV], (unsigned long long)s.events);
+    add_count(ct, c, 1ull);
+    atomicMax(&ct[C_MAXEV], s.events);
 }
 
 // Launch bounds of the event tracker: blocks of up to kEventBlock = 256
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
     // particles of an older one score into global memory
     int key_run[2] = {-1, -1};
     uint32_t key_batch[2] = {0, 0};
-    int fed[2] = {0, 0};
+    uint32_t fed[2] = {0, 0};
     int live[2] = {0, 0};
     uint32_t gen[2] = {0, 0};
     uint64_t cursor = 0, end = 0;
@@ -202,6 +202,7 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
     const int evict_max = (int)(W >> 4);
     uint32_t nlive = 0;
     int cur = 0;
+    uint32_t deposited = 0;  // FP64 walk: this lane's share of kDepositBound
 
     while (true) {
         unsigned char *buf = bank + cur * buf_bytes;
@@ -265,7 +266,7 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
             cursor += take;
             nlive += take;
             live[feed_reg] += (int)take;
-            fed[feed_reg] += (int)take;
+            fed[feed_reg] += take;
         }
         if (nlive == 0) break;
         __syncwarp();
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
             int reg = packed & 3;
             if (reg < 2 && (uint32_t)(packed >> 2) != gen[reg]) reg = 2;
             uint64_t goff = 0;
-            if (alive && reg == 2) {
+            if (alive && (reg == 2 || sizeof(P) == 8)) {  // FP64: long flights score globally from any region
                 const RunCase &rc = a.runs[run];
                 const uint64_t h = ((uint64_t)s.h_hi << 32) | s.h_lo;
                 const uint64_t batch = (h - rc.first) / rc.batch_len;
@@ -309,8 +310,17 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
                 int o = -1;
                 f.k0 = 0;
                 f.k1 = -1;
-                if (alive) o = step<P, false, G>(s, a.cases[ci], key, a.max_events, f, nullptr);
-                warp_deposit<P>(regions, rb, nbs, reg, a.t.flux, goff, f, lane);
+                if (alive) o = step<P, false, G>(s, a.cases[ci], key, a.max_events, f, nullptr, reg == 2);
+                deposited += warp_deposit<P>(regions, rb, nbs, reg, a.t.flux, goff, f, lane);
+                if constexpr (sizeof(P) == 8) {  // before a bin's sum can outgrow its 64 bits
+                    if (__any_sync(CLS_FULL_MASK, deposited >= kDepositBound)) {
+                        __syncwarp();
+                        for (int r = 0; r < 2; ++r)
+                            if (key_run[r] >= 0)
+                                flush_region<P>(regions + r * rb, a, a.runs[key_run[r]].case_index, key_batch[r], lane, false);
+                        deposited = 0;
+                    }
+                }
                 if (o >= 0) {
                     record_outcome(a, ci, s.h_lo, s.h_hi, o);
                     if (reg < 2) finish_event_history<P>(regions + reg * rb, nbs, s, o);
@@ -347,21 +357,21 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
         }
         // warp-aggregated event counters: one shared-memory atomic per counter
         for (int r = 0; r < 2; ++r) {
-            unsigned long long *ct = reinterpret_cast<unsigned long long *>(region_stats<P>(regions + r * rb, nbs) + S_NUM);
+            uint32_t *ct = region_counters(regions + r * rb, nbs);
             const unsigned long long v0 = warp_sum(r ? c1 : c0), v1 = warp_sum(r ? i1 : i0);
             const unsigned long long v2 = warp_sum(r ? f1 : f0), v3 = warp_sum(r ? e1 : e0);
             if (lane == 0) {
-                if (v0) atomicAdd(&ct[C_COLL], v0);
-                if (v1) atomicAdd(&ct[C_INT], v1);
-                if (v2) atomicAdd(&ct[C_REFL], v2);
-                if (v3) atomicAdd(&ct[C_EVENTS], v3);
+                if (v0) add_count(ct, C_COLL, v0);
+                if (v1) add_count(ct, C_INT, v1);
+                if (v2) add_count(ct, C_REFL, v2);
+                if (v3) add_count(ct, C_EVENTS, v3);
             }
         }
         __syncwarp();
         nlive = out;
         cur ^= 1;
         // FP32 regions: bound the partial sums
-        if (a.flush_every) {
+        if constexpr (sizeof(P) == 4) {
             for (int r = 0; r < 2; ++r) {
                 if (fed[r] >= a.flush_every && key_run[r] >= 0) {
                     flush_region<P>(regions + r * rb, a, a.runs[key_run[r]].case_index, key_batch[r], lane);

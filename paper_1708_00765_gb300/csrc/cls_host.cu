@@ -49,6 +49,11 @@ struct Options {
 // persistent launch with its own chunk counter.
 constexpr int kMaxGroups = 10;  // 2 schedules x 5 geometries
 
+// Work counters on the device: one per group, then the claimed histories of
+// every piece of the history-tracker groups (LaunchArgs::claimed), at most
+// kMaxPieces (or one per case) in a group and 64 per case.
+constexpr uint64_t kMaxPieces = 32768;
+
 }  // namespace
 
 struct cls_handle {
@@ -124,6 +129,16 @@ OutcomeRecord *outcome_record(RunCase *runs, size_t ncases) {
     return reinterpret_cast<OutcomeRecord *>(reinterpret_cast<unsigned char *>(runs) + ncases * sizeof(RunCase));
 }
 
+// Copies of a case's statistics on the device, one of which a warp adds to
+// (global_stats in cls_device.cuh): fewer for very many cases.
+int stats_copies(size_t ncases) { return ncases <= 1024 ? 32 : ncases <= 8192 ? 4 : 1; }
+
+size_t stats_bytes(size_t ncases) { return ncases * stats_copies(ncases) * S_NUM * sizeof(double); }
+
+size_t counter_bytes(size_t ncases) {
+    return (kMaxGroups + std::min<size_t>(64 * ncases, ncases + kMaxGroups * kMaxPieces)) * sizeof(unsigned long long);
+}
+
 void free_tallies(cls_handle *h) {
     if (!h->ws) {
         cudaFree(h->d_flux);
@@ -166,7 +181,7 @@ DevLayout dev_layout(const cls_handle *h, size_t bank) {
     L.flux = o;
     o = up(o + nc * (size_t)h->nbatch * (size_t)h->nbins_stride * sizeof(double));
     L.stats = o;
-    o = up(o + nc * S_NUM * sizeof(double));
+    o = up(o + stats_bytes(nc));
     L.counters = o;
     o = up(o + nc * C_NUM * sizeof(unsigned long long));
     L.cases = o;
@@ -174,7 +189,7 @@ DevLayout dev_layout(const cls_handle *h, size_t bank) {
     L.runs = o;
     o = up(o + runs_bytes(nc));
     L.chunk = o;
-    o = up(o + kMaxGroups * sizeof(unsigned long long));
+    o = up(o + counter_bytes(nc));
     L.bank = o;
     L.total = up(o + bank);
     return L;
@@ -185,7 +200,7 @@ int alloc_tallies(cls_handle *h) {
     const size_t nc = h->cases.size();
     const size_t nflux = nc * (size_t)h->nbatch * (size_t)h->nbins_stride;
     if (cudaMalloc(&h->d_flux, nflux * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&h->d_stats, nc * S_NUM * sizeof(double)) != cudaSuccess ||
+        cudaMalloc(&h->d_stats, stats_bytes(nc)) != cudaSuccess ||
         cudaMalloc(&h->d_counters, nc * C_NUM * sizeof(unsigned long long)) != cudaSuccess) {
         free_tallies(h);
         cudaGetLastError();
@@ -197,7 +212,7 @@ int alloc_tallies(cls_handle *h) {
 int zero_tallies(cls_handle *h) {
     const size_t nc = h->cases.size();
     CLS_CUDA(cudaMemset(h->d_flux, 0, nc * (size_t)h->nbatch * h->nbins_stride * sizeof(double)));
-    CLS_CUDA(cudaMemset(h->d_stats, 0, nc * S_NUM * sizeof(double)));
+    CLS_CUDA(cudaMemset(h->d_stats, 0, stats_bytes(nc)));
     CLS_CUDA(cudaMemset(h->d_counters, 0, nc * C_NUM * sizeof(unsigned long long)));
     h->next_history.assign(nc, 0);
     h->n_hist.assign(nc, 0);
@@ -255,7 +270,7 @@ int create_common(const double *params, int ncases, bool batch, cls_handle **out
     int rc = CLS_OK;
     if (cudaMalloc(&h->d_cases, ncases * sizeof(CaseParams)) != cudaSuccess ||
         cudaMalloc(&h->d_runs, runs_bytes(ncases)) != cudaSuccess ||
-        cudaMalloc(&h->d_chunk_counter, kMaxGroups * sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMalloc(&h->d_chunk_counter, counter_bytes(ncases)) != cudaSuccess ||
         cudaMallocHost(&h->h_runs, runs_bytes(ncases)) != cudaSuccess) {
         rc = CLS_E_NOMEM;
     }
@@ -279,7 +294,7 @@ uint64_t batch_len_for(uint64_t n, int nbatch) {
 }
 
 int region_bytes_for(const cls_handle *h) {
-    return region_bytes(h->opt.precision == CLS_PREC_FP32, h->nbins_stride);
+    return region_bytes(h->nbins_stride);
 }
 
 // FP32 regions are flushed into the FP64 global tallies after this many
@@ -345,6 +360,7 @@ std::vector<Group> plan_groups(const cls_handle *h, std::vector<int> *gk) {
 // from 0 and chunk counter g.
 struct RunPlan {
     int ngroups = 0;
+    size_t counter_bytes = 0;  // of the work counters in use
     int sched[kMaxGroups];
     int geom[kMaxGroups];
     LaunchArgs a[kMaxGroups];
@@ -361,22 +377,34 @@ int prepare_run(cls_handle *h, uint64_t n, uint64_t seed, RunPlan *plan) {
     LaunchArgs a;
     std::memset(&a, 0, sizeof(a));
     a.cases = h->d_cases;
-    a.chunk = (uint32_t)h->opt.chunk;
-    a.t = Tallies{h->d_flux, h->d_stats, h->d_counters, h->nbatch, h->nbins_stride};
+    a.t = Tallies{h->d_flux, h->d_stats, h->d_counters, h->nbatch, h->nbins_stride, stats_copies(h->cases.size())};
     a.seed = seed;
     a.rk = make_round_keys(seed);
     a.max_events = h->opt.max_events;
     a.region_bytes = region_bytes_for(h);
-    a.flush_every = (h->opt.precision == CLS_PREC_FP32) ? kFp32FlushHistories : 0;
+    a.flush_every = kFp32FlushHistories;
+
     // the record's binding is read from device memory at every launch (graph
     // replays see the current buffer); while nothing is recorded the kernels are
     // given no record at all and skip that read
     a.outcomes = h->outcome_codes ? outcome_record(h->d_runs, nc) : nullptr;
     int idx = 0;
+    uint64_t pieces = 0;
     plan->ngroups = (int)groups.size();
     for (int g = 0; g < plan->ngroups; ++g) {
         const int off = idx;
         uint64_t chunks = 0;
+        LaunchArgs &ag = plan->a[g];
+        ag = a;
+        ag.chunk = (uint32_t)h->opt.chunk;
+        ag.nruns = groups[g].ncases;
+        ag.claimed = h->d_chunk_counter + kMaxGroups + pieces;
+        const uint64_t warps = (uint64_t)h->sm_count * (h->opt.precision == CLS_PREC_FP32 ? 28 : 20);
+        if (groups[g].sched != CLS_SCHED_EVENT) {
+            plan_pieces(ag, n, batch_len_for(n, h->nbatch), warps, kMaxPieces);
+            pieces += (uint64_t)ag.pieces_per_run * ag.nruns;
+        }
+        const double cost = groups[g].cost * (double)n;
         for (int i = 0; i < nc; ++i) {
             const int k = h->order[i];
             if (gk[k] != g) continue;
@@ -386,19 +414,17 @@ int prepare_run(cls_handle *h, uint64_t n, uint64_t seed, RunPlan *plan) {
             r.batch_len = batch_len_for(n, h->nbatch);
             r.chunk_begin = chunks;
             r.case_index = k;
-            r.pad = 0;
+            plan_claims(r, h->cases[k], cost, warps, ag.chunk, (uint32_t)h->opt.chunk);
             chunks += (n + h->opt.chunk - 1) / h->opt.chunk;
         }
-        LaunchArgs &ag = plan->a[g];
-        ag = a;
         ag.runs = h->d_runs + off;
-        ag.nruns = idx - off;
         ag.total_chunks = chunks;
         ag.chunk_counter = h->d_chunk_counter + g;
         ag.warp_counts = (groups[g].geom == 0 || groups[g].cost < kWarpCountCost * groups[g].ncases) ? 1 : 0;
         plan->sched[g] = groups[g].sched;
         plan->geom[g] = groups[g].geom;
     }
+    plan->counter_bytes = (kMaxGroups + pieces) * sizeof(unsigned long long);
     OutcomeRecord *rec = outcome_record(h->h_runs, nc);
     *rec = OutcomeRecord{nullptr, 0, 0};
     if (h->outcome_codes) {
@@ -437,7 +463,7 @@ int tracker_shape(cls_handle *h, int region_bytes, int sched, int geom, Shape *o
     const bool event = sched == CLS_SCHED_EVENT;
     const bool fp64 = h->opt.precision == CLS_PREC_FP64;
     // each warp owns two tally regions; wide meshes get fewer warps per block
-    const size_t per_warp = 2 * (size_t)region_bytes;
+    const size_t per_warp = event ? 2 * (size_t)region_bytes : history_warp_bytes(region_bytes);
     const int fit_warps = (int)std::min<size_t>(kMaxSmemPerBlock / per_warp, 8);
     if (fit_warps < 1) return CLS_E_INVAL;
     // the history trackers' launch bounds
@@ -605,7 +631,14 @@ int fetch_case(cls_handle *h, int k, std::vector<double> &flux, double stats[S_N
     const size_t nfl = (size_t)h->nbatch * h->nbins_stride;
     flux.resize(nfl);
     CLS_CUDA(cudaMemcpy(flux.data(), h->d_flux + (size_t)k * nfl, nfl * sizeof(double), cudaMemcpyDeviceToHost));
-    CLS_CUDA(cudaMemcpy(stats, h->d_stats + (size_t)k * S_NUM, S_NUM * sizeof(double), cudaMemcpyDeviceToHost));
+    const int copies = stats_copies(h->cases.size());
+    double st[32 * S_NUM];
+    CLS_CUDA(cudaMemcpy(st, h->d_stats + (size_t)k * copies * S_NUM, copies * S_NUM * sizeof(double),
+                        cudaMemcpyDeviceToHost));
+    for (int q = 0; q < S_NUM; ++q) {
+        stats[q] = 0.0;
+        for (int i = 0; i < copies; ++i) stats[q] += st[i * S_NUM + q];
+    }
     CLS_CUDA(cudaMemcpy(ct, h->d_counters + (size_t)k * C_NUM, C_NUM * sizeof(unsigned long long),
                         cudaMemcpyDeviceToHost));
     return CLS_OK;
@@ -996,7 +1029,7 @@ int cls_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
     if (rc) return rc;
     CLS_CUDA(cudaMemcpyAsync(h->d_runs, h->h_runs, runs_bytes(h->cases.size()), cudaMemcpyHostToDevice, s));
     CLS_CUDA(cudaEventRecord(h->runs_copied, s));
-    CLS_CUDA(cudaMemsetAsync(h->d_chunk_counter, 0, kMaxGroups * sizeof(unsigned long long), s));
+    CLS_CUDA(cudaMemsetAsync(h->d_chunk_counter, 0, plan.counter_bytes, s));
     for (int g = 0; g < plan.ngroups && !rc; ++g) rc = launch_tracker(h, plan.a[g], plan.sched[g], plan.geom[g], sh[g], s);
     if (rc) return rc;
     rc = record_pair(h, s, false);
@@ -1026,8 +1059,7 @@ int cls_batch_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
     const int key[10] = {h->opt.precision, h->opt.schedule, h->opt.block, h->opt.chunk, (int)h->opt.max_events,
                          h->opt.blocks_per_sm, (int)(seed & 0x7fffffff), (int)(seed >> 31), h->opt.group_geometry,
                          h->outcome_codes != nullptr};
-    std::vector<uint64_t> tc(plan.ngroups);
-    for (int g = 0; g < plan.ngroups; ++g) tc[g] = plan.a[g].total_chunks;
+    const std::vector<uint64_t> tc = {n};  // the launches' work distribution is captured with them
     if (h->graph_exec && (tc != h->graph_total_chunks || std::memcmp(key, h->graph_key, sizeof(key))))
         destroy_graph(h);
     if (!h->graph_exec) {
@@ -1048,7 +1080,7 @@ int cls_batch_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
             h->join_events.push_back(e);
         }
         CLS_CUDA(cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e = cudaMemsetAsync(h->d_chunk_counter, 0, kMaxGroups * sizeof(unsigned long long), h->capture_stream);
+        cudaError_t e = cudaMemsetAsync(h->d_chunk_counter, 0, plan.counter_bytes, h->capture_stream);
         if (e == cudaSuccess && plan.ngroups > 1) e = cudaEventRecord(h->join_events[0], h->capture_stream);
         int lrc = (e == cudaSuccess) ? CLS_OK : CLS_E_CUDA;
         for (int g = 0; g < plan.ngroups && !lrc; ++g) {
@@ -1262,7 +1294,7 @@ int cls_bind_workspace(cls_handle *h, void *d_workspace, size_t bytes) {
         int rc = CLS_OK;
         if (cudaMalloc(&h->d_cases, h->cases.size() * sizeof(CaseParams)) != cudaSuccess ||
             cudaMalloc(&h->d_runs, runs_bytes(h->cases.size())) != cudaSuccess ||
-            cudaMalloc(&h->d_chunk_counter, kMaxGroups * sizeof(unsigned long long)) != cudaSuccess) {
+            cudaMalloc(&h->d_chunk_counter, counter_bytes(h->cases.size())) != cudaSuccess) {
             cudaGetLastError();
             rc = CLS_E_NOMEM;
         }

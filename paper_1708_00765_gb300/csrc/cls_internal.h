@@ -43,7 +43,8 @@ struct RunCase {
     uint64_t batch_len;
     uint64_t chunk_begin;
     int32_t case_index;  // index into the CaseParams array / tally blocks
-    int32_t pad;
+    uint16_t claim_bits; // history tracker: a claim in this run takes at most chunk 2^claim_bits histories
+    uint16_t refill_min; // history tracker: lanes that wait before histories end and start
 };
 
 // The caller's per-history outcome record (cls_record_outcomes), kept in
@@ -67,7 +68,7 @@ enum Event { EV_LEAK_X0 = 0, EV_LEAK_XL = 1, EV_REFLECT = 2, EV_SCATTER = 3, EV_
 
 // Device tallies of all cases.  Case k owns
 //   flux     + k * nbatch * nbins_stride   [nbatch][nbins_stride] doubles
-//   stats    + k * S_NUM                   doubles
+//   stats    + k * stats_copies * S_NUM    [stats_copies][S_NUM] doubles, to be summed
 //   counters + k * C_NUM                   u64
 struct Tallies {
     double *flux;
@@ -75,6 +76,7 @@ struct Tallies {
     unsigned long long *counters;
     int nbatch;
     int nbins_stride;
+    int stats_copies;
 };
 
 // The ten round keys of Philox4x32-10 for one seed: (k0, k1) of round r are
@@ -102,14 +104,21 @@ struct LaunchArgs {
     const CaseParams *cases;
     const RunCase *runs;  // in chunk order (largest estimated cost first)
     int nruns;
-    uint32_t chunk;       // histories per chunk (divides 1024)
-    uint64_t total_chunks;
-    unsigned long long *chunk_counter;  // zeroed before each launch
+    uint32_t chunk;       // event tracker: histories per chunk (divides 1024); history tracker: the least that a warp claims
+    uint64_t total_chunks;              // event tracker
+    unsigned long long *chunk_counter;  // zeroed before each launch; history tracker: its tickets
+    // history tracker: each run entry's histories in pieces of piece_len (whole
+    // statistics batches; the last one shorter), pieces_per_run of them; the
+    // histories claimed of piece p (of run entry p / pieces_per_run) are counted
+    // in claimed[p], zeroed before each launch; `team` warps start on each piece
+    unsigned long long *claimed;
+    uint64_t piece_len;
+    uint32_t pieces_per_run, team;
     Tallies t;
     uint64_t seed;
     uint32_t max_events;
     int region_bytes;     // bytes per warp tally region (see region_bytes())
-    int flush_every;      // flush a region after this many histories were fed into it (0: never)
+    uint32_t flush_every; // FP32: flush a region after this many histories were fed into it
     int warp_counts;      // history tracker: its short-history instance (warp-summed counters, sparse deposits)
     const OutcomeRecord *outcomes;  // per-history outcome record, or nullptr (never recorded)
     // event schedule only
@@ -130,25 +139,28 @@ struct TraceArgs {
     int *n_rows;
 };
 
-// A warp tally region: the bins, then S_NUM FP64 statistics and C_NUM u64
+// A warp tally region: the bins, then S_NUM FP64 statistics and C_NUM
 // counters, then each lane's own copy of the per-history statistics (S_NUM x
-// 32 doubles, statistic-major), which a lane updates without atomics when its
-// history ends and the flush sums over the warp; padded to 16 bytes.
-//   FP64 walk: nbins_stride FP64 bins, each flight scored bin by bin.
-//   FP32 walk: nbins_stride + 1 entries of a fixed-point difference array
-//     (u64, 32 fraction bits): a flight adds its end-bin partials and its
-//     interior-bin length with at most four integer atomics, and the flush
-//     takes the exact prefix sum, so the FP32 walk's deposits are summed
-//     without rounding (FP64 is used from the flush on).
-__host__ __device__ inline int region_bins_bytes(bool fixed, int nbins_stride) {
-    return 8 * (nbins_stride + (fixed ? 1 : 0));
+// 32 words of 8 bytes, statistic-major), which a lane updates without atomics
+// when its history ends and the flush sums over the warp; padded to 16 bytes.
+// The bins are nbins_stride + 1 entries of a fixed-point difference array: a
+// flight adds its end-bin partials and its interior-bin length with at most
+// four integer additions, whatever its length, and the flush takes the exact
+// prefix sum (FP64 is used from the flush on).  Entries and counters are 64
+// bits in two arrays of 32-bit halves, low halves first: shared memory adds 32
+// bits natively, 64 bits only by a compare-and-swap loop (cls_device.cuh).
+__host__ __device__ inline int region_bins_bytes(int nbins_stride) { return 8 * (nbins_stride + 1); }
+__host__ __device__ inline int region_lane_stats_offset(int nbins_stride) {
+    return region_bins_bytes(nbins_stride) + 8 * (S_NUM + C_NUM);
 }
-__host__ __device__ inline int region_lane_stats_offset(bool fixed, int nbins_stride) {
-    return region_bins_bytes(fixed, nbins_stride) + 8 * (S_NUM + C_NUM);
+__host__ __device__ inline int region_bytes(int nbins_stride) {
+    return (region_lane_stats_offset(nbins_stride) + 8 * 32 * S_NUM + 15) & ~15;
 }
-__host__ __device__ inline int region_bytes(bool fixed, int nbins_stride) {
-    return (region_lane_stats_offset(fixed, nbins_stride) + 8 * 32 * S_NUM + 15) & ~15;
-}
+
+// Dynamic shared memory of a warp of the history tracker: two tally regions and
+// its feeding state (cls_device.cuh's WarpFeed).
+constexpr int kWarpFeedBytes = 112;
+inline size_t history_warp_bytes(int region) { return 2 * (size_t)region + kWarpFeedBytes; }
 
 // Largest block of the event tracker (its launch bounds: 2 such blocks per SM).
 constexpr int kEventBlockThreads = 256;

@@ -28,14 +28,17 @@ namespace {
 
 using namespace cls;
 
+constexpr int kNoallocMaxPieces = 64 * CLS_NOALLOC_MAX_CASES;
+
 struct NoallocScratch {
     CaseParams cases[CLS_NOALLOC_MAX_CASES];
     RunCase runs[CLS_NOALLOC_MAX_CASES];
     unsigned long long chunk_counter;
+    unsigned long long claimed[kNoallocMaxPieces];
 };
 
 // The static scratch: every device that loads the library holds one copy of
-// it (about 16 KB) until the process exits.
+// it (about 48 KB) until the process exits.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoallocScratch)];
 
 // One call's case parameters and work list, handed to the set-up kernel by
@@ -51,11 +54,12 @@ static_assert(sizeof(NoallocImage) < 32000, "kernel arguments are limited to 32 
 
 // Writes the call's cases and work list into the scratch and clears the work
 // counter; runs before the tracker on the same stream.
-__global__ void noalloc_setup(NoallocScratch *scratch, const NoallocImage img) {
+__global__ void noalloc_setup(NoallocScratch *scratch, const NoallocImage img, int npieces) {
     for (int i = threadIdx.x; i < img.ncases; i += blockDim.x) {
         scratch->cases[i] = img.cases[i];
         scratch->runs[i] = img.runs[i];
     }
+    for (int i = threadIdx.x; i < npieces; i += blockDim.x) scratch->claimed[i] = 0ull;
     if (threadIdx.x == 0) scratch->chunk_counter = 0ull;
 }
 
@@ -115,36 +119,37 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
     img.ncases = ncases;
     const uint64_t q = 1024ull * (uint64_t)nbatch;
     const uint64_t batch_len = 1024ull * ((n + q - 1) / q > 0 ? (n + q - 1) / q : 1);
-    const int chunk = 256;
-    uint64_t chunk_begin = 0;
-    for (int k = 0; k < ncases; ++k) {
-        img.cases[k] = make_case(params + 9 * (size_t)k, (uint32_t)k);
-        RunCase &r = img.runs[k];
-        r.first = first;
-        r.n = n;
-        r.batch_len = batch_len;
-        r.chunk_begin = chunk_begin;
-        r.case_index = k;
-        chunk_begin += (n + chunk - 1) / chunk;
-    }
-
+    const uint64_t tracker_warps = (uint64_t)sm_count * 20;
     LaunchArgs a;
     std::memset(&a, 0, sizeof(a));
     a.cases = scratch->cases;
     a.runs = scratch->runs;
     a.nruns = ncases;
-    a.chunk = chunk;
-    a.total_chunks = chunk_begin;
+    plan_pieces(a, n, batch_len, tracker_warps, kNoallocMaxPieces);
     a.chunk_counter = &scratch->chunk_counter;
-    a.t = Tallies{d_flux, d_stats, d_counters, nbatch, nbins_stride};
+    a.claimed = scratch->claimed;
+    a.t = Tallies{d_flux, d_stats, d_counters, nbatch, nbins_stride, 1};
     a.seed = seed;
     a.rk = make_round_keys(seed);
     a.max_events = 100000000u;
-    a.region_bytes = region_bytes(false, nbins_stride);
-    a.flush_every = 0;
+    a.region_bytes = region_bytes(nbins_stride);
     a.warp_counts = 1;
 
-    const size_t per_warp = 2 * (size_t)a.region_bytes;
+    double cost = 0.0;
+    for (int k = 0; k < ncases; ++k) {
+        img.cases[k] = make_case(params + 9 * (size_t)k, (uint32_t)k);
+        cost += img.cases[k].cost * (double)n;
+    }
+    for (int k = 0; k < ncases; ++k) {
+        RunCase &r = img.runs[k];
+        r.first = first;
+        r.n = n;
+        r.batch_len = batch_len;
+        r.case_index = k;
+        plan_claims(r, img.cases[k], cost, tracker_warps, a.chunk, 256);  // the chunk option's default
+    }
+
+    const size_t per_warp = history_warp_bytes(a.region_bytes);
     int warps = (int)((200 * 1024) / per_warp);
     warps = warps > kHistoryBlockFp64 / 32 ? kHistoryBlockFp64 / 32 : warps;
     if (warps < 1) return CLS_E_INVAL;
@@ -156,7 +161,7 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
     if (bps < 1) return CLS_E_INVAL;
 
     cudaStream_t s = (cudaStream_t)stream;
-    noalloc_setup<<<1, 64, 0, s>>>(scratch, img);
+    noalloc_setup<<<1, 256, 0, s>>>(scratch, img, (int)(a.pieces_per_run * a.nruns));
     if (cudaGetLastError() != cudaSuccess) return CLS_E_CUDA;
     history_kernel<double, 0><<<sm_count * bps, block, smem, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? CLS_OK : CLS_E_CUDA;
