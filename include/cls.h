@@ -215,7 +215,9 @@ int cls_reset(cls_handle *h);
  * current cases and options -- flux tallies [cases][nbatch][nbins_stride]
  * doubles, statistics, counters, the case table, the work list, the work
  * counters and, when the handle's schedule (or a case's) is the event schedule
- * or still automatic, the event tracker's particle bank for the current launch
+ * or still automatic, the event tracker's particle bank, else the buffer in
+ * which the history tracker leaves a launch's last histories (optional: with
+ * less room it walks them itself), for the current launch
  * shape (for an automatic schedule, the larger of the autotuner's event
  * candidates).  Errors: CLS_E_INVAL, CLS_E_CUDA. */
 int cls_workspace_bytes(cls_handle *h, size_t *bytes);
@@ -413,7 +415,7 @@ int cls_debug_fixed32(const float *c, int n, unsigned long long *out);
  * options; per-history event cap 1e8).  The call is asynchronous, so it cannot
  * report capped histories as CLS_E_EVENT_LIMIT: they show in d_counters[k][7].
  *
- * Scratch (case parameters, work list, work counters; about 48 KB) lives in a
+ * Scratch (case parameters, work list, work counters; about 560 KB) lives in a
  * static device array that every GPU loading the library holds until the
  * process exits.  The first call on each device looks up that array's device
  * address (with the device current) and keeps it for the life of the process;

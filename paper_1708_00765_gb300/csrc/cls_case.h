@@ -45,39 +45,70 @@ inline double cost_estimate(const CaseParams &c) {
 }
 
 // How a history-tracker launch of n histories in each of `nruns` run entries is
-// claimed by about `warps` warps (LaunchArgs): pieces of whole statistics
-// batches, at most max_pieces of them; as many warps start on a piece as it
-// takes to employ all; and the least a warp claims is 32 histories, a warp's
-// lanes, or where that would not go round, a power of two below.
-inline void plan_pieces(LaunchArgs &a, uint64_t n, uint64_t batch_len, uint64_t warps, uint64_t max_pieces) {
+// claimed (LaunchArgs): pieces of whole statistics batches, at most max_pieces
+// of them; as many warps start on a piece as it takes to employ all; and the
+// least a warp claims is 32 histories, a warp's lanes, or where that would not
+// go round, a power of two below.  `warps`: about as many as the launch has.
+// Runs of up to kNarrowHistories histories for each warp of the narrow walk go
+// to it alone (a.narrow): measured on the 3D box in FP64, 1e4 histories (5.5 a
+// warp) take 1.04 ms there and 1.10 ms in the tracker, 1e5 take 6.4 and 2.6 ms;
+// on the rod in FP32, 55 and 84 us, 260 and 113 us.
+constexpr double kNarrowHistories = 8.0;
+// Launches whose histories average this many events or more by the estimate
+// hand their warps' last histories over to the narrow walk: it walks a history
+// twice as fast, but only one per warp.  Measured: the diffusive box (153
+// events) at 1e6 histories in FP32 20.4 -> 18.7 ms, in FP64 75 -> 66 ms; the
+// box L = 10 (47 events) at 1e5 in FP64 2.6 -> 2.8 ms.
+constexpr double kHandOverEvents = 128.0;
+
+// Estimated events per history: about cost^(3/4) (the cost estimate is within a
+// factor of two for short histories and several times too high for scattering media).
+inline double estimated_events(double cost) { return std::pow(std::max(cost, 1.0), 0.75); }
+
+inline void plan_pieces(LaunchArgs &a, uint64_t n, uint64_t batch_len, double mean_cost, int sm_count, bool fp32,
+                        uint64_t max_pieces) {
+    const double total = (double)n * a.nruns;
+    const double narrow_warps = (double)sm_count * kNarrowBlocks * (kNarrowBlock / 32);
+    a.narrow = total <= kNarrowHistories * narrow_warps;
+    const double warps = a.narrow ? std::min(total, narrow_warps) : sm_count * (fp32 ? 28.0 : 20.0);
     const uint64_t used = (n + batch_len - 1) / batch_len;  // batches
     const uint64_t per_run = std::max<uint64_t>(1, std::min<uint64_t>(std::min<uint64_t>(used, 64), max_pieces / a.nruns));
     const uint64_t batches = (used + per_run - 1) / per_run;
     a.piece_len = batches * batch_len;
     a.pieces_per_run = (uint32_t)((used + batches - 1) / batches);
-    const uint64_t pieces = (uint64_t)a.pieces_per_run * a.nruns;
-    a.team = (uint32_t)((warps + pieces - 1) / pieces);
-    const double per_warp = (double)n * a.nruns / (double)warps;
-    a.chunk = 32;
-    while (a.chunk > 1 && (double)a.chunk > per_warp) a.chunk >>= 1;
+    a.team = (uint32_t)std::ceil(warps / ((double)a.pieces_per_run * a.nruns));
+    a.hand_over = estimated_events(mean_cost) >= kHandOverEvents ? kHandOver : 0;
+    a.chunk = a.narrow ? 1 : 32;
+    while (a.chunk > 1 && (double)a.chunk > total / warps) a.chunk >>= 1;
+}
+
+// Blocks of the narrow walk: as many as the run has histories for its warps.
+inline int narrow_grid(const LaunchArgs &a, uint64_t n, int sm_count) {
+    const int full = sm_count * kNarrowBlocks, warps = kNarrowBlock / 32;
+    return a.narrow ? (int)std::min((double)full, std::ceil((double)n * a.nruns / warps)) : full;
+}
+
+inline size_t narrow_smem(const LaunchArgs &a, bool fp64) {
+    return (size_t)(kNarrowBlock / 32) * (narrow_memory_bytes(fp64) + a.region_bytes);
 }
 
 // Claim limit and refill threshold of a run entry (RunCase), from the
 // estimated cost of its histories and of all histories of the launch.  A claim
 // takes at most 1/8 of a warp's share of the launch by that estimate (a sweep's
 // longest cases have a hundred times its shortest's events), and at most 32
-// times the chunk option.  Events per history are about cost^(3/4)
-// (measured: the estimate is within a factor of two for short histories and
-// several times too high for scattering media).
-inline void plan_claims(RunCase &r, const CaseParams &c, double launch_cost, uint64_t warps, uint32_t chunk,
+// times the chunk option.
+inline void plan_claims(RunCase &r, const CaseParams &c, double launch_cost, int sm_count, uint32_t chunk,
                         uint32_t option) {
-    const double share = launch_cost / (8.0 * (double)warps * std::max(c.cost, 1.0) * chunk);
+    const double share = launch_cost / (8.0 * 24.0 * sm_count * std::max(c.cost, 1.0) * chunk);  // 24: about the warps of an SM
     const double most = std::min(share, 32.0 * option / chunk);
     int bits = 0;
     while (bits < 40 && std::ldexp(1.0, bits + 1) <= most) ++bits;
     r.claim_bits = (uint16_t)bits;
-    const double events = std::pow(std::max(c.cost, 1.0), 0.75);
-    r.refill_min = (uint16_t)std::min(12.0, std::max(2.0, std::floor(5.2 * std::sqrt(32.0 / events) + 0.5)));
+    // lanes die 32 / events per step, and waiting idles half of refill_min of them.  Measured, 2 / 4 / 8 / 12 / 16
+    // lanes: box L = 10 (47 events, FP32, 1e8) 101 / 97 / 100 / 107 / 118 ms; sweep (5 events, 256 x 1e6) 50.8 /
+    // 49.4 / 47.3 / 46.5 / 47.1 ms
+    const double wait = std::floor(5.2 * std::sqrt(32.0 / estimated_events(c.cost)) + 0.5);
+    r.refill_min = (uint16_t)std::min(12.0, std::max(2.0, wait));
 }
 
 // The kernels' view of one validated case: p_0 = Lambda_0 / (Lambda_0 +

@@ -182,6 +182,7 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
     const size_t gwarp = (size_t)blockIdx.x * (blockDim.x >> 5) + warp;
     unsigned char *bank = reinterpret_cast<unsigned char *>(a.bank) + gwarp * 2 * buf_bytes;
     const RoundKeys &key = a.rk;
+    PhiloxDraws<P, G, false> draws{key};
     const int nbs = a.t.nbins_stride;
     const unsigned lt_mask = (1u << lane) - 1u;
 
@@ -310,7 +311,7 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
                 int o = -1;
                 f.k0 = 0;
                 f.k1 = -1;
-                if (alive) o = step<P, false, G>(s, a.cases[ci], key, a.max_events, f, nullptr, reg == 2);
+                if (alive) o = step<P, false, G>(s, a.cases[ci], draws, a.max_events, f, nullptr, reg == 2);
                 deposited += warp_deposit<P>(regions, rb, nbs, reg, a.t.flux, goff, f, lane);
                 if constexpr (sizeof(P) == 8) {  // before a bin's sum can outgrow its 64 bits
                     if (__any_sync(CLS_FULL_MASK, deposited >= kDepositBound)) {

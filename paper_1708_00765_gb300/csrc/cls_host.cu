@@ -49,10 +49,11 @@ struct Options {
 // persistent launch with its own chunk counter.
 constexpr int kMaxGroups = 10;  // 2 schedules x 5 geometries
 
-// Work counters on the device: one per group, then the claimed histories of
+// Work counters on the device: three per group, then the claimed histories of
 // every piece of the history-tracker groups (LaunchArgs::claimed), at most
 // kMaxPieces (or one per case) in a group and 64 per case.
 constexpr uint64_t kMaxPieces = 32768;
+constexpr int kGroupCounters = 3 * kMaxGroups;  // each group's tickets; histories handed over; and taken
 
 }  // namespace
 
@@ -136,7 +137,7 @@ int stats_copies(size_t ncases) { return ncases <= 1024 ? 32 : ncases <= 8192 ? 
 size_t stats_bytes(size_t ncases) { return ncases * stats_copies(ncases) * S_NUM * sizeof(double); }
 
 size_t counter_bytes(size_t ncases) {
-    return (kMaxGroups + std::min<size_t>(64 * ncases, ncases + kMaxGroups * kMaxPieces)) * sizeof(unsigned long long);
+    return (kGroupCounters + std::min<size_t>(64 * ncases, ncases + kMaxGroups * kMaxPieces)) * sizeof(unsigned long long);
 }
 
 void free_tallies(cls_handle *h) {
@@ -398,10 +399,10 @@ int prepare_run(cls_handle *h, uint64_t n, uint64_t seed, RunPlan *plan) {
         ag = a;
         ag.chunk = (uint32_t)h->opt.chunk;
         ag.nruns = groups[g].ncases;
-        ag.claimed = h->d_chunk_counter + kMaxGroups + pieces;
-        const uint64_t warps = (uint64_t)h->sm_count * (h->opt.precision == CLS_PREC_FP32 ? 28 : 20);
+        ag.claimed = h->d_chunk_counter + kGroupCounters + pieces;
         if (groups[g].sched != CLS_SCHED_EVENT) {
-            plan_pieces(ag, n, batch_len_for(n, h->nbatch), warps, kMaxPieces);
+            plan_pieces(ag, n, batch_len_for(n, h->nbatch), groups[g].cost / groups[g].ncases, h->sm_count,
+                        h->opt.precision == CLS_PREC_FP32, kMaxPieces);
             pieces += (uint64_t)ag.pieces_per_run * ag.nruns;
         }
         const double cost = groups[g].cost * (double)n;
@@ -414,17 +415,19 @@ int prepare_run(cls_handle *h, uint64_t n, uint64_t seed, RunPlan *plan) {
             r.batch_len = batch_len_for(n, h->nbatch);
             r.chunk_begin = chunks;
             r.case_index = k;
-            plan_claims(r, h->cases[k], cost, warps, ag.chunk, (uint32_t)h->opt.chunk);
+            plan_claims(r, h->cases[k], cost, h->sm_count, ag.chunk, (uint32_t)h->opt.chunk);
             chunks += (n + h->opt.chunk - 1) / h->opt.chunk;
         }
         ag.runs = h->d_runs + off;
         ag.total_chunks = chunks;
         ag.chunk_counter = h->d_chunk_counter + g;
+        ag.handed = h->d_chunk_counter + kMaxGroups + g;
+        ag.taken = h->d_chunk_counter + 2 * kMaxGroups + g;
         ag.warp_counts = (groups[g].geom == 0 || groups[g].cost < kWarpCountCost * groups[g].ncases) ? 1 : 0;
         plan->sched[g] = groups[g].sched;
         plan->geom[g] = groups[g].geom;
     }
-    plan->counter_bytes = (kMaxGroups + pieces) * sizeof(unsigned long long);
+    plan->counter_bytes = (kGroupCounters + pieces) * sizeof(unsigned long long);
     OutcomeRecord *rec = outcome_record(h->h_runs, nc);
     *rec = OutcomeRecord{nullptr, 0, 0};
     if (h->outcome_codes) {
@@ -452,7 +455,9 @@ struct Shape {
     int grid, block;
     size_t smem;
     uint32_t bank_slots;  // event schedule: slots per block and buffer
-    size_t bank_off;      // event schedule: this launch's slice of the bank
+    size_t bank_off;      // this launch's slice of the bank: the event schedule's particles, the
+                          // history schedule's hand-over buffer
+    uint32_t straggler_cap;  // history schedule: slots of that buffer
 };
 
 size_t shape_bank_bytes(const cls_handle *h, const Shape &sh) {
@@ -485,13 +490,16 @@ int tracker_shape(cls_handle *h, int region_bytes, int sched, int geom, Shape *o
     out->smem = smem;
     out->bank_slots = event ? (uint32_t)(h->opt.bank > 0 ? ((h->opt.bank + 31) & ~31) : 128) : 0u;
     out->bank_off = 0;
+    out->straggler_cap = event ? 0u : (uint32_t)(out->grid * (block / 32) * kHandOver);
     return CLS_OK;
 }
 
-// Shapes of a run's launches; the event launches take consecutive slices of
-// one particle bank (grid warps x 2 buffers x slots x fields x 16 B each, all
-// of a run's launches may run at once).  *bank: the bytes they need together.
-int plan_shapes(cls_handle *h, const RunPlan &plan, Shape *sh, size_t *bank) {
+// Shapes of a run's launches, which take consecutive slices of one bank (all of
+// a run's launches may run at once): the event launches grid warps x 2 buffers x
+// slots x fields x 16 B each, the history launches, after them, their hand-over
+// buffers.  *bank: the bytes they need together; a hand-over buffer is cut
+// where it would end beyond `limit` (the tracker walks what it cannot hand over).
+int plan_shapes(cls_handle *h, const RunPlan &plan, Shape *sh, size_t *bank, size_t limit = ~(size_t)0) {
     *bank = 0;
     for (int g = 0; g < plan.ngroups; ++g) {
         const int rc = tracker_shape(h, plan.a[g].region_bytes, plan.sched[g], plan.geom[g], &sh[g]);
@@ -501,8 +509,18 @@ int plan_shapes(cls_handle *h, const RunPlan &plan, Shape *sh, size_t *bank) {
             *bank += (shape_bank_bytes(h, sh[g]) + 255) & ~(size_t)255;
         }
     }
+    for (int g = 0; g < plan.ngroups; ++g) {
+        if (plan.sched[g] == CLS_SCHED_EVENT) continue;
+        sh[g].bank_off = *bank;
+        const size_t room = *bank < (limit & ~(size_t)255) ? ((limit & ~(size_t)255) - *bank) / kStragglerBytes : 0;
+        sh[g].straggler_cap = (uint32_t)std::min<size_t>(sh[g].straggler_cap, room);
+        *bank += ((size_t)sh[g].straggler_cap * kStragglerBytes + 255) & ~(size_t)255;
+    }
     return CLS_OK;
 }
+
+// Bytes of the bank that runs may use: a bound workspace's beyond its other buffers.
+size_t bank_limit(const cls_handle *h) { return h->ws ? h->ws_bytes - h->ws_bank_off : ~(size_t)0; }
 
 // Make sure the particle bank holds `need` bytes.  Done before any graph capture.
 int ensure_bank(cls_handle *h, size_t need) {
@@ -527,15 +545,11 @@ int ensure_bank(cls_handle *h, size_t need) {
     return CLS_OK;
 }
 
-// Bytes of event bank the handle's current options need: none unless the
-// handle's schedule (or a case's) is the event schedule or still automatic
-// (then the larger of the autotuner's event candidates, every group on the
-// event schedule).
+// Bytes of bank the handle's current options need (plan_shapes; for an
+// automatic schedule the largest of the autotuner's event candidates, every
+// group on the event schedule).
 int bank_need(cls_handle *h, size_t *need) {
     *need = 0;
-    bool event = h->opt.schedule == CLS_SCHED_EVENT || h->opt.schedule == CLS_SCHED_AUTO;
-    for (size_t k = 0; k < h->cases.size(); ++k) event |= case_schedule(h, (int)k) == CLS_SCHED_EVENT;
-    if (!event) return CLS_OK;
     const Options saved = h->opt;
     const int saved_bps = h->used_blocks_per_sm;
     int rc = CLS_OK;
@@ -582,7 +596,7 @@ int carve_workspace(cls_handle *h, size_t bank) {
     return zero_tallies(h);
 }
 
-int launch_tracker(cls_handle *h, LaunchArgs a, int sched, int geom, const Shape &sh, cudaStream_t s) {
+int launch_tracker(cls_handle *h, LaunchArgs a, int sched, int geom, const Shape &sh, uint64_t n, cudaStream_t s) {
     cudaError_t e;
     const bool fp64 = h->opt.precision == CLS_PREC_FP64;
     if (sched == CLS_SCHED_EVENT) {
@@ -592,8 +606,17 @@ int launch_tracker(cls_handle *h, LaunchArgs a, int sched, int geom, const Shape
         e = fp64 ? launch_event_fp64(a, sh.grid, sh.block, sh.smem, s, geom)
                  : launch_event_fp32(a, sh.grid, sh.block, sh.smem, s, geom);
     } else {
-        e = fp64 ? launch_history_fp64(a, sh.grid, sh.block, sh.smem, s, geom)
-                 : launch_history_fp32(a, sh.grid, sh.block, sh.smem, s, geom);
+        a.stragglers = static_cast<unsigned char *>(h->d_bank) + sh.bank_off;
+        a.straggler_cap = sh.straggler_cap;
+        e = cudaSuccess;
+        if (!a.narrow)
+            e = fp64 ? launch_history_fp64(a, sh.grid, sh.block, sh.smem, s, geom)
+                     : launch_history_fp32(a, sh.grid, sh.block, sh.smem, s, geom);
+        if (e != cudaSuccess) return CLS_E_CUDA;
+        if (!a.narrow && a.hand_over == 0) return CLS_OK;
+        const int grid = narrow_grid(a, n, h->sm_count);
+        const size_t smem = narrow_smem(a, fp64);
+        e = fp64 ? launch_narrow_fp64(a, grid, smem, s, geom) : launch_narrow_fp32(a, grid, smem, s, geom);
     }
     return cuda_fail(e);
 }
@@ -1022,7 +1045,7 @@ int cls_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
     if (rc) return rc;
     Shape sh[kMaxGroups];
     size_t bank = 0;
-    rc = plan_shapes(h, plan, sh, &bank);
+    rc = plan_shapes(h, plan, sh, &bank, bank_limit(h));
     if (!rc) rc = ensure_bank(h, bank);
     if (rc) return rc;
     rc = record_pair(h, s, true);
@@ -1030,7 +1053,7 @@ int cls_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
     CLS_CUDA(cudaMemcpyAsync(h->d_runs, h->h_runs, runs_bytes(h->cases.size()), cudaMemcpyHostToDevice, s));
     CLS_CUDA(cudaEventRecord(h->runs_copied, s));
     CLS_CUDA(cudaMemsetAsync(h->d_chunk_counter, 0, plan.counter_bytes, s));
-    for (int g = 0; g < plan.ngroups && !rc; ++g) rc = launch_tracker(h, plan.a[g], plan.sched[g], plan.geom[g], sh[g], s);
+    for (int g = 0; g < plan.ngroups && !rc; ++g) rc = launch_tracker(h, plan.a[g], plan.sched[g], plan.geom[g], sh[g], n, s);
     if (rc) return rc;
     rc = record_pair(h, s, false);
     if (rc) return rc;
@@ -1065,7 +1088,7 @@ int cls_batch_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
     if (!h->graph_exec) {
         Shape sh[kMaxGroups];
         size_t bank = 0;
-        rc = plan_shapes(h, plan, sh, &bank);
+        rc = plan_shapes(h, plan, sh, &bank, bank_limit(h));
         if (!rc) rc = ensure_bank(h, bank);
         if (rc) return rc;
         if (!h->capture_stream) CLS_CUDA(cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking));
@@ -1086,7 +1109,7 @@ int cls_batch_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
         for (int g = 0; g < plan.ngroups && !lrc; ++g) {
             cudaStream_t gs = g == 0 ? h->capture_stream : h->aux_streams[g - 1];
             if (g > 0 && cudaStreamWaitEvent(gs, h->join_events[0], 0) != cudaSuccess) lrc = CLS_E_CUDA;
-            if (!lrc) lrc = launch_tracker(h, plan.a[g], plan.sched[g], plan.geom[g], sh[g], gs);
+            if (!lrc) lrc = launch_tracker(h, plan.a[g], plan.sched[g], plan.geom[g], sh[g], n, gs);
             if (!lrc && g > 0 && (cudaEventRecord(h->join_events[g], gs) != cudaSuccess ||
                                   cudaStreamWaitEvent(h->capture_stream, h->join_events[g], 0) != cudaSuccess))
                 lrc = CLS_E_CUDA;

@@ -114,6 +114,13 @@ struct LaunchArgs {
     unsigned long long *claimed;
     uint64_t piece_len;
     uint32_t pieces_per_run, team;
+    // histories handed from the history tracker to the narrow walk: slots of
+    // kStragglerBytes, the number handed over and taken (zeroed before each run)
+    unsigned char *stragglers;
+    unsigned long long *handed, *taken;
+    uint32_t straggler_cap;
+    int hand_over;        // history tracker: a warp with at most this many histories left, and none to claim, hands them over
+    int narrow;           // the narrow walk takes the whole run, from the pieces
     Tallies t;
     uint64_t seed;
     uint32_t max_events;
@@ -157,6 +164,14 @@ __host__ __device__ inline int region_bytes(int nbins_stride) {
     return (region_lane_stats_offset(nbins_stride) + 8 * 32 * S_NUM + 15) & ~15;
 }
 
+// The narrow walk (narrow_kernel): its blocks, the histories a warp of the
+// history tracker hands over to it at most, and the bytes of one; its dynamic
+// shared memory per warp is the draw buffer and feeding state, then one region.
+constexpr int kNarrowBlock = 128, kNarrowBlocks = 3;
+constexpr int kHandOver = 4;
+constexpr int kStragglerBytes = 128;
+__host__ __device__ constexpr int narrow_memory_bytes(bool fp64) { return (fp64 ? 4096 : 1280) + 112; }
+
 // Dynamic shared memory of a warp of the history tracker: two tally regions and
 // its feeding state (cls_device.cuh's WarpFeed).
 constexpr int kWarpFeedBytes = 112;
@@ -188,6 +203,8 @@ cudaError_t launch_history_fp64(const LaunchArgs &a, int grid, int block, size_t
 cudaError_t launch_history_fp32(const LaunchArgs &a, int grid, int block, size_t smem, cudaStream_t s, int geom);
 cudaError_t launch_event_fp64(const LaunchArgs &a, int grid, int block, size_t smem, cudaStream_t s, int geom);
 cudaError_t launch_event_fp32(const LaunchArgs &a, int grid, int block, size_t smem, cudaStream_t s, int geom);
+cudaError_t launch_narrow_fp64(const LaunchArgs &a, int grid, size_t smem, cudaStream_t s, int geom);
+cudaError_t launch_narrow_fp32(const LaunchArgs &a, int grid, size_t smem, cudaStream_t s, int geom);
 cudaError_t launch_trace_fp64(const TraceArgs &a, cudaStream_t s);
 cudaError_t launch_trace_fp32(const TraceArgs &a, cudaStream_t s);
 cudaError_t occupancy_history_fp64(int block, size_t smem, int *blocks_per_sm, int geom);

@@ -29,16 +29,18 @@ namespace {
 using namespace cls;
 
 constexpr int kNoallocMaxPieces = 64 * CLS_NOALLOC_MAX_CASES;
+constexpr int kNoallocStragglers = 4096;  // histories handed to the narrow walk; the tracker walks any others to their ends
 
 struct NoallocScratch {
     CaseParams cases[CLS_NOALLOC_MAX_CASES];
     RunCase runs[CLS_NOALLOC_MAX_CASES];
-    unsigned long long chunk_counter;
+    unsigned long long chunk_counter, handed, taken;
     unsigned long long claimed[kNoallocMaxPieces];
+    __align__(16) unsigned char stragglers[kNoallocStragglers * kStragglerBytes];
 };
 
 // The static scratch: every device that loads the library holds one copy of
-// it (about 48 KB) until the process exits.
+// it (about 560 KB) until the process exits.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoallocScratch)];
 
 // One call's case parameters and work list, handed to the set-up kernel by
@@ -60,7 +62,7 @@ __global__ void noalloc_setup(NoallocScratch *scratch, const NoallocImage img, i
         scratch->runs[i] = img.runs[i];
     }
     for (int i = threadIdx.x; i < npieces; i += blockDim.x) scratch->claimed[i] = 0ull;
-    if (threadIdx.x == 0) scratch->chunk_counter = 0ull;
+    if (threadIdx.x == 0) scratch->chunk_counter = scratch->handed = scratch->taken = 0ull;
 }
 
 constexpr int kMaxDevices = 64;
@@ -119,15 +121,23 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
     img.ncases = ncases;
     const uint64_t q = 1024ull * (uint64_t)nbatch;
     const uint64_t batch_len = 1024ull * ((n + q - 1) / q > 0 ? (n + q - 1) / q : 1);
-    const uint64_t tracker_warps = (uint64_t)sm_count * 20;
     LaunchArgs a;
     std::memset(&a, 0, sizeof(a));
     a.cases = scratch->cases;
     a.runs = scratch->runs;
     a.nruns = ncases;
-    plan_pieces(a, n, batch_len, tracker_warps, kNoallocMaxPieces);
+    double cost = 0.0;
+    for (int k = 0; k < ncases; ++k) {
+        img.cases[k] = make_case(params + 9 * (size_t)k, (uint32_t)k);
+        cost += img.cases[k].cost * (double)n;
+    }
+    plan_pieces(a, n, batch_len, cost / (double)n / ncases, sm_count, false, kNoallocMaxPieces);
     a.chunk_counter = &scratch->chunk_counter;
     a.claimed = scratch->claimed;
+    a.handed = &scratch->handed;
+    a.taken = &scratch->taken;
+    a.stragglers = scratch->stragglers;
+    a.straggler_cap = kNoallocStragglers;
     a.t = Tallies{d_flux, d_stats, d_counters, nbatch, nbins_stride, 1};
     a.seed = seed;
     a.rk = make_round_keys(seed);
@@ -135,18 +145,13 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
     a.region_bytes = region_bytes(nbins_stride);
     a.warp_counts = 1;
 
-    double cost = 0.0;
-    for (int k = 0; k < ncases; ++k) {
-        img.cases[k] = make_case(params + 9 * (size_t)k, (uint32_t)k);
-        cost += img.cases[k].cost * (double)n;
-    }
     for (int k = 0; k < ncases; ++k) {
         RunCase &r = img.runs[k];
         r.first = first;
         r.n = n;
         r.batch_len = batch_len;
         r.case_index = k;
-        plan_claims(r, img.cases[k], cost, tracker_warps, a.chunk, 256);  // the chunk option's default
+        plan_claims(r, img.cases[k], cost, sm_count, a.chunk, 256);  // the chunk option's default
     }
 
     const size_t per_warp = history_warp_bytes(a.region_bytes);
@@ -163,6 +168,8 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
     cudaStream_t s = (cudaStream_t)stream;
     noalloc_setup<<<1, 256, 0, s>>>(scratch, img, (int)(a.pieces_per_run * a.nruns));
     if (cudaGetLastError() != cudaSuccess) return CLS_E_CUDA;
-    history_kernel<double, 0><<<sm_count * bps, block, smem, s>>>(a);
-    return cudaGetLastError() == cudaSuccess ? CLS_OK : CLS_E_CUDA;
+    if (!a.narrow) history_kernel<double, 0><<<sm_count * bps, block, smem, s>>>(a);
+    if (cudaGetLastError() != cudaSuccess) return CLS_E_CUDA;
+    if (!a.narrow && a.hand_over == 0) return CLS_OK;
+    return launch_narrow_fp64(a, narrow_grid(a, n, sm_count), narrow_smem(a, true), s, 0) == cudaSuccess ? CLS_OK : CLS_E_CUDA;
 }
