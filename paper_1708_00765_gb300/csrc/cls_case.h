@@ -145,6 +145,10 @@ inline CaseParams make_case(const double *p, uint32_t case_id) {
     }
     c.thr_p053 = unit_threshold(c.p0, 53);
     c.thr_p024 = (uint32_t)unit_threshold((double)c.p0_f, 24);
+    // products of these in FP32 neither overflow nor lose bits
+    auto moderate = [](double v) { return v >= 0x1p-60 && v <= 0x1p60; };
+    c.filter = moderate(c.L) && moderate(c.lambda[0]) && moderate(c.lambda[1]) &&
+               (p[0] == 0 || moderate(1.0 / p[0])) && (p[1] == 0 || moderate(1.0 / p[1]));
     c.cost = cost_estimate(c);
     return c;
 }

@@ -345,7 +345,7 @@ template <typename P>
 struct History {
     P r[3];
     P w[3];
-    P iw[3];          // 1 / w (infinite when the component is 0)
+    P iw[3];          // 1 / w (infinite when the component is 0); [1] and [2] in the FP64 narrow walk only
     int m;
     uint32_t j;       // per-history draw index
     uint32_t c2, c3;  // words 2, 3 of the last Philox block (odd draws)
@@ -486,42 +486,25 @@ __device__ __forceinline__ CaseRegs<P> load_case(const CaseParams &c) {
 }
 
 template <typename P>
+__device__ __forceinline__ P recip_or_inf(P w) {
+    return Real<P>::is_zero(w) ? Real<P>::inf() : Real<P>::recip(w);
+}
+
+template <typename P>
 __device__ __forceinline__ void set_direction(History<P> &s, P wx, P wy, P wz) {
-    using R = Real<P>;
     s.w[0] = wx;
     s.w[1] = wy;
     s.w[2] = wz;
-    if constexpr (sizeof(P) == 8) {  // one copy of the integer reciprocal, three passes
-        P a = wx, b = wy, c = wz, r0 = P(0), r1 = P(0), r2 = P(0);
-#pragma unroll 1
-        for (int t = 0; t < 3; ++t) {
-            r0 = r1;
-            r1 = r2;
-            r2 = R::is_zero(a) ? R::inf() : R::recip(a);
-            a = b;
-            b = c;
-        }
-        s.iw[0] = r0;
-        s.iw[1] = r1;
-        s.iw[2] = r2;
-    } else {
-        s.iw[0] = R::is_zero(wx) ? R::inf() : R::recip(wx);
-        s.iw[1] = R::is_zero(wy) ? R::inf() : R::recip(wy);
-        s.iw[2] = R::is_zero(wz) ? R::inf() : R::recip(wz);
-    }
+    s.iw[0] = recip_or_inf(wx);
 }
 
-// Direction (wx, 0, 0) of the slab and the x-projected box: no reciprocal of
-// the zero components
+// Direction (wx, 0, 0) of the slab and the x-projected box
 template <typename P>
 __device__ __forceinline__ void set_direction_x(History<P> &s, P wx) {
-    using R = Real<P>;
     s.w[0] = wx;
     s.w[1] = P(0);
     s.w[2] = P(0);
-    s.iw[0] = R::is_zero(wx) ? R::inf() : R::recip(wx);
-    s.iw[1] = R::inf();
-    s.iw[2] = R::inf();
+    s.iw[0] = recip_or_inf(wx);
 }
 
 // Draw the pending direction of a 3D or extruded walk: mu, then the azimuth
@@ -589,8 +572,6 @@ __device__ __forceinline__ void source(History<P> &s, const CaseParams &cp, cons
             s.w[1] = P(0);
             s.w[2] = P(0);
             s.iw[0] = w;
-            s.iw[1] = R::inf();
-            s.iw[2] = R::inf();
         }
     } else if (gd == 11 || gd == 13) {
         uint32_t hi, lo;  // slab, projected box: mu = sqrt(xi)
@@ -601,8 +582,6 @@ __device__ __forceinline__ void source(History<P> &s, const CaseParams &cp, cons
         s.w[1] = P(0);
         s.w[2] = P(0);
         s.iw[0] = P(1);
-        s.iw[1] = R::inf();
-        s.iw[2] = R::inf();
     }
     s.m = draw_below(s, key, cp.thr_p053, cp.thr_p024) ? 0 : 1;
 }
@@ -788,6 +767,160 @@ __device__ __forceinline__ P face_distance(P r, P w, P iw, P L) {
     return R::is_zero(w) ? R::inf() : d;
 }
 
+// The next event: the flight's length and what ends it.
+template <typename P>
+struct Choice {
+    P l;
+    bool bnd, coll;   // boundary, collision; else interface
+    int face;         // 0: x = 0, 1: x = L, 2: lateral
+    bool on_y, on_z;  // reflection on a y and / or z face
+};
+
+// The smallest of the collision, interface and boundary distances: x faces,
+// then the lateral faces of the box; boundary, else collision, else interface.
+template <typename P, int G, typename Case>
+__device__ __forceinline__ Choice<P> choose_event(const History<P> &s, const Case &cp, P l_c, P l_i, P iy, P iz) {
+    using R = Real<P>;
+    const int gd = geometry<G>(cp);
+    const P INF = R::inf(), L = R::L(cp);
+    Choice<P> c;
+    c.face = R::pos(s.w[0]) ? 1 : 0;
+    P l_b = face_distance(s.r[0], s.w[0], s.iw[0], L);
+    P l_y = INF, l_z = INF;
+    if (gd == 3 || gd == 2) {  // lateral faces: y (and z in the box; the extruded geometry has none)
+        l_y = face_distance(s.r[1], s.w[1], iy, L);
+        if (R::lt(l_y, l_b)) {
+            l_b = l_y;
+            c.face = 2;
+        }
+        if (gd == 3) {
+            l_z = face_distance(s.r[2], s.w[2], iz, L);
+            if (R::lt(l_z, l_b)) {
+                l_b = l_z;
+                c.face = 2;
+            }
+        }
+    }
+    c.bnd = R::le(l_b, l_c) && R::le(l_b, l_i);
+    c.coll = !c.bnd && R::le(l_c, l_i);
+    c.l = c.bnd ? l_b : (c.coll ? l_c : l_i);
+    c.on_y = c.bnd && c.face == 2 && R::eq(l_y, l_b);
+    c.on_z = c.bnd && c.face == 2 && R::eq(l_z, l_b);
+    return c;
+}
+
+// l_c from -ln(1 - u) of its draw
+template <typename P, typename Case>
+__device__ __forceinline__ P collision_distance(const Case &cp, int m, P e_c) {
+    using R = Real<P>;
+    return R::pos(R::sigma(cp, m)) ? R::nonneg(e_c * R::inv_sigma(cp, m)) : R::inf();
+}
+
+// l_i from -ln(1 - u) of its draw
+template <typename P, int G, typename Case>
+__device__ __forceinline__ P interface_distance(const History<P> &s, const Case &cp, int m, P e_i) {
+    using R = Real<P>;
+    const int gd = geometry<G>(cp);
+    P l_i = R::lambda(cp, m) * e_i;
+    if (gd == 11) l_i *= R::abs(s.iw[0]);  // slab: the chord projected on x, Lambda/|mu|
+    else if (gd == 2) l_i /= sqrt(P(1) - s.w[2] * s.w[2]);  // extruded: in-plane chord along the flight
+    return R::nonneg(l_i);
+}
+
+// |x| in float, truncated to 21 bits, for 0 or 2^-126 <= |x| < 2^128 (smaller: 0)
+__device__ __forceinline__ float coarse(double x) {
+    const uint32_t h = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+    return h < (897u << 20) ? 0.0f : __uint_as_float((h << 3) + 0x40000000u);
+}
+
+// The event of the FP64 walk with one exact distance instead of five.  The
+// five are first bounded in FP32 (a filtered predicate in the sense of Fortune
+// and Van Wyk, Proc. 9th ACM Symp. Computational Geometry, 1993), and where
+// the nearest is certain only its distance is evaluated in FP64: one logarithm
+// instead of two, at most one reciprocal (of a lateral face's direction), one
+// product.  Bounds: positions and directions lose 2^-20 of their values, so a
+// boundary distance lies within L 2^-18/|w| of (target - r)/|w| in FP32;
+// -ln(1 - u) from the draw's high word (2^-33 of u, so 2^-17 of 1 - u > 2^-16)
+// and the hardware's log2 (2^-22 relative) lies within 2^-14, the parameters'
+// and 1/|w|'s relative roundings (below 2^-18 of at most 11.1) included.  The
+// rest, about 2 draws in 10^4, and cases of extreme magnitudes (filter) take
+// all five exactly.  Results are the exact comparison's.  FP64 instructions
+// take 64 cycles per warp and scheduler here, FP32 ones one or two.  Measured
+// (FP64): the box L = 10, 1e7 histories, 45.7 -> 41.1 ms; extruded 3e5 1457 ->
+// 1237 us; warp instructions per event of the box 76 -> 60.
+template <int G, typename Case>
+__device__ __forceinline__ Choice<double> choose_filtered(const History<double> &s, const Case &cp, int m, uint32_t hi,
+                                                          uint32_t lo, uint32_t ihi, uint32_t ilo) {
+    using R = Real<double>;
+    const int gd = geometry<G>(cp);
+    const bool box = gd == 3, lateral = box || gd == 2;
+    const float L = cp.L_f, err = L * 0x1p-18f;
+    // the nearest so far and its bounds, and the least lower bound of the others
+    int which = 0;  // 0, 1, 2: x, y, z face; 3: collision; 4: interface
+    float low = 0.0f, high = 0.0f, rest = __int_as_float(0x7f800000);
+    auto face = [&](int axis, float *a, float *b) {
+        const float r = coarse(s.r[axis]), iw = Real<float>::recip(coarse(s.w[axis]));
+        const float d = __double2hiint(s.w[axis]) >= 0 ? L - r : r;
+        *a = (d - err) * iw;
+        *b = (d + err) * iw;
+    };
+    auto consider = [&](int q, float a, float b) {
+        const bool nearer = b < high;
+        rest = fminf(rest, nearer ? low : a);
+        low = nearer ? a : low;
+        high = nearer ? b : high;
+        which = nearer ? q : which;
+    };
+    face(0, &low, &high);
+    float a, b;
+    if (lateral) {
+        face(1, &a, &b);
+        consider(1, a, b);
+        if (box) {
+            face(2, &a, &b);
+            consider(2, a, b);
+        }
+    }
+    const float kErr = 0x1p-14f, kLn2 = 0.693147180559945f;
+    const float e_c = -kLn2 * __log2f((float)~hi * 0x1p-32f), e_i = -kLn2 * __log2f((float)~ihi * 0x1p-32f);
+    if (cp.sigma_f[m] > 0.0f) consider(3, (e_c - kErr) * cp.inv_sigma_f[m], (e_c + kErr) * cp.inv_sigma_f[m]);
+    float la = cp.lambda_f[m], lb = la;
+    if (gd == 11) {
+        la *= Real<float>::recip(coarse(s.w[0]));
+        lb = la;
+    } else if (gd == 2) {  // 1 - wz^2 within 2^-18
+        const float wz = coarse(s.w[2]), q = fmaf(-wz, wz, 1.0f);
+        la *= rsqrtf(q + 0x1p-18f);
+        lb *= rsqrtf(q - 0x1p-18f);
+    }
+    consider(4, (e_i - kErr) * la, (e_i + kErr) * lb);
+    const bool sure = high < rest && cp.filter && hi < 0xFFFF0000u && ihi < 0xFFFF0000u;
+
+    Choice<double> c;
+    if (sure) {
+        c.bnd = which < 3;
+        c.coll = which == 3;
+        c.face = which == 0 ? (R::pos(s.w[0]) ? 1 : 0) : 2;
+        c.on_y = which == 1;
+        c.on_z = which == 2;
+        if (c.bnd) {
+            const double r = which == 0 ? s.r[0] : which == 1 ? s.r[1] : s.r[2];
+            const double w = which == 0 ? s.w[0] : which == 1 ? s.w[1] : s.w[2];
+            c.l = face_distance(r, w, which == 0 ? s.iw[0] : R::recip(w), R::L(cp));
+        } else {
+            const double e = exp_variate_shared(c.coll ? R::k53(hi, lo) : R::k53(ihi, ilo));
+            c.l = c.coll ? R::nonneg(e * R::inv_sigma(cp, m)) : interface_distance<double, G>(s, cp, m, e);
+        }
+    } else {
+        double x_c, x_i;
+        R::exp_variates(hi, lo, ihi, ilo, &x_c, &x_i);
+        c = choose_event<double, G>(s, cp, collision_distance<double>(cp, m, x_c),
+                                    interface_distance<double, G>(s, cp, m, x_i), recip_or_inf(s.w[1]),
+                                    recip_or_inf(s.w[2]));
+    }
+    return c;
+}
+
 // Where step takes its random numbers from.  PhiloxDraws: the lane's own
 // Philox blocks, computed as they are needed; with DEFER a 3D or extruded
 // scatter leaves its direction pending for the caller's resolve_direction.
@@ -795,19 +928,29 @@ template <typename P, int G, bool DEFER>
 struct PhiloxDraws {
     const RoundKeys &key;
 
-    // collision, then interface distance.  One Philox block serves both draws
-    // (draw_pair), except in the FP32 x-projected walk, where holding the pair
-    // spills registers (measured 10% slower there, 4-7% faster elsewhere).
-    __device__ __forceinline__ void distances(History<P> &s, P *e_c, P *e_i) {
+    // The event, from the draws of the collision, then the interface distance.
+    // One Philox block serves both draws (draw_pair), except in the FP32
+    // x-projected walk, where holding the pair spills registers (measured 10%
+    // slower there, 4-7% faster elsewhere).
+    template <typename Case>
+    __device__ __forceinline__ Choice<P> choose(History<P> &s, const Case &cp, int m) {
         uint32_t hi, lo, ihi, ilo;
-        if constexpr (sizeof(P) == 4 && G == 13) {
-            draw_words(s, key, hi, lo);
-            *e_c = Real<P>::exp_variate(hi, lo);
-            draw_words(s, key, ihi, ilo);
-            *e_i = Real<P>::exp_variate(ihi, ilo);
-        } else {
+        if constexpr (sizeof(P) == 8) {
             draw_pair(s, key, hi, lo, ihi, ilo);
-            Real<P>::exp_variates(hi, lo, ihi, ilo, e_c, e_i);
+            return choose_filtered<G>(s, cp, m, hi, lo, ihi, ilo);
+        } else {
+            P e_c, e_i;
+            if constexpr (G == 13) {
+                draw_words(s, key, hi, lo);
+                e_c = Real<P>::exp_variate(hi, lo);
+                draw_words(s, key, ihi, ilo);
+                e_i = Real<P>::exp_variate(ihi, ilo);
+            } else {
+                draw_pair(s, key, hi, lo, ihi, ilo);
+                Real<P>::exp_variates(hi, lo, ihi, ilo, &e_c, &e_i);
+            }
+            return choose_event<P, G>(s, cp, collision_distance<P>(cp, m, e_c), interface_distance<P, G>(s, cp, m, e_i),
+                                      Real<P>::recip(s.w[1]), Real<P>::recip(s.w[2]));
         }
     }
     __device__ __forceinline__ bool below(History<P> &s, unsigned long long thr53, uint32_t thr24) {
@@ -868,10 +1011,18 @@ struct NarrowDraws {
             }
         }
     }
-    __device__ __forceinline__ void distances(History<P> &s, P *ec, P *ei) {
+    template <typename Case>
+    __device__ __forceinline__ Choice<P> choose(History<P> &s, const Case &cp, int m) {
         s.j += 2u;
-        *ec = e_c;
-        *ei = e_i;
+        P iy, iz;
+        if constexpr (sizeof(P) == 8) {
+            iy = s.iw[1];
+            iz = s.iw[2];
+        } else {
+            iy = Real<P>::recip(s.w[1]);
+            iz = Real<P>::recip(s.w[2]);
+        }
+        return choose_event<P, G>(s, cp, collision_distance<P>(cp, m, e_c), interface_distance<P, G>(s, cp, m, e_i), iy, iz);
     }
     __device__ __forceinline__ bool below(History<P> &s, unsigned long long thr53, uint32_t thr24) {
         ++s.j;
@@ -922,51 +1073,17 @@ __device__ __forceinline__ int step(History<P> &s, const Case &cp, Draws &draws,
     }
     ++s.events;
     const int m = s.m;
-    const P INF = R::inf();
     const P L = R::L(cp);
 
-    // collision, then interface distance
-    P e_c, e_i;
-    draws.distances(s, &e_c, &e_i);
-    const P l_c = R::pos(R::sigma(cp, m)) ? R::nonneg(e_c * R::inv_sigma(cp, m)) : INF;
-    P l_i = R::lambda(cp, m) * e_i;
-    if (gd == 11) l_i *= R::abs(s.iw[0]);  // slab: the chord projected on x, Lambda/|mu|
-    else if (gd == 2) l_i /= sqrt(P(1) - s.w[2] * s.w[2]);  // extruded: in-plane chord along the flight
-    l_i = R::nonneg(l_i);
-
-    // boundary distance: x faces, then the lateral faces of the box
-    // (the face ahead minus the position) / omega, on every lane; infinite for omega = 0
-    int face = R::pos(s.w[0]) ? 1 : 0;  // 0: x = 0, 1: x = L, 2: lateral
-    P l_b = face_distance(s.r[0], s.w[0], s.iw[0], L);
-    P l_y = INF, l_z = INF;
-    const bool box = gd == 3;
-    const bool lateral = box || gd == 2;  // lateral faces: y (and z in the box; the extruded geometry has none)
-    if (lateral) {
-        l_y = face_distance(s.r[1], s.w[1], s.iw[1], L);
-        if (R::lt(l_y, l_b)) {
-            l_b = l_y;
-            face = 2;
-        }
-        if (box) {
-            l_z = face_distance(s.r[2], s.w[2], s.iw[2], L);
-            if (R::lt(l_z, l_b)) {
-                l_b = l_z;
-                face = 2;
-            }
-        }
-    }
-
-    // the event: boundary, else collision, else interface.  Every lane then
-    // moves and scores its flight on one converged path.
-    const bool bnd = R::le(l_b, l_c) && R::le(l_b, l_i);
-    const bool coll = !bnd && R::le(l_c, l_i);
-    const bool leak = bnd && face != 2;
-    const P l = bnd ? l_b : (coll ? l_c : l_i);
-    const P x1 = leak ? ((face == 0) ? P(0) : L) : s.r[0] + l * s.w[0];
+    // Every lane moves and scores its flight on one converged path.
+    const Choice<P> c = draws.choose(s, cp, m);
+    const bool bnd = c.bnd, coll = c.coll, leak = bnd && c.face != 2;
+    const P l = c.l;
+    const P x1 = leak ? ((c.face == 0) ? P(0) : L) : s.r[0] + l * s.w[0];
     plan_flight(f, s, cp, s.r[0], x1, l, m, global);
     s.r[0] = x1;
-    if (lateral) {
-        if (bnd && face == 2 && R::eq(l_y, l_b)) {  // specular reflection on a y face
+    if (gd == 3 || gd == 2) {
+        if (c.on_y) {  // specular reflection on a y face
             s.r[1] = R::pos(s.w[1]) ? L : P(0);
             s.w[1] = R::flip(s.w[1]);
             s.iw[1] = R::flip(s.iw[1]);
@@ -974,8 +1091,8 @@ __device__ __forceinline__ int step(History<P> &s, const Case &cp, Draws &draws,
             s.r[1] += l * s.w[1];
         }
     }
-    if (box) {
-        if (bnd && face == 2 && R::eq(l_z, l_b)) {  // and/or on a z face
+    if (gd == 3) {
+        if (c.on_z) {  // and/or on a z face
             s.r[2] = R::pos(s.w[2]) ? L : P(0);
             s.w[2] = R::flip(s.w[2]);
             s.iw[2] = R::flip(s.iw[2]);
@@ -984,7 +1101,7 @@ __device__ __forceinline__ int step(History<P> &s, const Case &cp, Draws &draws,
         }
     }
     if (leak) {
-        const int ev = (face == 0) ? EV_LEAK_X0 : EV_LEAK_XL;
+        const int ev = (c.face == 0) ? EV_LEAK_X0 : EV_LEAK_XL;
         trace_row<P, TRACE>(tr, ev, s, (double)l);
         return ev;
     }
@@ -1693,7 +1810,7 @@ __device__ __forceinline__ void end_history(unsigned char *regions, const Launch
 // A history handed from the history tracker to the narrow walk.
 template <typename P>
 struct Straggler {
-    P r[3], w[3], iw[3], track0, track1;
+    P r[3], w[3], iw, track0, track1;
     uint32_t h_lo, h_hi, cid, j, events, n_int, m, lcase, lbatch;
 };
 static_assert(sizeof(Straggler<float>) <= kStragglerBytes && sizeof(Straggler<double>) <= kStragglerBytes,
@@ -1714,8 +1831,8 @@ __device__ __forceinline__ bool hand_over(const LaunchArgs &a, const History<P> 
     for (int i = 0; i < 3; ++i) {
         t.r[i] = s.r[i];
         t.w[i] = s.w[i];
-        t.iw[i] = s.iw[i];
     }
+    t.iw = s.iw[0];
     t.track0 = s.track0;
     t.track1 = s.track1;
     t.h_lo = s.h_lo;
@@ -1884,7 +2001,8 @@ __device__ __forceinline__ void fill_draws(DrawBuffer<P> &b, int at, uint32_t bl
             b.w[1][at + t] = d.w[1];
             if constexpr (sizeof(P) == 8) {
                 b.iw[0][at + t] = d.iw[0];
-                b.iw[1][at + t] = d.iw[1];
+                b.iw[1][at + t] = recip_or_inf(d.w[1]);
+                d.iw[2] = recip_or_inf(d.w[2]);
             }
         }
         b.w[2][at + t] = d.w[2];
@@ -1948,8 +2066,8 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
             for (int q = 0; q < 3; ++q) {
                 s.r[q] = t.r[q];
                 s.w[q] = t.w[q];
-                s.iw[q] = t.iw[q];
             }
+            s.iw[0] = t.iw;
             s.track0 = t.track0;
             s.track1 = t.track1;
             s.h_lo = t.h_lo;
@@ -1961,6 +2079,10 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
             s.m = (int)t.m;
             lcase = (int)t.lcase;
             lbatch = t.lbatch;
+        }
+        if constexpr (sizeof(P) == 8) {
+            s.iw[1] = recip_or_inf(s.w[1]);
+            s.iw[2] = recip_or_inf(s.w[2]);
         }
         if (key_case != lcase || key_batch != lbatch) {
             if (key_case >= 0) flush_region<P>(region, a, key_case, key_batch, lane, key_case != lcase);

@@ -23,10 +23,10 @@
 
 namespace cls {
 
-// Bank fields (16 bytes each, SoA): FP32 uses 4, FP64 uses 8.
+// Bank fields (16 bytes each, SoA): FP32 uses 4, FP64 uses 7.
 //   FP32: [0] (x, y, z, track0) [1] (wx, wy, wz, track1) [2] meta0 [3] meta1
-//   FP64: [0] (x, y) [1] (z, track0) [2] (wx, wy) [3] (wz, track1) [4] (iwx, iwy)
-//         [5] (iwz, -) [6] meta0 [7] meta1
+//   FP64: [0] (x, y) [1] (z, track0) [2] (wx, wy) [3] (wz, track1) [4] (iwx, -)
+//         [5] meta0 [6] meta1
 //   meta0 = (h_lo, h_hi, j, c2); meta1 = (c3, m | region << 1 | generation << 3, events, run)
 //   (region 0 or 1: a warp tally region of that generation; 2: global tallies)
 template <typename P>
@@ -37,7 +37,7 @@ struct BankLayout<float> {
 };
 template <>
 struct BankLayout<double> {
-    static constexpr int kFields = 8;
+    static constexpr int kFields = 7;
 };
 
 template <typename P>
@@ -91,10 +91,9 @@ __device__ __forceinline__ void bank_store<double>(unsigned char *buf, uint32_t 
     reinterpret_cast<double2 *>(buf + f)[slot] = make_double2(s.r[2], s.track0);
     reinterpret_cast<double2 *>(buf + 2 * f)[slot] = make_double2(s.w[0], s.w[1]);
     reinterpret_cast<double2 *>(buf + 3 * f)[slot] = make_double2(s.w[2], s.track1);
-    reinterpret_cast<double2 *>(buf + 4 * f)[slot] = make_double2(s.iw[0], s.iw[1]);
-    reinterpret_cast<double2 *>(buf + 5 * f)[slot] = make_double2(s.iw[2], 0.0);
-    reinterpret_cast<uint4 *>(buf + 6 * f)[slot] = make_uint4(s.h_lo, s.h_hi, s.j, s.c2);
-    reinterpret_cast<uint4 *>(buf + 7 * f)[slot] =
+    reinterpret_cast<double2 *>(buf + 4 * f)[slot] = make_double2(s.iw[0], 0.0);
+    reinterpret_cast<uint4 *>(buf + 5 * f)[slot] = make_uint4(s.h_lo, s.h_hi, s.j, s.c2);
+    reinterpret_cast<uint4 *>(buf + 6 * f)[slot] =
         make_uint4(s.c3, (uint32_t)s.m | ((uint32_t)reg << 1), s.events, (uint32_t)run);
 }
 
@@ -107,9 +106,8 @@ __device__ __forceinline__ void bank_load<double>(const unsigned char *buf, uint
     const double2 c = reinterpret_cast<const double2 *>(buf + 2 * f)[slot];
     const double2 d = reinterpret_cast<const double2 *>(buf + 3 * f)[slot];
     const double2 e = reinterpret_cast<const double2 *>(buf + 4 * f)[slot];
-    const double2 g = reinterpret_cast<const double2 *>(buf + 5 * f)[slot];
-    const uint4 m0 = reinterpret_cast<const uint4 *>(buf + 6 * f)[slot];
-    const uint4 m1 = reinterpret_cast<const uint4 *>(buf + 7 * f)[slot];
+    const uint4 m0 = reinterpret_cast<const uint4 *>(buf + 5 * f)[slot];
+    const uint4 m1 = reinterpret_cast<const uint4 *>(buf + 6 * f)[slot];
     s.r[0] = a.x;
     s.r[1] = a.y;
     s.r[2] = b.x;
@@ -119,8 +117,6 @@ __device__ __forceinline__ void bank_load<double>(const unsigned char *buf, uint
     s.w[2] = d.x;
     s.track1 = d.y;
     s.iw[0] = e.x;
-    s.iw[1] = e.y;
-    s.iw[2] = g.x;
     s.h_lo = m0.x;
     s.h_hi = m0.y;
     s.j = m0.z;

@@ -32,6 +32,7 @@ struct CaseParams {
     int32_t nbins;
     uint32_t case_id;  // Philox counter word 3
     int32_t source;    // 0 incident flux on x = 0 (suite I), 1 uniform isotropic volume source (suite II)
+    int32_t filter;    // the FP64 walk may compare distances in FP32 first (choose): the parameters' magnitudes allow it
     double cost;    // host estimate of events per history (ordering only)
 };
 
