@@ -6,6 +6,7 @@
 // FP64 (paper Sec. 2 observables; standard errors per Sec. 5 / Eq.
 // combined_var usage: per-history for R, T, A and <phi>, batch means for phi(x)).
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <map>
@@ -57,6 +58,71 @@ constexpr int kGroupCounters = 3 * kMaxGroups;  // each group's tickets; histori
 
 }  // namespace
 
+// ------------------------------------------------------------ tally reader
+// What cls_tallies reads of one case, in pinned host memory that the kernel
+// writes directly: the flux profile and its batch-means error, the statistics
+// and counters.  A call used to copy the case's flux of all batches (51 KB for
+// 100 bins), statistics and counters with three synchronous copies and reduce
+// them on the host: 55 us a call, 14 of the 54 ms of a pass over the 256-case
+// sweep at 1e6 histories per case.  One small launch and one
+// wait: 23 us (16 in the library, the rest in the Python binding).
+namespace {
+
+struct TallyView {
+    double *flux, *sigma;             // [nbins], host
+    double *stats;                    // [S_NUM], host
+    unsigned long long *counters;     // [C_NUM], host
+    const double *batch_histories;    // [nbatch], host
+};
+
+constexpr int kTallyBins = 32, kTallySlices = 8, kMaxBatches = 1024;
+
+// Block (kTallyBins, kTallySlices): 32 bins, the batches in 8 interleaved
+// slices.  phi = sum_b flux_b / (N dx); its variance B/(B-1) sum_b (n_b/N)^2
+// (X_b - phi)^2 over the B = `used` batches that hold histories (finalize_raw).
+__global__ void tally_kernel(const double *flux, const double *stats, const unsigned long long *counters, int copies,
+                             int nbins, int stride, int nbatch, int used, double N, double dx, TallyView out) {
+    __shared__ double part[kTallySlices][kTallyBins];
+    __shared__ double phi_of[kTallyBins];
+    __shared__ double histories[kMaxBatches];
+    const int x = threadIdx.x, y = threadIdx.y, k = blockIdx.x * kTallyBins + x;
+    for (int b = y * kTallyBins + x; b < nbatch; b += kTallyBins * kTallySlices) histories[b] = out.batch_histories[b];
+    double v = 0.0;
+    if (k < nbins)
+        for (int b = y; b < nbatch; b += kTallySlices) v += flux[(size_t)b * stride + k];
+    part[y][x] = v;
+    __syncthreads();
+    if (y == 0) {
+        for (int i = 1; i < kTallySlices; ++i) v += part[i][x];
+        phi_of[x] = v / (N * dx);
+    }
+    __syncthreads();
+    const double phi = phi_of[x];
+    double acc = 0.0;
+    if (k < nbins)
+        for (int b = y; b < nbatch; b += kTallySlices) {
+            const double nb = histories[b];
+            if (!(nb > 0.0)) continue;
+            const double d = flux[(size_t)b * stride + k] / (nb * dx) - phi, w = nb / N;
+            acc += w * w * d * d;
+        }
+    part[y][x] = acc;
+    __syncthreads();
+    if (y == 0 && k < nbins) {
+        for (int i = 1; i < kTallySlices; ++i) acc += part[i][x];
+        out.flux[k] = phi;
+        out.sigma[k] = used < 2 ? NAN : sqrt(acc * used / (used - 1.0));
+    }
+    if (blockIdx.x == 0 && y == 1 && x < S_NUM) {
+        double t = 0.0;
+        for (int i = 0; i < copies; ++i) t += stats[i * S_NUM + x];
+        out.stats[x] = t;
+    }
+    if (blockIdx.x == 0 && y == 2 && x < C_NUM) out.counters[x] = counters[x];
+}
+
+}  // namespace
+
 struct cls_handle {
     int device = 0;
     int sm_count = 0;
@@ -76,7 +142,7 @@ struct cls_handle {
     unsigned long long *d_counters = nullptr;
     unsigned long long *d_chunk_counter = nullptr;
     // per-run work
-    RunCase *h_runs = nullptr;  // pinned; the OutcomeRecord follows the cases' RunCases
+    RunCase *h_runs = nullptr;  // pinned; the OutcomeRecord follows the cases' RunCases, then the tally reader's memory
     RunCase *d_runs = nullptr;
     uint8_t *outcome_codes = nullptr;  // caller's per-history outcome buffer (device), or null
     uint64_t outcome_cap = 0;
@@ -101,6 +167,8 @@ struct cls_handle {
     cudaStream_t last_stream = nullptr;
     bool ran = false;
     std::vector<cudaEvent_t> ev_pairs;  // start/stop per pending run
+    std::vector<cudaEvent_t> ev_free;   // events of runs that have been timed, for the next ones
+    std::map<std::array<long, 6>, int> occupancy;  // blocks per SM of the trackers, by their launch shape
     double seconds = 0.0;
     // batch graph: group 0 is captured on capture_stream, group g > 0 on
     // aux_streams[g - 1], forked after the counter reset and joined at the end
@@ -123,8 +191,25 @@ int cuda_fail(cudaError_t e) { return e == cudaSuccess ? CLS_OK : CLS_E_CUDA; }
         if (_e != cudaSuccess) return CLS_E_CUDA;   \
     } while (0)
 
+// Pinned bytes of the tally reader after the work list: flux, sigma, batch
+// histories, statistics, counters.
+size_t tally_view_offset(size_t ncases);
+
+TallyView tally_view(cls_handle *h) {
+    double *p = reinterpret_cast<double *>(reinterpret_cast<unsigned char *>(h->h_runs) + tally_view_offset(h->cases.size()));
+    const int nb = h->nbins_max;
+    return TallyView{p, p + nb, p + 2 * nb, reinterpret_cast<unsigned long long *>(p + 2 * nb + S_NUM),
+                     p + 2 * nb + S_NUM + C_NUM};
+}
+
 // The run's work list: one RunCase per case, then the OutcomeRecord.
 size_t runs_bytes(size_t ncases) { return ncases * sizeof(RunCase) + sizeof(OutcomeRecord); }
+
+size_t tally_view_offset(size_t ncases) { return (runs_bytes(ncases) + 63) & ~(size_t)63; }
+
+size_t pinned_bytes(size_t ncases, int nbins_max) {
+    return tally_view_offset(ncases) + (2 * (size_t)nbins_max + S_NUM + C_NUM + kMaxBatches) * sizeof(double);
+}
 
 OutcomeRecord *outcome_record(RunCase *runs, size_t ncases) {
     return reinterpret_cast<OutcomeRecord *>(reinterpret_cast<unsigned char *>(runs) + ncases * sizeof(RunCase));
@@ -272,7 +357,7 @@ int create_common(const double *params, int ncases, bool batch, cls_handle **out
     if (cudaMalloc(&h->d_cases, ncases * sizeof(CaseParams)) != cudaSuccess ||
         cudaMalloc(&h->d_runs, runs_bytes(ncases)) != cudaSuccess ||
         cudaMalloc(&h->d_chunk_counter, counter_bytes(ncases)) != cudaSuccess ||
-        cudaMallocHost(&h->h_runs, runs_bytes(ncases)) != cudaSuccess) {
+        cudaMallocHost(&h->h_runs, pinned_bytes(ncases, h->nbins_max)) != cudaSuccess) {
         rc = CLS_E_NOMEM;
     }
     if (!rc) rc = alloc_tallies(h);
@@ -478,10 +563,17 @@ int tracker_shape(cls_handle *h, int region_bytes, int sched, int geom, Shape *o
     int bps = h->opt.blocks_per_sm;
     if (bps <= 0) {
         const int g = geom;
-        cudaError_t e = event ? (fp64 ? occupancy_event_fp64(block, smem, &bps, g) : occupancy_event_fp32(block, smem, &bps, g))
-                              : (fp64 ? occupancy_history_fp64(block, smem, &bps, g)
-                                      : occupancy_history_fp32(block, smem, &bps, g));
-        if (e != cudaSuccess) return CLS_E_CUDA;
+        const std::array<long, 6> shape = {event, fp64, g, block, (long)smem, h->device};
+        const auto known = h->occupancy.find(shape);
+        if (known != h->occupancy.end()) {
+            bps = known->second;
+        } else {
+            cudaError_t e = event ? (fp64 ? occupancy_event_fp64(block, smem, &bps, g) : occupancy_event_fp32(block, smem, &bps, g))
+                                  : (fp64 ? occupancy_history_fp64(block, smem, &bps, g)
+                                          : occupancy_history_fp32(block, smem, &bps, g));
+            if (e != cudaSuccess) return CLS_E_CUDA;
+            h->occupancy[shape] = bps;
+        }
         if (bps < 1) return CLS_E_INVAL;  // the block does not fit on an SM
     }
     h->used_blocks_per_sm = bps;
@@ -623,18 +715,31 @@ int launch_tracker(cls_handle *h, LaunchArgs a, int sched, int geom, const Shape
 
 int record_pair(cls_handle *h, cudaStream_t s, bool start) {
     if (start) {
-        cudaEvent_t e0, e1;
-        CLS_CUDA(cudaEventCreate(&e0));
-        if (cudaEventCreate(&e1) != cudaSuccess) {
-            cudaEventDestroy(e0);
-            return CLS_E_CUDA;
+        while (h->ev_free.size() < 2) {
+            cudaEvent_t e;
+            CLS_CUDA(cudaEventCreate(&e));
+            h->ev_free.push_back(e);
         }
-        h->ev_pairs.push_back(e0);
-        h->ev_pairs.push_back(e1);
+        for (int i = 0; i < 2; ++i) {
+            h->ev_pairs.push_back(h->ev_free.back());
+            h->ev_free.pop_back();
+        }
     }
     return cuda_fail(cudaEventRecord(h->ev_pairs[h->ev_pairs.size() - (start ? 2 : 1)], s));
 }
 
+// The timed runs' events go back for the next runs (a few: a program that never
+// reads its tallies leaves a pair for each run).
+void release_events(cls_handle *h) {
+    for (cudaEvent_t e : h->ev_pairs) {
+        if (h->ev_free.size() < 8) h->ev_free.push_back(e);
+        else cudaEventDestroy(e);
+    }
+    h->ev_pairs.clear();
+}
+
+// Wait for the last run, with whatever the caller has enqueued behind it, and
+// add the device times of the runs since the last call.
 int sync_and_time(cls_handle *h) {
     if (!h->ran) return CLS_E_STATE;
     CLS_CUDA(cudaSetDevice(h->device));
@@ -643,10 +748,8 @@ int sync_and_time(cls_handle *h) {
         float ms = 0.f;
         CLS_CUDA(cudaEventElapsedTime(&ms, h->ev_pairs[i], h->ev_pairs[i + 1]));
         h->seconds += ms * 1e-3;
-        cudaEventDestroy(h->ev_pairs[i]);
-        cudaEventDestroy(h->ev_pairs[i + 1]);
     }
-    h->ev_pairs.clear();
+    release_events(h);
     return CLS_OK;
 }
 
@@ -671,10 +774,9 @@ int fetch_case(cls_handle *h, int k, std::vector<double> &flux, double stats[S_N
 // R, T, A per-history Bernoulli means with sqrt(p(1-p)/(N-1)); <phi> the mean
 // track length with its per-history standard error; phi_k = sum_b flux[b][k] /
 // (N dx) with the batch-means error B/(B-1) sum_b (n_b/N)^2 (X_b - X)^2.
-int finalize_raw(const cls_raw_t &raw, const double *flux, int flux_stride, const uint64_t *bh, double L,
-                 cls_tallies_t *out) {
+int finalize_counts(const cls_raw_t &raw, cls_tallies_t *out) {
     const double N = (double)raw.n_histories;
-    if (!(N > 0) || raw.nbins < 1 || raw.nbatch < 1 || !(L > 0)) return CLS_E_INVAL;
+    if (!(N > 0)) return CLS_E_INVAL;
     out->n_histories = raw.n_histories;
     out->nR = raw.nR;
     out->nT = raw.nT;
@@ -698,6 +800,14 @@ int finalize_raw(const cls_raw_t &raw, const double *flux, int flux_stride, cons
     out->sigma_total_flux = N > 1 ? std::sqrt(var / (N - 1.0)) : NAN;
     out->track0 = raw.track[0] / N;
     out->track1 = raw.track[1] / N;
+    return raw.n_capped ? CLS_E_EVENT_LIMIT : CLS_OK;
+}
+
+int finalize_raw(const cls_raw_t &raw, const double *flux, int flux_stride, const uint64_t *bh, double L,
+                 cls_tallies_t *out) {
+    const double N = (double)raw.n_histories;
+    if (!(N > 0) || raw.nbins < 1 || raw.nbatch < 1 || !(L > 0)) return CLS_E_INVAL;
+    finalize_counts(raw, out);
     const int nb = raw.nbins;
     const double dx = L / nb;
     int B = 0;
@@ -747,16 +857,37 @@ void raw_of(const cls_handle *h, int k, const double st[S_NUM], const unsigned l
 
 int tallies_of(cls_handle *h, int k, cls_tallies_t *out) {
     if (!h || !out || k < 0 || k >= (int)h->cases.size()) return CLS_E_INVAL;
+    if (!h->ran) return CLS_E_STATE;
+    CLS_CUDA(cudaSetDevice(h->device));
+    const CaseParams &c = h->cases[k];
+    const TallyView v = tally_view(h);
+    double *bh = const_cast<double *>(v.batch_histories);
+    int used = 0;
+    for (int b = 0; b < h->nbatch; ++b) {
+        bh[b] = (double)h->batch_hist[k][b];
+        used += h->batch_hist[k][b] > 0;
+    }
+    // runs still in flight on other streams than the last one's
+    for (size_t i = 0; i + 3 < h->ev_pairs.size(); i += 2)
+        CLS_CUDA(cudaStreamWaitEvent(h->last_stream, h->ev_pairs[i + 1], 0));
+    const int copies = stats_copies(h->cases.size());
+    tally_kernel<<<(c.nbins + kTallyBins - 1) / kTallyBins, dim3(kTallyBins, kTallySlices), 0, h->last_stream>>>(
+        h->d_flux + (size_t)k * h->nbatch * h->nbins_stride, h->d_stats + (size_t)k * copies * S_NUM,
+        h->d_counters + (size_t)k * C_NUM, copies, c.nbins, h->nbins_stride, h->nbatch, used, (double)h->n_hist[k],
+        c.L / c.nbins, v);
+    CLS_CUDA(cudaGetLastError());
     int rc = sync_and_time(h);
     if (rc) return rc;
-    std::vector<double> flux;
-    double st[S_NUM];
     unsigned long long ct[C_NUM];
-    rc = fetch_case(h, k, flux, st, ct);
-    if (rc) return rc;
+    double st[S_NUM];
+    std::memcpy(ct, v.counters, sizeof(ct));
+    std::memcpy(st, v.stats, sizeof(st));
     cls_raw_t raw;
     raw_of(h, k, st, ct, &raw);
-    rc = finalize_raw(raw, flux.data(), h->nbins_stride, h->batch_hist[k].data(), h->cases[k].L, out);
+    rc = finalize_counts(raw, out);
+    if (rc == CLS_E_INVAL) return rc;
+    if (out->flux) std::memcpy(out->flux, v.flux, c.nbins * sizeof(double));
+    if (out->flux_sigma) std::memcpy(out->flux_sigma, v.sigma, c.nbins * sizeof(double));
     out->seconds = h->seconds;
     return rc;
 }
@@ -942,7 +1073,7 @@ int cls_set_option(cls_handle *h, int key, int64_t v) {
         o.chunk = (int)v;
         break;
     case CLS_OPT_NBATCH:
-        if (v < 2 || v > 1024) return CLS_E_INVAL;
+        if (v < 2 || v > kMaxBatches) return CLS_E_INVAL;
         if (v != h->nbatch) {
             // changes the tally layout: only allowed before the first run
             if (h->ran) return CLS_E_STATE;
@@ -1285,6 +1416,7 @@ void cls_destroy(cls_handle *h) {
     for (cudaStream_t a : h->aux_streams) cudaStreamDestroy(a);
     for (cudaEvent_t e : h->join_events) cudaEventDestroy(e);
     for (cudaEvent_t e : h->ev_pairs) cudaEventDestroy(e);
+    for (cudaEvent_t e : h->ev_free) cudaEventDestroy(e);
     if (h->runs_copied) cudaEventDestroy(h->runs_copied);
     free_device(h);
     if (h->h_runs) cudaFreeHost(h->h_runs);
