@@ -626,10 +626,9 @@ __device__ __forceinline__ void add_track(History<P> &s, P l, int m) {
 }
 
 template <typename Case>
-__device__ __forceinline__ void plan_flight(Flight<float> &f, History<float> &s, const Case &cp, float x0,
-                                            float x1, float l, int m, bool) {
+__device__ __forceinline__ void plan_flight(Flight<float> &f, const Case &cp, float x0, float x1, float l, float wx,
+                                            float iwx, bool) {
     using R = Real<float>;
-    add_track(s, l, m);
     f.k0 = 0;
     f.k1 = -1;
     if (!R::pos(l)) return;
@@ -637,7 +636,7 @@ __device__ __forceinline__ void plan_flight(Flight<float> &f, History<float> &s,
     const float inv_dx = R::inv_dx(cp);
     // the x-extent clipped to [0, L]
     const float a = R::nonneg(x0), b = R::nonneg(x1);
-    if (R::is_zero(s.w[0])) {
+    if (R::is_zero(wx)) {
         const int k = R::floor_index(a * inv_dx, nb - 1);
         f.k0 = f.k1 = k;
         f.tail = k == nb - 1;
@@ -660,7 +659,7 @@ __device__ __forceinline__ void plan_flight(Flight<float> &f, History<float> &s,
         f.a0 = l;
         return;
     }
-    const float c = R::dx(cp) * R::abs(s.iw[0]);
+    const float c = R::dx(cp) * R::abs(iwx);
     f.a0 = R::nonneg(fmaf(-R::frac(ulo, k0), c, c));
     f.a1 = R::frac(uhi, k1) * c;
     f.c = c;
@@ -711,10 +710,9 @@ __device__ __forceinline__ void plan_flight_real(Flight<double> &f, double ulo, 
 }
 
 template <typename Case>
-__device__ __forceinline__ void plan_flight(Flight<double> &f, History<double> &s, const Case &cp, double x0,
-                                            double x1, double l, int m, bool global) {
+__device__ __forceinline__ void plan_flight(Flight<double> &f, const Case &cp, double x0, double x1, double l, double wx,
+                                            double iwx, bool global) {
     using R = Real<double>;
-    add_track(s, l, m);
     f.k0 = 0;
     f.k1 = -1;
     f.real = global;
@@ -739,15 +737,15 @@ __device__ __forceinline__ void plan_flight(Flight<double> &f, History<double> &
         F1 = ~0ull;
     }
     k0 = min(k0, nb - 1);
-    if (R::is_zero(s.w[0])) k1 = k0 = (R::lt(a, b) ? k0 : k1);  // the bin that contains x0
+    if (R::is_zero(wx)) k1 = k0 = (R::lt(a, b) ? k0 : k1);  // the bin that contains x0
     f.k0 = k0;
     f.k1 = k1;
     f.tail = k1 == nb - 1;
     // in bin widths: a flight inside one bin scores its length itself, else
     // 1/|wx| in a whole bin
-    const double v = k0 == k1 ? l * inv_dx : R::abs(s.iw[0]);
+    const double v = k0 == k1 ? l * inv_dx : R::abs(iwx);
     if (global || (int)((unsigned long long)__double_as_longlong(v) >> 52) >= 1023 + kFixed64MaxExp) {
-        plan_flight_real(f, ulo, uhi, l, R::dx(cp) * R::abs(s.iw[0]));
+        plan_flight_real(f, ulo, uhi, l, R::dx(cp) * R::abs(iwx));
         return;
     }
     const unsigned long long q = fixed64(v);
@@ -953,6 +951,10 @@ struct PhiloxDraws {
                                       Real<P>::recip(s.w[1]), Real<P>::recip(s.w[2]));
         }
     }
+    template <typename Case>
+    __device__ __forceinline__ void score(Flight<P> &f, const History<P> &s, const Case &cp, P x1, P l, bool global) {
+        plan_flight(f, cp, s.r[0], x1, l, s.w[0], s.iw[0], global);
+    }
     __device__ __forceinline__ bool below(History<P> &s, unsigned long long thr53, uint32_t thr24) {
         return draw_below(s, key, thr53, thr24);
     }
@@ -975,54 +977,78 @@ struct PhiloxDraws {
 template <typename P>
 struct DrawBuffer {
     static constexpr int kDraws = 64;  // two for each lane of the warp
+    float4 w[kDraws];                  // w[0], w[1], w[2], -
+    float e[kDraws];
     uint32_t hi[kDraws];
-    P e[kDraws];
-    P w[3][kDraws];
 };
 template <>
 struct DrawBuffer<double> {
     static constexpr int kDraws = 64;
+    double2 w01[kDraws], w2i0[kDraws], i12[kDraws];  // (w[0], w[1]), (w[2], 1/w[0]), (1/w[1], 1/w[2])
     double e[kDraws];
-    double w[3][kDraws], iw[3][kDraws];
-    uint32_t hi[kDraws], lo[kDraws];
+    uint2 word[kDraws];                              // (hi, lo)
 };
+
 template <typename P, int G>
 struct NarrowDraws {
     // the draws of one event: j, j + 1 (distances), j + 2 (scatter or absorb), j + 3, j + 4 (direction)
     P e_c, e_i, wx, wy, wz, ix, iy, iz;
     uint32_t t_hi, t_lo, x_hi;
 
+    P x0, x1, l, fw, fiw;  // the flight made: its x, length, direction cosine and its reciprocal
+
     __device__ __forceinline__ void fetch(const DrawBuffer<P> &b, int slot) {
         e_c = b.e[slot];
         e_i = b.e[slot + 1];
-        t_hi = b.hi[slot + 2];
-        if constexpr (sizeof(P) == 8) t_lo = b.lo[slot + 2];
-        if constexpr (G == 0 || G == 1) x_hi = b.hi[slot + 3];
-        if constexpr (G != 1) wz = b.w[2][slot + 3];
-        if constexpr (G == 0 || G == 2 || G == 3) {
-            wx = b.w[0][slot + 3];
-            wy = b.w[1][slot + 3];
-        }
         if constexpr (sizeof(P) == 8) {
-            if constexpr (G != 1) iz = b.iw[2][slot + 3];
-            if constexpr (G == 0 || G == 2 || G == 3) {
-                ix = b.iw[0][slot + 3];
-                iy = b.iw[1][slot + 3];
+            const uint2 t = b.word[slot + 2];
+            t_hi = t.x;
+            t_lo = t.y;
+            if constexpr (G == 0 || G == 1) x_hi = b.word[slot + 3].x;
+            if constexpr (G != 1) {
+                const double2 w2i0 = b.w2i0[slot + 3];
+                wz = w2i0.x;
+                ix = w2i0.y;
+            }
+            if constexpr (G != 1 && G != 11 && G != 13) {
+                const double2 w01 = b.w01[slot + 3], i12 = b.i12[slot + 3];
+                wx = w01.x;
+                wy = w01.y;
+                iy = i12.x;
+                iz = i12.y;
+            }
+        } else {
+            t_hi = b.hi[slot + 2];
+            t_lo = 0;
+            if constexpr (G == 0 || G == 1) x_hi = b.hi[slot + 3];
+            if constexpr (G != 1) {
+                const float4 w = b.w[slot + 3];
+                wx = w.x;
+                wy = w.y;
+                wz = w.z;
             }
         }
     }
     template <typename Case>
+    __device__ __forceinline__ void score(Flight<P> &, const History<P> &s, const Case &, P x, P length, bool) {
+        x0 = s.r[0];
+        x1 = x;
+        l = length;
+        fw = s.w[0];
+        fiw = s.iw[0];
+    }
+    template <typename Case>
     __device__ __forceinline__ Choice<P> choose(History<P> &s, const Case &cp, int m) {
         s.j += 2u;
-        P iy, iz;
+        P i1, i2;
         if constexpr (sizeof(P) == 8) {
-            iy = s.iw[1];
-            iz = s.iw[2];
+            i1 = s.iw[1];
+            i2 = s.iw[2];
         } else {
-            iy = Real<P>::recip(s.w[1]);
-            iz = Real<P>::recip(s.w[2]);
+            i1 = Real<P>::recip(s.w[1]);
+            i2 = Real<P>::recip(s.w[2]);
         }
-        return choose_event<P, G>(s, cp, collision_distance<P>(cp, m, e_c), interface_distance<P, G>(s, cp, m, e_i), iy, iz);
+        return choose_event<P, G>(s, cp, collision_distance<P>(cp, m, e_c), interface_distance<P, G>(s, cp, m, e_i), i1, i2);
     }
     __device__ __forceinline__ bool below(History<P> &s, unsigned long long thr53, uint32_t thr24) {
         ++s.j;
@@ -1036,7 +1062,7 @@ struct NarrowDraws {
         ++s.j;
         if constexpr (sizeof(P) == 8) {
             s.w[0] = wz;
-            s.iw[0] = iz;
+            s.iw[0] = G == 0 ? iz : ix;
         } else {
             set_direction_x(s, wz);
         }
@@ -1080,7 +1106,8 @@ __device__ __forceinline__ int step(History<P> &s, const Case &cp, Draws &draws,
     const bool bnd = c.bnd, coll = c.coll, leak = bnd && c.face != 2;
     const P l = c.l;
     const P x1 = leak ? ((c.face == 0) ? P(0) : L) : s.r[0] + l * s.w[0];
-    plan_flight(f, s, cp, s.r[0], x1, l, m, global);
+    add_track(s, l, m);
+    draws.score(f, s, cp, x1, l, global);
     s.r[0] = x1;
     if (gd == 3 || gd == 2) {
         if (c.on_y) {  // specular reflection on a y face
@@ -1960,8 +1987,8 @@ __global__ void __launch_bounds__(HistoryBounds<P, G>::threads, HistoryBounds<P,
 // history's next 64 draws at once -- Philox blocks, exponential variates, and
 // the direction a scatter at each draw would take, with its reciprocals -- and
 // only distances, the event and the move are left on the chain, which every
-// lane follows; the case's parameters stay in registers, and the four
-// additions of a flight's deposit go to four lanes.  The arithmetic is step's
+// lane follows; the case's parameters stay in registers, and the flights are
+// scored 32 at a time, one by each lane.  The arithmetic is step's
 // on the same draws, so results do not change.  Measured: 1000 histories
 // of the 3D box 1.07 -> 0.61 ms in FP64 and 345 -> 198 us in FP32, of the
 // diffusive box in FP32 5.1 -> 2.8 ms (0.45 us per event of the longest).
@@ -1977,36 +2004,42 @@ __device__ __forceinline__ void fill_draws(DrawBuffer<P> &b, int at, uint32_t bl
     R::exp_variates(o.x, o.y, o.z, o.w, &e0, &e1);
     b.e[at] = e0;
     b.e[at + 1] = e1;
-    b.hi[at] = o.x;
-    b.hi[at + 1] = o.z;
     if constexpr (sizeof(P) == 8) {
-        b.lo[at] = o.y;
-        b.lo[at + 1] = o.w;
+        b.word[at] = make_uint2(o.x, o.y);
+        b.word[at + 1] = make_uint2(o.z, o.w);
+    } else {
+        b.hi[at] = o.x;
+        b.hi[at + 1] = o.z;
     }
     if constexpr (G == 1) return;
     uint32_t mu_hi = o.x, mu_lo = o.y, phi_hi = o.z, phi_lo = o.w;
 #pragma unroll 1
     for (int t = 0; t < 2; ++t) {
-        History<P> d;
         if constexpr (G == 11 || G == 13) {
-            set_direction_x(d, R::two_u_minus_one(mu_hi, mu_lo));
-            d.w[2] = d.w[0];
-            d.iw[2] = d.iw[0];
+            const P mu = R::two_u_minus_one(mu_hi, mu_lo);
+            if constexpr (sizeof(P) == 8) b.w2i0[at + t] = make_double2(mu, recip_or_inf(mu));
+            else b.w[at + t] = make_float4(0.0f, 0.0f, mu, 0.0f);
         } else {
             P mu, st, sn, cs;
             R::direction_cosines(mu_hi, mu_lo, false, &mu, &st);
             R::sincos_2pi(phi_hi, phi_lo, &sn, &cs);
-            set_direction(d, st * cs, st * sn, mu);
-            b.w[0][at + t] = d.w[0];
-            b.w[1][at + t] = d.w[1];
+            const P wx = st * cs, wy = st * sn;
             if constexpr (sizeof(P) == 8) {
-                b.iw[0][at + t] = d.iw[0];
-                b.iw[1][at + t] = recip_or_inf(d.w[1]);
-                d.iw[2] = recip_or_inf(d.w[2]);
+                double v = wx, r0 = 0.0, r1 = 0.0, r2 = 0.0;
+#pragma unroll 1
+                for (int q = 0; q < 3; ++q) {  // one copy of the reciprocal
+                    r0 = r1;
+                    r1 = r2;
+                    r2 = recip_or_inf(v);
+                    v = q == 0 ? wy : mu;
+                }
+                b.w01[at + t] = make_double2(wx, wy);
+                b.w2i0[at + t] = make_double2(mu, r0);
+                b.i12[at + t] = make_double2(r1, r2);
+            } else {
+                b.w[at + t] = make_float4(wx, wy, mu, 0.0f);
             }
         }
-        b.w[2][at + t] = d.w[2];
-        if constexpr (sizeof(P) == 8) b.iw[2][at + t] = d.iw[2];
         mu_hi = o.z;
         mu_lo = o.w;
         phi_hi = n_hi;
@@ -2019,6 +2052,10 @@ struct NarrowMemory {  // dynamic shared memory of a warp, followed by its tally
     DrawBuffer<P> draws;
     WarpFeed feed;
 };
+static_assert(sizeof(NarrowMemory<float>) <= narrow_memory_bytes(false) &&
+                  sizeof(NarrowMemory<double>) <= narrow_memory_bytes(true) && narrow_memory_bytes(false) % 16 == 0 &&
+                  narrow_memory_bytes(true) % 16 == 0,
+              "the host sizes the narrow walk's shared memory");
 
 template <typename P, int G>
 __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(const LaunchArgs a) {
@@ -2041,6 +2078,25 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
 
     int key_case = -1;  // the region's (case, batch)
     uint32_t key_batch = 0, fed = 0, deposited = 0;
+    // flights still to be scored, one in each lane below `held`
+    P x0 = P(0), x1 = P(0), l = P(0), fw = P(0), fiw = P(0);
+    int held = 0;
+    auto score_held = [&]() {
+        Flight<P> f;
+        f.k0 = 0;
+        f.k1 = -1;
+        if (lane < held) plan_flight(f, a.cases[key_case], x0, x1, l, fw, fiw, false);
+        const uint64_t goff = ((uint64_t)key_case * (uint64_t)a.t.nbatch + key_batch) * (uint64_t)nbs;
+        deposited += warp_deposit<P>(region, a.region_bytes, nbs, 0, a.t.flux, goff, f, lane);
+        held = 0;
+        if constexpr (sizeof(P) == 8) {  // before a bin's sum can outgrow its 64 bits
+            if (__any_sync(CLS_FULL_MASK, deposited >= kDepositBound)) {
+                __syncwarp();
+                flush_region<P>(region, a, key_case, key_batch, lane, false);
+                deposited = 0;
+            }
+        }
+    };
     while (true) {
         // the next history: all lanes hold its state
         History<P> s;
@@ -2085,11 +2141,12 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
             s.iw[2] = recip_or_inf(s.w[2]);
         }
         if (key_case != lcase || key_batch != lbatch) {
+            if (held > 0) score_held();
+            __syncwarp();
             if (key_case >= 0) flush_region<P>(region, a, key_case, key_batch, lane, key_case != lcase);
             key_case = lcase;
             key_batch = lbatch;
         }
-        double *gbins = a.t.flux + ((uint64_t)lcase * (uint64_t)a.t.nbatch + lbatch) * (uint64_t)nbs;
         const CaseRegs<P> cp = load_case<P>(a.cases[lcase]);
         uint32_t base = s.j & ~1u, top = 0;  // draws base .. top - 1 are in the buffer
         int ev = -1;
@@ -2104,26 +2161,17 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
             NarrowDraws<P, G> draws;
             draws.fetch(mem.draws, (int)(s.j - base));
             Flight<P> f;
+            draws.l = P(0);
             ev = step<P, false, G>(s, cp, draws, a.max_events, f, nullptr, false);
-            if (f.k1 >= f.k0) {
-                if (!scores_global(f, 0)) {
-                    const FixedFlight q(f);
-                    const unsigned long long x = lane == 0 ? q.q0 : lane == 1 ? q.d1 : lane == 2 ? q.d2 : q.d3;
-                    const int k = (lane < 2 ? f.k0 : f.k1) + (lane & 1);
-                    if (lane < 2 || (lane == 2 && q.inter) || (lane == 3 && q.multi)) add_entry(region, nbs, k, x);
-                    if constexpr (sizeof(P) == 8) {  // before a bin's sum can outgrow its 64 bits (one history: 2^31)
-                        deposited += q.bound;
-                        if (deposited >= 16u * kDepositBound) {
-                            __syncwarp();
-                            flush_region<P>(region, a, key_case, key_batch, lane, false);
-                            deposited = 0;
-                        }
-                    }
-                } else {
-                    for (int k = f.k0 + lane; k <= f.k1; k += 32)
-                        atomicAdd(&gbins[k], k == f.k0 ? flight_real(f.a0) : k == f.k1 ? flight_real(f.a1) : flight_real(f.c));
-                }
+            // the flight waits in one lane's registers until 32 are scored together
+            if (lane == held) {
+                x0 = draws.x0;
+                x1 = draws.x1;
+                l = draws.l;
+                fw = draws.fw;
+                fiw = draws.fiw;
             }
+            if (++held == 32) score_held();
         }
         if (lane == 0) {
             uint32_t n_coll, n_refl;
@@ -2131,10 +2179,13 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
         }
         __syncwarp();
         if (sizeof(P) == 4 && ++fed >= a.flush_every) {  // FP32: before a bin's sum can outgrow its 64 bits
+            if (held > 0) score_held();
+            __syncwarp();
             flush_region<P>(region, a, key_case, key_batch, lane);
             fed = 0;
         }
     }
+    if (held > 0) score_held();
     __syncwarp();
     if (key_case >= 0) flush_region<P>(region, a, key_case, key_batch, lane);
 }

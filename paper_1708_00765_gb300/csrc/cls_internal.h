@@ -165,17 +165,18 @@ __host__ __device__ inline int region_bytes(int nbins_stride) {
     return (region_lane_stats_offset(nbins_stride) + 8 * 32 * S_NUM + 15) & ~15;
 }
 
+constexpr int kWarpFeedBytes = 112;  // of WarpFeed (cls_device.cuh)
+
 // The narrow walk (narrow_kernel): its blocks, the histories a warp of the
 // history tracker hands over to it at most, and the bytes of one; its dynamic
 // shared memory per warp is the draw buffer and feeding state, then one region.
 constexpr int kNarrowBlock = 128, kNarrowBlocks = 3;
 constexpr int kHandOver = 4;
 constexpr int kStragglerBytes = 128;
-__host__ __device__ constexpr int narrow_memory_bytes(bool fp64) { return (fp64 ? 4096 : 1280) + 112; }
+__host__ __device__ constexpr int narrow_memory_bytes(bool fp64) { return (fp64 ? 4096 : 1536) + kWarpFeedBytes; }
 
 // Dynamic shared memory of a warp of the history tracker: two tally regions and
 // its feeding state (cls_device.cuh's WarpFeed).
-constexpr int kWarpFeedBytes = 112;
 inline size_t history_warp_bytes(int region) { return 2 * (size_t)region + kWarpFeedBytes; }
 
 // Largest block of the event tracker (its launch bounds: 2 such blocks per SM).
