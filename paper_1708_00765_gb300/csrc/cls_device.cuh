@@ -82,11 +82,6 @@ __device__ __forceinline__ double exp_variate_shared(unsigned long long k) {
     return exp_variate(k, IntLogTables{cls_logn_tab, cls_logt_tab});
 }
 
-// (sin, cos) of 2 pi u for u = k 2^-53, from the shared-memory table
-__device__ __forceinline__ void sincos_2pi_shared(unsigned long long k, double *sn, double *cs) {
-    sincos_2pi_int(k, cls_sincos_tab, sn, cs);
-}
-
 // the integer E as a double, exactly (|E| < 2^51), by the 1.5 2^52 shift
 __device__ __forceinline__ double small_int_to_double(long long e) {
     return __longlong_as_double(0x4338000000000000ll + e) - 0x1.8p52;
@@ -156,28 +151,42 @@ struct Real<double> {
     static __device__ __forceinline__ double sqrt_uniform(uint32_t hi, uint32_t lo) {
         return sqrt_int(U128{k53(hi, lo) << 1, 0ull}, 54);
     }
-    // A new direction's cosine mu and st = sqrt(1 - mu^2) from the draw u of mu:
-    // cosine law mu = sqrt(u), st = sqrt(1 - u); isotropic mu = 2u - 1,
-    // st = sqrt(4 u (1 - u)), with 1 - u and 4 u (1 - u) exact integers
-    static __device__ __forceinline__ void direction_cosines(uint32_t hi, uint32_t lo, bool cosine, double *mu,
-                                                             double *st) {
+    // A new direction from the draws u of mu and v of phi = 2 pi v: cosine law
+    // mu = sqrt(u), st = sqrt(1 - u); isotropic mu = 2u - 1, st = sqrt(4 u (1 -
+    // u)), with 1 - u and 4 u (1 - u) exact integers; a = st cos phi, b = st sin
+    // phi multiplied in integers before their one rounding (an FP64 product
+    // costs 64 cycles of its warp, an integer one 16).
+    static __device__ __forceinline__ void direction(uint32_t hi, uint32_t lo, uint32_t phi_hi, uint32_t phi_lo,
+                                                     bool cosine, double *mu, double *a, double *b) {
         const unsigned long long k = k53(hi, lo), n = (1ull << 53) - k;
         // sqrt(u) (the cosine law only: a lane starts the loop at t = 1
-        // otherwise), then st, through one copy of sqrt_int
+        // otherwise), then st, through one copy of sqrt_q61
         const U128 x1 = cosine ? U128{n << 1, 0ull} : U128{(k * n) << 2, (umulhi64(k, n) << 2) | ((k * n) >> 62)};
         const int s1 = cosine ? 54 : 106;
         U128 x = cosine ? U128{k << 1, 0ull} : x1;
-        int scale = s1;
-        double r0 = 0.0, r1 = 0.0;
+        int scale = s1, e0 = 0, e1 = 0;
+        uint64_t q0 = 0, q1 = 0;
 #pragma unroll 1
         for (int t = cosine ? 0 : 1; t < 2; ++t) {
-            r0 = r1;
-            r1 = sqrt_int(x, scale);
+            q0 = q1;
+            e0 = e1;
+            q1 = sqrt_q61(x, scale, &e1);
             x = x1;
             scale = s1;
         }
-        *mu = cosine ? r0 : two_u_minus_one(hi, lo);
-        *st = r1;
+        *mu = cosine ? fixed_to_double((int64_t)q0, e0 - 61) : two_u_minus_one(hi, lo);
+        int64_t sn, cs;
+        sincos_2pi_q62(k53(phi_hi, phi_lo), cls_sincos_tab, &sn, &cs);
+        int64_t v = cs;
+        double r0 = 0.0, r1 = 0.0;
+#pragma unroll 1
+        for (int t = 0; t < 2; ++t) {
+            r0 = r1;
+            r1 = sqrt_times_q62(q1, e1, v);
+            v = sn;
+        }
+        *a = r0;
+        *b = r1;
     }
     // 1 - u, exactly: (2^53 - k) 2^-53
     static __device__ __forceinline__ double one_minus(uint32_t hi, uint32_t lo) {
@@ -259,10 +268,6 @@ struct Real<double> {
     }
     // 1/a in integer arithmetic (Newton-Raphson, cls_intmath.h)
     static __device__ __forceinline__ double recip(double a) { return recip_int(a); }
-    // (sin, cos) of 2 pi u from the draw's words
-    static __device__ __forceinline__ void sincos_2pi(uint32_t hi, uint32_t lo, double *s, double *co) {
-        sincos_2pi_shared(k53(hi, lo), s, co);
-    }
 };
 
 // FP32 tracking: position, direction and distances in float; the flights'
@@ -281,11 +286,6 @@ struct Real<float> {
         return r;
     }
     static __device__ __forceinline__ float sqrt_uniform(uint32_t hi, uint32_t lo) { return fast_sqrt(uniform(hi, lo)); }
-    static __device__ __forceinline__ void direction_cosines(uint32_t hi, uint32_t lo, bool cosine, float *mu,
-                                                            float *st) {
-        *mu = cosine ? sqrt_uniform(hi, lo) : two_u_minus_one(hi, lo);
-        *st = fast_sqrt(1.0f - *mu * *mu);
-    }
     static __device__ __forceinline__ float one_minus(uint32_t hi, uint32_t) {
         return (float)((1u << 24) - (hi >> 8)) * 0x1p-24f;
     }
@@ -332,11 +332,14 @@ struct Real<float> {
         return r;
     }
     // (sin, cos)(2 pi u) = -(sin, cos)(2 pi (u - 1/2)), the argument in [-pi, pi)
-    static __device__ __forceinline__ void sincos_2pi(uint32_t hi, uint32_t lo, float *s, float *co) {
+    static __device__ __forceinline__ void direction(uint32_t hi, uint32_t lo, uint32_t phi_hi, uint32_t phi_lo,
+                                                     bool cosine, float *mu, float *a, float *b) {
+        *mu = cosine ? sqrt_uniform(hi, lo) : two_u_minus_one(hi, lo);
+        const float st = fast_sqrt(1.0f - *mu * *mu);
         float sn, cs;
-        __sincosf(6.28318530717958647692f * (uniform(hi, lo) - 0.5f), &sn, &cs);
-        *s = -sn;
-        *co = -cs;
+        __sincosf(6.28318530717958647692f * (uniform(phi_hi, phi_lo) - 0.5f), &sn, &cs);
+        *a = st * -cs;
+        *b = st * -sn;
     }
 };
 
@@ -519,10 +522,8 @@ __device__ __forceinline__ void resolve_direction(History<P> &s, const CaseParam
     const bool cosine = s.pend == DIR_SOURCE_COSINE;
     uint32_t hi, lo, phi_hi, phi_lo;
     draw_pair(s, key, hi, lo, phi_hi, phi_lo);  // mu, then phi
-    P mu, st, sn, cs;
-    Real<P>::direction_cosines(hi, lo, cosine, &mu, &st);
-    Real<P>::sincos_2pi(phi_hi, phi_lo, &sn, &cs);
-    const P a = st * cs, b = st * sn;
+    P mu, a, b;
+    Real<P>::direction(hi, lo, phi_hi, phi_lo, cosine, &mu, &a, &b);
     set_direction(s, cosine ? mu : a, cosine ? a : b, cosine ? b : mu);
     if (s.pend != DIR_SCATTER) s.m = draw_below(s, key, cp.thr_p053, cp.thr_p024) ? 0 : 1;
     s.pend = DIR_NONE;
@@ -870,13 +871,13 @@ __device__ __forceinline__ Choice<double> choose_filtered(const History<double> 
         which = nearer ? q : which;
     };
     face(0, &low, &high);
-    float a, b;
+    float fa, fb;
     if (lateral) {
-        face(1, &a, &b);
-        consider(1, a, b);
+        face(1, &fa, &fb);
+        consider(1, fa, fb);
         if (box) {
-            face(2, &a, &b);
-            consider(2, a, b);
+            face(2, &fa, &fb);
+            consider(2, fa, fb);
         }
     }
     const float kErr = 0x1p-14f, kLn2 = 0.693147180559945f;
@@ -892,6 +893,7 @@ __device__ __forceinline__ Choice<double> choose_filtered(const History<double> 
         lb *= rsqrtf(q - 0x1p-18f);
     }
     consider(4, (e_i - kErr) * la, (e_i + kErr) * lb);
+    // (a certain face is never one of direction 0, whose bounds are infinite)
     const bool sure = high < rest && cp.filter && hi < 0xFFFF0000u && ihi < 0xFFFF0000u;
 
     Choice<double> c;
@@ -901,14 +903,23 @@ __device__ __forceinline__ Choice<double> choose_filtered(const History<double> 
         c.face = which == 0 ? (R::pos(s.w[0]) ? 1 : 0) : 2;
         c.on_y = which == 1;
         c.on_z = which == 2;
+        // the two factors of the distance, one product for all lanes
+        double a, b;
         if (c.bnd) {
             const double r = which == 0 ? s.r[0] : which == 1 ? s.r[1] : s.r[2];
             const double w = which == 0 ? s.w[0] : which == 1 ? s.w[1] : s.w[2];
-            c.l = face_distance(r, w, which == 0 ? s.iw[0] : R::recip(w), R::L(cp));
+            a = (R::pos(w) ? R::L(cp) : 0.0) - r;
+            b = which == 0 ? s.iw[0] : R::recip(w);
         } else {
-            const double e = exp_variate_shared(c.coll ? R::k53(hi, lo) : R::k53(ihi, ilo));
-            c.l = c.coll ? R::nonneg(e * R::inv_sigma(cp, m)) : interface_distance<double, G>(s, cp, m, e);
+            a = exp_variate_shared(c.coll ? R::k53(hi, lo) : R::k53(ihi, ilo));
+            b = c.coll ? R::inv_sigma(cp, m) : R::lambda(cp, m);
         }
+        double l = a * b;
+        if (which == 4) {
+            if (gd == 11) l *= R::abs(s.iw[0]);
+            else if (gd == 2) l /= sqrt(1.0 - s.w[2] * s.w[2]);
+        }
+        c.l = R::nonneg(l);
     } else {
         double x_c, x_i;
         R::exp_variates(hi, lo, ihi, ilo, &x_c, &x_i);
@@ -2020,10 +2031,8 @@ __device__ __forceinline__ void fill_draws(DrawBuffer<P> &b, int at, uint32_t bl
             if constexpr (sizeof(P) == 8) b.w2i0[at + t] = make_double2(mu, recip_or_inf(mu));
             else b.w[at + t] = make_float4(0.0f, 0.0f, mu, 0.0f);
         } else {
-            P mu, st, sn, cs;
-            R::direction_cosines(mu_hi, mu_lo, false, &mu, &st);
-            R::sincos_2pi(phi_hi, phi_lo, &sn, &cs);
-            const P wx = st * cs, wy = st * sn;
+            P mu, wx, wy;
+            R::direction(mu_hi, mu_lo, phi_hi, phi_lo, false, &mu, &wx, &wy);
             if constexpr (sizeof(P) == 8) {
                 double v = wx, r0 = 0.0, r1 = 0.0, r2 = 0.0;
 #pragma unroll 1

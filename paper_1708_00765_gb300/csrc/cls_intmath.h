@@ -167,8 +167,9 @@ CLS_HD double exp_variate(uint64_t k, IntLogTables tab) {
     return u128_to_double(m, 120);
 }
 
-// v 2^-62 rounded to the nearest double, for a signed Q62 value v
-CLS_HD double q62_to_double(int64_t v) {
+// v 2^e rounded to the nearest double (ties to even), for a signed v and a
+// normal result
+CLS_HD double fixed_to_double(int64_t v, int e) {
     if (v == 0) return 0.0;
     const uint64_t sgn = v < 0 ? (1ull << 63) : 0ull;
     const uint64_t a = v < 0 ? 0ull - (uint64_t)v : (uint64_t)v;
@@ -178,13 +179,16 @@ CLS_HD double q62_to_double(int64_t v) {
     const uint64_t round = (x >> 10) & 1ull;
     const uint64_t sticky = x & 0x3FFull;
     mant += round & ((sticky != 0ull ? 1ull : 0ull) | (mant & 1ull));
-    const uint64_t ex = (uint64_t)(63 - lz - 62 + 1023 - 1);
+    const uint64_t ex = (uint64_t)(63 - lz + e + 1023 - 1);
     return bits_to_double(sgn | ((ex << 52) + mant));
 }
 
-// (sin, cos) of 2 pi u for u = k 2^-53, 0 <= k < 2^53; sc: {sin, cos} of
+// v 2^-62 rounded to the nearest double, for a signed Q62 value v
+CLS_HD double q62_to_double(int64_t v) { return fixed_to_double(v, -62); }
+
+// (sin, cos) of 2 pi u in Q62 for u = k 2^-53, 0 <= k < 2^53; sc: {sin, cos} of
 // 2 pi j/256 times 2^62.
-CLS_HD void sincos_2pi_int(uint64_t k, const int64_t (*sc)[2], double *sn, double *cs) {
+CLS_HD void sincos_2pi_q62(uint64_t k, const int64_t (*sc)[2], int64_t *sn, int64_t *cs) {
     const uint64_t j = (k + (1ull << 44)) >> 45;           // nearest tabulated angle, 0..256
     const int64_t t = (int64_t)k - (int64_t)(j << 45);     // in [-2^44, 2^44)
     const int64_t S = sc[j & 255ull][0], C = sc[j & 255ull][1];
@@ -209,8 +213,16 @@ CLS_HD void sincos_2pi_int(uint64_t k, const int64_t (*sc)[2], double *sn, doubl
     // sin(a + delta) = S + S cm1 + C sin(delta); cos(a + delta) = C + C cm1 - S sin(delta)  (Q62)
     const int64_t s_cm1 = mulq63(S, cm1), c_cm1 = mulq63(C, cm1);
     const int64_t c_sd = smulhi64(C, sd) >> 5, s_sd = smulhi64(S, sd) >> 5;   // (Q62 Q69) >> 69
-    *sn = q62_to_double(S + s_cm1 + c_sd);
-    *cs = q62_to_double(C + c_cm1 - s_sd);
+    *sn = S + s_cm1 + c_sd;
+    *cs = C + c_cm1 - s_sd;
+}
+
+// The same as doubles.
+CLS_HD void sincos_2pi_int(uint64_t k, const int64_t (*sc)[2], double *sn, double *cs) {
+    int64_t s, c;
+    sincos_2pi_q62(k, sc, &s, &c);
+    *sn = q62_to_double(s);
+    *cs = q62_to_double(c);
 }
 
 // floor(a d / 2^62) for a in (0, 2^62] and signed d
@@ -270,14 +282,15 @@ CLS_HD double recip_int(double a) {
     return bits_to_double((b & (1ull << 63)) | ((e << 52) + mant));
 }
 
-// sqrt(X 2^-scale) rounded to the nearest double, for 0 <= X < 2^127 and even
-// scale: Newton-Raphson iteration for the reciprocal square root,
+// sqrt(X 2^-scale) = q 2^(e - 61) with q in [2^60, 2^61] (q = 0 for X = 0),
+// for 0 <= X < 2^127 and even scale: Newton-Raphson iteration for the reciprocal square root,
 // y <- y + y (1 - v y^2)/2, on v = X 2^-2t in [1/4, 1) from the FP32
 // approximate reciprocal square root of v's leading 24 bits (relative error
 // below 2^-22): one step in 32-bit arithmetic (to about 2^-29), one in Q61
-// fixed point, then sqrt(v) = v y and one rounding: within an ulp.
-CLS_HD double sqrt_int(U128 X, int scale) {
-    if ((X.hi | X.lo) == 0ull) return 0.0;
+// fixed point, then sqrt(v) = v y.
+CLS_HD uint64_t sqrt_q61(U128 X, int scale, int *e) {
+    *e = 0;
+    if ((X.hi | X.lo) == 0ull) return 0ull;
     // normalise by an even shift: v = X' 2^-128 in [1/4, 1)
     const int lz = X.hi ? clz64(X.hi) : 64 + clz64(X.lo);
     const int sh = lz & ~1;
@@ -311,15 +324,28 @@ CLS_HD double sqrt_int(U128 X, int scale) {
         const int64_t t = (int64_t)(umulhi64(vy, (uint64_t)y) << 4);  // v y^2, Q62
         y += mulq62(y, ((1ll << 62) - t) >> 1);                      // + y (1 - v y^2)/2
     }
-    const uint64_t q = umulhi64(v, (uint64_t)y);  // sqrt(v) = v y, Q61, in [2^60, 2^61]
+    // sqrt(X 2^-scale) = sqrt(v) 2^((128 - sh - scale)/2)
+    *e = (128 - sh - scale) / 2;
+    return umulhi64(v, (uint64_t)y);  // sqrt(v) = v y, Q61, in [2^60, 2^61]
+}
+
+// sqrt(X 2^-scale) rounded to the nearest double: within an ulp.
+CLS_HD double sqrt_int(U128 X, int scale) {
+    int e2;
+    const uint64_t q = sqrt_q61(X, scale, &e2);
+    if (q == 0ull) return 0.0;
     const int qz = clz64(q);
     const uint64_t n = q << qz;
     uint64_t mant = n >> 11;
     mant += ((n >> 10) & 1ull) & (((n & 0x3FFull) != 0ull ? 1ull : 0ull) | (mant & 1ull));
-    // sqrt(X 2^-scale) = sqrt(v) 2^((128 - sh - scale)/2)
-    const int e2 = (128 - sh - scale) / 2;
     const uint64_t e = (uint64_t)(63 - qz - 61 + e2 + 1023 - 1);
     return bits_to_double((e << 52) + mant);
+}
+
+// The product of q 2^(e - 61) (sqrt_q61) and a Q62 value c (|c| <= 2^62), one
+// rounding: its 2^-60 of q's magnitude is exact before it.
+CLS_HD double sqrt_times_q62(uint64_t q, int e, int64_t c) {
+    return fixed_to_double(smulhi64((int64_t)(q << 1), c), e - 60);
 }
 
 }  // namespace cls
