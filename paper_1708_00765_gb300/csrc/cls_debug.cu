@@ -36,9 +36,7 @@ __global__ void uniform_kernel(uint64_t seed, uint32_t case_id, const uint64_t *
     const cls::RoundKeys key = cls::make_round_keys(seed);
     cls::History<double> s64;
     cls::History<float> s32;
-    s64.h_lo = s32.h_lo = (uint32_t)h[i];
-    s64.h_hi = s32.h_hi = (uint32_t)(h[i] >> 32);
-    s64.cid = s32.cid = case_id;
+    s64.key = s32.key = cls::history_key(h[i], case_id, key);
     // the cached odd words come from the even draw before them
     const uint32_t jj = (uint32_t)j[i];
     s64.j = s32.j = jj & ~1u;

@@ -42,25 +42,26 @@ struct BankLayout<double> {
 
 template <typename P>
 __device__ __forceinline__ void bank_store(unsigned char *buf, uint32_t S, uint32_t slot, const History<P> &s, int run,
-                                           int reg);
+                                           int reg, const RoundKeys &rk);
 template <typename P>
 __device__ __forceinline__ void bank_load(const unsigned char *buf, uint32_t S, uint32_t slot, History<P> &s, int &run,
-                                          int &reg);
+                                          int &reg, const RoundKeys &rk);
 
 template <>
 __device__ __forceinline__ void bank_store<float>(unsigned char *buf, uint32_t S, uint32_t slot, const History<float> &s,
-                                                  int run, int reg) {
+                                                  int run, int reg, const RoundKeys &rk) {
+    const uint64_t h = history_id(s.key, rk);
     const size_t f = (size_t)S * 16;
     reinterpret_cast<float4 *>(buf)[slot] = make_float4(s.r[0], s.r[1], s.r[2], s.track0);
     reinterpret_cast<float4 *>(buf + f)[slot] = make_float4(s.w[0], s.w[1], s.w[2], s.track1);
-    reinterpret_cast<uint4 *>(buf + 2 * f)[slot] = make_uint4(s.h_lo, s.h_hi, s.j, s.c2);
+    reinterpret_cast<uint4 *>(buf + 2 * f)[slot] = make_uint4((uint32_t)h, (uint32_t)(h >> 32), s.j, s.c2);
     reinterpret_cast<uint4 *>(buf + 3 * f)[slot] =
         make_uint4(s.c3, (uint32_t)s.m | ((uint32_t)reg << 1), s.events, (uint32_t)run);
 }
 
 template <>
 __device__ __forceinline__ void bank_load<float>(const unsigned char *buf, uint32_t S, uint32_t slot, History<float> &s,
-                                                 int &run, int &reg) {
+                                                 int &run, int &reg, const RoundKeys &rk) {
     const size_t f = (size_t)S * 16;
     const float4 a = reinterpret_cast<const float4 *>(buf)[slot];
     const float4 b = reinterpret_cast<const float4 *>(buf + f)[slot];
@@ -72,8 +73,7 @@ __device__ __forceinline__ void bank_load<float>(const unsigned char *buf, uint3
     s.track0 = a.w;
     set_direction<float>(s, b.x, b.y, b.z);
     s.track1 = b.w;
-    s.h_lo = c.x;
-    s.h_hi = c.y;
+    s.key = history_key(((uint64_t)c.y << 32) | c.x, 0u, rk);
     s.j = c.z;
     s.c2 = c.w;
     s.c3 = d.x;
@@ -85,21 +85,22 @@ __device__ __forceinline__ void bank_load<float>(const unsigned char *buf, uint3
 
 template <>
 __device__ __forceinline__ void bank_store<double>(unsigned char *buf, uint32_t S, uint32_t slot,
-                                                   const History<double> &s, int run, int reg) {
+                                                   const History<double> &s, int run, int reg, const RoundKeys &rk) {
+    const uint64_t h = history_id(s.key, rk);
     const size_t f = (size_t)S * 16;
     reinterpret_cast<double2 *>(buf)[slot] = make_double2(s.r[0], s.r[1]);
     reinterpret_cast<double2 *>(buf + f)[slot] = make_double2(s.r[2], s.track0);
     reinterpret_cast<double2 *>(buf + 2 * f)[slot] = make_double2(s.w[0], s.w[1]);
     reinterpret_cast<double2 *>(buf + 3 * f)[slot] = make_double2(s.w[2], s.track1);
     reinterpret_cast<double2 *>(buf + 4 * f)[slot] = make_double2(s.iw[0], 0.0);
-    reinterpret_cast<uint4 *>(buf + 5 * f)[slot] = make_uint4(s.h_lo, s.h_hi, s.j, s.c2);
+    reinterpret_cast<uint4 *>(buf + 5 * f)[slot] = make_uint4((uint32_t)h, (uint32_t)(h >> 32), s.j, s.c2);
     reinterpret_cast<uint4 *>(buf + 6 * f)[slot] =
         make_uint4(s.c3, (uint32_t)s.m | ((uint32_t)reg << 1), s.events, (uint32_t)run);
 }
 
 template <>
 __device__ __forceinline__ void bank_load<double>(const unsigned char *buf, uint32_t S, uint32_t slot,
-                                                  History<double> &s, int &run, int &reg) {
+                                                  History<double> &s, int &run, int &reg, const RoundKeys &rk) {
     const size_t f = (size_t)S * 16;
     const double2 a = reinterpret_cast<const double2 *>(buf)[slot];
     const double2 b = reinterpret_cast<const double2 *>(buf + f)[slot];
@@ -117,8 +118,7 @@ __device__ __forceinline__ void bank_load<double>(const unsigned char *buf, uint
     s.w[2] = d.x;
     s.track1 = d.y;
     s.iw[0] = e.x;
-    s.h_lo = m0.x;
-    s.h_hi = m0.y;
+    s.key = history_key(((uint64_t)m0.y << 32) | m0.x, 0u, rk);
     s.j = m0.z;
     s.c2 = m0.w;
     s.c3 = m1.x;
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
                 const CaseParams &cp = a.cases[a.runs[feed_run].case_index];
                 History<P> s;
                 source<P, G>(s, cp, key, cursor + lane);
-                bank_store<P>(buf, W, nlive + lane, s, feed_run, feed_reg | (int)(gen[feed_reg] << 2));
+                bank_store<P>(buf, W, nlive + lane, s, feed_run, feed_reg | (int)(gen[feed_reg] << 2), key);
             }
             cursor += take;
             nlive += take;
@@ -286,16 +286,16 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
             Flight<P> f;
             int run = 0, packed = 0;
             bool alive = slot < nlive;
-            if (alive) bank_load<P>(buf, W, slot, s, run, packed);
+            if (alive) bank_load<P>(buf, W, slot, s, run, packed, key);
             const int ci = alive ? a.runs[run].case_index : 0;
-            s.cid = a.cases[ci].case_id;  // Philox counter word 3 (not stored in the bank)
+            s.key.cid = a.cases[ci].case_id;  // Philox counter word 3 (not stored in the bank)
             // the particle's region, or 2 if that region has since changed key
             int reg = packed & 3;
             if (reg < 2 && (uint32_t)(packed >> 2) != gen[reg]) reg = 2;
             uint64_t goff = 0;
             if (alive && (reg == 2 || sizeof(P) == 8)) {  // FP64: long flights score globally from any region
                 const RunCase &rc = a.runs[run];
-                const uint64_t h = ((uint64_t)s.h_hi << 32) | s.h_lo;
+                const uint64_t h = history_id(s.key, key);
                 const uint64_t batch = (h - rc.first) / rc.batch_len;
                 goff = ((uint64_t)ci * (uint64_t)a.t.nbatch + batch) * (uint64_t)nbs;
             }
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
                     }
                 }
                 if (o >= 0) {
-                    record_outcome(a, ci, s.h_lo, s.h_hi, o);
+                    record_outcome(a, ci, s.key, o);
                     if (reg < 2) finish_event_history<P>(regions + reg * rb, nbs, s, o);
                     else finish_history_global<P>(a, ci, s, o, false);
                     alive = false;
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
             live[1] -= __popc(__ballot_sync(CLS_FULL_MASK, died && reg == 1));
             const int store_tag = (reg < 2) ? (reg | (int)(gen[reg] << 2)) : 2;
             const unsigned b = __ballot_sync(CLS_FULL_MASK, alive);
-            if (alive) bank_store<P>(nxt, W, out + __popc(b & lt_mask), s, run, store_tag);
+            if (alive) bank_store<P>(nxt, W, out + __popc(b & lt_mask), s, run, store_tag, key);
             out += __popc(b);
         }
         // warp-aggregated event counters: one shared-memory atomic per counter
