@@ -49,27 +49,40 @@ inline double cost_estimate(const CaseParams &c) {
 // of them; as many warps start on a piece as it takes to employ all; and the
 // least a warp claims is 32 histories, a warp's lanes, or where that would not
 // go round, a power of two below.  `warps`: about as many as the launch has.
-// Runs of up to kNarrowHistories histories for each warp of the narrow walk go
-// to it alone (a.narrow): measured on the 3D box in FP64, 1e4 histories (5.5 a
-// warp) take 1.04 ms there and 1.10 ms in the tracker, 1e5 take 6.4 and 2.6 ms;
-// on the rod in FP32, 55 and 84 us, 260 and 113 us.
-constexpr double kNarrowHistories = 8.0;
-// Launches whose histories average this many events or more by the estimate
-// hand their warps' last histories over to the narrow walk: it walks a history
-// twice as fast, but only one per warp.  Measured: the diffusive box (153
-// events) at 1e6 histories in FP32 20.4 -> 18.7 ms, in FP64 75 -> 66 ms; the
-// box L = 10 (47 events) at 1e5 in FP64 2.6 -> 2.8 ms.
-constexpr double kHandOverEvents = 128.0;
+// Runs of up to narrow_histories histories for each warp of the narrow walk go to
+// it alone (a.narrow).  Measured, us in the tracker / the narrow walk at 14
+// histories a warp (25,000): FP32 box L = 10 525 / 320, rod 91 / 67, diffusive box
+// 2947 / 2546, and at 22 571 / 492, 107 / 97, 4756 / 3763; FP64 rod 135 / 119, slab
+// 171 / 167, but extruded 569 / 902, box 1788 / 1826.
+inline double narrow_histories(bool fp32, int geom) {
+    return fp32 ? 24.0 : geom == 1 || geom == 11 || geom == 13 ? 14.0 : 8.0;
+}
 
 // Estimated events per history: about cost^(3/4) (the cost estimate is within a
 // factor of two for short histories and several times too high for scattering media).
 inline double estimated_events(double cost) { return std::pow(std::max(cost, 1.0), 0.75); }
 
-inline void plan_pieces(LaunchArgs &a, uint64_t n, uint64_t batch_len, double mean_cost, int sm_count, bool fp32,
+// Warps of a launch hand their last histories over to the narrow walk, which
+// walks a history two to four times as fast, but only one per warp: the last
+// kHandOver where histories average kHandOverEvents or more by the estimate,
+// else the last two, except in the FP64 walks with two or three axes, whose
+// draws cost the narrow walk most.  Measured, none / 2 / 4 handed over: diffusive
+// box (153 events) 1e6 in FP32 20.4 / 14.7 / 13.3 ms, 1e5 10.1 / 8.3 / 6.3 ms; box
+// L = 10 (47 events) in FP32 1e6 1.74 / 1.57 / 1.56 ms, 1e5 781 / 678 / 665 us, in
+// FP64 1e5 2.15 / 2.25 / 2.45 ms; slab 1e5 in FP64 275 / 233 / 234 us.
+constexpr double kHandOverEvents = 128.0;
+
+inline int hand_over_for(double events, bool fp32, int geom) {
+    if (events >= kHandOverEvents) return kHandOver;
+    return fp32 || geom == 1 || geom == 11 || geom == 13 ? 2 : 0;
+}
+
+
+inline void plan_pieces(LaunchArgs &a, uint64_t n, uint64_t batch_len, double mean_cost, int geom, int sm_count, bool fp32,
                         uint64_t max_pieces) {
     const double total = (double)n * a.nruns;
     const double narrow_warps = (double)sm_count * kNarrowBlocks * (kNarrowBlock / 32);
-    a.narrow = total <= kNarrowHistories * narrow_warps;
+    a.narrow = total <= narrow_histories(fp32, geom) * narrow_warps;
     const double warps = a.narrow ? std::min(total, narrow_warps) : sm_count * (fp32 ? 28.0 : 20.0);
     const uint64_t used = (n + batch_len - 1) / batch_len;  // batches
     const uint64_t per_run = std::max<uint64_t>(1, std::min<uint64_t>(std::min<uint64_t>(used, 64), max_pieces / a.nruns));
@@ -77,7 +90,7 @@ inline void plan_pieces(LaunchArgs &a, uint64_t n, uint64_t batch_len, double me
     a.piece_len = batches * batch_len;
     a.pieces_per_run = (uint32_t)((used + batches - 1) / batches);
     a.team = (uint32_t)std::ceil(warps / ((double)a.pieces_per_run * a.nruns));
-    a.hand_over = estimated_events(mean_cost) >= kHandOverEvents ? kHandOver : 0;
+    a.hand_over = hand_over_for(estimated_events(mean_cost), fp32, geom);
     a.chunk = a.narrow ? 1 : 32;
     while (a.chunk > 1 && (double)a.chunk > total / warps) a.chunk >>= 1;
 }

@@ -486,7 +486,7 @@ int prepare_run(cls_handle *h, uint64_t n, uint64_t seed, RunPlan *plan) {
         ag.nruns = groups[g].ncases;
         ag.claimed = h->d_chunk_counter + kGroupCounters + pieces;
         if (groups[g].sched != CLS_SCHED_EVENT) {
-            plan_pieces(ag, n, batch_len_for(n, h->nbatch), groups[g].cost / groups[g].ncases, h->sm_count,
+            plan_pieces(ag, n, batch_len_for(n, h->nbatch), groups[g].cost / groups[g].ncases, groups[g].geom, h->sm_count,
                         h->opt.precision == CLS_PREC_FP32, kMaxPieces);
             pieces += (uint64_t)ag.pieces_per_run * ag.nruns;
         }

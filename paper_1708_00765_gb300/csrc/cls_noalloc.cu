@@ -131,7 +131,7 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
         img.cases[k] = make_case(params + 9 * (size_t)k, (uint32_t)k);
         cost += img.cases[k].cost * (double)n;
     }
-    plan_pieces(a, n, batch_len, cost / (double)n / ncases, sm_count, false, kNoallocMaxPieces);
+    plan_pieces(a, n, batch_len, cost / (double)n / ncases, 0, sm_count, false, kNoallocMaxPieces);
     a.chunk_counter = &scratch->chunk_counter;
     a.claimed = scratch->claimed;
     a.handed = &scratch->handed;
