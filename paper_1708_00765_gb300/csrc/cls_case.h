@@ -119,9 +119,9 @@ inline void plan_claims(RunCase &r, const CaseParams &c, double launch_cost, int
     r.claim_bits = (uint16_t)bits;
     // lanes die 32 / events per step, and waiting idles half of refill_min of them.  Measured, 2 / 4 / 8 / 12 / 16
     // lanes: box L = 10 (47 events, FP32, 1e8) 101 / 97 / 100 / 107 / 118 ms; sweep (5 events, 256 x 1e6) 50.8 /
-    // 49.4 / 47.3 / 46.5 / 47.1 ms
-    const double wait = std::floor(5.2 * std::sqrt(32.0 / estimated_events(c.cost)) + 0.5);
-    r.refill_min = (uint16_t)std::min(12.0, std::max(2.0, wait));
+    // 49.4 / 47.3 / 46.5 / 47.1 ms; by this rule 46.2 ms, with 5.2 and at most 12 lanes 46.8
+    const double wait = std::floor(6.5 * std::sqrt(32.0 / estimated_events(c.cost)) + 0.5);
+    r.refill_min = (uint16_t)std::min(16.0, std::max(2.0, wait));
 }
 
 // The kernels' view of one validated case: p_0 = Lambda_0 / (Lambda_0 +

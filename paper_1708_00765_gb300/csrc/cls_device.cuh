@@ -411,7 +411,6 @@ template <typename P>
 struct Flight {
     int k0, k1;
     P a0, a1, c;
-    bool tail;  // k1 is the mesh's last bin: the difference array's end marker falls past the mesh
 };
 
 // FP64 walk: the same in fixed point, units of 2^-kFixed64Bits bin widths,
@@ -421,7 +420,7 @@ template <>
 struct Flight<double> {
     int k0, k1;
     unsigned long long a0, a1, c;
-    bool tail, real;
+    bool real;
 };
 
 __device__ __forceinline__ double flight_real(unsigned long long a) { return __longlong_as_double((long long)a); }
@@ -679,7 +678,6 @@ __device__ __forceinline__ void plan_flight(Flight<float> &f, const Case &cp, fl
     if (R::is_zero(wx)) {
         const int k = R::floor_index(a * inv_dx, nb - 1);
         f.k0 = f.k1 = k;
-        f.tail = k == nb - 1;
         f.a0 = l;
         return;
     }
@@ -694,7 +692,6 @@ __device__ __forceinline__ void plan_flight(Flight<float> &f, const Case &cp, fl
     const int k1 = R::floor_index(uhi, nb - 1);
     f.k0 = k0;
     f.k1 = k1;
-    f.tail = k1 == nb - 1;
     if (k0 == k1) {  // the flight lies inside one bin: its length itself
         f.a0 = l;
         return;
@@ -780,7 +777,6 @@ __device__ __forceinline__ void plan_flight(Flight<double> &f, const Case &cp, d
     if (R::is_zero(wx)) k1 = k0 = (R::lt(a, b) ? k0 : k1);  // the bin that contains x0
     f.k0 = k0;
     f.k1 = k1;
-    f.tail = k1 == nb - 1;
     // in bin widths: a flight inside one bin scores its length itself, else
     // 1/|wx| in a whole bin
     const double v = k0 == k1 ? l * inv_dx : R::abs(iwx);
@@ -1225,12 +1221,17 @@ __device__ __forceinline__ int step(History<P> &s, const Case &cp, Draws &draws,
 // entries of 200: 14 cycles per warp and scheduler, against 62 for a 64-bit
 // integer atomic and 94 for a double (both are compare-and-swap loops, and
 // slow down further where lanes meet: 90 and 250 on 20 entries; the halves
-// stay at 14).
+// stay at 14).  The high half is added even where it is zero: the walk is short
+// of integer instructions, not of shared-memory ones (testing it first: box L =
+// 10, FP32, 1e8 histories 93.5 ms, adding it always 91.9).
 __device__ __forceinline__ void add_halves(uint32_t *lo, uint32_t *hi, unsigned long long x) {
     const uint32_t xl = (uint32_t)x;
     const uint32_t old = atomicAdd(lo, xl);
-    const uint32_t h = (uint32_t)(x >> 32) + (old + xl < old ? 1u : 0u);
-    if (h != 0u) atomicAdd(hi, h);
+    uint32_t h;  // the high half and the carry of old + xl
+    asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %1, %2;\n\taddc.u32 %0, %3, 0;\n\t}"
+        : "=r"(h)
+        : "r"(old), "r"(xl), "r"((uint32_t)(x >> 32)));
+    atomicAdd(hi, h);
 }
 
 template <typename P>
@@ -1334,11 +1335,7 @@ __device__ __forceinline__ void derive_counts(const History<P> &s, const CasePar
     *n_refl = s.events - *n_coll - s.n_int - leaked;
 }
 
-// Outcome and event counters of the lanes whose history ended this step
-// (`ended`, scoring into region lreg < 2).  When several lanes ended they are
-// summed over the warp per region (ballot counts, warp reductions of 16-bit
-// halves) and one lane adds each to the region, else each lane adds its own:
-// short histories that end together do not serialise on shared atomics.
+// Outcome and event counters of a finished history.
 __device__ __forceinline__ void count_one(uint32_t *ct, int outcome, uint32_t n_coll, uint32_t n_int, uint32_t n_refl,
                                           uint32_t events) {
     const int c = (outcome == EV_LEAK_X0) ? C_R : (outcome == EV_LEAK_XL) ? C_T : (outcome == EV_ABSORB) ? C_A : C_CAPPED;
@@ -1348,51 +1345,6 @@ __device__ __forceinline__ void count_one(uint32_t *ct, int outcome, uint32_t n_
     if (n_refl) add_count(ct, C_REFL, n_refl);
     add_count(ct, C_EVENTS, events);
     atomicMax(&ct[C_MAXEV], events);
-}
-
-__device__ __forceinline__ unsigned long long warp_sum32(bool mine, uint32_t x, bool small) {
-    const uint32_t v = mine ? x : 0u;
-    if (small) return __reduce_add_sync(CLS_FULL_MASK, v);  // 32 values below 2^27 sum below 2^32
-    return (unsigned long long)__reduce_add_sync(CLS_FULL_MASK, v & 0xFFFFu) +
-           ((unsigned long long)__reduce_add_sync(CLS_FULL_MASK, v >> 16) << 16);
-}
-
-template <typename P>
-__device__ __forceinline__ void warp_count(unsigned char *regions, int rbytes, int nbs, bool ended, int lreg,
-                                           const History<P> &s, uint32_t n_coll, uint32_t n_refl, int outcome, int lane,
-                                           bool small) {
-    const unsigned em = __ballot_sync(CLS_FULL_MASK, ended);
-    if (em == 0u) return;
-    if (__popc(em) < 4) {
-        if (ended)
-            count_one(region_counters(regions + lreg * rbytes, nbs), outcome, n_coll, s.n_int, n_refl, s.events);
-        return;
-    }
-#pragma unroll 1
-    for (int r = 0; r < 2; ++r) {
-        const bool mine = ended && lreg == r;
-        const unsigned m = __ballot_sync(CLS_FULL_MASK, mine);
-        if (m == 0u) continue;
-        const unsigned nr = __popc(__ballot_sync(CLS_FULL_MASK, mine && outcome == EV_LEAK_X0));
-        const unsigned nt = __popc(__ballot_sync(CLS_FULL_MASK, mine && outcome == EV_LEAK_XL));
-        const unsigned na = __popc(__ballot_sync(CLS_FULL_MASK, mine && outcome == EV_ABSORB));
-        const unsigned ncap = __popc(m) - nr - nt - na;
-        const unsigned long long nc = warp_sum32(mine, n_coll, small), ni = warp_sum32(mine, s.n_int, small);
-        const unsigned long long nf = warp_sum32(mine, n_refl, small), ne = warp_sum32(mine, s.events, small);
-        const unsigned mx = __reduce_max_sync(CLS_FULL_MASK, mine ? s.events : 0u);
-        if (lane == __ffs(m) - 1) {
-            uint32_t *ct = region_counters(regions + r * rbytes, nbs);
-            if (nr) add_count(ct, C_R, nr);
-            if (nt) add_count(ct, C_T, nt);
-            if (na) add_count(ct, C_A, na);
-            if (ncap) add_count(ct, C_CAPPED, ncap);
-            if (nc) add_count(ct, C_COLL, nc);
-            if (ni) add_count(ct, C_INT, ni);
-            if (nf) add_count(ct, C_REFL, nf);
-            add_count(ct, C_EVENTS, ne);
-            atomicMax(&ct[C_MAXEV], mx);
-        }
-    }
 }
 
 // The interior bins of the flights that score into the global bins, spread
@@ -1421,6 +1373,11 @@ __device__ __forceinline__ void spread_interior(double *gflux, uint64_t goff, in
         const uint64_t ogoff = __shfl_sync(CLS_FULL_MASK, goff, o);
         if (t < total) atomicAdd(&gflux[ogoff + ob + t], oc);
     }
+}
+
+// The global bins of (case, batch), as an offset into the flux array.
+__device__ __forceinline__ uint64_t bins_offset(const Tallies &t, int lcase, uint32_t lbatch) {
+    return ((uint64_t)lcase * (uint64_t)t.nbatch + lbatch) * (uint64_t)t.nbins_stride;
 }
 
 // Bound on a region's bins between two flushes (FP64 walk): each lane sums the
@@ -1467,16 +1424,14 @@ struct FixedFlight {
 // Score the warp's flights.
 //   Region lanes: the difference array's entries (FixedFlight), two integer
 //   additions for a flight inside one bin, three when it spans two, four
-//   otherwise.  With SKIP, an entry that adds zero is left out (q0 = qc when
-//   the flight covers its first bin whole, q1 = qc when it covers its last bin
-//   whole), and so is the end marker D[k1+1] of a flight whose last bin is the
-//   mesh's (the flush never reads past the last bin).
+//   otherwise.
 //   Lanes that score globally (scores_global) add FP64 values to the bins of
-//   their (case, batch) at gflux + goff, interior bins spread over the warp.
+//   their (case, batch), interior bins spread over the warp.
 // Returns the lane's share of DepositBound.
-template <typename P, bool SKIP = false>
-__device__ __forceinline__ uint32_t warp_deposit(unsigned char *regions, int rbytes, int nbs, int lreg, double *gflux,
-                                                 uint64_t goff, const Flight<P> &f, int lane) {
+template <typename P>
+__device__ __forceinline__ uint32_t warp_deposit(unsigned char *regions, int rbytes, const Tallies &t, int lreg, int lcase,
+                                                 uint32_t lbatch, const Flight<P> &f, int lane) {
+    const int nbs = t.nbins_stride;
     const bool has = f.k1 >= f.k0, global = scores_global(f, lreg);
     uint32_t bound = 0;
     if (has) {
@@ -1485,26 +1440,20 @@ __device__ __forceinline__ uint32_t warp_deposit(unsigned char *regions, int rby
             unsigned char *region = regions + lreg * rbytes;
             const FixedFlight q(f);
             bound = q.bound;
-            if constexpr (SKIP) {
-                if (q.q0 != 0ull) add_entry(region, nbs, f.k0, q.q0);
-                if (q.d1 != 0ull && (q.multi || !f.tail)) add_entry(region, nbs, f.k0 + 1, q.d1);
-                if (q.inter && q.d2 != 0ull) add_entry(region, nbs, f.k1, q.d2);
-                if (q.multi && !f.tail) add_entry(region, nbs, f.k1 + 1, q.d3);
-            } else {
-                add_entry(region, nbs, f.k0, q.q0);
-                add_entry(region, nbs, f.k0 + 1, q.d1);
-                if (q.inter) add_entry(region, nbs, f.k1, q.d2);
-                if (q.multi) add_entry(region, nbs, f.k1 + 1, q.d3);
-            }
+            add_entry(region, nbs, f.k0, q.q0);
+            add_entry(region, nbs, f.k0 + 1, q.d1);
+            if (q.inter) add_entry(region, nbs, f.k1, q.d2);
+            if (q.multi) add_entry(region, nbs, f.k1 + 1, q.d3);
         } else {
-            double *gbins = gflux + goff;
+            double *gbins = t.flux + bins_offset(t, lcase, lbatch);
             atomicAdd(&gbins[f.k0], flight_real(f.a0));
             if (f.k1 > f.k0) atomicAdd(&gbins[f.k1], flight_real(f.a1));
         }
     }
     const int ni = (has && global) ? max(f.k1 - f.k0 - 1, 0) : 0;
     // one vote instead of the scan when no lane has any
-    if (__any_sync(CLS_FULL_MASK, ni > 0)) spread_interior(gflux, goff, f.k0, flight_real(f.c), ni, lane);
+    if (__any_sync(CLS_FULL_MASK, ni > 0))
+        spread_interior(t.flux, bins_offset(t, lcase, lbatch), f.k0, flight_real(f.c), ni, lane);
     return bound;
 }
 
@@ -1866,20 +1815,19 @@ struct HistoryBounds<float, G> {
     static constexpr int threads = history_threads_fp32(G), blocks = 4;
 };
 
-// The end of a lane's history: outcome record, statistics, and (unless COUNT is
-// false, for lanes that score into a region) its counters.
-template <typename P, int G, bool COUNT>
+// The end of a lane's history: outcome record, statistics and counters.
+template <typename P, int G>
 __device__ __forceinline__ void end_history(unsigned char *regions, const LaunchArgs &a, const History<P> &s, int out,
-                                            int lreg, int lcase, int lane, uint32_t *n_coll, uint32_t *n_refl) {
-    derive_counts<P, G>(s, a.cases[lcase], out, n_coll, n_refl);
+                                            int lreg, int lcase, int lane) {
+    uint32_t n_coll, n_refl;
+    derive_counts<P, G>(s, a.cases[lcase], out, &n_coll, &n_refl);
     record_outcome(a, lcase, s.key, out);
     if (lreg < 2) {
         unsigned char *region = regions + lreg * a.region_bytes;
         if (!finish_history<P>(region, a.t.nbins_stride, s, lane)) add_history_stats_global<P>(a, lcase, s);
-        if constexpr (COUNT)
-            count_one(region_counters(region, a.t.nbins_stride), out, *n_coll, s.n_int, *n_refl, s.events);
+        count_one(region_counters(region, a.t.nbins_stride), out, n_coll, s.n_int, n_refl, s.events);
     } else {
-        finish_history_global<P>(a, lcase, s, out, true, *n_coll, *n_refl);
+        finish_history_global<P>(a, lcase, s, out, true, n_coll, n_refl);
     }
 }
 
@@ -1923,20 +1871,7 @@ __device__ __forceinline__ bool hand_over(const LaunchArgs &a, const History<P> 
     return true;
 }
 
-// WC: the instance for launches of short histories, in which many histories
-// end in the same step and many flights touch the slab's faces.  Its
-// history-end counters are summed over the warp first (warp_count; otherwise
-// each lane adds its own, count_one), and its deposits skip the difference
-// array's zero entries and the end markers past the mesh (warp_deposit's
-// SKIP): a flight from x = 0 or to x = L, over whole bins at that end, needs
-// one or two shared atomics instead of four, and the lanes born at x = 0 no
-// longer queue on the same entries.  The mixed-geometry kernel serves batch
-// sweeps and always takes it.  Measured on the 256-case sweep: 10% faster
-// (rods 12%) for the summed counters, 6.7% more for the skipped entries; on
-// the 3D box's 47-event histories the first costs 1% and the second 2%, so
-// the host picks the instance per launch.  A template parameter rather than a
-// runtime switch: carrying both paths measured 1% slower on the 3D box.
-template <typename P, int G, bool WC = (G == 0)>
+template <typename P, int G>
 __global__ void __launch_bounds__(HistoryBounds<P, G>::threads, HistoryBounds<P, G>::blocks) history_kernel(const LaunchArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
@@ -1974,14 +1909,7 @@ __global__ void __launch_bounds__(HistoryBounds<P, G>::threads, HistoryBounds<P,
         // History ends and births, together, once several lanes wait for them:
         // both are long stretches of code for the few lanes concerned.
         if (__popc(idle) >= wait) {
-            uint32_t n_coll = 0, n_refl = 0;
-            if (out >= 0) end_history<P, G, !(WC || G == 0)>(regions, a, s, out, lreg, lcase, lane, &n_coll, &n_refl);
-            // short histories often end together: their counters are then summed
-            // over the warp first (the host asks for it when a launch's cases average
-            // few events per history, and always for the mixed-geometry kernel)
-            if constexpr (WC || G == 0)
-                warp_count<P>(regions, rb, a.t.nbins_stride, out >= 0 && lreg < 2, lreg, s, n_coll, n_refl, out, lane,
-                              a.max_events < (1u << 27));
+            if (out >= 0) end_history<P, G>(regions, a, s, out, lreg, lcase, lane);
             out = out >= 0 ? kEmpty : out;
             if (!exhausted) {
                 exhausted = refill<P, G>(regions, rb, feed, a, s, out, lreg, lcase, lbatch, wait, lane);
@@ -2004,10 +1932,7 @@ __global__ void __launch_bounds__(HistoryBounds<P, G>::threads, HistoryBounds<P,
             const int ev = step<P, false, G>(s, a.cases[lcase], draws, a.max_events, f, nullptr, lreg == 2);
             out = ev < 0 ? kWalking : ev;
         }
-        const uint64_t goff = scores_global(f, lreg)
-                                  ? ((uint64_t)lcase * (uint64_t)a.t.nbatch + lbatch) * (uint64_t)a.t.nbins_stride
-                                  : 0ull;
-        deposited += warp_deposit<P, WC>(regions, rb, a.t.nbins_stride, lreg, a.t.flux, goff, f, lane);
+        deposited += warp_deposit<P>(regions, rb, a.t, lreg, lcase, lbatch, f, lane);
         if constexpr (sizeof(P) == 8) {  // before a bin's sum can outgrow its 64 bits
             if (__any_sync(CLS_FULL_MASK, deposited >= kDepositBound)) {
                 __syncwarp();
@@ -2106,7 +2031,7 @@ static_assert(sizeof(NarrowMemory<float>) <= narrow_memory_bytes(false) &&
 template <typename P, int G>
 __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(const LaunchArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x & 31, nbs = a.t.nbins_stride;
+    const int lane = threadIdx.x & 31;
     unsigned long long count = 0;
     if (!a.narrow) {
         count = min(*a.handed, (unsigned long long)a.straggler_cap);
@@ -2132,8 +2057,7 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
         f.k0 = 0;
         f.k1 = -1;
         if (lane < held) plan_flight(f, a.cases[key_case], x0, x1, l, fw, fiw, false);
-        const uint64_t goff = ((uint64_t)key_case * (uint64_t)a.t.nbatch + key_batch) * (uint64_t)nbs;
-        deposited += warp_deposit<P>(region, a.region_bytes, nbs, 0, a.t.flux, goff, f, lane);
+        deposited += warp_deposit<P>(region, a.region_bytes, a.t, 0, key_case, key_batch, f, lane);
         held = 0;
         if constexpr (sizeof(P) == 8) {  // before a bin's sum can outgrow its 64 bits
             if (__any_sync(CLS_FULL_MASK, deposited >= kDepositBound)) {
@@ -2217,10 +2141,7 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
             }
             if (++held == 32) score_held();
         }
-        if (lane == 0) {
-            uint32_t n_coll, n_refl;
-            end_history<P, G, true>(region, a, s, ev, 0, lcase, lane, &n_coll, &n_refl);
-        }
+        if (lane == 0) end_history<P, G>(region, a, s, ev, 0, lcase, lane);
         __syncwarp();
         if (sizeof(P) == 4 && ++fed >= a.flush_every) {  // FP32: before a bin's sum can outgrow its 64 bits
             if (held > 0) score_held();

@@ -292,12 +292,10 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
             // the particle's region, or 2 if that region has since changed key
             int reg = packed & 3;
             if (reg < 2 && (uint32_t)(packed >> 2) != gen[reg]) reg = 2;
-            uint64_t goff = 0;
+            uint32_t batch = 0;
             if (alive && (reg == 2 || sizeof(P) == 8)) {  // FP64: long flights score globally from any region
                 const RunCase &rc = a.runs[run];
-                const uint64_t h = history_id(s.key, key);
-                const uint64_t batch = (h - rc.first) / rc.batch_len;
-                goff = ((uint64_t)ci * (uint64_t)a.t.nbatch + batch) * (uint64_t)nbs;
+                batch = (uint32_t)((history_id(s.key, key) - rc.first) / rc.batch_len);
             }
             const uint32_t ev0 = alive ? s.events : 0u;
             s.n_coll = s.n_int = s.n_refl = 0;
@@ -308,7 +306,7 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
                 f.k0 = 0;
                 f.k1 = -1;
                 if (alive) o = step<P, false, G>(s, a.cases[ci], draws, a.max_events, f, nullptr, reg == 2);
-                deposited += warp_deposit<P>(regions, rb, nbs, reg, a.t.flux, goff, f, lane);
+                deposited += warp_deposit<P>(regions, rb, a.t, reg, ci, batch, f, lane);
                 if constexpr (sizeof(P) == 8) {  // before a bin's sum can outgrow its 64 bits
                     if (__any_sync(CLS_FULL_MASK, deposited >= kDepositBound)) {
                         __syncwarp();

@@ -13,13 +13,6 @@ namespace {
 
 template <int G>
 cudaError_t launch_history_g(const LaunchArgs &a, int grid, int block, size_t smem, cudaStream_t s) {
-    if (G != 0 && a.warp_counts) {
-        static std::atomic<unsigned long long> optin_wc{0};
-        const cudaError_t e = ensure_smem_optin(history_kernel<double, G, true>, optin_wc);
-        if (e != cudaSuccess) return e;
-        history_kernel<double, G, true><<<grid, block, smem, s>>>(a);
-        return cudaGetLastError();
-    }
     static std::atomic<unsigned long long> optin{0};
     const cudaError_t e = ensure_smem_optin(history_kernel<double, G>, optin);
     if (e != cudaSuccess) return e;

@@ -403,11 +403,6 @@ struct Group {
     int ncases;
 };
 
-// A launch whose cases average fewer estimated events per history than this
-// runs the tracker's short-history instance (history-end counters summed over
-// the warp, deposits that skip zero and past-the-mesh difference entries).
-constexpr double kWarpCountCost = 32.0;
-
 std::vector<Group> plan_groups(const cls_handle *h, std::vector<int> *gk) {
     std::vector<Group> groups;
     const int nc = (int)h->cases.size();
@@ -508,7 +503,6 @@ int prepare_run(cls_handle *h, uint64_t n, uint64_t seed, RunPlan *plan) {
         ag.chunk_counter = h->d_chunk_counter + g;
         ag.handed = h->d_chunk_counter + kMaxGroups + g;
         ag.taken = h->d_chunk_counter + 2 * kMaxGroups + g;
-        ag.warp_counts = (groups[g].geom == 0 || groups[g].cost < kWarpCountCost * groups[g].ncases) ? 1 : 0;
         plan->sched[g] = groups[g].sched;
         plan->geom[g] = groups[g].geom;
     }

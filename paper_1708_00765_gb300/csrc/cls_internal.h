@@ -127,7 +127,6 @@ struct LaunchArgs {
     uint32_t max_events;
     int region_bytes;     // bytes per warp tally region (see region_bytes())
     uint32_t flush_every; // FP32: flush a region after this many histories were fed into it
-    int warp_counts;      // history tracker: its short-history instance (warp-summed counters, sparse deposits)
     const OutcomeRecord *outcomes;  // per-history outcome record, or nullptr (never recorded)
     // event schedule only
     void *bank;            // grid warps x 2 buffers x bank_slots particles (SoA)

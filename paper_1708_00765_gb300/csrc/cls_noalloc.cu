@@ -143,7 +143,6 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
     a.rk = make_round_keys(seed);
     a.max_events = 100000000u;
     a.region_bytes = region_bytes(nbins_stride);
-    a.warp_counts = 1;
 
     for (int k = 0; k < ncases; ++k) {
         RunCase &r = img.runs[k];
