@@ -415,7 +415,7 @@ int cls_debug_fixed32(const float *c, int n, unsigned long long *out);
  * options; per-history event cap 1e8).  The call is asynchronous, so it cannot
  * report capped histories as CLS_E_EVENT_LIMIT: they show in d_counters[k][7].
  *
- * Scratch (case parameters, work list, work counters; about 560 KB) lives in a
+ * Scratch (case parameters, work list, work counters; about 620 KB) lives in a
  * static device array that every GPU loading the library holds until the
  * process exits.  The first call on each device looks up that array's device
  * address (with the device current) and keeps it for the life of the process;

@@ -1318,33 +1318,39 @@ __device__ __forceinline__ bool finish_history(unsigned char *region, int nbs, c
     return true;
 }
 
-// A finished history's collisions and reflections, from its draw index and its
-// other counters (the walk need not count them): the source takes a fixed
-// number of draws, every event two, every collision one and every scatter one
+// Draws that the source takes.
+template <int G>
+__device__ __forceinline__ uint32_t source_draws(const CaseParams &cp) {
+    const int gd = geometry<G>(cp);
+    const uint32_t volume = cp.source == 1;
+    return gd == 3 ? 5u + volume : gd == 2 ? 4u + volume : gd == 1 ? 1u + 2u * volume : 2u + volume;
+}
+
+// A finished history's collisions and reflections since its draw index was
+// base_j, from that and its other counters since then (the walk need not count
+// them): every event takes two draws, every collision one and every scatter one
 // more (a direction cosine) or two (mu and phi); and every event is a
 // collision, an interface crossing, a reflection or the final leak.
 template <typename P, int G>
-__device__ __forceinline__ void derive_counts(const History<P> &s, const CaseParams &cp, int outcome, uint32_t *n_coll,
-                                              uint32_t *n_refl) {
+__device__ __forceinline__ void derive_counts(const History<P> &s, const CaseParams &cp, int outcome, uint32_t base_j,
+                                              uint32_t events, uint32_t *n_coll, uint32_t *n_refl) {
     const int gd = geometry<G>(cp);
-    const bool wide = gd == 3 || gd == 2, volume = cp.source == 1;
-    const uint32_t source = gd == 3 ? 5u + volume : gd == 2 ? 4u + volume : gd == 1 ? 1u + 2u * volume : 2u + volume;
     const uint32_t absorbed = outcome == EV_ABSORB, leaked = outcome == EV_LEAK_X0 || outcome == EV_LEAK_XL;
-    const uint32_t extra = s.j - source - 2u * s.events;  // of collisions and scatters
-    *n_coll = wide ? (extra + 2u * absorbed) / 3u : (extra + absorbed) / 2u;
-    *n_refl = s.events - *n_coll - s.n_int - leaked;
+    const uint32_t extra = s.j - base_j - 2u * events;  // of collisions and scatters
+    *n_coll = gd == 3 || gd == 2 ? (extra + 2u * absorbed) / 3u : (extra + absorbed) / 2u;
+    *n_refl = events - *n_coll - s.n_int - leaked;
 }
 
 // Outcome and event counters of a finished history.
 __device__ __forceinline__ void count_one(uint32_t *ct, int outcome, uint32_t n_coll, uint32_t n_int, uint32_t n_refl,
-                                          uint32_t events) {
+                                          uint32_t events, uint32_t longest) {
     const int c = (outcome == EV_LEAK_X0) ? C_R : (outcome == EV_LEAK_XL) ? C_T : (outcome == EV_ABSORB) ? C_A : C_CAPPED;
     add_count(ct, c, 1ull);
     if (n_coll) add_count(ct, C_COLL, n_coll);
     if (n_int) add_count(ct, C_INT, n_int);
     if (n_refl) add_count(ct, C_REFL, n_refl);
     add_count(ct, C_EVENTS, events);
-    atomicMax(&ct[C_MAXEV], events);
+    atomicMax(&ct[C_MAXEV], longest);
 }
 
 // The interior bins of the flights that score into the global bins, spread
@@ -1499,7 +1505,7 @@ __device__ __forceinline__ void add_history_stats_global(const LaunchArgs &a, in
 template <typename P>
 __device__ __forceinline__ void finish_history_global(const LaunchArgs &a, int case_index, const History<P> &s,
                                                       int outcome, bool with_event_counts, uint32_t n_coll = 0,
-                                                      uint32_t n_refl = 0) {
+                                                      uint32_t n_refl = 0, uint32_t events = 0) {
     add_history_stats_global<P>(a, case_index, s);
     unsigned long long *ct = a.t.counters + (size_t)case_index * C_NUM;
     const int c = (outcome == EV_LEAK_X0) ? C_R : (outcome == EV_LEAK_XL) ? C_T : (outcome == EV_ABSORB) ? C_A : C_CAPPED;
@@ -1508,7 +1514,7 @@ __device__ __forceinline__ void finish_history_global(const LaunchArgs &a, int c
         if (n_coll) atomicAdd(&ct[C_COLL], (unsigned long long)n_coll);
         if (s.n_int) atomicAdd(&ct[C_INT], (unsigned long long)s.n_int);
         if (n_refl) atomicAdd(&ct[C_REFL], (unsigned long long)n_refl);
-        atomicAdd(&ct[C_EVENTS], (unsigned long long)s.events);
+        atomicAdd(&ct[C_EVENTS], (unsigned long long)events);
     }
     atomicMax(&ct[C_MAXEV], (unsigned long long)s.events);
 }
@@ -1815,28 +1821,31 @@ struct HistoryBounds<float, G> {
     static constexpr int threads = history_threads_fp32(G), blocks = 4;
 };
 
-// The end of a lane's history: outcome record, statistics and counters.
+// The end of a lane's history: outcome record, statistics and counters (those
+// since its draw index was base_j and its events base_events).
 template <typename P, int G>
 __device__ __forceinline__ void end_history(unsigned char *regions, const LaunchArgs &a, const History<P> &s, int out,
-                                            int lreg, int lcase, int lane) {
+                                            int lreg, int lcase, uint32_t base_j, uint32_t base_events, int lane) {
+    const uint32_t events = s.events - base_events;
     uint32_t n_coll, n_refl;
-    derive_counts<P, G>(s, a.cases[lcase], out, &n_coll, &n_refl);
+    derive_counts<P, G>(s, a.cases[lcase], out, base_j, events, &n_coll, &n_refl);
     record_outcome(a, lcase, s.key, out);
     if (lreg < 2) {
         unsigned char *region = regions + lreg * a.region_bytes;
         if (!finish_history<P>(region, a.t.nbins_stride, s, lane)) add_history_stats_global<P>(a, lcase, s);
-        count_one(region_counters(region, a.t.nbins_stride), out, n_coll, s.n_int, n_refl, s.events);
+        count_one(region_counters(region, a.t.nbins_stride), out, n_coll, s.n_int, n_refl, events, s.events);
     } else {
-        finish_history_global<P>(a, lcase, s, out, true, n_coll, n_refl);
+        finish_history_global<P>(a, lcase, s, out, true, n_coll, n_refl, events);
     }
 }
 
-// A history handed from the history tracker to the narrow walk.
+// A history handed from a tracker to the narrow walk, with the draw index and
+// events up to which its collisions, crossings and reflections are counted.
 template <typename P>
 struct Straggler {
     P r[3], w[3], iw, track0, track1;
     HistoryKey key;
-    uint32_t j, events, n_int, m, lcase, lbatch;
+    uint32_t j, events, n_int, m, lcase, lbatch, base_j, base_events;
 };
 static_assert(sizeof(Straggler<float>) <= kStragglerBytes && sizeof(Straggler<double>) <= kStragglerBytes,
               "the host sizes the hand-over buffer");
@@ -1846,7 +1855,7 @@ static_assert(sizeof(Straggler<float>) <= kStragglerBytes && sizeof(Straggler<do
 // lane's history was taken (all but those beyond the buffer's capacity).
 template <typename P>
 __device__ __forceinline__ bool hand_over(const LaunchArgs &a, const History<P> &s, int lcase, uint32_t lbatch,
-                                          unsigned live, int lane) {
+                                          uint32_t base_j, uint32_t base_events, unsigned live, int lane) {
     unsigned slot = 0;
     if (lane == 0) slot = (unsigned)atomicAdd(a.handed, (unsigned long long)__popc(live));
     slot = __shfl_sync(CLS_FULL_MASK, slot, 0) + __popc(live & ((1u << lane) - 1u));
@@ -1867,6 +1876,8 @@ __device__ __forceinline__ bool hand_over(const LaunchArgs &a, const History<P> 
     t.m = (uint32_t)s.m;
     t.lcase = (uint32_t)lcase;
     t.lbatch = lbatch;
+    t.base_j = base_j;
+    t.base_events = base_events;
     *reinterpret_cast<Straggler<P> *>(a.stragglers + (size_t)slot * kStragglerBytes) = t;
     return true;
 }
@@ -1909,7 +1920,8 @@ __global__ void __launch_bounds__(HistoryBounds<P, G>::threads, HistoryBounds<P,
         // History ends and births, together, once several lanes wait for them:
         // both are long stretches of code for the few lanes concerned.
         if (__popc(idle) >= wait) {
-            if (out >= 0) end_history<P, G>(regions, a, s, out, lreg, lcase, lane);
+            if (out >= 0)
+                end_history<P, G>(regions, a, s, out, lreg, lcase, source_draws<G>(a.cases[lcase]), 0u, lane);
             out = out >= 0 ? kEmpty : out;
             if (!exhausted) {
                 exhausted = refill<P, G>(regions, rb, feed, a, s, out, lreg, lcase, lbatch, wait, lane);
@@ -1920,7 +1932,7 @@ __global__ void __launch_bounds__(HistoryBounds<P, G>::threads, HistoryBounds<P,
             const unsigned live = __ballot_sync(CLS_FULL_MASK, out == kWalking);
             if (exhausted && live != 0u && __popc(live) <= a.hand_over) {
                 if (out == kWalking) resolve_direction<P, G>(s, a.cases[lcase], key);
-                if (hand_over<P>(a, s, lcase, lbatch, live, lane)) out = kEmpty;
+                if (hand_over<P>(a, s, lcase, lbatch, source_draws<G>(a.cases[lcase]), 0u, live, lane)) out = kEmpty;
             }
             if (__all_sync(CLS_FULL_MASK, out != kWalking)) break;
         }
@@ -2071,7 +2083,7 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
         // the next history: all lanes hold its state
         History<P> s;
         int lcase;
-        uint32_t lbatch;
+        uint32_t lbatch, base_j, base_events;
         if (a.narrow) {
             if (feed->pos == feed->pos_end && !claim(feed, a, lane)) break;
             const RunCase &rc = a.runs[feed->piece / a.pieces_per_run];
@@ -2082,6 +2094,8 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
             lcase = rc.case_index;
             lbatch = (uint32_t)(pos / rc.batch_len);
             source<P, G>(s, a.cases[lcase], a.rk, rc.first + pos);
+            base_j = s.j;
+            base_events = 0;
         } else {
             unsigned long long i;
             if (lane == 0) i = atomicAdd(a.taken, 1ull);
@@ -2103,6 +2117,8 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
             s.m = (int)t.m;
             lcase = (int)t.lcase;
             lbatch = t.lbatch;
+            base_j = t.base_j;
+            base_events = t.base_events;
         }
         if constexpr (sizeof(P) == 8) {
             s.iw[1] = recip_or_inf(s.w[1]);
@@ -2141,7 +2157,7 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
             }
             if (++held == 32) score_held();
         }
-        if (lane == 0) end_history<P, G>(region, a, s, ev, 0, lcase, lane);
+        if (lane == 0) end_history<P, G>(region, a, s, ev, 0, lcase, base_j, base_events, lane);
         __syncwarp();
         if (sizeof(P) == 4 && ++fed >= a.flush_every) {  // FP32: before a bin's sum can outgrow its 64 bits
             if (held > 0) score_held();

@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
     uint32_t gen[2] = {0, 0};
     uint64_t cursor = 0, end = 0;
     int feed_reg = 0, feed_run = 0;
-    bool exhausted = false, have_pending = false;
+    bool exhausted = false, have_pending = false, handing = a.hand_over > 0;
     unsigned long long pending = 0;
     // a region still serving more particles than this is drained rather than evicted
     const int evict_max = (int)(W >> 4);
@@ -275,6 +275,8 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
         // bank every events_per_pass events: the longest histories of a launch
         // (10^4 events and more) would otherwise pay a bank round trip every few
         // events while the rest of the GPU idles.
+        // And once at most hand_over of them are left it hands those over to the
+        // narrow walk, if there is room (asked once).
         const bool tail = exhausted && nlive <= 32u;
         const uint32_t epp = tail ? 0xFFFFFFFFu : a.events_per_pass;
         // collisions, interface crossings, reflections, events of this pass, per region
@@ -301,7 +303,8 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
             s.n_coll = s.n_int = s.n_refl = 0;
             bool died = false;
             for (uint32_t e = 0; e < epp; ++e) {
-                if (!__any_sync(CLS_FULL_MASK, alive)) break;
+                const unsigned walking = __ballot_sync(CLS_FULL_MASK, alive);
+                if (walking == 0u || (tail && handing && __popc(walking) <= a.hand_over)) break;
                 int o = -1;
                 f.k0 = 0;
                 f.k1 = -1;
@@ -345,6 +348,19 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
             }
             live[0] -= __popc(__ballot_sync(CLS_FULL_MASK, died && reg == 0));
             live[1] -= __popc(__ballot_sync(CLS_FULL_MASK, died && reg == 1));
+            if (tail && handing) {
+                handing = false;
+                const unsigned walking = __ballot_sync(CLS_FULL_MASK, alive);
+                if (walking != 0u) {
+                    if (alive) {
+                        const RunCase &rc = a.runs[run];
+                        batch = (uint32_t)((history_id(s.key, key) - rc.first) / rc.batch_len);
+                    }
+                    // this pass and the earlier ones have counted its events so far
+                    s.n_int = 0;
+                    if (hand_over<P>(a, s, ci, batch, s.j, s.events, walking, lane)) alive = false;
+                }
+            }
             const int store_tag = (reg < 2) ? (reg | (int)(gen[reg] << 2)) : 2;
             const unsigned b = __ballot_sync(CLS_FULL_MASK, alive);
             if (alive) bank_store<P>(nxt, W, out + __popc(b & lt_mask), s, run, store_tag, key);

@@ -484,6 +484,9 @@ int prepare_run(cls_handle *h, uint64_t n, uint64_t seed, RunPlan *plan) {
             plan_pieces(ag, n, batch_len_for(n, h->nbatch), groups[g].cost / groups[g].ncases, groups[g].geom, h->sm_count,
                         h->opt.precision == CLS_PREC_FP32, kMaxPieces);
             pieces += (uint64_t)ag.pieces_per_run * ag.nruns;
+        } else {
+            ag.hand_over = hand_over_for(estimated_events(groups[g].cost / groups[g].ncases),
+                                         h->opt.precision == CLS_PREC_FP32, groups[g].geom);
         }
         const double cost = groups[g].cost * (double)n;
         for (int i = 0; i < nc; ++i) {
@@ -534,9 +537,9 @@ struct Shape {
     int grid, block;
     size_t smem;
     uint32_t bank_slots;  // event schedule: slots per block and buffer
-    size_t bank_off;      // this launch's slice of the bank: the event schedule's particles, the
-                          // history schedule's hand-over buffer
-    uint32_t straggler_cap;  // history schedule: slots of that buffer
+    size_t bank_off;      // event schedule: its particles' slice of the bank
+    size_t straggler_off;    // the hand-over buffer's slice
+    uint32_t straggler_cap;  // and its slots
 };
 
 size_t shape_bank_bytes(const cls_handle *h, const Shape &sh) {
@@ -576,14 +579,15 @@ int tracker_shape(cls_handle *h, int region_bytes, int sched, int geom, Shape *o
     out->smem = smem;
     out->bank_slots = event ? (uint32_t)(h->opt.bank > 0 ? ((h->opt.bank + 31) & ~31) : 128) : 0u;
     out->bank_off = 0;
-    out->straggler_cap = event ? 0u : (uint32_t)(out->grid * (block / 32) * kHandOver);
+    out->straggler_off = 0;
+    out->straggler_cap = (uint32_t)(out->grid * (block / 32) * kHandOver);
     return CLS_OK;
 }
 
 // Shapes of a run's launches, which take consecutive slices of one bank (all of
 // a run's launches may run at once): the event launches grid warps x 2 buffers x
-// slots x fields x 16 B each, the history launches, after them, their hand-over
-// buffers.  *bank: the bytes they need together; a hand-over buffer is cut
+// slots x fields x 16 B each, and every launch, after them, its hand-over
+// buffer.  *bank: the bytes they need together; a hand-over buffer is cut
 // where it would end beyond `limit` (the tracker walks what it cannot hand over).
 int plan_shapes(cls_handle *h, const RunPlan &plan, Shape *sh, size_t *bank, size_t limit = ~(size_t)0) {
     *bank = 0;
@@ -596,8 +600,7 @@ int plan_shapes(cls_handle *h, const RunPlan &plan, Shape *sh, size_t *bank, siz
         }
     }
     for (int g = 0; g < plan.ngroups; ++g) {
-        if (plan.sched[g] == CLS_SCHED_EVENT) continue;
-        sh[g].bank_off = *bank;
+        sh[g].straggler_off = *bank;
         const size_t room = *bank < (limit & ~(size_t)255) ? ((limit & ~(size_t)255) - *bank) / kStragglerBytes : 0;
         sh[g].straggler_cap = (uint32_t)std::min<size_t>(sh[g].straggler_cap, room);
         *bank += ((size_t)sh[g].straggler_cap * kStragglerBytes + 255) & ~(size_t)255;
@@ -685,6 +688,8 @@ int carve_workspace(cls_handle *h, size_t bank) {
 int launch_tracker(cls_handle *h, LaunchArgs a, int sched, int geom, const Shape &sh, uint64_t n, cudaStream_t s) {
     cudaError_t e;
     const bool fp64 = h->opt.precision == CLS_PREC_FP64;
+    a.stragglers = static_cast<unsigned char *>(h->d_bank) + sh.straggler_off;
+    a.straggler_cap = sh.straggler_cap;
     if (sched == CLS_SCHED_EVENT) {
         a.bank = static_cast<unsigned char *>(h->d_bank) + sh.bank_off;
         a.bank_slots = sh.bank_slots;
@@ -692,18 +697,15 @@ int launch_tracker(cls_handle *h, LaunchArgs a, int sched, int geom, const Shape
         e = fp64 ? launch_event_fp64(a, sh.grid, sh.block, sh.smem, s, geom)
                  : launch_event_fp32(a, sh.grid, sh.block, sh.smem, s, geom);
     } else {
-        a.stragglers = static_cast<unsigned char *>(h->d_bank) + sh.bank_off;
-        a.straggler_cap = sh.straggler_cap;
         e = cudaSuccess;
         if (!a.narrow)
             e = fp64 ? launch_history_fp64(a, sh.grid, sh.block, sh.smem, s, geom)
                      : launch_history_fp32(a, sh.grid, sh.block, sh.smem, s, geom);
-        if (e != cudaSuccess) return CLS_E_CUDA;
-        if (!a.narrow && a.hand_over == 0) return CLS_OK;
-        const int grid = narrow_grid(a, n, h->sm_count);
-        const size_t smem = narrow_smem(a, fp64);
-        e = fp64 ? launch_narrow_fp64(a, grid, smem, s, geom) : launch_narrow_fp32(a, grid, smem, s, geom);
     }
+    if (e != cudaSuccess || (!a.narrow && a.hand_over == 0)) return cuda_fail(e);
+    const int grid = narrow_grid(a, n, h->sm_count);
+    const size_t smem = narrow_smem(a, fp64);
+    e = fp64 ? launch_narrow_fp64(a, grid, smem, s, geom) : launch_narrow_fp32(a, grid, smem, s, geom);
     return cuda_fail(e);
 }
 

@@ -115,12 +115,12 @@ struct LaunchArgs {
     unsigned long long *claimed;
     uint64_t piece_len;
     uint32_t pieces_per_run, team;
-    // histories handed from the history tracker to the narrow walk: slots of
+    // histories handed from the trackers to the narrow walk: slots of
     // kStragglerBytes, the number handed over and taken (zeroed before each run)
     unsigned char *stragglers;
     unsigned long long *handed, *taken;
     uint32_t straggler_cap;
-    int hand_over;        // history tracker: a warp with at most this many histories left, and none to claim, hands them over
+    int hand_over;        // a tracker's warp with at most this many histories left, and none to claim, hands them over
     int narrow;           // the narrow walk takes the whole run, from the pieces
     Tallies t;
     uint64_t seed;
@@ -171,7 +171,7 @@ constexpr int kWarpFeedBytes = 112;  // of WarpFeed (cls_device.cuh)
 // shared memory per warp is the draw buffer and feeding state, then one region.
 constexpr int kNarrowBlock = 128, kNarrowBlocks = 3;
 constexpr int kHandOver = 4;
-constexpr int kStragglerBytes = 128;
+constexpr int kStragglerBytes = 144;
 __host__ __device__ constexpr int narrow_memory_bytes(bool fp64) { return (fp64 ? 4096 : 1536) + kWarpFeedBytes; }
 
 // Dynamic shared memory of a warp of the history tracker: two tally regions and

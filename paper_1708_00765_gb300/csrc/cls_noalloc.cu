@@ -40,7 +40,7 @@ struct NoallocScratch {
 };
 
 // The static scratch: every device that loads the library holds one copy of
-// it (about 560 KB) until the process exits.
+// it (about 620 KB) until the process exits.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoallocScratch)];
 
 // One call's case parameters and work list, handed to the set-up kernel by
