@@ -14,7 +14,7 @@
 //    one rounding to the nearest double: within one ulp;
 //  * sine and cosine by angle addition from the nearest of 256 tabulated
 //    angles (|delta| <= pi/256) with the Taylor series of sin(delta) and
-//    cos(delta) - 1, in Q62-Q69 fixed point: absolute error below 2^-60 before
+//    cos(delta) - 1, in Q62-Q69 fixed point: absolute error below 2^-59 before
 //    the final rounding to double.
 //
 // Host and device compile the same code (the host build serves tests).
@@ -104,6 +104,47 @@ CLS_HD double u128_to_double(U128 m, int scale) {
     return bits_to_double((ex << 52) + mant);
 }
 
+CLS_HD uint32_t umulhi32(uint32_t a, uint32_t b) {
+#ifdef __CUDA_ARCH__
+    return __umulhi(a, b);
+#else
+    return (uint32_t)(((uint64_t)a * b) >> 32);
+#endif
+}
+
+// The products below are written out in 32-bit halves, for the operands' known
+// sizes: a general 64 x 64 product takes four wide multiplies (4 cycles of a
+// warp's multiplier each) and a dozen more instructions for its carries and
+// signs.
+
+// a^2 2^-63 for a < 2^55, to the nearest unit
+CLS_HD uint64_t square_q63(uint64_t a) {
+    const uint32_t h = (uint32_t)(a >> 32), l = (uint32_t)a;
+    return (((uint64_t)h * h) << 1) + ((((uint64_t)h * l << 1) + umulhi32(l, l) + (1u << 30)) >> 31);
+}
+
+// a/3 for |a| < 2^55, within 2 units: 1/3 = (2^32/3)(1 + 2^-32) 2^-32
+CLS_HD int64_t third(int64_t a) {
+    const int64_t t = (int64_t)(int32_t)(a >> 32) * 0x55555555 + (int64_t)umulhi32((uint32_t)a, 0x55555555u);
+    return t + (t >> 32);
+}
+
+// a b 2^-63 for a < 2^46, b < 2^63, to the nearest unit
+CLS_HD uint64_t mul46_q63(uint64_t a, uint64_t b) {
+    const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
+    return (((uint64_t)ah * bh) << 1) + (((uint64_t)ah * bl + (uint64_t)al * bh + umulhi32(al, bl) + (1u << 30)) >> 31);
+}
+
+// E ln2 2^120
+CLS_HD void ln2_times(uint32_t E, uint64_t *lo, uint64_t *hi) {
+    const uint64_t p0 = (uint64_t)E * (uint32_t)CLS_LN2_Q120_LO;
+    const uint64_t p1 = (uint64_t)E * (uint32_t)(CLS_LN2_Q120_LO >> 32) + (p0 >> 32);
+    const uint64_t p2 = (uint64_t)E * (uint32_t)CLS_LN2_Q120_HI + (p1 >> 32);
+    const uint32_t p3 = E * (uint32_t)(CLS_LN2_Q120_HI >> 32) + (uint32_t)(p2 >> 32);
+    *lo = (p1 << 32) | (uint32_t)p0;
+    *hi = ((uint64_t)p3 << 32) | (uint32_t)p2;
+}
+
 // Tables in the memory the caller reads them from (shared memory on the GPU).
 struct IntLogTables {
     const uint16_t *n;      // N_i
@@ -143,18 +184,19 @@ CLS_HD double exp_variate(uint64_t k, IntLogTables tab) {
     // (|r| < 2^-8.6): q0 in Q63; q1 (times r^2 < 2^-17) and q2 (times
     // r^4 < 2^-34) in Q31, their products with r^2 2^47 and r^4 2^62 in 32 bits.
     const int32_t r31 = (int32_t)(R >> 32);
-    const int64_t r2 = mulq63(R, R);                                                   // r^2 2^63
-    const int64_t q0 = -(1ll << 62) + mulq63(R, 0x2AAAAAAAAAAAAAABll);                 // -1/2 + r/3
+    const uint64_t Ra = (uint64_t)(R < 0 ? -R : R);                                    // |r| 2^63 < 2^54.4
+    const uint64_t r2 = square_q63(Ra);                                                // r^2 2^63 < 2^46
+    const int64_t q0 = -(1ll << 62) + third(R);                                        // -1/2 + r/3
     const int32_t q1 = -0x20000000 + (int32_t)(((int64_t)r31 * 0x1999999A) >> 31);    // -1/4 + r/5
     const int32_t q2 = -0x15555555 + (int32_t)(((int64_t)r31 * 0x12492492) >> 31);    // -1/6 + r/7
     const int32_t r2s = (int32_t)(r2 >> 16);                                           // r^2 2^47
     const int32_t r4s = (int32_t)(((int64_t)r2s * r2s) >> 32);                         // r^4 2^62
-    const int64_t P = q0 + (((int64_t)q1 * r2s) >> 15) + (((int64_t)q2 * r4s) >> 30);  // Q63
-    const int64_t rq = R + mulq63(r2, P);                                              // ln(1 + r) 2^63
+    const int64_t P = q0 + (((int64_t)q1 * r2s) >> 15) + (((int64_t)q2 * r4s) >> 30);  // Q63, in (-0.51, -0.49)
+    const int64_t rq = R - (int64_t)mul46_q63(r2, (uint64_t)-P);                       // ln(1 + r) 2^63
     // ln(1 - u) 2^120 = T_i - E ln2 + rq 2^57, two's complement (negative)
     const uint64_t t_lo = tab.t[i][0], t_hi = tab.t[i][1];
-    const uint64_t e_lo = CLS_LN2_Q120_LO * (uint64_t)E;
-    const uint64_t e_hi = CLS_LN2_Q120_HI * (uint64_t)E + umulhi64(CLS_LN2_Q120_LO, (uint64_t)E);
+    uint64_t e_lo, e_hi;
+    ln2_times((uint32_t)E, &e_lo, &e_hi);
     uint64_t s_lo = t_lo - e_lo;
     uint64_t s_hi = t_hi - e_hi - (t_lo < e_lo ? 1ull : 0ull);
     const uint64_t a_lo = (uint64_t)rq << 57;
@@ -162,23 +204,23 @@ CLS_HD double exp_variate(uint64_t k, IntLogTables tab) {
     const uint64_t x_lo = s_lo + a_lo;
     s_hi += a_hi + (x_lo < s_lo ? 1ull : 0ull);
     s_lo = x_lo;
-    // magnitude -s
-    const U128 m = {0ull - s_lo, ~s_hi + (s_lo == 0ull ? 1ull : 0ull)};
-    return u128_to_double(m, 120);
+    // magnitude -s, in [2^-9, 2^5.3]: the leading one within the high word's top
+    // 17 bits; rounded to nearest, half up (the bits below 2^-120 are unknown)
+    const uint64_t m_lo = 0ull - s_lo, m_hi = ~s_hi + (s_lo == 0ull ? 1ull : 0ull);
+    const int z = clz64(m_hi);                                   // 2 .. 17
+    const uint64_t x = (m_hi << z) | (m_lo >> (64 - z));
+    const uint64_t mant = ((x >> 10) + 1ull) >> 1;
+    return bits_to_double(((uint64_t)(127 - z - 120 + 1023 - 1) << 52) + mant);
 }
 
-// v 2^e rounded to the nearest double (ties to even), for a signed v and a
-// normal result
+// v 2^e rounded to the nearest double (ties away), for a signed v and a normal
+// result
 CLS_HD double fixed_to_double(int64_t v, int e) {
     if (v == 0) return 0.0;
     const uint64_t sgn = v < 0 ? (1ull << 63) : 0ull;
     const uint64_t a = v < 0 ? 0ull - (uint64_t)v : (uint64_t)v;
     const int lz = clz64(a);
-    const uint64_t x = a << lz;  // leading one at bit 63
-    uint64_t mant = x >> 11;
-    const uint64_t round = (x >> 10) & 1ull;
-    const uint64_t sticky = x & 0x3FFull;
-    mant += round & ((sticky != 0ull ? 1ull : 0ull) | (mant & 1ull));
+    const uint64_t mant = (((a << lz) >> 10) + 1ull) >> 1;  // leading one at bit 52
     const uint64_t ex = (uint64_t)(63 - lz + e + 1023 - 1);
     return bits_to_double(sgn | ((ex << 52) + mant));
 }
@@ -192,27 +234,28 @@ CLS_HD void sincos_2pi_q62(uint64_t k, const int64_t (*sc)[2], int64_t *sn, int6
     const uint64_t j = (k + (1ull << 44)) >> 45;           // nearest tabulated angle, 0..256
     const int64_t t = (int64_t)k - (int64_t)(j << 45);     // in [-2^44, 2^44)
     const int64_t S = sc[j & 255ull][0], C = sc[j & 255ull][1];
-    // delta = 2 pi t 2^-53 in Q69 (|delta| < 2^-6.3)
-    const int64_t dh = smulhi64(t, CLS_TWO_PI_Q60);
-    const uint64_t dl = (uint64_t)t * (uint64_t)CLS_TWO_PI_Q60;
-    const int64_t d = (int64_t)(((uint64_t)dh << 20) | (dl >> 44));
-    const int64_t d2 = smulhi64(d, d) >> 11;                               // delta^2, Q63
+    // |delta| = 2 pi |t| 2^-53 in Q68 (below 2^-6.3); sin(delta) takes t's sign
+    const uint64_t d = umulhi64((uint64_t)(t < 0 ? -t : t) << 19, (uint64_t)CLS_TWO_PI_Q60);
+    const uint64_t d2 = umulhi64(d, d) >> 9;                               // delta^2, Q63, below 2^50.4
     // sin(delta) = delta - delta d2 (1/6 - d2 (1/120 - d2/5040))
     // cos(delta) - 1 = -d2 (1/2 - d2 (1/24 - d2/720))
     // The inner terms need only 32-bit operands: b = 1/120 - d2/5040 (used
     // times delta d2^2 < 2^-31) in Q31, and the products d2 b and d2/720
     // (used times delta d2 < 2^-18, and d2^2 < 2^-25) from d2 2^43 and
-    // 32-bit coefficients, each within 2^-43.
+    // 32-bit coefficients, each within 2^-43; d2 (1/24 - d2/720) (used times
+    // d2 < 2^-12.6) from d2 2^43 and 32 bits, within 2^-47.
     const int32_t d2h = (int32_t)(d2 >> 20);                                            // d2 2^43
     const int32_t b31 = 0x01111111 - (int32_t)(((int64_t)d2h * 0x00068068) >> 43);       // 1/120 - d2/5040, Q31
-    const int64_t a = 0x1555555555555555ll - (((int64_t)d2h * b31) >> 11);              // 1/6 - d2 b
-    const int64_t sd = d - mulq63(mulq63(d, d2), a);                                    // Q69
-    const int64_t e = 0x0555555555555555ll - (((int64_t)d2h * 0x002D82D8) >> 11);       // 1/24 - d2/720
-    const int64_t h = (1ll << 62) - mulq63(d2, e);                                      // 1/2 - d2 e
-    const int64_t cm1 = -mulq63(d2, h);                                        // Q63
-    // sin(a + delta) = S + S cm1 + C sin(delta); cos(a + delta) = C + C cm1 - S sin(delta)  (Q62)
-    const int64_t s_cm1 = mulq63(S, cm1), c_cm1 = mulq63(C, cm1);
-    const int64_t c_sd = smulhi64(C, sd) >> 5, s_sd = smulhi64(S, sd) >> 5;   // (Q62 Q69) >> 69
+    const uint64_t a = 0x1555555555555555ull - (uint64_t)(((int64_t)d2h * b31) >> 11);  // 1/6 - d2 b, Q63
+    const uint64_t d3 = umulhi64(umulhi64(d, d2) << 15, a);                             // (Q67 << 15) Q63 -> Q81
+    const uint64_t sd = d - (d3 >> 13);                                                 // |sin(delta)|, Q68
+    const uint32_t e = 0xAAAAAAABu - (uint32_t)(((int64_t)d2h * 0x05B05B06) >> 43);     // 1/24 - d2/720, Q36
+    const uint64_t h = (1ull << 62) - (((uint64_t)(uint32_t)d2h * e) >> 16);            // 1/2 - d2 e, Q63
+    const uint64_t cm = umulhi64(d2 << 1, h);                                           // 1 - cos(delta), Q63
+    // sin(a + delta) = S - S cm + C sin(delta); cos(a + delta) = C - C cm - S sin(delta)  (Q62)
+    const int64_t Sn = t < 0 ? -S : S, Cn = t < 0 ? -C : C;
+    const int64_t s_cm1 = -(smulhi64(S, (int64_t)(cm << 1))), c_cm1 = -(smulhi64(C, (int64_t)(cm << 1)));
+    const int64_t c_sd = smulhi64(Cn, (int64_t)sd) >> 4, s_sd = smulhi64(Sn, (int64_t)sd) >> 4;   // (Q62 Q68) >> 68
     *sn = S + s_cm1 + c_sd;
     *cs = C + c_cm1 - s_sd;
 }
@@ -266,18 +309,15 @@ CLS_HD double recip_int(double a) {
     const uint32_t m31 = (uint32_t)(M >> 21);                         // m 2^31, truncated
     const int64_t e0 = (int64_t)((1ull << 62) - (uint64_t)m31 * y31);  // (1 - m y0) 2^62, |.| < 2^41
     int64_t y = (int64_t)((uint64_t)y31 << 31) + (int64_t)y31 * (e0 >> 31);  // y1 2^62
-    // second step in Q62
+    // second step in Q61: 1 - m y < 2^-29, so its product with y needs 32 bits of each
     {
-        const uint64_t hi = umulhi64(M, (uint64_t)y), lo = M * (uint64_t)y;
-        const int64_t t = (int64_t)((hi << 12) | (lo >> 52));         // m y 2^62
-        y += mulq62(y, (1ll << 62) - t);
+        const int64_t t = (1ll << 61) - (int64_t)umulhi64(M << 11, (uint64_t)y);  // (1 - m y) 2^61, |.| < 2^32
+        y += ((int64_t)(int32_t)(t >> 1) * (int32_t)(y >> 32)) >> 28;
     }
     // 1/|a| = y 2^-62 2^(1023 - ex), rounded to 53 bits
     const uint64_t x = (uint64_t)y;
     const int lz = clz64(x);
-    const uint64_t n = x << lz;
-    uint64_t mant = n >> 11;
-    mant += ((n >> 10) & 1ull) & (((n & 0x3FFull) != 0ull ? 1ull : 0ull) | (mant & 1ull));
+    const uint64_t mant = (((x << lz) >> 10) + 1ull) >> 1;
     const uint64_t e = (uint64_t)(63 - lz - 62 + (1023 - ex) + 1023 - 1);
     return bits_to_double((b & (1ull << 63)) | ((e << 52) + mant));
 }
@@ -318,15 +358,13 @@ CLS_HD uint64_t sqrt_q61(U128 X, int scale, int *e) {
     const uint32_t vy30 = (uint32_t)(((uint64_t)v32 * y30) >> 32);     // v y0 2^30
     const int64_t e0 = (int64_t)((1ull << 60) - (uint64_t)vy30 * y30);  // (1 - v y0^2) 2^60
     int64_t y = (int64_t)((uint64_t)y30 << 31) + (int64_t)y30 * (e0 >> 30);  // y1 2^61
-    // second step in Q61
-    {
-        const uint64_t vy = umulhi64(v, (uint64_t)y);                 // v y, Q61
-        const int64_t t = (int64_t)(umulhi64(vy, (uint64_t)y) << 4);  // v y^2, Q62
-        y += mulq62(y, ((1ll << 62) - t) >> 1);                      // + y (1 - v y^2)/2
-    }
     // sqrt(X 2^-scale) = sqrt(v) 2^((128 - sh - scale)/2)
     *e = (128 - sh - scale) / 2;
-    return umulhi64(v, (uint64_t)y);  // sqrt(v) = v y, Q61, in [2^60, 2^61]
+    // second step in Q61, taken on v y = sqrt(v): v y + v y (1 - v y^2)/2, whose
+    // last factor is below 2^-28, so the product needs 32 bits of each
+    const uint64_t vy = umulhi64(v, (uint64_t)y);                               // Q61
+    const int64_t t = (1ll << 58) - (int64_t)umulhi64(vy, (uint64_t)y);         // (1 - v y^2) 2^58, |.| < 2^30
+    return (uint64_t)((int64_t)vy + (((int64_t)(int32_t)t * (int32_t)(vy >> 31)) >> 28));  // in [2^60, 2^61]
 }
 
 // sqrt(X 2^-scale) rounded to the nearest double: within an ulp.
@@ -335,9 +373,7 @@ CLS_HD double sqrt_int(U128 X, int scale) {
     const uint64_t q = sqrt_q61(X, scale, &e2);
     if (q == 0ull) return 0.0;
     const int qz = clz64(q);
-    const uint64_t n = q << qz;
-    uint64_t mant = n >> 11;
-    mant += ((n >> 10) & 1ull) & (((n & 0x3FFull) != 0ull ? 1ull : 0ull) | (mant & 1ull));
+    const uint64_t mant = (((q << qz) >> 10) + 1ull) >> 1;
     const uint64_t e = (uint64_t)(63 - qz - 61 + e2 + 1023 - 1);
     return bits_to_double((e << 52) + mant);
 }
