@@ -385,6 +385,17 @@ struct Real<float> {
 };
 
 // ----------------------------------------------------------- history state
+// The mesh coordinate of a history's position: its bin, and the fraction of the
+// bin width with 64 bits (all ones at x = L).  Carried by the FP64 walk, where
+// the end of a flight is the start of the next; the FP32 walk forms both anew.
+template <typename P>
+struct MeshPoint {};
+template <>
+struct MeshPoint<double> {
+    uint32_t k;
+    unsigned long long F;
+};
+
 template <typename P>
 struct History {
     P r[3];
@@ -397,6 +408,7 @@ struct History {
     uint32_t events, n_coll, n_int, n_refl;
     uint32_t pend;    // direction still to draw (DIR_*), 3D and extruded geometries
     P track0, track1; // per-history track length in material 0 / 1
+    MeshPoint<P> at;  // where r[0] lies on the mesh (not in the narrow walk)
 };
 
 // A new direction of the 3D or extruded walk is drawn by resolve_direction,
@@ -569,6 +581,11 @@ __device__ __forceinline__ void resolve_direction(History<P> &s, const CaseParam
     s.pend = DIR_NONE;
 }
 
+template <typename Case>
+__device__ __forceinline__ void set_mesh_point(History<double> &s, const Case &cp);
+template <typename Case>
+__device__ __forceinline__ void set_mesh_point(History<float> &s, const Case &cp);
+
 // Source: position and direction first, then the material label.  With
 // DEFER, a 3D or extruded source leaves its direction and label pending for
 // the caller's resolve_direction.
@@ -584,9 +601,13 @@ __device__ __forceinline__ void source(History<P> &s, const CaseParams &cp, cons
     s.r[0] = P(0);
     s.r[1] = P(0);
     s.r[2] = P(0);
+    if constexpr (sizeof(P) == 8) s.at = MeshPoint<P>{0u, 0ull};
     const P L = R::L(cp);
     if (gd == 3 || gd == 2) {
-        if (cp.source == 1) s.r[0] = L * draw(s, key);  // suite II: uniform position, isotropic direction
+        if (cp.source == 1) {  // suite II: uniform position, isotropic direction
+            s.r[0] = L * draw(s, key);
+            set_mesh_point(s, cp);
+        }
         if (gd == 3) {  // y, then z
             uint32_t yh, yl, zh, zl;
             draw_pair(s, key, yh, yl, zh, zl);
@@ -601,6 +622,7 @@ __device__ __forceinline__ void source(History<P> &s, const CaseParams &cp, cons
     }
     if (cp.source == 1) {
         s.r[0] = L * draw(s, key);
+        set_mesh_point(s, cp);
         if (gd == 11 || gd == 13) {
             set_direction_x(s, draw_iso(s, key));
         } else {
@@ -710,14 +732,24 @@ __device__ __forceinline__ void plan_flight(Flight<float> &f, const Case &cp, fl
 constexpr int kFixed64Bits = 48;
 constexpr int kFixed64MaxExp = 9;
 
-// A bin coordinate u = x / dx >= 0 (below 2^12): its integer part, and its
-// fraction with 64 bits.
-__device__ __forceinline__ unsigned long long split_coordinate(double u, int *k) {
+// The mesh coordinate of x, clipped to [0, L], from u = x / dx (below 2^12).
+template <typename Case>
+__device__ __forceinline__ MeshPoint<double> mesh_point(const Case &cp, double x) {
+    using R = Real<double>;
+    const double L = R::L(cp), c = R::nonneg(x);
+    const double u = (R::lt(L, c) ? L : c) * R::inv_dx(cp);
     const unsigned long long b = (unsigned long long)__double_as_longlong(u);
     const int e = (int)(b >> 52) - 1023;
     const unsigned long long M = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    *k = e >= 0 ? (int)(M >> (52 - e)) : 0;
-    return e >= -12 ? M << (12 + e) : M >> min(-12 - e, 63);
+    MeshPoint<double> p;
+    p.k = e >= 0 ? (uint32_t)(M >> (52 - e)) : 0u;
+    p.F = e >= -12 ? M << (12 + e) : M >> min(-12 - e, 63);
+    const uint32_t last = (uint32_t)cp.nbins - 1u;
+    if (p.k > last) {  // x = L: the whole of the last bin
+        p.k = last;
+        p.F = ~0ull;
+    }
+    return p;
 }
 
 // round(v 2^kFixed64Bits) for 0 <= v < 2^kFixed64MaxExp, half up
@@ -728,9 +760,12 @@ __device__ __forceinline__ unsigned long long fixed64(double v) {
     return sh <= 0 ? M << -sh : ((M >> min(sh - 1, 63)) + 1ull) >> 1;
 }
 
-// round(F c 2^-64), half up
+// round(F c 2^-64) within a unit, for c < 2^58: three of the four half products
 __device__ __forceinline__ unsigned long long mul_fraction(unsigned long long F, unsigned long long c) {
-    return __umul64hi(F, c) + ((F * c) >> 63);
+    const uint32_t fh = (uint32_t)(F >> 32), fl = (uint32_t)F, ch = (uint32_t)(c >> 32), cl = (uint32_t)c;
+    const unsigned long long t = (unsigned long long)fh * cl;
+    const unsigned long long mid = (unsigned long long)fl * ch + (uint32_t)t + 0xC0000000ull;  // below 2^59; 3/4: the product left out is 1/4 on average
+    return (unsigned long long)fh * ch + (t >> 32) + (mid >> 32);
 }
 
 // The flight in FP64, for the global bins: bit patterns of a0, a1 and c.
@@ -747,41 +782,26 @@ __device__ __forceinline__ void plan_flight_real(Flight<double> &f, double ulo, 
 }
 
 template <typename Case>
-__device__ __forceinline__ void plan_flight(Flight<double> &f, const Case &cp, double x0, double x1, double l, double wx,
-                                            double iwx, bool global) {
+__device__ __forceinline__ void plan_flight(Flight<double> &f, const Case &cp, const MeshPoint<double> &from,
+                                            const MeshPoint<double> &to, double x0, double x1, double l, double iwx,
+                                            bool global) {
     using R = Real<double>;
     f.k0 = 0;
     f.k1 = -1;
     f.real = global;
     if (!R::pos(l)) return;
-    const int nb = cp.nbins;
-    const double inv_dx = R::inv_dx(cp);
-    // the x-extent clipped to [0, L]; every value below is >= 0, so min and
-    // max are the integer comparisons of R::lt
-    const double a = R::nonneg(x0), b = R::nonneg(x1);
-    const double L = R::L(cp);
-    const double lo = R::lt(a, b) ? a : b;
-    double hi = R::lt(a, b) ? b : a;
-    hi = R::lt(L, hi) ? L : hi;
-    // bin coordinates x / dx: bin index = integer part; the end bins receive
-    // (1 - frac) dx / |wx| and frac dx / |wx|
-    const double ulo = lo * inv_dx, uhi = hi * inv_dx;
-    int k0, k1;
-    const unsigned long long F0 = split_coordinate(ulo, &k0);
-    unsigned long long F1 = split_coordinate(uhi, &k1);
-    if (k1 >= nb) {  // x = L: the whole of the last bin
-        k1 = nb - 1;
-        F1 = ~0ull;
-    }
-    k0 = min(k0, nb - 1);
-    if (R::is_zero(wx)) k1 = k0 = (R::lt(a, b) ? k0 : k1);  // the bin that contains x0
+    const bool up = R::lt(R::nonneg(x0), R::nonneg(x1));
+    const int k0 = (int)(up ? from.k : to.k), k1 = (int)(up ? to.k : from.k);
+    const unsigned long long F0 = up ? from.F : to.F, F1 = up ? to.F : from.F;
     f.k0 = k0;
     f.k1 = k1;
     // in bin widths: a flight inside one bin scores its length itself, else
     // 1/|wx| in a whole bin
-    const double v = k0 == k1 ? l * inv_dx : R::abs(iwx);
+    const double v = k0 == k1 ? l * R::inv_dx(cp) : R::abs(iwx);
     if (global || (int)((unsigned long long)__double_as_longlong(v) >> 52) >= 1023 + kFixed64MaxExp) {
-        plan_flight_real(f, ulo, uhi, l, R::dx(cp) * R::abs(iwx));
+        const double a = up ? x0 : x1, b = up ? x1 : x0, L = R::L(cp);
+        plan_flight_real(f, R::nonneg(a) * R::inv_dx(cp), (R::lt(L, R::nonneg(b)) ? L : R::nonneg(b)) * R::inv_dx(cp), l,
+                         R::dx(cp) * R::abs(iwx));
         return;
     }
     const unsigned long long q = fixed64(v);
@@ -789,6 +809,21 @@ __device__ __forceinline__ void plan_flight(Flight<double> &f, const Case &cp, d
     f.a1 = mul_fraction(F1, q);
     f.c = q;
 }
+
+// A flight by its ends alone.
+template <typename Case>
+__device__ __forceinline__ void plan_flight(Flight<double> &f, const Case &cp, double x0, double x1, double l, double,
+                                            double iwx, bool global) {
+    plan_flight(f, cp, mesh_point(cp, x0), mesh_point(cp, x1), x0, x1, l, iwx, global);
+}
+
+// Where a history's position lies on the mesh, when it has been set.
+template <typename Case>
+__device__ __forceinline__ void set_mesh_point(History<double> &s, const Case &cp) {
+    s.at = mesh_point(cp, s.r[0]);
+}
+template <typename Case>
+__device__ __forceinline__ void set_mesh_point(History<float> &, const Case &) {}
 
 // Distance along the flight to the face ahead on one axis: (L - r)/omega
 // moving up, (0 - r)/omega moving down, clamped at 0; infinite when omega is
@@ -998,8 +1033,14 @@ struct PhiloxDraws {
         }
     }
     template <typename Case>
-    __device__ __forceinline__ void score(Flight<P> &f, const History<P> &s, const Case &cp, P x1, P l, bool global) {
-        plan_flight(f, cp, s.r[0], x1, l, s.w[0], s.iw[0], global);
+    __device__ __forceinline__ void score(Flight<P> &f, History<P> &s, const Case &cp, P x1, P l, bool global) {
+        if constexpr (sizeof(P) == 8) {
+            const MeshPoint<P> to = mesh_point(cp, x1);
+            plan_flight(f, cp, s.at, to, s.r[0], x1, l, s.iw[0], global);
+            s.at = to;
+        } else {
+            plan_flight(f, cp, s.r[0], x1, l, s.w[0], s.iw[0], global);
+        }
     }
     __device__ __forceinline__ bool below(History<P> &s, unsigned long long thr53, uint32_t thr24) {
         return draw_below(s, key, thr53, thr24);

@@ -290,7 +290,8 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
             bool alive = slot < nlive;
             if (alive) bank_load<P>(buf, W, slot, s, run, packed, key);
             const int ci = alive ? a.runs[run].case_index : 0;
-            s.key.cid = a.cases[ci].case_id;  // Philox counter word 3 (not stored in the bank)
+            s.key.cid = a.cases[ci].case_id;  // Philox counter word 3 and the mesh point are not stored in the bank
+            if (alive) set_mesh_point(s, a.cases[ci]);
             // the particle's region, or 2 if that region has since changed key
             int reg = packed & 3;
             if (reg < 2 && (uint32_t)(packed >> 2) != gen[reg]) reg = 2;
