@@ -513,7 +513,8 @@ def sweep_arms(args, rank, world, pg, local, pool):
     t32 = max_over_ranks(pg, sum(times))
     tal32 = [b32.tallies(k) for k in range(nc)]
     # end to end through the C ABI: each step's run (its work list copied from pinned
-    # host memory) and every case's tallies (device-to-host copy, FP64 normalisation)
+    # host memory) and every case's tallies (reduced over the batches by a small kernel
+    # that reads the batches' history counts from, and writes its result to, pinned memory)
     barrier(pg)
     torch.cuda.synchronize()
     t0 = time.perf_counter()
@@ -534,8 +535,8 @@ def sweep_arms(args, rank, world, pg, local, pool):
                                         / args.steps for g in sorted({int(c[7]) for c in cases})},
         "launch_ms": [1e3 * x for x in times], "ops_per_step": ops32, "events_per_step": events32}
     out["e2e"] = {"value": world * nc * n * E2E_STEPS / e2e_s, "unit": "histories/s", "steps": E2E_STEPS,
-                  "h2d_bytes_per_step": nc * 40 + 24,
-                  "d2h_bytes_per_step": nc * (64 * SWEEP_BINS * 8 + 4 * 8 + 9 * 8)}
+                  "h2d_bytes_per_step": nc * 40 + 24 + nc * 64 * 8,
+                  "d2h_bytes_per_step": nc * (2 * SWEEP_BINS * 8 + 4 * 8 + 9 * 8)}
 
     if not args.no_fp64:
         # ---- FP64 plain: one handle and one launch per case, default launch shape, no graph
@@ -678,8 +679,8 @@ def box_arms(args, rank, world, pg, local):
     clk = merge_clocks(samplers) if samplers else None
     clk_mhz = (clk or {}).get("sm_mhz") or 2070.0
     full = n == workloads.BOX_L10_HISTORIES
-    names = {"fp64": ("history_kernel<double, 3, 0>", "box"), "fp32": ("history_kernel<float, 3, 0>", "box"),
-             "fp64_x": ("history_kernel<double, 13, 0>", "box_x"), "fp32_x": ("history_kernel<float, 13, 0>", "box_x")}
+    names = {"fp64": ("history_kernel<double, 3>", "box"), "fp32": ("history_kernel<float, 3>", "box"),
+             "fp64_x": ("history_kernel<double, 13>", "box_x"), "fp32_x": ("history_kernel<float, 13>", "box_x")}
     for arm, r in results.items():
         k, w = names[arm]
         r["roofline"] = roofline(k, w, r["ops_per_launch"], r["launch_s"], r["events_per_launch"], clk_mhz, full)
@@ -801,16 +802,16 @@ def headline(args, rank, world, pg, local):
 
 def launches_per_replay(tuned, cases) -> int:
     """Kernel launches in one replay of the sweep's graph: one per geometry when the
-    autotuner groups the cases by geometry, else one mixed launch."""
-    return len({int(c[7]) for c in cases}) if tuned.get("group_geometry", 0) else 1
+    autotuner groups the cases by geometry, else one mixed launch; each is followed by
+    the narrow walk of the histories its warps hand over."""
+    return 2 * (len({int(c[7]) for c in cases}) if tuned.get("group_geometry", 0) else 1)
 
 
 def sweep_kernels(tuned) -> str:
-    """The FP32 sweep's kernels: one mixed-geometry launch, or one per geometry (rods,
-    boxes; their cases' short histories take the warp-summed-counters instance)."""
+    """The FP32 sweep's kernels: one mixed-geometry launch, or one per geometry (rods, boxes)."""
     if tuned.get("group_geometry", 0):
-        return "history_kernel<float, 1, 1> + history_kernel<float, 3, 1>"
-    return "history_kernel<float, 0, 1>"
+        return "history_kernel<float, 1> + history_kernel<float, 3>"
+    return "history_kernel<float, 0>"
 
 
 def box_only(args, rank, world, pg, local):
@@ -864,7 +865,7 @@ def diffusive_workload(args, rank, world, pg, local):
     clk_mhz = sampler.summary().get("sm_mhz") or 2070.0
     full = n == workloads.BOX_DIFFUSIVE_HISTORIES
     for sched, r in out.items():
-        r["roofline"] = roofline("history_kernel<float, 3, 0>" if sched == "history" else "event_kernel<float, 3>",
+        r["roofline"] = roofline("history_kernel<float, 3>" if sched == "history" else "event_kernel<float, 3>",
                                  "diffusive", r["ops_per_launch"], r["launch_s"],
                                  r["events_per_launch"], clk_mhz, full)
     if rank == 0:

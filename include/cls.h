@@ -215,9 +215,9 @@ int cls_reset(cls_handle *h);
  * current cases and options -- flux tallies [cases][nbatch][nbins_stride]
  * doubles, statistics, counters, the case table, the work list, the work
  * counters and, when the handle's schedule (or a case's) is the event schedule
- * or still automatic, the event tracker's particle bank, else the buffer in
- * which the history tracker leaves a launch's last histories (optional: with
- * less room it walks them itself), for the current launch
+ * or still automatic, the event tracker's particle bank, and the buffer in
+ * which the trackers leave a launch's last histories (where options set after
+ * the binding leave less room, they walk those themselves), for the current launch
  * shape (for an automatic schedule, the larger of the autotuner's event
  * candidates).  Errors: CLS_E_INVAL, CLS_E_CUDA. */
 int cls_workspace_bytes(cls_handle *h, size_t *bytes);

@@ -44,16 +44,14 @@ inline double cost_estimate(const CaseParams &c) {
     return 1.0 + rate * path;
 }
 
-// How a history-tracker launch of n histories in each of `nruns` run entries is
-// claimed (LaunchArgs): pieces of whole statistics batches, at most max_pieces
-// of them; as many warps start on a piece as it takes to employ all; and the
-// least a warp claims is 32 histories, a warp's lanes, or where that would not
-// go round, a power of two below.  `warps`: about as many as the launch has.
-// Runs of up to narrow_histories histories for each warp of the narrow walk go to
-// it alone (a.narrow).  Measured, us in the tracker / the narrow walk at 14
-// histories a warp (25,000): FP32 box L = 10 525 / 320, rod 91 / 67, diffusive box
-// 2947 / 2546, and at 22 571 / 492, 107 / 97, 4756 / 3763; FP64 rod 135 / 119, slab
-// 171 / 167, but extruded 569 / 902, box 1788 / 1826.
+// Runs of up to this many histories for each warp of the narrow walk go to it
+// alone (LaunchArgs::narrow).  Measured, us in the tracker / the narrow walk.
+// FP64, 8 a warp (14,000): 3D case 3a 848 / 670, box L = 10 1239 / 1224, extruded
+// 448 / 582 (at 4000: 410 / 324), case 1b, of 4 events, 84 / 174 (at 1000: 68 /
+// 50); slab 146 / 108, rod 204 / 168.  FP32, 22 a warp (40,000): 3D case 3a 310 /
+// 264, extruded 218 / 212, rod 168 / 151, case 1b 83 / 101 (at 20,000: 69 / 61).
+// The crossing follows the longest history's length over the mean's, which
+// no estimate here knows, so the line is where most cases cross.
 inline double narrow_histories(bool fp32, int geom) {
     return fp32 ? 24.0 : geom == 1 || geom == 11 || geom == 13 ? 14.0 : 8.0;
 }
@@ -77,7 +75,11 @@ inline int hand_over_for(double events, bool fp32, int geom) {
     return fp32 || geom == 1 || geom == 11 || geom == 13 ? 2 : 0;
 }
 
-
+// How a history-tracker launch of n histories in each of `nruns` run entries is
+// claimed (LaunchArgs): pieces of whole statistics batches, at most max_pieces
+// of them; as many warps start on a piece as it takes to employ all; and the
+// least a warp claims is 32 histories, a warp's lanes, or where that would not
+// go round, a power of two below.
 inline void plan_pieces(LaunchArgs &a, uint64_t n, uint64_t batch_len, double mean_cost, int geom, int sm_count, bool fp32,
                         uint64_t max_pieces) {
     const double total = (double)n * a.nruns;

@@ -1837,7 +1837,12 @@ __device__ __forceinline__ bool refill(unsigned char *regions, int rb, WarpFeed 
 // Persistent kernel.  Each warp claims ranges of consecutive histories (claim);
 // lanes whose histories have ended take the next histories of the warp's claim
 // (ballot + prefix popcount), several lanes at a time, so lanes stay busy across
-// history and claim boundaries.  Each warp owns two shared-memory tally
+// history and claim boundaries.  Bound by issue (FP32) and by instruction supply
+// and the FP64 pipe (FP64).  Before fixed-point bins in 32-bit halves, claims
+// from pieces, batched ends and births, events chosen by FP32 bounds and the
+// shorter integer routines / now: box L = 10 in FP64 1e7 histories 56.6 / 33.2
+// ms, in FP32 1e8 109.3 / 90.8 ms; 256-case sweep in FP32 at 1e6 a case 54.3 /
+// 37.4 ms.  Each warp owns two shared-memory tally
 // regions keyed by (case, batch); a region is flushed to global memory when
 // its key changes, after flush_every histories (FP32) or kDepositBound (FP64),
 // or when the warp retires.
@@ -1852,7 +1857,8 @@ __device__ __forceinline__ bool refill(unsigned char *regions, int rb, WarpFeed 
 // the one-dimensional walks (rod, slab, x-projected box), whose state fits:
 // the FP64 walk is latency-bound, and more resident warps hide its
 // integer-arithmetic and shared-memory latencies (measured: 5% faster for the
-// x-projected box at 6, no gain for the 3D box, which would spill).
+// x-projected box at 6; for the 3D and mixed walks 6 blocks gain 1% on the box
+// at 1e7 histories, 41.1 -> 40.6 ms then, and lose 3-5% on smaller runs).
 template <typename P, int G>
 struct HistoryBounds {
     static constexpr int threads = kHistoryBlockFp64, blocks = (G == 1 || G == 11 || G == 13) ? 6 : 5;
@@ -2015,9 +2021,10 @@ __global__ void __launch_bounds__(HistoryBounds<P, G>::threads, HistoryBounds<P,
 // only distances, the event and the move are left on the chain, which every
 // lane follows; the case's parameters stay in registers, and the flights are
 // scored 32 at a time, one by each lane.  The arithmetic is step's
-// on the same draws, so results do not change.  Measured: 1000 histories
-// of the 3D box 1.07 -> 0.61 ms in FP64 and 345 -> 198 us in FP32, of the
-// diffusive box in FP32 5.1 -> 2.8 ms (0.45 us per event of the longest).
+// on the same draws, so results do not change.  Measured: 1000 histories of
+// the 3D box in FP64 753 us by the tracker, 483 us here; the diffusive box,
+// 1e6 histories in FP32, 20.4 ms without the hand-over, 12.8 ms with it.  An
+// event of a lone history takes 0.23 us in FP32 and 1.5 us in FP64.
 // The two draws of a lane's Philox block into the buffer, at `at` and at + 1.
 template <typename P, int G>
 __device__ __forceinline__ void fill_draws(DrawBuffer<P> &b, int at, uint32_t block, const History<P> &s,

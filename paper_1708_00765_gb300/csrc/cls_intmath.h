@@ -9,9 +9,9 @@
 // point:
 //  * the logarithm by the table-driven reduction of Tang (ACM TOMS 16, 1990)
 //    with an exact 64-bit product for the reduced argument, the Taylor series
-//    of ln(1 + r) by Horner's rule in Q31/Q63 (precision tapered to what each
+//    of ln(1 + r) in Q31/Q63 grouped in pairs (precision tapered to what each
 //    term needs), the sum in 128-bit fixed point with 120 fraction bits, and
-//    one rounding to the nearest double: within one ulp;
+//    one rounding to the nearest double: within 0.6 ulp;
 //  * sine and cosine by angle addition from the nearest of 256 tabulated
 //    angles (|delta| <= pi/256) with the Taylor series of sin(delta) and
 //    cos(delta) - 1, in Q62-Q69 fixed point: absolute error below 2^-59 before
