@@ -1986,7 +1986,7 @@ __global__ void __launch_bounds__(HistoryBounds<P, G>::threads, HistoryBounds<P,
         f.k0 = 0;
         f.k1 = -1;
         if (out == kWalking) {
-            // directions of the lanes born in this round and of those that scattered in the last
+            // directions of the lanes born in this step and of those that scattered in the last
             resolve_direction<P, G>(s, a.cases[lcase], key);
             const int ev = step<P, false, G>(s, a.cases[lcase], draws, a.max_events, f, nullptr, lreg == 2);
             out = ev < 0 ? kWalking : ev;
