@@ -587,8 +587,9 @@ int tracker_shape(cls_handle *h, int region_bytes, int sched, int geom, Shape *o
 // Shapes of a run's launches, which take consecutive slices of one bank (all of
 // a run's launches may run at once): the event launches grid warps x 2 buffers x
 // slots x fields x 16 B each, and every launch, after them, its hand-over
-// buffer.  *bank: the bytes they need together; a hand-over buffer is cut
-// where it would end beyond `limit` (the tracker walks what it cannot hand over).
+// buffer, if it hands histories over at all.  *bank: the bytes they need
+// together; a hand-over buffer is cut where it would end beyond `limit` (the
+// tracker walks what it cannot hand over).
 int plan_shapes(cls_handle *h, const RunPlan &plan, Shape *sh, size_t *bank, size_t limit = ~(size_t)0) {
     *bank = 0;
     for (int g = 0; g < plan.ngroups; ++g) {
@@ -603,6 +604,7 @@ int plan_shapes(cls_handle *h, const RunPlan &plan, Shape *sh, size_t *bank, siz
         sh[g].straggler_off = *bank;
         const size_t room = *bank < (limit & ~(size_t)255) ? ((limit & ~(size_t)255) - *bank) / kStragglerBytes : 0;
         sh[g].straggler_cap = (uint32_t)std::min<size_t>(sh[g].straggler_cap, room);
+        if (plan.a[g].narrow || plan.a[g].hand_over == 0) sh[g].straggler_cap = 0;
         *bank += ((size_t)sh[g].straggler_cap * kStragglerBytes + 255) & ~(size_t)255;
     }
     return CLS_OK;
@@ -622,8 +624,11 @@ int ensure_bank(cls_handle *h, size_t need) {
         return CLS_OK;
     }
     if (need <= h->bank_bytes) return CLS_OK;
-    CLS_CUDA(cudaDeviceSynchronize());
-    cudaFree(h->d_bank);
+    if (h->d_bank) {
+        CLS_CUDA(cudaDeviceSynchronize());
+        destroy_graph(h);  // the captured launches name the old bank
+        cudaFree(h->d_bank);
+    }
     h->d_bank = nullptr;
     h->bank_bytes = 0;
     if (cudaMalloc(&h->d_bank, need) != cudaSuccess) {
@@ -632,6 +637,29 @@ int ensure_bank(cls_handle *h, size_t need) {
     }
     h->bank_bytes = need;
     return CLS_OK;
+}
+
+// Shapes of a run's launches, and the bank they need.  The hand-over buffers
+// are a help, not a need: where memory is short, or the stream is being captured
+// and nothing can be allocated, they are cut to what there is.
+int plan_bank(cls_handle *h, const RunPlan &plan, Shape *sh, cudaStream_t s) {
+    size_t bank = 0;
+    int rc = plan_shapes(h, plan, sh, &bank, bank_limit(h));
+    if (rc) return rc;
+    if (!h->ws && bank > h->bank_bytes) {
+        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess) cudaGetLastError();
+        if (capturing != cudaStreamCaptureStatusNone) {
+            rc = plan_shapes(h, plan, sh, &bank, h->bank_bytes);
+            if (rc) return rc;
+        }
+    }
+    rc = ensure_bank(h, bank);
+    if (rc == CLS_E_NOMEM) {
+        rc = plan_shapes(h, plan, sh, &bank, 0);
+        if (!rc) rc = ensure_bank(h, bank);
+    }
+    return rc;
 }
 
 // Bytes of bank the handle's current options need (plan_shapes; for an
@@ -653,6 +681,8 @@ int bank_need(cls_handle *h, size_t *need) {
             plan.sched[g] = groups[g].sched;
             plan.geom[g] = groups[g].geom;
             plan.a[g].region_bytes = region_bytes_for(h);
+            plan.a[g].narrow = 0;
+            plan.a[g].hand_over = kHandOver;
         }
         Shape sh[kMaxGroups];
         size_t bank = 0;
@@ -1171,9 +1201,7 @@ int cls_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
     int rc = prepare_run(h, n, seed, &plan);
     if (rc) return rc;
     Shape sh[kMaxGroups];
-    size_t bank = 0;
-    rc = plan_shapes(h, plan, sh, &bank, bank_limit(h));
-    if (!rc) rc = ensure_bank(h, bank);
+    rc = plan_bank(h, plan, sh, s);
     if (rc) return rc;
     rc = record_pair(h, s, true);
     if (rc) return rc;
@@ -1214,9 +1242,7 @@ int cls_batch_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
         destroy_graph(h);
     if (!h->graph_exec) {
         Shape sh[kMaxGroups];
-        size_t bank = 0;
-        rc = plan_shapes(h, plan, sh, &bank, bank_limit(h));
-        if (!rc) rc = ensure_bank(h, bank);
+        rc = plan_bank(h, plan, sh, s);
         if (rc) return rc;
         if (!h->capture_stream) CLS_CUDA(cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking));
         while ((int)h->aux_streams.size() < plan.ngroups - 1) {
