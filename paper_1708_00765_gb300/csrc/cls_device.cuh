@@ -2205,7 +2205,10 @@ __global__ void __launch_bounds__(kNarrowBlock, kNarrowBlocks) narrow_kernel(con
             }
             if (++held == 32) score_held();
         }
-        if (lane == 0) end_history<P, G>(region, a, s, ev, 0, lcase, base_j, base_events, lane);
+        // the event tracker's regions sum t^2 in FP64: so its stragglers', in FP32,
+        // go straight to the FP64 statistics
+        if (lane == 0)
+            end_history<P, G>(region, a, s, ev, sizeof(P) == 4 && a.bank != nullptr ? 2 : 0, lcase, base_j, base_events, lane);
         __syncwarp();
         if (sizeof(P) == 4 && ++fed >= a.flush_every) {  // FP32: before a bin's sum can outgrow its 64 bits
             if (held > 0) score_held();

@@ -146,3 +146,17 @@ def test_histories_beyond_the_hand_over_buffer_are_walked_to_their_ends():
     assert [int(v) for v in counters[0].cpu()] == [int(o[k]) for k in keys]
     assert float(stats[0, 0]) == pytest.approx(o["sum_t"], rel=1e-12)
     np.testing.assert_allclose(flux[0].sum(0).cpu().numpy(), o["flux"].sum(0), rtol=1e-12)
+
+
+@pytest.mark.parametrize("n", [1, 3])
+def test_event_stragglers_keep_their_statistics_in_fp64(n):
+    """The event tracker sums t^2 in FP64, in FP32 walks too: of one history it is the square of its track
+    length, and of three no less than a third of the squared sum, to FP64 rounding, wherever they ended."""
+    p = (1.0, 10.0, 0.5, 0.2, 0.999, 0.999, 8.0, 3, 60)
+    for seed in range(8):
+        t = run(p, n, seed, precision="fp32", schedule="event")
+        assert t["sum_t"] == pytest.approx(sum(t["track"]), rel=1e-14)
+        if n == 1:
+            assert t["sum_t2"] == pytest.approx(t["sum_t"] ** 2, rel=1e-14)
+        else:
+            assert t["sum_t"] ** 2 / n * (1 - 1e-14) <= t["sum_t2"] <= t["sum_t"] ** 2 * (1 + 1e-14)
