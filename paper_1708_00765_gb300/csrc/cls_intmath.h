@@ -11,10 +11,10 @@
 //    with an exact 64-bit product for the reduced argument, the Taylor series
 //    of ln(1 + r) in Q31/Q63 grouped in pairs (precision tapered to what each
 //    term needs), the sum in 128-bit fixed point with 120 fraction bits, and
-//    one rounding to the nearest double: within 0.6 ulp;
+//    one rounding to the nearest double: within 0.57 ulp;
 //  * sine and cosine by angle addition from the nearest of 256 tabulated
 //    angles (|delta| <= pi/256) with the Taylor series of sin(delta) and
-//    cos(delta) - 1, in Q62-Q69 fixed point: absolute error below 2^-59 before
+//    cos(delta) - 1, in Q62-Q81 fixed point: absolute error below 2^-60 before
 //    the final rounding to double.
 //
 // Host and device compile the same code (the host build serves tests).
@@ -129,10 +129,10 @@ CLS_HD int64_t third(int64_t a) {
     return t + (t >> 32);
 }
 
-// a b 2^-63 for a < 2^46, b < 2^63, to the nearest unit
-CLS_HD uint64_t mul46_q63(uint64_t a, uint64_t b) {
+// a b 2^-55 for a < 2^46, b < 2^63, to the nearest unit
+CLS_HD uint64_t mul46_q71(uint64_t a, uint64_t b) {
     const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
-    return (((uint64_t)ah * bh) << 1) + (((uint64_t)ah * bl + (uint64_t)al * bh + umulhi32(al, bl) + (1u << 30)) >> 31);
+    return (((uint64_t)ah * bh) << 9) + (((uint64_t)ah * bl + (uint64_t)al * bh + umulhi32(al, bl) + (1u << 22)) >> 23);
 }
 
 // E ln2 2^120
@@ -192,15 +192,15 @@ CLS_HD double exp_variate(uint64_t k, IntLogTables tab) {
     const int32_t r2s = (int32_t)(r2 >> 16);                                           // r^2 2^47
     const int32_t r4s = (int32_t)(((int64_t)r2s * r2s) >> 32);                         // r^4 2^62
     const int64_t P = q0 + (((int64_t)q1 * r2s) >> 15) + (((int64_t)q2 * r4s) >> 30);  // Q63, in (-0.51, -0.49)
-    const int64_t rq = R - (int64_t)mul46_q63(r2, (uint64_t)-P);                       // ln(1 + r) 2^63
-    // ln(1 - u) 2^120 = T_i - E ln2 + rq 2^57, two's complement (negative)
+    const int64_t rq = (R << 8) - (int64_t)mul46_q71(r2, (uint64_t)-P);                // ln(1 + r) 2^71
+    // ln(1 - u) 2^120 = T_i - E ln2 + rq 2^49, two's complement (negative)
     const uint64_t t_lo = tab.t[i][0], t_hi = tab.t[i][1];
     uint64_t e_lo, e_hi;
     ln2_times((uint32_t)E, &e_lo, &e_hi);
     uint64_t s_lo = t_lo - e_lo;
     uint64_t s_hi = t_hi - e_hi - (t_lo < e_lo ? 1ull : 0ull);
-    const uint64_t a_lo = (uint64_t)rq << 57;
-    const uint64_t a_hi = (uint64_t)(rq >> 7);
+    const uint64_t a_lo = (uint64_t)rq << 49;
+    const uint64_t a_hi = (uint64_t)(rq >> 15);
     const uint64_t x_lo = s_lo + a_lo;
     s_hi += a_hi + (x_lo < s_lo ? 1ull : 0ull);
     s_lo = x_lo;
@@ -242,19 +242,21 @@ CLS_HD void sincos_2pi_q62(uint64_t k, const int64_t (*sc)[2], int64_t *sn, int6
     // The inner terms need only 32-bit operands: b = 1/120 - d2/5040 (used
     // times delta d2^2 < 2^-31) in Q31, and the products d2 b and d2/720
     // (used times delta d2 < 2^-18, and d2^2 < 2^-25) from d2 2^43 and
-    // 32-bit coefficients, each within 2^-43; d2 (1/24 - d2/720) (used times
-    // d2 < 2^-12.6) from d2 2^43 and 32 bits, within 2^-47.
+    // 32-bit coefficients, each within 2^-43; 1/24 - d2/720 (used times d2^2 <
+    // 2^-25) to 2^-37, its product with d2 in full.  The two terms of a sum are
+    // floored in opposite directions.
     const int32_t d2h = (int32_t)(d2 >> 20);                                            // d2 2^43
     const int32_t b31 = 0x01111111 - (int32_t)(((int64_t)d2h * 0x00068068) >> 43);       // 1/120 - d2/5040, Q31
     const uint64_t a = 0x1555555555555555ull - (uint64_t)(((int64_t)d2h * b31) >> 11);  // 1/6 - d2 b, Q63
     const uint64_t d3 = umulhi64(umulhi64(d, d2) << 15, a);                             // (Q67 << 15) Q63 -> Q81
     const uint64_t sd = d - (d3 >> 13);                                                 // |sin(delta)|, Q68
-    const uint32_t e = 0xAAAAAAABu - (uint32_t)(((int64_t)d2h * 0x05B05B06) >> 43);     // 1/24 - d2/720, Q36
-    const uint64_t h = (1ull << 62) - (((uint64_t)(uint32_t)d2h * e) >> 16);            // 1/2 - d2 e, Q63
+    const uint32_t e = 0xAAAAAAABu - (uint32_t)(((int64_t)d2h * 0x05B05B06 + 0x6AAAAAAAAAAll) >> 43);  // 1/24 - d2/720, Q36, within half a unit
+    const uint64_t de = (uint64_t)(uint32_t)(d2 >> 19) * e + umulhi32((uint32_t)(d2 << 13), e);    // d2 e, Q80
+    const uint64_t h = (1ull << 62) - (de >> 17);                                       // 1/2 - d2 e, Q63
     const uint64_t cm = umulhi64(d2 << 1, h);                                           // 1 - cos(delta), Q63
     // sin(a + delta) = S - S cm + C sin(delta); cos(a + delta) = C - C cm - S sin(delta)  (Q62)
     const int64_t Sn = t < 0 ? -S : S, Cn = t < 0 ? -C : C;
-    const int64_t s_cm1 = -(smulhi64(S, (int64_t)(cm << 1))), c_cm1 = -(smulhi64(C, (int64_t)(cm << 1)));
+    const int64_t s_cm1 = -smulhi64(S, (int64_t)(cm << 1)), c_cm1 = smulhi64(C, -(int64_t)(cm << 1));
     const int64_t c_sd = smulhi64(Cn, (int64_t)sd) >> 4, s_sd = smulhi64(Sn, (int64_t)sd) >> 4;   // (Q62 Q68) >> 68
     *sn = S + s_cm1 + c_sd;
     *cs = C + c_cm1 - s_sd;
@@ -268,17 +270,12 @@ CLS_HD void sincos_2pi_int(uint64_t k, const int64_t (*sc)[2], double *sn, doubl
     *cs = q62_to_double(c);
 }
 
-// floor(a d / 2^62) for a in (0, 2^62] and signed d
-CLS_HD int64_t mulq62(int64_t a, int64_t d) {
-    return (int64_t)(((uint64_t)smulhi64(a, d) << 2) | (((uint64_t)a * (uint64_t)d) >> 62));
-}
-
 // 1/a for a normal double a: Newton-Raphson iteration for the reciprocal,
 // y <- y + y (1 - m y) (each step squares the relative error; P. Markstein,
 // IBM J. Res. Dev. 34, 1990), on the significand m in [1, 2) from the FP32
 // approximate reciprocal of its leading 24 bits (relative error below 2^-22):
-// one step in 32-bit arithmetic (to about 2^-30), one in Q62 fixed point (to
-// about 2^-59), then one rounding to the nearest double: within an ulp of 1/a.
+// one step in 32-bit arithmetic (to 2^-31), one in Q62 fixed point (to 2^-61),
+// then one rounding to the nearest double: within 0.504 ulp of 1/a.
 // Zero, subnormal, infinite and NaN a take the division.
 CLS_HD double recip_int(double a) {
     uint64_t b;
@@ -304,15 +301,17 @@ CLS_HD double recip_int(double a) {
     memcpy(&rb, &rf, sizeof rb);
     const int re = (int)((rb >> 23) & 0xFF) - 127;                    // -1, or 0 when y0 = 1
     // first step in 32-bit arithmetic (y0 and m to 31 fraction bits): y1
-    // within about 2^-30 of 1/m
+    // within 2^-31 of 1/m, nearly all of it m's truncation
     const uint32_t y31 = ((rb & 0x7FFFFFu) | 0x800000u) << (8 + re);  // y0 2^31, at most 2^31
     const uint32_t m31 = (uint32_t)(M >> 21);                         // m 2^31, truncated
     const int64_t e0 = (int64_t)((1ull << 62) - (uint64_t)m31 * y31);  // (1 - m y0) 2^62, |.| < 2^41
-    int64_t y = (int64_t)((uint64_t)y31 << 31) + (int64_t)y31 * (e0 >> 31);  // y1 2^62
-    // second step in Q61: 1 - m y < 2^-29, so its product with y needs 32 bits of each
+    int64_t y = (int64_t)((uint64_t)y31 << 31) + (((int64_t)y31 * (int32_t)(e0 >> 20)) >> 11);  // y1 2^62
+    // second step in Q62: 1 - m y lies in (-2^-31, 2^-41), so it takes 32 bits; y (1 - m y) =
+    // (1 - m y) - (1 - y) (1 - m y), with 1 - y in 32 bits
     {
-        const int64_t t = (1ll << 61) - (int64_t)umulhi64(M << 11, (uint64_t)y);  // (1 - m y) 2^61, |.| < 2^32
-        y += ((int64_t)(int32_t)(t >> 1) * (int32_t)(y >> 32)) >> 28;
+        const int64_t t = (1ll << 62) - (int64_t)umulhi64(M << 11, (uint64_t)y << 1);
+        const int32_t z = (int32_t)((uint64_t)((1ll << 62) - y + (1ll << 30)) >> 31);  // 1 - y, Q31
+        y += t - (((int64_t)(int32_t)t * z + (1ll << 30)) >> 31);
     }
     // 1/|a| = y 2^-62 2^(1023 - ex), rounded to 53 bits
     const uint64_t x = (uint64_t)y;
@@ -327,7 +326,7 @@ CLS_HD double recip_int(double a) {
 // y <- y + y (1 - v y^2)/2, on v = X 2^-2t in [1/4, 1) from the FP32
 // approximate reciprocal square root of v's leading 24 bits (relative error
 // below 2^-22): one step in 32-bit arithmetic (to about 2^-29), one in Q61
-// fixed point, then sqrt(v) = v y.
+// fixed point, taken on sqrt(v) = v y: within 2^-58.5.
 CLS_HD uint64_t sqrt_q61(U128 X, int scale, int *e) {
     *e = 0;
     if ((X.hi | X.lo) == 0ull) return 0ull;
@@ -363,8 +362,9 @@ CLS_HD uint64_t sqrt_q61(U128 X, int scale, int *e) {
     // second step in Q61, taken on v y = sqrt(v): v y + v y (1 - v y^2)/2, whose
     // last factor is below 2^-28, so the product needs 32 bits of each
     const uint64_t vy = umulhi64(v, (uint64_t)y);                               // Q61
-    const int64_t t = (1ll << 58) - (int64_t)umulhi64(vy, (uint64_t)y);         // (1 - v y^2) 2^58, |.| < 2^30
-    return (uint64_t)((int64_t)vy + (((int64_t)(int32_t)t * (int32_t)(vy >> 31)) >> 28));  // in [2^60, 2^61]
+    // (1 - v y^2) 2^59, |.| < 2^31: the product's floor counted as its middle
+    const int64_t t = (1ll << 59) - 1 - (int64_t)(umulhi64(vy, (uint64_t)y) << 1);
+    return (uint64_t)((int64_t)vy + (((int64_t)(int32_t)t * (int32_t)(vy >> 31)) >> 29));  // in [2^60, 2^61]
 }
 
 // sqrt(X 2^-scale) rounded to the nearest double: within an ulp.
