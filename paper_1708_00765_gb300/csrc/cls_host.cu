@@ -177,8 +177,8 @@ struct cls_handle {
     std::vector<cudaEvent_t> join_events;  // [0]: the fork, [g]: group g's end
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t graph_exec = nullptr;
-    std::vector<uint64_t> graph_total_chunks;
-    int graph_key[10] = {0};
+    std::array<uint64_t, 2> graph_run{};  // the histories per case and the seed it was captured for
+    int graph_key[8] = {0};
 };
 
 namespace {
@@ -1234,11 +1234,11 @@ int cls_batch_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
     // ranges) before replaying the graph.  The groups' launches are parallel
     // branches of the graph: the second starts its blocks as the first one's
     // drain, so their tails overlap.
-    const int key[10] = {h->opt.precision, h->opt.schedule, h->opt.block, h->opt.chunk, (int)h->opt.max_events,
-                         h->opt.blocks_per_sm, (int)(seed & 0x7fffffff), (int)(seed >> 31), h->opt.group_geometry,
-                         h->outcome_codes != nullptr};
-    const std::vector<uint64_t> tc = {n};  // the launches' work distribution is captured with them
-    if (h->graph_exec && (tc != h->graph_total_chunks || std::memcmp(key, h->graph_key, sizeof(key))))
+    const int key[8] = {h->opt.precision, h->opt.schedule, h->opt.block, h->opt.chunk, (int)h->opt.max_events,
+                        h->opt.blocks_per_sm, h->opt.group_geometry, h->outcome_codes != nullptr};
+    // the launches' work distribution and round keys are captured with them
+    const std::array<uint64_t, 2> run = {n, seed};
+    if (h->graph_exec && (run != h->graph_run || std::memcmp(key, h->graph_key, sizeof(key))))
         destroy_graph(h);
     if (!h->graph_exec) {
         Shape sh[kMaxGroups];
@@ -1279,7 +1279,7 @@ int cls_batch_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
             destroy_graph(h);
             return CLS_E_CUDA;
         }
-        h->graph_total_chunks = tc;
+        h->graph_run = run;
         std::memcpy(h->graph_key, key, sizeof(key));
     }
     rc = record_pair(h, s, true);
