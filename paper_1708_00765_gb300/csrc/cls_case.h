@@ -8,6 +8,7 @@
 #include <cstring>
 
 #include "../../include/cls.h"
+#include "cls_fixed.h"
 #include "cls_internal.h"
 
 namespace cls {
@@ -83,7 +84,7 @@ inline int hand_over_for(double events, bool fp32, int geom) {
 inline void plan_pieces(LaunchArgs &a, uint64_t n, uint64_t batch_len, double mean_cost, int geom, int sm_count, bool fp32,
                         uint64_t max_pieces) {
     const double total = (double)n * a.nruns;
-    const double narrow_warps = (double)sm_count * kNarrowBlocks * (kNarrowBlock / 32);
+    const double narrow_warps = (double)sm_count * kNarrowBlocks * narrow_block_warps(!fp32, a.region_bytes);
     a.narrow = total <= narrow_histories(fp32, geom) * narrow_warps;
     const double warps = a.narrow ? std::min(total, narrow_warps) : sm_count * (fp32 ? 28.0 : 20.0);
     const uint64_t used = (n + batch_len - 1) / batch_len;  // batches
@@ -98,13 +99,13 @@ inline void plan_pieces(LaunchArgs &a, uint64_t n, uint64_t batch_len, double me
 }
 
 // Blocks of the narrow walk: as many as the run has histories for its warps.
-inline int narrow_grid(const LaunchArgs &a, uint64_t n, int sm_count) {
-    const int full = sm_count * kNarrowBlocks, warps = kNarrowBlock / 32;
+inline int narrow_grid(const LaunchArgs &a, bool fp64, uint64_t n, int sm_count) {
+    const int full = sm_count * kNarrowBlocks, warps = narrow_block_warps(fp64, a.region_bytes);
     return a.narrow ? (int)std::min((double)full, std::ceil((double)n * a.nruns / warps)) : full;
 }
 
 inline size_t narrow_smem(const LaunchArgs &a, bool fp64) {
-    return (size_t)(kNarrowBlock / 32) * (narrow_memory_bytes(fp64) + a.region_bytes);
+    return (size_t)narrow_block_warps(fp64, a.region_bytes) * (narrow_memory_bytes(fp64) + a.region_bytes);
 }
 
 // Claim limit and refill threshold of a run entry (RunCase), from the
@@ -164,6 +165,8 @@ inline CaseParams make_case(const double *p, uint32_t case_id) {
     auto moderate = [](double v) { return v >= 0x1p-60 && v <= 0x1p60; };
     c.filter = moderate(c.L) && moderate(c.lambda[0]) && moderate(c.lambda[1]) &&
                (p[0] == 0 || moderate(1.0 / p[0])) && (p[1] == 0 || moderate(1.0 / p[1]));
+    c.fix_bits = fixed_bits(c.dx, c.sigma, c.lambda);
+    c.fix_unit = std::ldexp(c.dx, -c.fix_bits);
     c.cost = cost_estimate(c);
     return c;
 }

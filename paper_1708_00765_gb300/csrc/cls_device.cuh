@@ -20,6 +20,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "cls_fixed.h"
 #include "cls_internal.h"
 #include "cls_intmath.h"
 
@@ -160,7 +161,7 @@ struct CaseRegs {
 };
 
 
-// FP64 walk: every quantity in double; shared-memory tally bins in double.
+// FP64 walk: every quantity in double; shared-memory tally bins in fixed point.
 // Comparisons of distances (non-negative after clamping) and sign tests run on
 // the IEEE bit patterns in the integer pipes, which order non-negative doubles
 // like the numbers they encode; the FP64 pipe is left to the arithmetic.
@@ -425,17 +426,21 @@ struct Flight {
     P a0, a1, c;
 };
 
-// FP64 walk: the same in fixed point, units of 2^-kFixed64Bits bin widths,
-// formed in integer arithmetic (plan_flight).  A flight that scores straight
-// into the global bins (`real`) holds the bit patterns of the doubles instead.
+// FP64 walk: the same in fixed point, units of 2^-fix_bits bin widths
+// (cls_fixed.h), formed in integer arithmetic (plan_flight).  A flight that
+// scores straight into the global bins (`real`) holds the bit patterns of the
+// doubles instead, in the low words.
 template <>
 struct Flight<double> {
     int k0, k1;
-    unsigned long long a0, a1, c;
+    Fix96 a0, a1, c;
     bool real;
 };
 
-__device__ __forceinline__ double flight_real(unsigned long long a) { return __longlong_as_double((long long)a); }
+__device__ __forceinline__ double flight_real(const Fix96 &a) { return __hiloint2double((int)a.w1, (int)a.w0); }
+__device__ __forceinline__ Fix96 flight_bits(double v) {
+    return Fix96{(uint32_t)__double2loint(v), (uint32_t)__double2hiint(v), 0u};
+}
 __device__ __forceinline__ double flight_real(float a) { return (double)a; }
 
 // whether the flight scores straight into the global bins (a lane whose region
@@ -724,14 +729,6 @@ __device__ __forceinline__ void plan_flight(Flight<float> &f, const Case &cp, fl
     f.c = c;
 }
 
-// FP64 walk.  Fixed point: 48 fraction bits of a bin width, a rounding of
-// 2^-49 bin widths per deposit, below the 2^-53 relative rounding of a sum of
-// more than 16 bin widths; and 2^15 bin widths of headroom per bin between two
-// flushes (DepositBound).  Lengths of 2^kFixed64MaxExp bin widths and more (a
-// grazing flight, |wx| < 2^-9) go to the global bins in FP64.
-constexpr int kFixed64Bits = 48;
-constexpr int kFixed64MaxExp = 9;
-
 // The mesh coordinate of x, clipped to [0, L], from u = x / dx (below 2^12).
 template <typename Case>
 __device__ __forceinline__ MeshPoint<double> mesh_point(const Case &cp, double x) {
@@ -752,33 +749,17 @@ __device__ __forceinline__ MeshPoint<double> mesh_point(const Case &cp, double x
     return p;
 }
 
-// round(v 2^kFixed64Bits) for 0 <= v < 2^kFixed64MaxExp, half up
-__device__ __forceinline__ unsigned long long fixed64(double v) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    const int sh = 52 - kFixed64Bits - ((int)(b >> 52) - 1023);
-    const unsigned long long M = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    return sh <= 0 ? M << -sh : ((M >> min(sh - 1, 63)) + 1ull) >> 1;
-}
-
-// round(F c 2^-64) within a unit, for c < 2^58: three of the four half products
-__device__ __forceinline__ unsigned long long mul_fraction(unsigned long long F, unsigned long long c) {
-    const uint32_t fh = (uint32_t)(F >> 32), fl = (uint32_t)F, ch = (uint32_t)(c >> 32), cl = (uint32_t)c;
-    const unsigned long long t = (unsigned long long)fh * cl;
-    const unsigned long long mid = (unsigned long long)fl * ch + (uint32_t)t + 0xC0000000ull;  // below 2^59; 3/4: the product left out is 1/4 on average
-    return (unsigned long long)fh * ch + (t >> 32) + (mid >> 32);
-}
-
 // The flight in FP64, for the global bins: bit patterns of a0, a1 and c.
 __device__ __forceinline__ void plan_flight_real(Flight<double> &f, double ulo, double uhi, double l, double c) {
     using R = Real<double>;
     f.real = true;
     if (f.k0 == f.k1) {
-        f.a0 = (unsigned long long)__double_as_longlong(l);
+        f.a0 = flight_bits(l);
         return;
     }
-    f.a0 = (unsigned long long)__double_as_longlong(R::nonneg(fma(-R::frac(ulo, f.k0), c, c)));
-    f.a1 = (unsigned long long)__double_as_longlong(R::frac(uhi, f.k1) * c);
-    f.c = (unsigned long long)__double_as_longlong(c);
+    f.a0 = flight_bits(R::nonneg(fma(-R::frac(ulo, f.k0), c, c)));
+    f.a1 = flight_bits(R::frac(uhi, f.k1) * c);
+    f.c = flight_bits(c);
 }
 
 template <typename Case>
@@ -792,21 +773,22 @@ __device__ __forceinline__ void plan_flight(Flight<double> &f, const Case &cp, c
     if (!R::pos(l)) return;
     const bool up = R::lt(R::nonneg(x0), R::nonneg(x1));
     const int k0 = (int)(up ? from.k : to.k), k1 = (int)(up ? to.k : from.k);
-    const unsigned long long F0 = up ? from.F : to.F, F1 = up ? to.F : from.F;
     f.k0 = k0;
     f.k1 = k1;
     // in bin widths: a flight inside one bin scores its length itself, else
     // 1/|wx| in a whole bin
     const double v = k0 == k1 ? l * R::inv_dx(cp) : R::abs(iwx);
-    if (global || (int)((unsigned long long)__double_as_longlong(v) >> 52) >= 1023 + kFixed64MaxExp) {
+    const int F = cp.fix_bits;
+    if (global || (__double2hiint(v) >> 20) >= 1023 + kFixedDepositBits - F) {
         const double a = up ? x0 : x1, b = up ? x1 : x0, L = R::L(cp);
         plan_flight_real(f, R::nonneg(a) * R::inv_dx(cp), (R::lt(L, R::nonneg(b)) ? L : R::nonneg(b)) * R::inv_dx(cp), l,
                          R::dx(cp) * R::abs(iwx));
         return;
     }
-    const unsigned long long q = fixed64(v);
-    f.a0 = k0 == k1 ? q : q - mul_fraction(F0, q);
-    f.a1 = mul_fraction(F1, q);
+    const Fix96 q = fixed96(v, F);
+    const bool multi = k0 != k1;  // else a0 = q, a1 = 0
+    f.a0 = sub96(q, fraction96(multi ? (up ? from.F : to.F) : 0ull, q));
+    f.a1 = fraction96(multi ? (up ? to.F : from.F) : 0ull, q);
     f.c = q;
 }
 
@@ -1253,7 +1235,8 @@ __device__ __forceinline__ int step(History<P> &s, const Case &cp, Draws &draws,
 // cls_internal.h): the bins, FP64 statistics, counters and the lanes' own
 // copies of the per-history statistics.  The bins are a fixed-point difference
 // array, prefix-summed exactly at the flush: the FP32 walk's with 32 fraction
-// bits of track length, the FP64 walk's with kFixed64Bits of a bin width.
+// bits of track length, the FP64 walk's in 96 bits with fix_bits of a bin width
+// (cls_fixed.h).
 //
 // 64-bit additions in shared memory go through 32-bit halves: the low half's
 // atomic returns the old value, whose carry joins the high half.  Every wrap
@@ -1284,8 +1267,9 @@ __device__ __forceinline__ void add_entry(unsigned char *region, int nbs, int k,
     add_halves(lo, lo + nbs + 1, x);
 }
 
+template <typename P>
 __device__ __forceinline__ uint32_t *region_counters(unsigned char *region, int nbs) {
-    return reinterpret_cast<uint32_t *>(region + region_bins_bytes(nbs) + 8 * S_NUM);
+    return reinterpret_cast<uint32_t *>(region + region_bins_bytes(sizeof(P) == 8, nbs) + 8 * S_NUM);
 }
 
 // counter c of the region += x (C_MAXEV: maximum, below 2^32)
@@ -1316,7 +1300,7 @@ using LaneStat = typename std::conditional<kFixedStats<P>, unsigned long long, d
 
 template <typename P>
 __device__ __forceinline__ LaneStat<P> *region_lane_stats(unsigned char *region, int nbs) {
-    return reinterpret_cast<LaneStat<P> *>(region + region_lane_stats_offset(nbs));
+    return reinterpret_cast<LaneStat<P> *>(region + region_lane_stats_offset(sizeof(P) == 8, nbs));
 }
 
 // A history longer than this (in track length) keeps its statistics out of the
@@ -1325,8 +1309,9 @@ __device__ __forceinline__ LaneStat<P> *region_lane_stats(unsigned char *region,
 // histories between flushes (FP32 regions flush every 1024).
 constexpr float kFixedTrackMax = 8192.0f;
 
+template <typename P>
 __device__ __forceinline__ double *region_stats(unsigned char *region, int nbs) {
-    return reinterpret_cast<double *>(region + region_bins_bytes(nbs));
+    return reinterpret_cast<double *>(region + region_bins_bytes(sizeof(P) == 8, nbs));
 }
 
 // The history's track length t and t^2 into this lane's own copy of the
@@ -1428,45 +1413,70 @@ __device__ __forceinline__ uint64_t bins_offset(const Tallies &t, int lcase, uin
 }
 
 // Bound on a region's bins between two flushes (FP64 walk): each lane sums the
-// high words of its flights' largest deposits, at most 2^(kFixed64Bits - 32 +
-// kFixed64MaxExp) = 2^25 each, and the warp flushes once a lane's sum has
-// reached 2^25: no lane's passes 2^26, so no bin of the warp passes 2^63 units.
-// FP32 regions are flushed by the histories fed into them.
-constexpr uint32_t kDepositBound = 1u << (kFixed64Bits - 32 + kFixed64MaxExp);
-static_assert(32ull * 2 * kDepositBound <= 1ull << 31, "a bin's sum stays below 2^63 units");
+// high words of its flights' largest deposits, rounded up, at most 2^26 each, and
+// the warp flushes once a lane's sum has reached 2^26: no lane's passes 2^27, so
+// no bin of the warp reaches 2^96 units.  (For F = 64 that is 2^26 bin widths: in
+// practice only key changes flush.)  FP32 regions are flushed by the histories fed
+// into them.
+constexpr uint32_t kDepositBound = 1u << (kFixedDepositBits - 64);
+static_assert(32ull * 2 * kDepositBound <= 1ull << 32, "a bin's sum stays below 2^96 units");
 
 // A flight's entries in the difference array D (bin k = D[0] + ... + D[k]): its
 // bins are a0 in k0, c in each interior bin k0 < k < k1 and a1 in k1, each
 // rounded once to fixed point (q0, qc, q1; zero where the flight has no such
 // bin), so D[k0] += q0, D[k0+1] += d1 = qc - q0 (or q1 - q0 when k1 = k0 + 1),
 // D[k1] += d2 = q1 - qc (with interior bins), D[k1+1] += d3 = -q1 (beyond one
-// bin), modulo 2^64: the flush's prefix sum returns exactly the rounded
-// deposits, whatever the order of the additions.  bound: its share of
-// kDepositBound.
+// bin), modulo 2^64 (2^96 in the FP64 walk): the flush's prefix sum returns
+// exactly the rounded deposits, whatever the order of the additions.
 struct FixedFlight {
     bool multi, inter;
-    unsigned long long q0, q1, qc, d1, d2, d3;
-    uint32_t bound;
+    unsigned long long q0, d1, d2, d3;
     __device__ __forceinline__ explicit FixedFlight(const Flight<float> &f) : multi(f.k1 > f.k0), inter(f.k1 > f.k0 + 1) {
         q0 = fixed32(f.a0);
-        q1 = fixed32(multi ? f.a1 : 0.0f);
-        qc = fixed32(inter ? f.c : 0.0f);
-        bound = 0;
-        entries();
-    }
-    __device__ __forceinline__ explicit FixedFlight(const Flight<double> &f) : multi(f.k1 > f.k0), inter(f.k1 > f.k0 + 1) {
-        q0 = f.a0;
-        q1 = multi ? f.a1 : 0ull;
-        qc = inter ? f.c : 0ull;
-        bound = (uint32_t)(f.c >> 32) + 1u;
-        entries();
-    }
-    __device__ __forceinline__ void entries() {
+        const unsigned long long q1 = fixed32(multi ? f.a1 : 0.0f), qc = fixed32(inter ? f.c : 0.0f);
         d1 = (inter ? qc : q1) - q0;
         d2 = q1 - qc;
         d3 = 0ull - q1;
     }
 };
+
+// The flight's entries added to the difference array; returns its share of
+// kDepositBound.
+__device__ __forceinline__ uint32_t deposit_flight(unsigned char *region, int nbs, const Flight<float> &f) {
+    const FixedFlight q(f);
+    add_entry(region, nbs, f.k0, q.q0);
+    add_entry(region, nbs, f.k0 + 1, q.d1);
+    if (q.inter) add_entry(region, nbs, f.k1, q.d2);
+    if (q.multi) add_entry(region, nbs, f.k1 + 1, q.d3);
+    return 0u;
+}
+
+// 96-bit entry k: as with 64 bits (add_halves) each word's atomic returns the old
+// value, whose carry joins the next word.
+__device__ __forceinline__ void add_entry(unsigned char *region, int nbs, int k, Fix96 x) {
+    uint32_t *const p = reinterpret_cast<uint32_t *>(region) + k;
+    uint32_t old = atomicAdd(p, x.w0);
+    asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %2, %3;\n\taddc.cc.u32 %0, %0, 0;\n\taddc.u32 %1, %1, 0;\n\t}"
+        : "+r"(x.w1), "+r"(x.w2)
+        : "r"(old), "r"(x.w0));
+    old = atomicAdd(p + nbs + 1, x.w1);
+    asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %1, %2;\n\taddc.u32 %0, %0, 0;\n\t}"
+        : "+r"(x.w2)
+        : "r"(old), "r"(x.w1));
+    atomicAdd(p + 2 * (nbs + 1), x.w2);
+}
+
+// FP64 walk.  Entry by entry: the four entries' words sent out together, to wait
+// for shared memory twice instead of eight times, take more instructions and were
+// slower (1e6 histories: rod 369 against 361 us, slab 515 / 498).
+__device__ __forceinline__ uint32_t deposit_flight(unsigned char *region, int nbs, const Flight<double> &f) {
+    const bool multi = f.k1 > f.k0, inter = f.k1 > f.k0 + 1;
+    add_entry(region, nbs, f.k0, f.a0);
+    add_entry(region, nbs, f.k0 + 1, sub96(inter ? f.c : f.a1, f.a0));  // (a1 = 0 in a flight of one bin)
+    if (inter) add_entry(region, nbs, f.k1, sub96(f.a1, f.c));
+    if (multi) add_entry(region, nbs, f.k1 + 1, sub96(Fix96{0u, 0u, 0u}, f.a1));
+    return f.c.w2 + 1u;
+}
 
 // Score the warp's flights.
 //   Region lanes: the difference array's entries (FixedFlight), two integer
@@ -1484,13 +1494,7 @@ __device__ __forceinline__ uint32_t warp_deposit(unsigned char *regions, int rby
     if (has) {
         if (!global) {
             // predicated, not branched: every lane with a flight runs the same code
-            unsigned char *region = regions + lreg * rbytes;
-            const FixedFlight q(f);
-            bound = q.bound;
-            add_entry(region, nbs, f.k0, q.q0);
-            add_entry(region, nbs, f.k0 + 1, q.d1);
-            if (q.inter) add_entry(region, nbs, f.k1, q.d2);
-            if (q.multi) add_entry(region, nbs, f.k1 + 1, q.d3);
+            bound = deposit_flight(regions + lreg * rbytes, nbs, f);
         } else {
             double *gbins = t.flux + bins_offset(t, lcase, lbatch);
             atomicAdd(&gbins[f.k0], flight_real(f.a0));
@@ -1572,21 +1576,41 @@ __device__ __forceinline__ void flush_region(unsigned char *region, const Launch
     double *g = a.t.flux + ((size_t)case_index * a.t.nbatch + batch) * (size_t)nbs;
     // the exact prefix sum of the fixed-point difference array, 32 bins at a
     // time; its entry nb (past the last bin) sums to zero and is cleared
-    const double unit = sizeof(P) == 4 ? 0x1p-32 : a.cases[case_index].dx * (1.0 / (double)(1ull << kFixed64Bits));
     uint32_t *lo = reinterpret_cast<uint32_t *>(region), *hi = lo + nbs + 1;
-    unsigned long long carry = 0ull;
-    for (int base = 0; base <= nb; base += 32) {
-        const int k = base + lane;
-        unsigned long long d = (k <= nb) ? (unsigned long long)hi[k] << 32 | lo[k] : 0ull;
+    if constexpr (sizeof(P) == 4) {
+        unsigned long long carry = 0ull;
+        for (int base = 0; base <= nb; base += 32) {
+            const int k = base + lane;
+            unsigned long long d = (k <= nb) ? (unsigned long long)hi[k] << 32 | lo[k] : 0ull;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long v = __shfl_up_sync(CLS_FULL_MASK, d, o);
-            if (lane >= o) d += v;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long v = __shfl_up_sync(CLS_FULL_MASK, d, o);
+                if (lane >= o) d += v;
+            }
+            const long long q = (long long)(carry + d);  // the bin's deposits, in units
+            carry += __shfl_sync(CLS_FULL_MASK, d, 31);
+            if (k < nb && q != 0) atomicAdd(&g[k], (double)q * 0x1p-32);
+            if (k <= nb) lo[k] = hi[k] = 0u;
         }
-        const long long q = (long long)(carry + d);  // the bin's deposits, in units
-        carry += __shfl_sync(CLS_FULL_MASK, d, 31);
-        if (k < nb && q != 0) atomicAdd(&g[k], (double)q * unit);
-        if (k <= nb) lo[k] = hi[k] = 0u;
+    } else {
+        const double unit = a.cases[case_index].fix_unit;
+        uint32_t *top = hi + nbs + 1;
+        Fix96 carry{0u, 0u, 0u};
+        for (int base = 0; base <= nb; base += 32) {
+            const int k = base + lane;
+            Fix96 d = (k <= nb) ? Fix96{lo[k], hi[k], top[k]} : Fix96{0u, 0u, 0u};
+#pragma unroll 1
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t w0 = __shfl_up_sync(CLS_FULL_MASK, d.w0, o), w1 = __shfl_up_sync(CLS_FULL_MASK, d.w1, o),
+                               w2 = __shfl_up_sync(CLS_FULL_MASK, d.w2, o);
+                if (lane >= o) d = add96(d, Fix96{w0, w1, w2});
+            }
+            const Fix96 q = add96(carry, d);  // the bin's deposits, in units
+            carry = Fix96{__shfl_sync(CLS_FULL_MASK, q.w0, 31), __shfl_sync(CLS_FULL_MASK, q.w1, 31),
+                          __shfl_sync(CLS_FULL_MASK, q.w2, 31)};
+            if (k < nb && (q.w0 | q.w1 | q.w2) != 0u) atomicAdd(&g[k], fix96_to_double(q) * unit);
+            if (k <= nb) lo[k] = hi[k] = top[k] = 0u;
+        }
     }
     if (!ends) {
         __syncwarp();
@@ -1607,7 +1631,7 @@ __device__ __forceinline__ void flush_region(unsigned char *region, const Launch
         for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(CLS_FULL_MASK, v, o);
         if (lane == 0 && __double_as_longlong(v) != 0) atomicAdd(&gst[q], v);
     }
-    double *st = region_stats(region, nbs);
+    double *st = region_stats<P>(region, nbs);
     if (lane < S_NUM) {
         const double v = st[lane];
         if (v != 0.0) {
@@ -1616,7 +1640,7 @@ __device__ __forceinline__ void flush_region(unsigned char *region, const Launch
         }
     } else if (lane < S_NUM + C_NUM) {
         const int c = lane - S_NUM;
-        uint32_t *ct = region_counters(region, nbs);
+        uint32_t *ct = region_counters<P>(region, nbs);
         const unsigned long long v = (unsigned long long)ct[C_NUM + c] << 32 | ct[c];
         if (v != 0ull) {
             unsigned long long *gc = &a.t.counters[(size_t)case_index * C_NUM + c];
@@ -1880,7 +1904,7 @@ __device__ __forceinline__ void end_history(unsigned char *regions, const Launch
     if (lreg < 2) {
         unsigned char *region = regions + lreg * a.region_bytes;
         if (!finish_history<P>(region, a.t.nbins_stride, s, lane)) add_history_stats_global<P>(a, lcase, s);
-        count_one(region_counters(region, a.t.nbins_stride), out, n_coll, s.n_int, n_refl, events, s.events);
+        count_one(region_counters<P>(region, a.t.nbins_stride), out, n_coll, s.n_int, n_refl, events, s.events);
     } else {
         finish_history_global<P>(a, lcase, s, out, true, n_coll, n_refl, events);
     }

@@ -140,8 +140,8 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
 // event maximum (event and collision counts are added per pass).
 template <typename P>
 __device__ __forceinline__ void finish_event_history(unsigned char *region, int nbs, const History<P> &s, int outcome) {
-    double *st = region_stats(region, nbs);
-    uint32_t *ct = region_counters(region, nbs);
+    double *st = region_stats<P>(region, nbs);
+    uint32_t *ct = region_counters<P>(region, nbs);
     const double t0 = (double)s.track0;
     const double t1 = (double)s.track1;
     const double t = t0 + t1;
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(kEventBlock, kEventMinBlocks) event_kernel(con
         }
         // warp-aggregated event counters: one shared-memory atomic per counter
         for (int r = 0; r < 2; ++r) {
-            uint32_t *ct = region_counters(regions + r * rb, nbs);
+            uint32_t *ct = region_counters<P>(regions + r * rb, nbs);
             const unsigned long long v0 = warp_sum(r ? c1 : c0), v1 = warp_sum(r ? i1 : i0);
             const unsigned long long v2 = warp_sum(r ? f1 : f0), v3 = warp_sum(r ? e1 : e0);
             if (lane == 0) {

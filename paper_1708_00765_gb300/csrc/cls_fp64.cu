@@ -21,11 +21,11 @@ cudaError_t launch_history_g(const LaunchArgs &a, int grid, int block, size_t sm
 }
 
 template <int G>
-cudaError_t launch_narrow_g(const LaunchArgs &a, int grid, size_t smem, cudaStream_t s) {
+cudaError_t launch_narrow_g(const LaunchArgs &a, int grid, int block, size_t smem, cudaStream_t s) {
     static std::atomic<unsigned long long> optin{0};
     const cudaError_t e = ensure_smem_optin(narrow_kernel<double, G>, optin);
     if (e != cudaSuccess) return e;
-    narrow_kernel<double, G><<<grid, kNarrowBlock, smem, s>>>(a);
+    narrow_kernel<double, G><<<grid, block, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -43,14 +43,14 @@ cudaError_t launch_history_fp64(const LaunchArgs &a, int grid, int block, size_t
     }
 }
 
-cudaError_t launch_narrow_fp64(const LaunchArgs &a, int grid, size_t smem, cudaStream_t s, int geom) {
+cudaError_t launch_narrow_fp64(const LaunchArgs &a, int grid, int block, size_t smem, cudaStream_t s, int geom) {
     switch (geom) {
-    case 1: return launch_narrow_g<1>(a, grid, smem, s);
-    case 2: return launch_narrow_g<2>(a, grid, smem, s);
-    case 3: return launch_narrow_g<3>(a, grid, smem, s);
-    case 11: return launch_narrow_g<11>(a, grid, smem, s);
-    case 13: return launch_narrow_g<13>(a, grid, smem, s);
-    default: return launch_narrow_g<0>(a, grid, smem, s);
+    case 1: return launch_narrow_g<1>(a, grid, block, smem, s);
+    case 2: return launch_narrow_g<2>(a, grid, block, smem, s);
+    case 3: return launch_narrow_g<3>(a, grid, block, smem, s);
+    case 11: return launch_narrow_g<11>(a, grid, block, smem, s);
+    case 13: return launch_narrow_g<13>(a, grid, block, smem, s);
+    default: return launch_narrow_g<0>(a, grid, block, smem, s);
     }
 }
 

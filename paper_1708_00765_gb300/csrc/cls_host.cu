@@ -31,7 +31,6 @@ namespace {
 constexpr int kBatchQuantum = 1024;   // statistics batches are multiples of this many histories
 constexpr int kMaxCases = 65536;
 constexpr uint32_t kMaxEventsLimit = 1u << 28;
-constexpr size_t kMaxSmemPerBlock = 200 * 1024;  // opt-in dynamic shared memory per block
 
 struct Options {
     int precision = CLS_PREC_FP64;
@@ -380,7 +379,7 @@ uint64_t batch_len_for(uint64_t n, int nbatch) {
 }
 
 int region_bytes_for(const cls_handle *h) {
-    return region_bytes(h->nbins_stride);
+    return region_bytes(h->opt.precision == CLS_PREC_FP64, h->nbins_stride);
 }
 
 // FP32 regions are flushed into the FP64 global tallies after this many
@@ -733,9 +732,9 @@ int launch_tracker(cls_handle *h, LaunchArgs a, int sched, int geom, const Shape
                      : launch_history_fp32(a, sh.grid, sh.block, sh.smem, s, geom);
     }
     if (e != cudaSuccess || (!a.narrow && a.hand_over == 0)) return cuda_fail(e);
-    const int grid = narrow_grid(a, n, h->sm_count);
+    const int grid = narrow_grid(a, fp64, n, h->sm_count), block = 32 * narrow_block_warps(fp64, a.region_bytes);
     const size_t smem = narrow_smem(a, fp64);
-    e = fp64 ? launch_narrow_fp64(a, grid, smem, s, geom) : launch_narrow_fp32(a, grid, smem, s, geom);
+    e = fp64 ? launch_narrow_fp64(a, grid, block, smem, s, geom) : launch_narrow_fp32(a, grid, block, smem, s, geom);
     return cuda_fail(e);
 }
 

@@ -34,6 +34,8 @@ struct CaseParams {
     int32_t source;    // 0 incident flux on x = 0 (suite I), 1 uniform isotropic volume source (suite II)
     int32_t filter;    // the FP64 walk may compare distances in FP32 first (choose): the parameters' magnitudes allow it
     double cost;    // host estimate of events per history (ordering only)
+    double fix_unit;   // FP64 walk: the unit of its bins, dx 2^-fix_bits (cls_fixed.h)
+    int32_t fix_bits;
 };
 
 // Per-run work of one case: histories [first, first + n), statistics batch
@@ -153,15 +155,18 @@ struct TraceArgs {
 // The bins are nbins_stride + 1 entries of a fixed-point difference array: a
 // flight adds its end-bin partials and its interior-bin length with at most
 // four integer additions, whatever its length, and the flush takes the exact
-// prefix sum (FP64 is used from the flush on).  Entries and counters are 64
-// bits in two arrays of 32-bit halves, low halves first: shared memory adds 32
-// bits natively, 64 bits only by a compare-and-swap loop (cls_device.cuh).
-__host__ __device__ inline int region_bins_bytes(int nbins_stride) { return 8 * (nbins_stride + 1); }
-__host__ __device__ inline int region_lane_stats_offset(int nbins_stride) {
-    return region_bins_bytes(nbins_stride) + 8 * (S_NUM + C_NUM);
+// prefix sum (FP64 is used from the flush on).  Entries have 64 bits in the FP32
+// walk and 96 in the FP64 walk (cls_fixed.h), counters 64, in arrays of 32-bit
+// words, low words first: shared memory adds 32 bits natively, 64 bits only by a
+// compare-and-swap loop (cls_device.cuh).
+__host__ __device__ constexpr int region_bins_bytes(bool fp64, int nbins_stride) {
+    return fp64 ? (12 * (nbins_stride + 1) + 7) & ~7 : 8 * (nbins_stride + 1);
 }
-__host__ __device__ inline int region_bytes(int nbins_stride) {
-    return (region_lane_stats_offset(nbins_stride) + 8 * 32 * S_NUM + 15) & ~15;
+__host__ __device__ constexpr int region_lane_stats_offset(bool fp64, int nbins_stride) {
+    return region_bins_bytes(fp64, nbins_stride) + 8 * (S_NUM + C_NUM);
+}
+__host__ __device__ constexpr int region_bytes(bool fp64, int nbins_stride) {
+    return (region_lane_stats_offset(fp64, nbins_stride) + 8 * 32 * S_NUM + 15) & ~15;
 }
 
 constexpr int kWarpFeedBytes = 112;  // of WarpFeed (cls_device.cuh)
@@ -173,6 +178,15 @@ constexpr int kNarrowBlock = 128, kNarrowBlocks = 3;
 constexpr int kHandOver = 4;
 constexpr int kStragglerBytes = 144;
 __host__ __device__ constexpr int narrow_memory_bytes(bool fp64) { return (fp64 ? 4096 : 1536) + kWarpFeedBytes; }
+
+// Dynamic shared memory that a block may take (the opt-in the kernels are given).
+constexpr size_t kMaxSmemPerBlock = 200 * 1024;
+
+// Warps of a block of the narrow walk: fewer on the widest meshes.
+inline int narrow_block_warps(bool fp64, int region) {
+    const size_t fit = kMaxSmemPerBlock / ((size_t)narrow_memory_bytes(fp64) + region);
+    return fit < kNarrowBlock / 32 ? (int)fit : kNarrowBlock / 32;
+}
 
 // Dynamic shared memory of a warp of the history tracker: two tally regions and
 // its feeding state (cls_device.cuh's WarpFeed).
@@ -204,8 +218,8 @@ cudaError_t launch_history_fp64(const LaunchArgs &a, int grid, int block, size_t
 cudaError_t launch_history_fp32(const LaunchArgs &a, int grid, int block, size_t smem, cudaStream_t s, int geom);
 cudaError_t launch_event_fp64(const LaunchArgs &a, int grid, int block, size_t smem, cudaStream_t s, int geom);
 cudaError_t launch_event_fp32(const LaunchArgs &a, int grid, int block, size_t smem, cudaStream_t s, int geom);
-cudaError_t launch_narrow_fp64(const LaunchArgs &a, int grid, size_t smem, cudaStream_t s, int geom);
-cudaError_t launch_narrow_fp32(const LaunchArgs &a, int grid, size_t smem, cudaStream_t s, int geom);
+cudaError_t launch_narrow_fp64(const LaunchArgs &a, int grid, int block, size_t smem, cudaStream_t s, int geom);
+cudaError_t launch_narrow_fp32(const LaunchArgs &a, int grid, int block, size_t smem, cudaStream_t s, int geom);
 cudaError_t launch_trace_fp64(const TraceArgs &a, cudaStream_t s);
 cudaError_t launch_trace_fp32(const TraceArgs &a, cudaStream_t s);
 cudaError_t occupancy_history_fp64(int block, size_t smem, int *blocks_per_sm, int geom);

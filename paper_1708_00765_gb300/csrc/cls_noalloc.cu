@@ -131,6 +131,7 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
         img.cases[k] = make_case(params + 9 * (size_t)k, (uint32_t)k);
         cost += img.cases[k].cost * (double)n;
     }
+    a.region_bytes = region_bytes(true, nbins_stride);
     plan_pieces(a, n, batch_len, cost / (double)n / ncases, 0, sm_count, false, kNoallocMaxPieces);
     a.chunk_counter = &scratch->chunk_counter;
     a.claimed = scratch->claimed;
@@ -142,7 +143,6 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
     a.seed = seed;
     a.rk = make_round_keys(seed);
     a.max_events = 100000000u;
-    a.region_bytes = region_bytes(nbins_stride);
 
     for (int k = 0; k < ncases; ++k) {
         RunCase &r = img.runs[k];
@@ -154,7 +154,7 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
     }
 
     const size_t per_warp = history_warp_bytes(a.region_bytes);
-    int warps = (int)((200 * 1024) / per_warp);
+    int warps = (int)(kMaxSmemPerBlock / per_warp);
     warps = warps > kHistoryBlockFp64 / 32 ? kHistoryBlockFp64 / 32 : warps;
     if (warps < 1) return CLS_E_INVAL;
     const int block = 32 * warps;
@@ -170,5 +170,8 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
     if (!a.narrow) history_kernel<double, 0><<<sm_count * bps, block, smem, s>>>(a);
     if (cudaGetLastError() != cudaSuccess) return CLS_E_CUDA;
     if (!a.narrow && a.hand_over == 0) return CLS_OK;
-    return launch_narrow_fp64(a, narrow_grid(a, n, sm_count), narrow_smem(a, true), s, 0) == cudaSuccess ? CLS_OK : CLS_E_CUDA;
+    const int narrow_block = 32 * narrow_block_warps(true, a.region_bytes);
+    return launch_narrow_fp64(a, narrow_grid(a, true, n, sm_count), narrow_block, narrow_smem(a, true), s, 0) == cudaSuccess
+               ? CLS_OK
+               : CLS_E_CUDA;
 }

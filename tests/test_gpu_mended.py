@@ -31,3 +31,31 @@ def test_a_batch_seed_counts_with_all_its_bits():
                 assert g[key] == want, (k, key)
             assert g["sum_t"] == pytest.approx(sum(p["sum_t"] for p in parts), rel=1e-12)
         prob.close()
+
+
+THICK = [(1.0, 1.0, 1.0, 1.0, 0.5, 0.5, L, 1, 1) for L in (1e5, 1e6, 1e9, 1e12, 1e14, 1e16)] + [
+    (1.0, 1.0, 1.0, 1.0, 0.5, 0.5, 1e16, 3, 3),
+    (1e12, 1e-3, 1.0, 2.0, 0.0, 0.9, 10.0, 1, 4),       # one material a trillion times as thick as the other
+    (0.1, 1e6, 1.0, 1e-9, 0.9, 0.0, 10.0, 11, 50),      # a chord of 1e-9 between ordinary ones
+    (1e300, 1e300, 1.0, 1.0, 0.5, 0.5, 1e300, 1, 2),    # no fixed-point unit: every flight in FP64
+    (0.5, 5.0, 2.0, 0.5, 0.5, 0.9, 10.0, 1, 4096)]      # the widest mesh
+
+
+@pytest.mark.parametrize("schedule,n", [("history", 300), ("history", 40_000), ("event", 20_000)])
+@pytest.mark.parametrize("params", THICK)
+def test_flux_where_a_bin_is_very_many_flights_wide(params, schedule, n):
+    """The flux bins hold what the flights deposit, whatever their length in bin widths."""
+    assert_parity(run(params, n, 31, schedule=schedule), oracle.run(ocase(params), 31, 0, n))
+
+
+@pytest.mark.parametrize("schedule,n", [("history", 300), ("history", 40_000), ("event", 20_000)])
+@pytest.mark.parametrize("params", THICK)
+def test_flux_of_a_thick_volume_source_is_the_track_length(params, schedule, n):
+    """Histories born deep inside, where a coordinate does not resolve a flight: the bins sum to the
+    track length all the same."""
+    raw = run(params, n, 31, source="volume", schedule=schedule)
+    o = oracle.run(ocase(params, 1), 31, 0, n)
+    for k, ko in COUNTS.items():
+        assert raw[k] == o[ko], k
+    assert raw["sum_t"] == pytest.approx(o["sum_t"], rel=1e-12)
+    assert raw["flux"].sum() == pytest.approx(raw["sum_t"], rel=1e-12)
