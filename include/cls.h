@@ -171,7 +171,9 @@ int cls_get_option(const cls_handle *h, int key, int64_t *value);
  * of runs equals one long run (checkpoint / resume).  History h draws its random
  * numbers from Philox4x32-10 with key `seed` and counter (j/2, h, case), so a
  * run is fully determined by (seed, first history, n).  Asynchronous; the
- * caller must keep the handle alive until the stream has finished.
+ * caller must keep the handle alive until the stream has finished.  Runs of one
+ * handle follow one another on the device, whatever their streams (outside
+ * stream capture).
  * Errors: CLS_E_INVAL (n == 0), CLS_E_CUDA. */
 int cls_run(cls_handle *h, uint64_t n_histories, uint64_t seed, void *stream);
 

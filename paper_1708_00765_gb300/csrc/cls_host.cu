@@ -753,6 +753,19 @@ int record_pair(cls_handle *h, cudaStream_t s, bool start) {
     return cuda_fail(cudaEventRecord(h->ev_pairs[h->ev_pairs.size() - (start ? 2 : 1)], s));
 }
 
+// Runs of a handle share its work list, work counters, hand-over slots and tallies:
+// a run enqueued on another stream than the last one's waits on the device for that
+// one's end (ev_pairs is empty once it has been waited for).  A stream of the
+// per-thread default's name may be another thread's.  Nothing outside a capture can
+// be waited for within it.
+int order_after_last_run(cls_handle *h, cudaStream_t s) {
+    if (h->ev_pairs.empty() || (s == h->last_stream && s != cudaStreamPerThread)) return CLS_OK;
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess) cudaGetLastError();
+    if (capturing != cudaStreamCaptureStatusNone) return CLS_OK;
+    return cuda_fail(cudaStreamWaitEvent(s, h->ev_pairs.back(), 0));
+}
+
 // The timed runs' events go back for the next runs (a few: a program that never
 // reads its tallies leaves a pair for each run).
 void release_events(cls_handle *h) {
@@ -892,9 +905,6 @@ int tallies_of(cls_handle *h, int k, cls_tallies_t *out) {
         bh[b] = (double)h->batch_hist[k][b];
         used += h->batch_hist[k][b] > 0;
     }
-    // runs still in flight on other streams than the last one's
-    for (size_t i = 0; i + 3 < h->ev_pairs.size(); i += 2)
-        CLS_CUDA(cudaStreamWaitEvent(h->last_stream, h->ev_pairs[i + 1], 0));
     const int copies = stats_copies(h->cases.size());
     tally_kernel<<<(c.nbins + kTallyBins - 1) / kTallyBins, dim3(kTallyBins, kTallySlices), 0, h->last_stream>>>(
         h->d_flux + (size_t)k * h->nbatch * h->nbins_stride, h->d_stats + (size_t)k * copies * S_NUM,
@@ -1202,7 +1212,8 @@ int cls_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
     Shape sh[kMaxGroups];
     rc = plan_bank(h, plan, sh, s);
     if (rc) return rc;
-    rc = record_pair(h, s, true);
+    rc = order_after_last_run(h, s);
+    if (!rc) rc = record_pair(h, s, true);
     if (rc) return rc;
     CLS_CUDA(cudaMemcpyAsync(h->d_runs, h->h_runs, runs_bytes(h->cases.size()), cudaMemcpyHostToDevice, s));
     CLS_CUDA(cudaEventRecord(h->runs_copied, s));
@@ -1281,7 +1292,8 @@ int cls_batch_run(cls_handle *h, uint64_t n, uint64_t seed, void *stream) {
         h->graph_run = run;
         std::memcpy(h->graph_key, key, sizeof(key));
     }
-    rc = record_pair(h, s, true);
+    rc = order_after_last_run(h, s);
+    if (!rc) rc = record_pair(h, s, true);
     if (rc) return rc;
     CLS_CUDA(cudaMemcpyAsync(h->d_runs, h->h_runs, runs_bytes(h->cases.size()), cudaMemcpyHostToDevice, s));
     CLS_CUDA(cudaEventRecord(h->runs_copied, s));

@@ -59,3 +59,23 @@ def test_flux_of_a_thick_volume_source_is_the_track_length(params, schedule, n):
         assert raw[k] == o[ko], k
     assert raw["sum_t"] == pytest.approx(o["sum_t"], rel=1e-12)
     assert raw["flux"].sum() == pytest.approx(raw["sum_t"], rel=1e-12)
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_runs_of_one_handle_on_several_streams_follow_one_another(batch):
+    """Long and short runs in turn on three streams, nothing waited for in between."""
+    p = (1.0, 10.0, 0.5, 0.2, 0.999, 0.999, 8.0, 3, 60)
+    params = np.array([p, workloads.ROD_L10, p]) if batch else np.array([p])
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    sizes = [30_000, 500, 4_000, 4_000, 25_000, 100]
+    prob = cls.Problem(params if batch else p, batch=batch)
+    for i, n in enumerate(sizes):
+        prob.run(n, 7, stream=streams[i % 3])
+    for k in range(params.shape[0]):
+        g = prob.raw_tallies(k)
+        o = oracle.run(ocase(params[k]), 7, 0, sum(sizes), case_id=k)
+        for key, ko in COUNTS.items():
+            assert g[key] == o[ko], (k, key)
+        assert g["sum_t"] == pytest.approx(o["sum_t"], rel=1e-12)
+        np.testing.assert_allclose(g["flux"].sum(0), o["flux"].sum(0), rtol=1e-12)
+    prob.close()
