@@ -80,12 +80,13 @@ inline int hand_over_for(double events, bool fp32, int geom) {
 // claimed (LaunchArgs): pieces of whole statistics batches, at most max_pieces
 // of them; as many warps start on a piece as it takes to employ all; and the
 // least a warp claims is 32 histories, a warp's lanes, or where that would not
-// go round, a power of two below.
+// go round, a power of two below.  may_narrow: whether a run small enough goes to
+// the narrow walk.
 inline void plan_pieces(LaunchArgs &a, uint64_t n, uint64_t batch_len, double mean_cost, int geom, int sm_count, bool fp32,
-                        uint64_t max_pieces) {
+                        uint64_t max_pieces, bool may_narrow) {
     const double total = (double)n * a.nruns;
     const double narrow_warps = (double)sm_count * kNarrowBlocks * narrow_block_warps(!fp32, a.region_bytes);
-    a.narrow = total <= narrow_histories(fp32, geom) * narrow_warps;
+    a.narrow = may_narrow && total <= narrow_histories(fp32, geom) * narrow_warps;
     const double warps = a.narrow ? std::min(total, narrow_warps) : sm_count * (fp32 ? 28.0 : 20.0);
     const uint64_t used = (n + batch_len - 1) / batch_len;  // batches
     const uint64_t per_run = std::max<uint64_t>(1, std::min<uint64_t>(std::min<uint64_t>(used, 64), max_pieces / a.nruns));

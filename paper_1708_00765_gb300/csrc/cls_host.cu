@@ -126,6 +126,10 @@ struct cls_handle {
     int device = 0;
     int sm_count = 0;
     bool batch = false;
+    // an autotuner's twin: its runs stand for much longer ones, so they take the
+    // tracker whose shape is being chosen even where they are small enough for the
+    // narrow walk, which knows no block, chunk or blocks per SM to choose
+    bool pilot = false;
     std::vector<double> params;  // ncases x 9, as created
     int geom = 0;                // geometry shared by every case, 0 if mixed
     Options opt;
@@ -481,7 +485,7 @@ int prepare_run(cls_handle *h, uint64_t n, uint64_t seed, RunPlan *plan) {
         ag.claimed = h->d_chunk_counter + kGroupCounters + pieces;
         if (groups[g].sched != CLS_SCHED_EVENT) {
             plan_pieces(ag, n, batch_len_for(n, h->nbatch), groups[g].cost / groups[g].ncases, groups[g].geom, h->sm_count,
-                        h->opt.precision == CLS_PREC_FP32, kMaxPieces);
+                        h->opt.precision == CLS_PREC_FP32, kMaxPieces, !h->pilot);
             pieces += (uint64_t)ag.pieces_per_run * ag.nruns;
         } else {
             ag.hand_over = hand_over_for(estimated_events(groups[g].cost / groups[g].ncases),
@@ -1014,6 +1018,7 @@ int cls_autotune(cls_handle *h, uint64_t n_pilot, uint64_t seed, void *stream) {
     int rc = create_common(h->params.data(), ncases, h->batch, &t);
     if (rc) return rc;
     t->opt = h->opt;
+    t->pilot = true;
     std::vector<Tuned> cand;
     // a batch of several geometries also tries one launch per geometry against one mixed launch
     std::vector<int> groupings = {h->opt.group_geometry};
@@ -1339,6 +1344,7 @@ int cls_autotune_cases(cls_handle *h, uint64_t n_pilot, uint64_t seed, void *str
         rc = create_common(h->params.data() + 9 * (size_t)k, 1, false, &t);
         if (rc) break;
         t->opt = h->opt;
+        t->pilot = true;
         t->cases[0].case_id = h->cases[k].case_id;  // the case's own random numbers
         rc = cudaMemcpy(t->d_cases, t->cases.data(), sizeof(CaseParams), cudaMemcpyHostToDevice) == cudaSuccess
                  ? CLS_OK : CLS_E_CUDA;
@@ -1370,6 +1376,7 @@ int cls_autotune_cases(cls_handle *h, uint64_t n_pilot, uint64_t seed, void *str
         rc = create_common(h->params.data(), nc, true, &t);
         if (!rc) {
             t->opt = h->opt;
+            t->pilot = true;
             for (int i = 0; i < 2 && !rc; ++i) {
                 for (int k = 0; k < nc; ++k) t->case_sched[k] = i ? chosen[k] : CLS_SCHED_AUTO;
                 destroy_graph(t);

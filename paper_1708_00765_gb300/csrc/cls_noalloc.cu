@@ -132,7 +132,7 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
         cost += img.cases[k].cost * (double)n;
     }
     a.region_bytes = region_bytes(true, nbins_stride);
-    plan_pieces(a, n, batch_len, cost / (double)n / ncases, 0, sm_count, false, kNoallocMaxPieces);
+    plan_pieces(a, n, batch_len, cost / (double)n / ncases, 0, sm_count, false, kNoallocMaxPieces, true);
     a.chunk_counter = &scratch->chunk_counter;
     a.claimed = scratch->claimed;
     a.handed = &scratch->handed;

@@ -1,5 +1,9 @@
 """Calls that earlier kernels or their host code answered wrongly, each against the oracle: counts
 exact, sums to the parity tests' tolerances."""
+import json
+import os
+import tempfile
+
 import numpy as np
 import pytest
 
@@ -79,3 +83,34 @@ def test_runs_of_one_handle_on_several_streams_follow_one_another(batch):
         assert g["sum_t"] == pytest.approx(o["sum_t"], rel=1e-12)
         np.testing.assert_allclose(g["flux"].sum(0), o["flux"].sum(0), rtol=1e-12)
     prob.close()
+
+
+def launches(call):
+    """(name, grid, block) of every kernel that `call` launches."""
+    from torch.profiler import ProfilerActivity, profile
+    for f in (lambda: torch.zeros(8, device="cuda").add_(1), call):  # the first session records nothing
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            f()
+            torch.cuda.synchronize()
+    with tempfile.TemporaryDirectory() as d:
+        path = os.path.join(d, "trace.json")
+        prof.export_chrome_trace(path)
+        with open(path) as f:
+            events = json.load(f)["traceEvents"]
+    out = [(e["name"], e["args"]["grid"], e["args"]["block"]) for e in events if e.get("cat") == "kernel"]
+    if not out:
+        pytest.skip("the profiler records no kernels here")
+    return out
+
+
+@pytest.mark.parametrize("params,batch", [((*workloads.BOX_L10[:8], 37), False), (workloads.batch_sweep(2, seed=1, nbins=21), True)])
+def test_autotuner_pilots_run_the_tracker(params, batch):
+    """A pilot small enough for the narrow walk still times the tracker's launch shapes.  (These FP64
+    boxes' histories are too short for a hand-over, so no other use of the narrow walk is expected.)"""
+    prob = cls.Problem(params, batch=batch)
+    names = [k for k, _, _ in launches(lambda: prob.autotune(2048 + 16 * batch, seed=12))]
+    if batch:
+        names += [k for k, _, _ in launches(lambda: prob.autotune_cases(2048, seed=12))]
+    prob.close()
+    assert any("history_kernel" in k for k in names) and any("event_kernel" in k for k in names)
+    assert not any("narrow_kernel" in k for k in names)
