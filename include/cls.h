@@ -70,7 +70,8 @@ extern "C" {
 #define CLS_OPT_SCHEDULE 2      /* CLS_SCHED_HISTORY (default), CLS_SCHED_EVENT, CLS_SCHED_AUTO */
 #define CLS_OPT_BLOCK 3         /* threads per block, multiple of 32 in [32, 256]; the FP64
                                    history tracker uses at most 128, the FP32 history tracker
-                                   for the 3D box at most 224 (their launch bounds)          */
+                                   for the 3D box at most 224 (their launch bounds); runs of
+                                   few histories, one to a warp, at most 128                 */
 #define CLS_OPT_CHUNK 4         /* histories a warp claims at once: 32, 64, ..., 1024.  The  */
                                 /* history tracker claims at most 32 times as many while a  */
                                 /* run is long, and fewer (down to 32, or to 1 in runs too   */
@@ -78,7 +79,8 @@ extern "C" {
                                 /* this many                                                */
 #define CLS_OPT_NBATCH 5        /* statistics batches per run, 2..1024 (default 64)         */
 #define CLS_OPT_MAX_EVENTS 6    /* per-history event cap, 1..2^28 (default 1e8)             */
-#define CLS_OPT_BLOCKS_PER_SM 7 /* persistent grid = SMs x this; 0 = occupancy maximum     */
+#define CLS_OPT_BLOCKS_PER_SM 7 /* persistent grid = SMs x this; 0 = occupancy maximum (runs  */
+                                /* of few histories, one to a warp: 384 threads, at most)    */
 #define CLS_OPT_BANK 8          /* event schedule: bank particles per warp, 0..4096, rounded  */
                                 /* up to a multiple of 32 (0 = 128)                         */
 #define CLS_OPT_EVENTS_PER_PASS 9 /* event schedule: events per particle per pass (1..64)  */

@@ -81,11 +81,11 @@ inline int hand_over_for(double events, bool fp32, int geom) {
 // of them; as many warps start on a piece as it takes to employ all; and the
 // least a warp claims is 32 histories, a warp's lanes, or where that would not
 // go round, a power of two below.  may_narrow: whether a run small enough goes to
-// the narrow walk.
+// the narrow walk, whose launch shape is `narrow`.
 inline void plan_pieces(LaunchArgs &a, uint64_t n, uint64_t batch_len, double mean_cost, int geom, int sm_count, bool fp32,
-                        uint64_t max_pieces, bool may_narrow) {
+                        uint64_t max_pieces, bool may_narrow, const NarrowShape &narrow) {
     const double total = (double)n * a.nruns;
-    const double narrow_warps = (double)sm_count * kNarrowBlocks * narrow_block_warps(!fp32, a.region_bytes);
+    const double narrow_warps = (double)sm_count * narrow.blocks * narrow.warps;
     a.narrow = may_narrow && total <= narrow_histories(fp32, geom) * narrow_warps;
     const double warps = a.narrow ? std::min(total, narrow_warps) : sm_count * (fp32 ? 28.0 : 20.0);
     const uint64_t used = (n + batch_len - 1) / batch_len;  // batches
@@ -100,13 +100,9 @@ inline void plan_pieces(LaunchArgs &a, uint64_t n, uint64_t batch_len, double me
 }
 
 // Blocks of the narrow walk: as many as the run has histories for its warps.
-inline int narrow_grid(const LaunchArgs &a, bool fp64, uint64_t n, int sm_count) {
-    const int full = sm_count * kNarrowBlocks, warps = narrow_block_warps(fp64, a.region_bytes);
-    return a.narrow ? (int)std::min((double)full, std::ceil((double)n * a.nruns / warps)) : full;
-}
-
-inline size_t narrow_smem(const LaunchArgs &a, bool fp64) {
-    return (size_t)narrow_block_warps(fp64, a.region_bytes) * (narrow_memory_bytes(fp64) + a.region_bytes);
+inline int narrow_grid(const LaunchArgs &a, const NarrowShape &narrow, uint64_t n, int sm_count) {
+    const int full = sm_count * narrow.blocks;
+    return a.narrow ? (int)std::min((double)full, std::ceil((double)n * a.nruns / narrow.warps)) : full;
 }
 
 // Claim limit and refill threshold of a run entry (RunCase), from the

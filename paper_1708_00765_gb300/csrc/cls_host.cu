@@ -386,6 +386,10 @@ int region_bytes_for(const cls_handle *h) {
     return region_bytes(h->opt.precision == CLS_PREC_FP64, h->nbins_stride);
 }
 
+NarrowShape narrow_shape_for(const cls_handle *h, int region) {
+    return narrow_shape(h->opt.precision == CLS_PREC_FP64, region, h->opt.block, h->opt.blocks_per_sm);
+}
+
 // FP32 regions are flushed into the FP64 global tallies after this many
 // histories, which keeps each bin's fixed-point sum far below its 2^31 range.
 constexpr int kFp32FlushHistories = 1024;
@@ -485,7 +489,8 @@ int prepare_run(cls_handle *h, uint64_t n, uint64_t seed, RunPlan *plan) {
         ag.claimed = h->d_chunk_counter + kGroupCounters + pieces;
         if (groups[g].sched != CLS_SCHED_EVENT) {
             plan_pieces(ag, n, batch_len_for(n, h->nbatch), groups[g].cost / groups[g].ncases, groups[g].geom, h->sm_count,
-                        h->opt.precision == CLS_PREC_FP32, kMaxPieces, !h->pilot);
+                        h->opt.precision == CLS_PREC_FP32, kMaxPieces, !h->pilot,
+                        narrow_shape_for(h, ag.region_bytes));
             pieces += (uint64_t)ag.pieces_per_run * ag.nruns;
         } else {
             ag.hand_over = hand_over_for(estimated_events(groups[g].cost / groups[g].ncases),
@@ -598,6 +603,7 @@ int plan_shapes(cls_handle *h, const RunPlan &plan, Shape *sh, size_t *bank, siz
     for (int g = 0; g < plan.ngroups; ++g) {
         const int rc = tracker_shape(h, plan.a[g].region_bytes, plan.sched[g], plan.geom[g], &sh[g]);
         if (rc) return rc;
+        if (plan.a[g].narrow) h->used_blocks_per_sm = narrow_shape_for(h, plan.a[g].region_bytes).blocks;
         if (plan.sched[g] == CLS_SCHED_EVENT) {
             sh[g].bank_off = *bank;
             *bank += (shape_bank_bytes(h, sh[g]) + 255) & ~(size_t)255;
@@ -736,9 +742,9 @@ int launch_tracker(cls_handle *h, LaunchArgs a, int sched, int geom, const Shape
                      : launch_history_fp32(a, sh.grid, sh.block, sh.smem, s, geom);
     }
     if (e != cudaSuccess || (!a.narrow && a.hand_over == 0)) return cuda_fail(e);
-    const int grid = narrow_grid(a, fp64, n, h->sm_count), block = 32 * narrow_block_warps(fp64, a.region_bytes);
-    const size_t smem = narrow_smem(a, fp64);
-    e = fp64 ? launch_narrow_fp64(a, grid, block, smem, s, geom) : launch_narrow_fp32(a, grid, block, smem, s, geom);
+    const NarrowShape narrow = narrow_shape_for(h, a.region_bytes);
+    const int grid = narrow_grid(a, narrow, n, h->sm_count), block = 32 * narrow.warps;
+    e = fp64 ? launch_narrow_fp64(a, grid, block, narrow.smem, s, geom) : launch_narrow_fp32(a, grid, block, narrow.smem, s, geom);
     return cuda_fail(e);
 }
 

@@ -182,10 +182,24 @@ __host__ __device__ constexpr int narrow_memory_bytes(bool fp64) { return (fp64 
 // Dynamic shared memory that a block may take (the opt-in the kernels are given).
 constexpr size_t kMaxSmemPerBlock = 200 * 1024;
 
-// Warps of a block of the narrow walk: fewer on the widest meshes.
-inline int narrow_block_warps(bool fp64, int region) {
-    const size_t fit = kMaxSmemPerBlock / ((size_t)narrow_memory_bytes(fp64) + region);
-    return fit < kNarrowBlock / 32 ? (int)fit : kNarrowBlock / 32;
+// The narrow walk's launch: warps of a block and blocks per SM.
+struct NarrowShape {
+    int warps, blocks;
+    size_t smem;
+};
+
+// At most as many threads per block and blocks per SM as the caller's options ask
+// for (block in threads; blocks_per_sm 0: kNarrowBlocks of kNarrowBlock threads, or
+// as many warps in smaller blocks), and fewer warps on the widest meshes.
+inline NarrowShape narrow_shape(bool fp64, int region, int block, int blocks_per_sm) {
+    const size_t warp = (size_t)narrow_memory_bytes(fp64) + region, fit = kMaxSmemPerBlock / warp;
+    const int most = block < kNarrowBlock ? block / 32 : kNarrowBlock / 32;
+    const int blocks = kNarrowBlocks * (kNarrowBlock / 32) / most;
+    NarrowShape s;
+    s.warps = fit < (size_t)most ? (int)fit : most;
+    s.blocks = blocks_per_sm > 0 && blocks_per_sm < blocks ? blocks_per_sm : blocks;
+    s.smem = s.warps * warp;
+    return s;
 }
 
 // Dynamic shared memory of a warp of the history tracker: two tally regions and

@@ -132,7 +132,8 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
         cost += img.cases[k].cost * (double)n;
     }
     a.region_bytes = region_bytes(true, nbins_stride);
-    plan_pieces(a, n, batch_len, cost / (double)n / ncases, 0, sm_count, false, kNoallocMaxPieces, true);
+    const NarrowShape narrow = narrow_shape(true, a.region_bytes, kNarrowBlock, 0);
+    plan_pieces(a, n, batch_len, cost / (double)n / ncases, 0, sm_count, false, kNoallocMaxPieces, true, narrow);
     a.chunk_counter = &scratch->chunk_counter;
     a.claimed = scratch->claimed;
     a.handed = &scratch->handed;
@@ -170,8 +171,6 @@ extern "C" int cls_run_noalloc(const double *params, int ncases, uint64_t first,
     if (!a.narrow) history_kernel<double, 0><<<sm_count * bps, block, smem, s>>>(a);
     if (cudaGetLastError() != cudaSuccess) return CLS_E_CUDA;
     if (!a.narrow && a.hand_over == 0) return CLS_OK;
-    const int narrow_block = 32 * narrow_block_warps(true, a.region_bytes);
-    return launch_narrow_fp64(a, narrow_grid(a, true, n, sm_count), narrow_block, narrow_smem(a, true), s, 0) == cudaSuccess
-               ? CLS_OK
-               : CLS_E_CUDA;
+    const int grid = narrow_grid(a, narrow, n, sm_count);
+    return launch_narrow_fp64(a, grid, 32 * narrow.warps, narrow.smem, s, 0) == cudaSuccess ? CLS_OK : CLS_E_CUDA;
 }

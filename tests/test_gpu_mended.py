@@ -114,3 +114,32 @@ def test_autotuner_pilots_run_the_tracker(params, batch):
     prob.close()
     assert any("history_kernel" in k for k in names) and any("event_kernel" in k for k in names)
     assert not any("narrow_kernel" in k for k in names)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_small_runs_keep_to_the_callers_launch_shape(precision):
+    """The narrow walk takes no more blocks per SM and threads per block than asked for, says what it took,
+    and walks the same histories."""
+    p, n = (*workloads.ROD_L10[:8], 29), 900
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    prob = cls.Problem(p)
+    prob.set_option("precision", precision)
+    prob.run(n, 4)
+    assert prob.get_option("blocks_per_sm") == 3  # of 128 threads
+    prob.set_option("blocks_per_sm", 1)
+    prob.set_option("block", 64)
+    kernels = [k for k in launches(lambda: prob.run(n, 4)) if "narrow_kernel" in k[0]]
+    assert len(kernels) == 1 and kernels[0][1][0] <= sms and kernels[0][2][0] <= 64, kernels
+    assert prob.get_option("blocks_per_sm") == 1
+    prob.set_option("blocks_per_sm", 0)
+    prob.set_option("block", 32)
+    prob.run(n, 4)
+    assert prob.get_option("blocks_per_sm") == 12
+    g = prob.raw_tallies()
+    prob.close()
+    assert g["n_histories"] == 3 * n
+    if precision == "fp64":
+        o = oracle.run(ocase(p), 4, 0, 3 * n)
+        for k, ko in COUNTS.items():
+            assert g[k] == o[ko], k
+        np.testing.assert_allclose(g["flux"].sum(0), o["flux"].sum(0), rtol=1e-12)
