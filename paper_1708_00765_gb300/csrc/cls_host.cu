@@ -161,6 +161,11 @@ struct cls_handle {
     // event-schedule bank
     void *d_bank = nullptr;
     size_t bank_bytes = 0;
+    // slots for the histories that the trackers hand over (in a bound workspace:
+    // behind the event bank), and outgrown ones that launches may still use
+    unsigned char *d_stragglers = nullptr;
+    size_t stragglers_bytes = 0;
+    std::vector<void *> old_stragglers;
     // caller-owned device workspace (cls_bind_workspace) holding every device
     // buffer above, or null: the library's own allocations
     unsigned char *ws = nullptr;
@@ -247,12 +252,17 @@ void free_device(cls_handle *h) {
         cudaFree(h->d_runs);
         cudaFree(h->d_chunk_counter);
         cudaFree(h->d_bank);
+        cudaFree(h->d_stragglers);
+        for (void *p : h->old_stragglers) cudaFree(p);
     }
+    h->old_stragglers.clear();
     h->d_cases = nullptr;
     h->d_runs = nullptr;
     h->d_chunk_counter = nullptr;
     h->d_bank = nullptr;
     h->bank_bytes = 0;
+    h->d_stragglers = nullptr;
+    h->stragglers_bytes = 0;
 }
 
 // Byte offsets of the device buffers in a caller's workspace, each 256-byte
@@ -546,8 +556,8 @@ struct Shape {
     size_t smem;
     uint32_t bank_slots;  // event schedule: slots per block and buffer
     size_t bank_off;      // event schedule: its particles' slice of the bank
-    size_t straggler_off;    // the hand-over buffer's slice
-    uint32_t straggler_cap;  // and its slots
+    unsigned char *stragglers;  // its hand-over slots
+    uint32_t straggler_cap;
 };
 
 size_t shape_bank_bytes(const cls_handle *h, const Shape &sh) {
@@ -587,18 +597,18 @@ int tracker_shape(cls_handle *h, int region_bytes, int sched, int geom, Shape *o
     out->smem = smem;
     out->bank_slots = event ? (uint32_t)(h->opt.bank > 0 ? ((h->opt.bank + 31) & ~31) : 128) : 0u;
     out->bank_off = 0;
-    out->straggler_off = 0;
-    out->straggler_cap = (uint32_t)(out->grid * (block / 32) * kHandOver);
+    out->stragglers = nullptr;
+    out->straggler_cap = (uint32_t)(out->grid * (block / 32));  // one history a warp
     return CLS_OK;
 }
 
-// Shapes of a run's launches, which take consecutive slices of one bank (all of
-// a run's launches may run at once): the event launches grid warps x 2 buffers x
-// slots x fields x 16 B each, and every launch, after them, its hand-over
-// buffer, if it hands histories over at all.  *bank: the bytes they need
-// together; a hand-over buffer is cut where it would end beyond `limit` (the
-// tracker walks what it cannot hand over).
-int plan_shapes(cls_handle *h, const RunPlan &plan, Shape *sh, size_t *bank, size_t limit = ~(size_t)0) {
+// Shapes of a run's launches, which take consecutive slices of the event bank and
+// of the hand-over slots (all of a run's launches may run at once): the event
+// launches grid warps x 2 buffers x slots x fields x 16 B each, *bank bytes
+// together, and every launch that hands histories over its slots, cut where they
+// run out (the tracker walks what it cannot hand over).  *want: the bytes of all
+// slots uncut.
+int plan_shapes(cls_handle *h, const RunPlan &plan, Shape *sh, size_t *bank, size_t *want = nullptr) {
     *bank = 0;
     for (int g = 0; g < plan.ngroups; ++g) {
         const int rc = tracker_shape(h, plan.a[g].region_bytes, plan.sched[g], plan.geom[g], &sh[g]);
@@ -609,18 +619,25 @@ int plan_shapes(cls_handle *h, const RunPlan &plan, Shape *sh, size_t *bank, siz
             *bank += (shape_bank_bytes(h, sh[g]) + 255) & ~(size_t)255;
         }
     }
+    unsigned char *slots = h->d_stragglers;
+    size_t room = h->stragglers_bytes;
+    if (h->ws) {
+        const size_t left = h->ws_bytes - h->ws_bank_off;
+        slots = h->ws + h->ws_bank_off + *bank;
+        room = left > *bank ? left - *bank : 0;
+    }
+    if (want) *want = 0;
     for (int g = 0; g < plan.ngroups; ++g) {
-        sh[g].straggler_off = *bank;
-        const size_t room = *bank < (limit & ~(size_t)255) ? ((limit & ~(size_t)255) - *bank) / kStragglerBytes : 0;
-        sh[g].straggler_cap = (uint32_t)std::min<size_t>(sh[g].straggler_cap, room);
-        if (plan.a[g].narrow || plan.a[g].hand_over == 0) sh[g].straggler_cap = 0;
-        *bank += ((size_t)sh[g].straggler_cap * kStragglerBytes + 255) & ~(size_t)255;
+        sh[g].straggler_cap *= plan.a[g].narrow ? 0 : plan.a[g].hand_over;
+        if (want) *want += ((size_t)sh[g].straggler_cap * kStragglerBytes + 255) & ~(size_t)255;
+        sh[g].straggler_cap = (uint32_t)std::min<size_t>(sh[g].straggler_cap, room / kStragglerBytes);
+        sh[g].stragglers = slots;
+        const size_t taken = std::min(((size_t)sh[g].straggler_cap * kStragglerBytes + 255) & ~(size_t)255, room);
+        slots += taken;
+        room -= taken;
     }
     return CLS_OK;
 }
-
-// Bytes of the bank that runs may use: a bound workspace's beyond its other buffers.
-size_t bank_limit(const cls_handle *h) { return h->ws ? h->ws_bytes - h->ws_bank_off : ~(size_t)0; }
 
 // Make sure the particle bank holds `need` bytes.  Done before any graph capture.
 int ensure_bank(cls_handle *h, size_t need) {
@@ -648,30 +665,48 @@ int ensure_bank(cls_handle *h, size_t need) {
     return CLS_OK;
 }
 
-// Shapes of a run's launches, and the bank they need.  The hand-over buffers
-// are a help, not a need: where memory is short, or the stream is being captured
-// and nothing can be allocated, they are cut to what there is.
-int plan_bank(cls_handle *h, const RunPlan &plan, Shape *sh, cudaStream_t s) {
-    size_t bank = 0;
-    int rc = plan_shapes(h, plan, sh, &bank, bank_limit(h));
-    if (rc) return rc;
-    if (!h->ws && bank > h->bank_bytes) {
-        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess) cudaGetLastError();
-        if (capturing != cudaStreamCaptureStatusNone) {
-            rc = plan_shapes(h, plan, sh, &bank, h->bank_bytes);
-            if (rc) return rc;
+// Hand-over slots for runs that ask for `want` bytes of them: at least those of
+// every warp that fits an SM, for either precision, so that options seldom outgrow
+// them.  Taken by the first run that hands histories over (short runs never do, and
+// 1.4 MB at the handle's creation made that 70 -> 200 us), without waiting for the
+// device: outgrown slots stay until the handle has no runs in flight.
+// They are a help and no need: where memory is short, or the stream is being captured
+// and nothing can be allocated, the trackers walk what they cannot hand over.
+void reserve_stragglers(cls_handle *h, size_t want, cudaStream_t s) {
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess) cudaGetLastError();
+    if (capturing != cudaStreamCaptureStatusNone) return;
+    size_t bytes[2] = {0, 0};
+    for (const Group &g : plan_groups(h, nullptr))
+        for (int fp32 = 0; fp32 < 2; ++fp32) {
+            const size_t warps = (size_t)h->sm_count * (fp32 ? 32 : 25);
+            const size_t slots = warps * hand_over_for(estimated_events(g.cost / g.ncases), fp32, g.geom);
+            bytes[fp32] += (slots * kStragglerBytes + 255) & ~(size_t)255;
         }
+    want = std::max(want, std::max(bytes[0], bytes[1]));
+    void *p = nullptr;
+    if (cudaMalloc(&p, want) != cudaSuccess) {
+        cudaGetLastError();
+        return;
     }
-    rc = ensure_bank(h, bank);
-    if (rc == CLS_E_NOMEM) {
-        rc = plan_shapes(h, plan, sh, &bank, 0);
-        if (!rc) rc = ensure_bank(h, bank);
-    }
-    return rc;
+    if (h->d_stragglers) h->old_stragglers.push_back(h->d_stragglers);
+    h->d_stragglers = static_cast<unsigned char *>(p);
+    h->stragglers_bytes = want;
 }
 
-// Bytes of bank the handle's current options need (plan_shapes; for an
+// Shapes of a run's launches, and the event bank and hand-over slots they need.
+int plan_bank(cls_handle *h, const RunPlan &plan, Shape *sh, cudaStream_t s) {
+    size_t bank = 0, want = 0;
+    int rc = plan_shapes(h, plan, sh, &bank, &want);
+    if (!rc && !h->ws && want > h->stragglers_bytes) {
+        reserve_stragglers(h, want, s);
+        rc = plan_shapes(h, plan, sh, &bank);
+    }
+    return rc ? rc : ensure_bank(h, bank);
+}
+
+// Bytes of event bank and hand-over slots that the handle's current options need
+// in a workspace (plan_shapes; for an
 // automatic schedule the largest of the autotuner's event candidates, every
 // group on the event schedule).
 int bank_need(cls_handle *h, size_t *need) {
@@ -694,11 +729,11 @@ int bank_need(cls_handle *h, size_t *need) {
             plan.a[g].hand_over = kHandOver;
         }
         Shape sh[kMaxGroups];
-        size_t bank = 0;
-        rc = plan_shapes(h, plan, sh, &bank);
+        size_t bank = 0, slots = 0;
+        rc = plan_shapes(h, plan, sh, &bank, &slots);
         h->opt = saved;
         if (rc) break;
-        *need = std::max(*need, bank);
+        *need = std::max(*need, bank + slots);
     }
     h->opt = saved;
     h->used_blocks_per_sm = saved_bps;
@@ -727,7 +762,7 @@ int carve_workspace(cls_handle *h, size_t bank) {
 int launch_tracker(cls_handle *h, LaunchArgs a, int sched, int geom, const Shape &sh, uint64_t n, cudaStream_t s) {
     cudaError_t e;
     const bool fp64 = h->opt.precision == CLS_PREC_FP64;
-    a.stragglers = static_cast<unsigned char *>(h->d_bank) + sh.straggler_off;
+    a.stragglers = sh.stragglers;
     a.straggler_cap = sh.straggler_cap;
     if (sched == CLS_SCHED_EVENT) {
         a.bank = static_cast<unsigned char *>(h->d_bank) + sh.bank_off;
@@ -1450,6 +1485,11 @@ int cls_reset(cls_handle *h) {
     if (!h) return CLS_E_INVAL;
     CLS_CUDA(cudaSetDevice(h->device));
     if (h->last_stream || h->ran) CLS_CUDA(cudaDeviceSynchronize());
+    if (!h->old_stragglers.empty()) {
+        destroy_graph(h);
+        for (void *p : h->old_stragglers) cudaFree(p);
+        h->old_stragglers.clear();
+    }
     return zero_tallies(h);
 }
 

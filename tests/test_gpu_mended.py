@@ -143,3 +143,43 @@ def test_small_runs_keep_to_the_callers_launch_shape(precision):
         for k, ko in COUNTS.items():
             assert g[k] == o[ko], k
         np.testing.assert_allclose(g["flux"].sum(0), o["flux"].sum(0), rtol=1e-12)
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_history_runs_wait_for_nothing_on_the_device(batch):
+    """Runs that take their hand-over slots, and runs that outgrow them, return while the device is busy with
+    other work."""
+    params = np.array([workloads.ROD_L10[:8] + (20,)] * 3)
+    prob, warm = (cls.Problem(params if batch else params[0], batch=batch) for _ in range(2))
+    side, seeds, n = torch.cuda.Stream(), (3, 4, 5), 60_000
+
+    def three(p, stream):
+        p.set_option("blocks_per_sm", 1)
+        p.run(n, seeds[0], stream)
+        p.set_option("blocks_per_sm", 32)  # more warps, more slots
+        p.run(n, seeds[1], stream)
+        p.set_option("precision", "fp32")
+        p.set_option("precision", "fp64")
+        p.run(n, seeds[2], stream)
+
+    own = torch.cuda.Stream()
+    three(warm, own)  # kernels, streams and graphs are loaded and made at their first use
+    torch.cuda.synchronize()
+    done = torch.cuda.Event()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(2_000_000_000)  # about a second
+        done.record()
+    three(prob, own)
+    assert not done.query()
+    torch.cuda.synchronize()
+    for k in range(3 if batch else 1):
+        g = prob.raw_tallies(k)
+        parts = [oracle.run(ocase(params[k]), s, i * n, n, case_id=k) for i, s in enumerate(seeds)]
+        for key, ko in COUNTS.items():
+            assert g[key] == (max if key == "max_events" else sum)(o[ko] for o in parts), key
+        assert g["sum_t"] == pytest.approx(sum(o["sum_t"] for o in parts), rel=1e-12)
+    prob.reset()
+    prob.run(n, seeds[1], own)
+    assert prob.raw_tallies()["nR"] == oracle.run(ocase(params[0]), seeds[1], 0, n)["nR"]
+    prob.close()
+    warm.close()
