@@ -183,3 +183,23 @@ def test_history_runs_wait_for_nothing_on_the_device(batch):
     assert prob.raw_tallies()["nR"] == oracle.run(ocase(params[0]), seeds[1], 0, n)["nR"]
     prob.close()
     warm.close()
+
+
+def test_a_replayed_graph_starts_from_fresh_counters_and_slots():
+    """The second launch of one captured graph (the same size twice), for the tracker with hand-over and for
+    the narrow walk: work counters, claimed pieces and hand-over slots are used again."""
+    diffusive = (1.0, 10.0, 0.5, 0.2, 0.999, 0.999, 8.0, 3, 60)
+    params = np.array([workloads.ROD_L10[:8] + (30,), diffusive, workloads.ROD_L10[:8] + (60,), diffusive])
+    sizes = [14_000, 14_000, 600, 600, 14_000]
+    prob = cls.Problem(params, batch=True)
+    for n in sizes:
+        prob.run(n, 9)
+    for k in range(params.shape[0]):
+        g = prob.raw_tallies(k)
+        o = oracle.run(ocase(params[k]), 9, 0, sum(sizes), case_id=k)
+        for key, ko in COUNTS.items():
+            assert g[key] == o[ko], (k, key)
+        for key in ("sum_t", "sum_t2"):
+            assert g[key] == pytest.approx(o[key], rel=1e-12), (k, key)
+        np.testing.assert_allclose(g["flux"].sum(0)[: int(params[k, 8])], o["flux"].sum(0), rtol=1e-12)
+    prob.close()
