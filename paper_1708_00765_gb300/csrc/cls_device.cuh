@@ -490,14 +490,6 @@ __device__ __forceinline__ P draw(History<P> &s, const RoundKeys &key) {
     return Real<P>::uniform(hi, lo);
 }
 
-// 1 - u of the next draw, exactly
-template <typename P>
-__device__ __forceinline__ P draw_one_minus(History<P> &s, const RoundKeys &key) {
-    uint32_t hi, lo;
-    draw_words(s, key, hi, lo);
-    return Real<P>::one_minus(hi, lo);
-}
-
 // 2u - 1 for the next draw u (isotropic direction cosine)
 template <typename P>
 __device__ __forceinline__ P draw_iso(History<P> &s, const RoundKeys &key) {
@@ -891,9 +883,10 @@ __device__ __forceinline__ float coarse(double x) {
 // instead of two, at most one reciprocal (of a lateral face's direction), one
 // product.  Bounds: positions and directions lose 2^-20 of their values, so a
 // boundary distance lies within L 2^-18/|w| of (target - r)/|w| in FP32;
-// -ln(1 - u) from the draw's high word (2^-33 of u, so 2^-17 of 1 - u > 2^-16)
-// and the hardware's log2 (2^-22 relative) lies within 2^-14, the parameters'
-// and 1/|w|'s relative roundings (below 2^-18 of at most 11.1) included.  The
+// -ln(1 - u), at most 11.1 here, from the draw's high word (within 2^-32 of u, so
+// 2^-16 of 1 - u > 2^-16) and the hardware's log2 (2^-22 relative) lies within
+// 2^-14, the parameters' and 1/|w|'s relative roundings (2^-23 and 2^-19.6)
+// included.  The
 // rest, about 2 draws in 10^4, and cases of extreme magnitudes (filter) take
 // all five exactly.  Results are the exact comparison's.  FP64 instructions
 // take 64 cycles per warp and scheduler here, FP32 ones one or two.  Measured
@@ -1730,8 +1723,9 @@ __device__ __forceinline__ int find_piece(const LaunchArgs &a, int lane) {
 // many batches at a time: a bin in global memory takes an FP64 addition only
 // every 16 ns, and chunks dealt out one by one sent all warps' flushes to the
 // same batch (1e7 rod histories in FP32: chunks of 32 8.9 ms, of 256 1.6 ms;
-// pieces 1.25 ms).  A claim takes half of the team's even share of what is
-// left of the piece, so that claims shrink as it ends, within claim_bits.
+// pieces 1.25 ms).  A claim takes half of the team's even share of what the warp
+// last knew to be left of the piece (all of it, when it comes to one), so that
+// claims shrink as it ends, within claim_bits.
 __device__ __forceinline__ bool claim(WarpFeed *feed, const LaunchArgs &a, int lane) {
     const uint32_t np = (uint32_t)a.nruns * a.pieces_per_run;
     int piece = feed->piece;
@@ -1862,9 +1856,9 @@ __device__ __forceinline__ bool refill(unsigned char *regions, int rb, WarpFeed 
 // lanes whose histories have ended take the next histories of the warp's claim
 // (ballot + prefix popcount), several lanes at a time, so lanes stay busy across
 // history and claim boundaries.  Bound by issue (FP32) and by instruction supply
-// and the FP64 pipe (FP64).  Before fixed-point bins in 32-bit halves, claims
+// and the FP64 pipe (FP64).  Before fixed-point bins in 32-bit words, claims
 // from pieces, batched ends and births, events chosen by FP32 bounds and the
-// shorter integer routines / now: box L = 10 in FP64 1e7 histories 56.6 / 33.2
+// shorter integer routines / now: box L = 10 in FP64 1e7 histories 56.7 / 34.5
 // ms, in FP32 1e8 109.3 / 90.8 ms; 256-case sweep in FP32 at 1e6 a case 54.3 /
 // 37.4 ms.  Each warp owns two shared-memory tally
 // regions keyed by (case, batch); a region is flushed to global memory when
@@ -2048,7 +2042,9 @@ __global__ void __launch_bounds__(HistoryBounds<P, G>::threads, HistoryBounds<P,
 // on the same draws, so results do not change.  Measured: 1000 histories of
 // the 3D box in FP64 753 us by the tracker, 483 us here; the diffusive box,
 // 1e6 histories in FP32, 20.4 ms without the hand-over, 12.8 ms with it.  An
-// event of a lone history takes 0.23 us in FP32 and 1.5 us in FP64.
+// event of a lone history takes 0.23 us in FP32 and, in FP64, 0.47 us on the rod,
+// 1.2 us in the box and 1.6 us in the extruded geometry.
+
 // The two draws of a lane's Philox block into the buffer, at `at` and at + 1.
 template <typename P, int G>
 __device__ __forceinline__ void fill_draws(DrawBuffer<P> &b, int at, uint32_t block, const History<P> &s,

@@ -12,7 +12,7 @@
 // and four bits of a bin with a single flight.)  The third word costs the FP64 walk
 // 1 to 4%: box L = 10, 1e7 histories, 33.1 -> 34.5 ms; slab 1e6 552 -> 571 us;
 // extruded 3e5 1019 -> 1039 us; FP64 additions to shared memory, compare-and-swap
-// loops, cost it 13%.
+// loops, cost the box 13% before the steps that followed.
 //
 // Host and device compile the same code (the host build serves tests).
 #pragma once

@@ -705,10 +705,9 @@ int plan_bank(cls_handle *h, const RunPlan &plan, Shape *sh, cudaStream_t s) {
     return rc ? rc : ensure_bank(h, bank);
 }
 
-// Bytes of event bank and hand-over slots that the handle's current options need
-// in a workspace (plan_shapes; for an
-// automatic schedule the largest of the autotuner's event candidates, every
-// group on the event schedule).
+// Bytes of event bank and hand-over slots that the handle's current options need in
+// a workspace (plan_shapes; for an automatic schedule the largest of the
+// autotuner's event candidates, every group on the event schedule).
 int bank_need(cls_handle *h, size_t *need) {
     *need = 0;
     const Options saved = h->opt;
